@@ -106,7 +106,11 @@ SA_D BlockPlan plan_block(PlanArgs a, int z, int x, bool recheck, bool counts, B
         }
     }
     if (j < B) len_s[j] = len_now;
-    if (j == 0) out_s[0] = -1;
+    if (j == 0) {
+        out_s[0] = -1;              // a block beyond the last pair keeps these: split 0 of 1 of no sequence
+        out_s[1] = 0;
+        out_s[2] = 1;
+    }
     const int cap = a.max_pages * kPageTokens;
     const int tiles = (j < B) ? (min(max(len_now + (a.Knew ? 1 : 0), 0), cap) + 31) >> 5 : 0;
     __syncthreads();
