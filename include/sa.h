@@ -84,21 +84,15 @@ enum { SA_POT4 = 0, SA_POTM1 = 1, SA_POTM2 = 2, SA_POTM4 = 4, SA_INT8 = 8, SA_KV
 enum { SA_KLAYOUT_BYTE = 0, SA_KLAYOUT_NIBBLE = 1, SA_KLAYOUT_PLANAR = 2 };
 /* flags */
 #define SA_FLAG_HADAMARD 1u /* rotate Q and K by the normalised Walsh-Hadamard matrix before quantising */
-/* Decode kernels only, mantissa codes (PoT-M1 / M2 / M4) only, off by default: execute the left shift of
- * eq. (3), (4) on the integer multiplier.  Each key element is decoded once, for the whole query group, to
- * sigma * 2^(F - k - e) (0 for the zero code) and every (query, element) update is one integer multiply-add
- * by that power of two instead of a shift followed by the sign multiply-add.  The INT32 scores are the same
- * bit for bit.  This uses the multiplier array as a barrel shifter, so it is not the paper's multiplier-free
- * datapath; it is the mid-point between the shift kernels and the INT8 multiply-accumulate comparison
- * (section III), and is reported as such.  (PoT-4 has no shift left in its key loop: SA_ERR_UNSUPPORTED.) */
+/* Decode kernels only, mantissa codes (PoT-M1 / M2 / M4) only: the caller asks for scores formed on multipliers.  The
+ * default kernels do that already (each key element is decoded once, for the whole query group, and the scores are
+ * exact matrix products), so the flag selects the same kernels; it is kept for programs that set it.  (PoT-4:
+ * SA_ERR_UNSUPPORTED.) */
 #define SA_FLAG_SHIFT_BY_MULTIPLY 2u
-/* Decode kernels only, power-of-two codes only, off by default: every sign flip and add of the integer score
- * (eq. (3)) is issued as logic and add instructions (exclusive-or with the sign mask, subtract, add) instead
- * of one multiply-add by +1 / -1, so that no instruction of the score datapath touches the multiplier array.
- * The INT32 scores are the same bit for bit.  It is the strictly multiplier-free form of the default kernels
- * and is slower than them on this GPU, whose shift/logic/add pipe is the busier one; it exists to be measured
- * beside the default, SA_FLAG_SHIFT_BY_MULTIPLY and the INT8 multiply-accumulate comparison.  Excludes
- * SA_FLAG_SHIFT_BY_MULTIPLY. */
+/* Decode kernels only, power-of-two codes only, off by default: the paper's multiplier-free datapath.  Every shift, sign
+ * flip and add of the integer score (eq. (3)) is a shift, logic or add instruction on the CUDA cores; no instruction of
+ * the score datapath touches a multiplier or a tensor core.  The INT32 scores are the same bit for bit.  It is 2 - 5
+ * times slower than the default on this GPU and exists to be measured beside it.  Excludes SA_FLAG_SHIFT_BY_MULTIPLY. */
 #define SA_FLAG_ADD_ON_ALU 4u
 
 typedef struct {
@@ -182,17 +176,18 @@ sa_status sa_fill_kv(const sa_config* cfg, const sa_cache* cache, const uint16_t
 /* Decode attention over the quantised cache — the hot path (section II-B eq. (3), II-C eq. (4),
  * II-D eq. (5), II-E, II-F):
  *   Q is quantised (and rotated, if flagged) inside the kernel; for every cached key the integer
- *   score A = sum_m sigma * qhat * (2^k + j) << (F - k - e) is formed exactly in INT32 with
- *   shifts, sign flips and adds; logits z = A * Delta * s * 2^-F * log2(e) / sqrt(d) feed an
- *   online softmax whose running maximum is an integer in the log2 domain, so that every
- *   rescale is an exact power of two; O accumulates p * vhat * 2^-g (the paper's floating-point
- *   A.V); the key axis is split over thread blocks and the partial (M, l, O) triples are merged
- *   with exact power-of-two factors.
- *   The A.V products run on the tensor cores as tf32 x tf32 with FP32 accumulation (mma.m16n8k8): the INT8
- *   values are exact in tf32, and every weight p * 2^-g enters as the sum of two tf32 terms (its leading
- *   11 significant bits, and the remainder cut to 11 bits), so that a weight keeps about 21 significant
- *   bits: the relative error of one product is below 2^-21, against 2^-24 for an FP32 multiply; measured
- *   max |dO| against the CPU oracle is 2e-8 .. 6e-7.  The integer scores never touch the tensor cores.
+ *   score A = sum_m sigma * qhat * (2^k + j) << (F - k - e) is formed exactly (INT32); logits
+ *   z = A * Delta * s * 2^-F * log2(e) / sqrt(d) feed an online softmax whose running reference is an
+ *   integer in the log2 domain, so that every rescale is an exact power of two; O accumulates
+ *   p * vhat * 2^-g (the paper's floating-point A.V); the key axis is split over thread blocks and the
+ *   partial (M, l, O) triples are merged with exact power-of-two factors.
+ *   The scores are matrix products on the tensor cores, over the whole query group of a KV head: a decoded
+ *   key element is a 5-bit magnitude times a power of two, the queries are 8-bit integers, and binary16
+ *   operands with FP32 sums below 2^24 units (or INT8 operands with INT32 sums) give the integer of eq. (3)
+ *   without rounding.  SA_FLAG_ADD_ON_ALU forms the same integers by shifts and adds alone.
+ *   The A.V products run on the tensor cores with FP32 accumulation: the INT8 values are exact in binary16,
+ *   and every weight enters as the sum of two binary16 terms (22 significant bits down to 2^-17 of the
+ *   largest weight, an absolute 2^-38 of it below that); measured |dO| against the CPU oracle: 1e-6 relative.
  * Q [batch, n_q_heads, head_dim] binary16; O [batch, n_q_heads, head_dim] float.
  * A sequence with seq_lens[b] == 0 yields zeros.
  * dbg_scores (nullable): int32 [batch, n_q_heads, max_pages_per_seq * 64]; receives A for every

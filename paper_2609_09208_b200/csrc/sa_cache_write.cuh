@@ -16,6 +16,7 @@ struct CacheArgs {
     int batch, max_pages, n_pages, Hkv;
     size_t page_bytes, kcode_off, meta_off, v_off, plane_off;
     int hadamard;
+    int k;                    // mantissa bits (MODE 7 of write_token only)
 };
 
 template <int D, int K, bool NIB>
@@ -30,7 +31,7 @@ SA_D void write_token_quant(uint8_t* block, const CacheArgs& a, int t, int lane,
     if constexpr (K == 8) {
         smax = encode_key_int8_vec<EPL>(kb, lane, a.hadamard != 0, kc);      // uniform INT8: stored as is
     } else {
-        smax = encode_key_vec<EPL, K>(kb, lane, a.hadamard != 0, kc);
+        smax = encode_key_vec<EPL, K>(kb, lane, a.hadamard != 0, kc, a.k);
         // byte container: the physical byte (phys_byte); the sub-byte containers below work on the canonical
         // byte with its exponent field replaced by g = 7 - e (0 for the zero code), i.e. canonical ^ 0x70
 #pragma unroll
@@ -106,12 +107,13 @@ SA_D uint8_t* page_block(const CacheArgs& a, int b, int lp, int h) {
     return a.pages + ((size_t)pidx * a.Hkv + h) * a.page_bytes;
 }
 
-// MODE: 0..4 = power-of-two code with K mantissa bits (byte container), 8 = PoT-4 nibble, 9 / 10 = PoT-M1 /
+// MODE: 0..4 = power-of-two code with K mantissa bits (byte container), 7 = the same with a.k of them, 8 = PoT-4 nibble, 9 / 10 = PoT-M1 /
 // PoT-M2 in the dense planar container, 16 = FP16, 32 = uniform INT8 comparison code
 template <int D, int MODE>
 SA_D void write_token(uint8_t* block, const CacheArgs& a, int t, int lane, const uint16_t* krow,
                       const uint16_t* vrow) {
-    if constexpr (MODE == 16) write_token_fp16<D>(block, a, t, lane, krow, vrow);
+    if constexpr (MODE == 7) write_token_quant<D, -1, false>(block, a, t, lane, krow, vrow);
+    else if constexpr (MODE == 16) write_token_fp16<D>(block, a, t, lane, krow, vrow);
     else if constexpr (MODE == 8) write_token_quant<D, 0, true>(block, a, t, lane, krow, vrow);
     else if constexpr (MODE == 9) write_token_quant<D, 1, true>(block, a, t, lane, krow, vrow);
     else if constexpr (MODE == 10) write_token_quant<D, 2, true>(block, a, t, lane, krow, vrow);

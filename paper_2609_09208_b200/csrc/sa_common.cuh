@@ -26,6 +26,26 @@ constexpr int kNumSMsB200 = 148;          // the split plan's SM count where no 
 constexpr int kEmax = 6;                  // largest exponent of the 3-bit field
 constexpr int kMNone = -(1 << 29);        // running-maximum value meaning "no key seen yet"
 
+// Warps per block, resident blocks per SM and stage buffers per warp of a decode kernel (the kernels' launch bounds and
+// shared-memory plans are sized for exactly this, and the split plan counts on it).
+struct KernelShape {
+    int warps, blocks_per_sm, stages;
+};
+// Matrix kernels (sa_decode_mma.cuh).  kb: mantissa bits, 8 for INT8.
+constexpr KernelShape mma_shape(int d, int kb) {
+    return d == 128 ? KernelShape{6, 2, 2} : (kb == 1 || kb == 2) ? KernelShape{4, 4, 2} : KernelShape{8, 2, 2};
+}
+// Shift-and-add kernels (sa_decode_kernel.cuh): one stage buffer per warp where a second one would cost resident warps
+// (d = 128, where a tile is 8 KB, and PoT-M4 with its 32 KB table of query multiples).
+constexpr KernelShape shift_shape(int d, int kb) {
+    const int ns = (d == 128 || kb == 4) ? 1 : 2;
+    return (kb == 1 || kb == 2) ? KernelShape{4, 4, ns}
+           : (d == 64)          ? KernelShape{10, 2, ns}
+           : (kb == 4)          ? KernelShape{8, 2, ns}
+                                : KernelShape{4, 5, ns};
+}
+constexpr KernelShape kFp16Shape{4, 3, 2};
+
 // ---------------------------------------------------------------------------------------------
 // Host-side description of a validated configuration.
 // ---------------------------------------------------------------------------------------------
@@ -39,30 +59,10 @@ struct Plan {
     int f_extra;              // F - (6 + k): applied as one final left shift of the INT32 sum
     sa_layout lay;
     size_t plane_off;         // dense planar container: offset of the mantissa bit planes inside a block
+    KernelShape shape;        // of the decode kernel that serves this configuration
 };
 
 sa_status make_plan(const sa_config* cfg, Plan* out);
-// Warps per block and resident blocks per SM of the decode kernel that serves a code
-// (kb: 0 PoT-4, 1 / 2 / 4 mantissa codes, 8 INT8; the kernels' launch bounds and shared-memory
-// plans are sized for exactly this, and the split plan counts on it).  At d = 64 two blocks of ten
-// warps (20 warps at 96 registers): for PoT-M4 the ten warps share one 32 KB table of query
-// multiples, and for every code fewer, larger blocks mean fewer prologues and partials, which is
-// most of the time of a batch-1 step.  PoT-M1 / M2 keep four blocks of four warps: their finer
-// granularity serves the short and ragged batches those codes are specified for (measured: 16 %
-// faster there, 6 % slower at T = 32768, batch 1).  At d = 128 (8 KB tiles, one stage buffer per
-// warp) PoT-M4 runs two blocks of eight warps beside their 32 KB tables (16 warps at 128 registers;
-// measured 3 - 22 % faster than three blocks of four); the other codes keep blocks of four warps
-// (larger blocks measured 2 - 13 % slower for them from batch 8 on).
-struct KernelShape {
-    int warps, blocks_per_sm;
-};
-constexpr KernelShape decode_shape(int d, int kb) {
-    return (kb == 1 || kb == 2) ? KernelShape{4, 4}
-           : (d == 64)          ? KernelShape{10, 2}
-           : (kb == 4)          ? KernelShape{8, 2}
-                                : KernelShape{4, 5};
-}
-constexpr KernelShape kFp16Shape{4, 3};
 // Streaming multiprocessors of the current device (cudaDevAttrMultiProcessorCount, asked once per device; 148,
 // a B200, where no device answers, so that the size queries also work on a machine without a GPU).
 int sm_count();
@@ -109,8 +109,7 @@ SA_HD void half_normalise(uint32_t mag_bits, int* M, int* X) {
 //   u = a/s = rho * 2^-e0 with rho in [1, 2);  j = floor((rho - 1) 2^K);  with n = 2^K + j the
 //   neighbours on the grid are n and n + 1 (in units of 2^(-K-e0)), and the upper one is nearer
 //   in log2 exactly when rho^2 4^K >= n (n + 1).
-template <int K>
-SA_HD uint8_t encode_element(uint32_t a_bits, uint32_t s_bits) {
+SA_HD uint8_t encode_element_k(int K, uint32_t a_bits, uint32_t s_bits) {
     const uint32_t mag = a_bits & 0x7fffu;
     if (mag == 0) return 0x70;
     int Ma, Xa, Ms, Xs;
@@ -131,6 +130,8 @@ SA_HD uint8_t encode_element(uint32_t a_bits, uint32_t s_bits) {
     if (e0 >= 7) return 0x70;
     return (uint8_t)(((a_bits >> 15) << 7) | ((uint32_t)e0 << 4) | (j << (4 - K)));
 }
+template <int K>
+SA_HD uint8_t encode_element(uint32_t a_bits, uint32_t s_bits) { return encode_element_k(K, a_bits, s_bits); }
 
 // Power-of-two exponent g of the value scale: the largest g with amax * 2^g <= 127
 // (section II-E).  amax = M * 2^X, so amax * 2^g <= 127  <=>  M * 2^(X + g + 4) <= 2032.

@@ -1,20 +1,33 @@
-// Entry points of the decode path: argument checks, the split plan, and the dispatch to the decode
-// kernel's instantiations (sa_decode_kernel.cuh; one translation unit per key code) and the split-K merge.
-#include "sa_decode_kernel.cuh"
+// Entry points of the decode path: argument checks, the split plan, and the dispatch to the decode kernels — matrix
+// scores (sa_decode_mma.cuh) or, for SA_FLAG_ADD_ON_ALU and the score pass of the shift-based A.V option, shifts and adds
+// (sa_decode_kernel.cuh) — and the split-K merge.
+#include "sa_decode_common.cuh"
 
 using namespace sa;
 
 namespace sa {
 void launch_decode_fp16_main(const Plan& p, const DecodeArgs& a, int GT, cudaStream_t s);   // sa_decode_fp16.cu
+void launch_mma_byte(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t s);         // sa_decode_mma_*.cu
+void launch_mma_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s);
+void launch_mma_dense(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t s);
+void launch_mma_int8(int d, const DecodeArgs& a, dim3 grid, cudaStream_t s);
+void launch_shift_pot4(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);   // sa_decode_pot*.cu
+void launch_shift_potm1(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
+void launch_shift_potm2(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
+void launch_shift_potm4(int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
+
 // The decode kernel for these arguments (the score pass of the shift-A.V option when a.zr is set).
 void launch_decode_main(const Plan& p, const DecodeArgs& a, int GT, cudaStream_t s) {
     const dim3 grid((unsigned)a.n_splits, (unsigned)(p.Hkv * (p.G / GT)), (unsigned)a.batch);
-    const int mode = a.zr ? 2 : (p.mulshift ? 1 : (p.addalu ? 3 : 0));   // a.zr: score pass of the shift-based A.V option
-    if (p.int8) launch_decode_int8(p.d, a, GT, grid, s);
-    else if (p.k == 0) launch_decode_pot4(p.nibble, p.d, mode, a, GT, grid, s);
-    else if (p.k == 1) launch_decode_potm1(p.nibble, p.d, mode, a, GT, grid, s);
-    else if (p.k == 2) launch_decode_potm2(p.nibble, p.d, mode, a, GT, grid, s);
-    else launch_decode_potm4(p.d, mode, a, GT, grid, s);
+    const bool sp = a.zr != nullptr;
+    if (!sp && !p.addalu) {
+        if (p.int8) launch_mma_int8(p.d, a, grid, s);
+        else if (p.nibble) launch_mma_dense(p.d, p.k, a, grid, s);
+        else launch_mma_byte(p.d, p.k, a, grid, s);
+    } else if (p.k == 0) launch_shift_pot4(p.nibble, p.d, sp, a, GT, grid, s);
+    else if (p.k == 1) launch_shift_potm1(p.nibble, p.d, sp, a, GT, grid, s);
+    else if (p.k == 2) launch_shift_potm2(p.nibble, p.d, sp, a, GT, grid, s);
+    else launch_shift_potm4(p.d, sp, a, GT, grid, s);
 }
 }  // namespace sa
 
@@ -33,9 +46,7 @@ extern "C" sa_status sa_decode_attention_stages(const sa_config* cfg, const sa_c
     if (st != SA_OK) return st;
     if (dbg_scores && (reinterpret_cast<uintptr_t>(dbg_scores) & 3)) return SA_ERR_ALIGNMENT;
     a.dbg_scores = dbg_scores;
-    // logits in the log2 domain: A * Delta * s * 2^-F * log2(e) / sqrt(d)
-    a.zscale = (float)(1.4426950408889634 / sqrt((double)p.d) / (double)(1LL << p.F));
-    if (p.int8) a.zscale = (float)(1.4426950408889634 / sqrt((double)p.d) / 127.0);   // key unit = scale / 127
+    set_scales(p, !p.addalu, &a);   // logits in the log2 domain: A * Delta * s * 2^-F * log2(e) / sqrt(d)
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (stages & 1) {
         launch_decode_main(p, a, GT, s);
@@ -56,12 +67,12 @@ extern "C" sa_status sa_debug_decode_lost_copy(const sa_config* cfg, const sa_ca
     st = make_decode_args(p, cache, Q, O, workspace, workspace_bytes, &a, &GT);
     if (st != SA_OK) return st;
     if (b < 0 || b >= a.batch || kv_head < 0 || kv_head >= p.Hkv || tile < 0) return SA_ERR_INVALID_ARG;
-    a.zscale = (float)(1.4426950408889634 / sqrt((double)p.d) / (double)(1LL << p.F));
+    set_scales(p, true, &a);
     a.lost_b = b;
     a.lost_kvh = kv_head;
     a.lost_tile = tile;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    launch_decode_potm4_lost_copy(a, dim3((unsigned)a.n_splits, (unsigned)p.Hkv, (unsigned)a.batch), s);
+    launch_mma_lost_copy(a, dim3((unsigned)a.n_splits, (unsigned)p.Hkv, (unsigned)a.batch), s);
     if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
     return launch_merge(p, a, s);
 }
@@ -103,9 +114,7 @@ sa_status sa::decode_step_impl(const sa_config* cfg, const sa_cache* cache, cons
     a.Knew = K_new;
     a.Vnew = V_new;
     a.wait_first = q_after_wait ? 1 : 0;
-    a.zscale = (float)(1.4426950408889634 / sqrt((double)p.d) / (double)(1LL << p.F));
-    if (p.int8) a.zscale = (float)(1.4426950408889634 / sqrt((double)p.d) / 127.0);
-    if (p.fp16) a.zscale = (float)(1.4426950408889634 / sqrt((double)p.d));
+    set_scales(p, !p.addalu, &a);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (p.fp16) launch_decode_fp16_main(p, a, GT, s);
     else launch_decode_main(p, a, GT, s);

@@ -3,6 +3,8 @@
 // dimension; the merge rule follows from the integer running maximum of section II-E:
 // M* = max_s M_s, every partial is rescaled by the exact factor 2^(M_s - M*)).
 #pragma once
+#include <cmath>
+
 #include "sa_common.cuh"
 #include "sa_mma.cuh"
 
@@ -21,6 +23,8 @@ struct DecodeArgs {
     int batch, Hq, Hkv, G, max_pages, n_pages, n_splits, f_extra, hadamard;
     size_t page_bytes, kcode_off, meta_off, v_off, plane_off;
     float zscale;
+    int gt, k;                // query heads per block; mantissa bits (the matrix kernels take both at run time)
+    float score_unit;         // integer score = raw product sum of the matrix kernels * score_unit (test hook)
     uint32_t one;             // the value 1, opaque to the compiler (adds issued as multiply-add)
     // Shift-based A.V option (eq. (6), (7)); all null / 0 on the default path.
     int32_t* zr;              // [batch][Hq][dbg_stride] rounded logits, written by the score pass
@@ -467,6 +471,9 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     a->v_off = p.lay.v_off;
     a->plane_off = p.plane_off;
     a->zscale = 0.0f;
+    a->gt = GT;
+    a->k = p.k;
+    a->score_unit = 1.0f;
     a->one = 1u;
     a->zr = nullptr;
     a->stat_m = nullptr;
@@ -483,8 +490,7 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
         a->plan = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)S * c->batch * p.Hq * (p.d + 2) * sizeof(float));
         // blocks per grid row that a batch of unequal lengths is cut into: the grid, rounded down to whole waves of
         // resident blocks (equal blocks gain nothing from a last, partly filled wave)
-        const KernelShape shape = p.fp16 ? kFp16Shape : decode_shape(p.d, p.int8 ? 8 : p.k);
-        const long long rows = (long long)p.Hkv * (p.G / GT), slots = (long long)sm_count() * shape.blocks_per_sm;
+        const long long rows = (long long)p.Hkv * (p.G / GT), slots = (long long)sm_count() * p.shape.blocks_per_sm;
         long long per_row = (long long)S * c->batch;
         if (per_row * rows > slots) per_row = ((per_row * rows) / slots) * slots / rows;
         a->bal_target = (int)(per_row < c->batch ? c->batch : per_row);
@@ -493,9 +499,23 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     return SA_OK;
 }
 
+// Logit scale (the queries' Delta and the keys' s_j still to be multiplied in) of the kernel that serves the plan.
+// matrix: the products of sa_score_mma.cuh, whose sums come in units of 2^-(14 + k) (INT8, nibbles: 1) whatever F is.
+inline void set_scales(const Plan& p, bool matrix, DecodeArgs* a) {
+    const double base = 1.4426950408889634 / sqrt((double)p.d);
+    if (p.fp16) a->zscale = (float)base;
+    else if (p.int8) a->zscale = (float)(base / 127.0);                       // key unit = scale / 127
+    else if (!matrix) a->zscale = (float)(base / (double)(1LL << p.F));
+    else if (p.nibble && p.k == 0) a->zscale = (float)(base / 64.0);
+    else {
+        a->zscale = (float)(base * 256.0);
+        a->score_unit = (float)(1 << (14 + p.k));
+    }
+}
+
 inline sa_status launch_merge(const Plan& p, const DecodeArgs& a, cudaStream_t s) {
     const int rows = a.batch * a.Hq;
-    const int early = (!p.fp16 && decode_shape(p.d, p.int8 ? 8 : p.k).warps >= 8) ? 1 : 0;
+    const int early = (!p.fp16 && p.shape.warps >= 8) ? 1 : 0;
     BumpArgs bump{a.Knew ? const_cast<int32_t*>(a.seq_lens) : nullptr, a.page_table, a.max_pages, a.n_pages, a.Hq, early, a.plan};
     cudaError_t err;
     const bool small = a.n_splits <= kMergeSmallSplits;

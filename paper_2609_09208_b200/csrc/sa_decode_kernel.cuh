@@ -1,13 +1,15 @@
-// The decode kernel template and its launcher; included by the translation units that instantiate it
-// (sa_decode_k*.cu, one per key code so that they compile in parallel).
+// The shift-and-add decode kernel and its launcher; included by the translation units that instantiate it
+// (sa_decode_pot*.cu, one per key code so that they compile in parallel).
 #pragma once
-// Decode attention over the power-of-two key cache: the hot path.
+// Decode attention whose integer scores are formed by shifts, sign flips and adds alone, as the paper writes them
+// (section II-B eq. (3), II-D eq. (5)).  It serves SA_FLAG_ADD_ON_ALU and the score pass of the shift-based A.V option;
+// the default kernel (sa_decode_mma.cuh) forms the same integers as matrix products, at 2 - 5 times the rate.
 //
-// Grid (split, KV head x query chunk, sequence); 4, 8 or 10 warps per block (decode_shape).  A block
+// Grid (split, KV head x query chunk, sequence); 4, 8 or 10 warps per block (shift_shape).  A block
 // quantises its GT query heads into shared memory (ahead of its wait on the preceding kernel),
 // then each of its warps walks its own 32-key tiles of the block's slice of the key axis with a
 // private online-softmax state, so the main loop has no block-wide barrier.  Per tile: lane = key
-// for the integer scores (section II-B eq. (3) with the mantissa code of eq. (5)), warp-wide maxima
+// for the integer scores, warp-wide maxima
 // and an integer running maximum in the log2 domain (section II-E); then the floating-point A.V
 // over the INT8 values as small tensor-core products
 // O^T[dims][queries] += V^T[dims][keys] P^T[keys][queries] (mma.m16n8k8, tf32 operands: the INT8
@@ -40,47 +42,41 @@ template <int D, int KB, bool NIB, int GT>
 struct DecodeSmem {
     static constexpr int NP = (GT + 1) / 2;        // query pairs
     static constexpr bool kTable = (KB == 1 || KB == 2 || KB == 4);   // mantissa codes: table datapath
-    static constexpr int NW = decode_shape(D, KB).warps;
+    static constexpr int NW = shift_shape(D, KB).warps;
     static constexpr int CH = NIB ? D / 32 : D / 16;
     static constexpr int PLANES = (NIB && kTable) ? KB : 0;           // dense planar container: mantissa bit planes
     using Stage = TileStage<CH, true, D, PLANES, D / 8>;
     // Stage buffers per warp: two (the next tile is in flight while this one is computed), except where a
     // second buffer would cost resident warps — d = 128 (a tile is 8 KB) and PoT-M4 (32 KB table): there one,
     // and the other warps of the SM cover the copy instead.
-    static constexpr int NS = (D == 128 || KB == 4) ? 1 : kStages;
+    static constexpr int NS = shift_shape(D, KB).stages;
     static constexpr int kStageOff = 0;
     static constexpr int kMbarOff = NW * NS * Stage::kBytes;
-    // PoT-4: the shifted packed query pairs [D][8][NP]; INT8: D/4 x GT words of four queries; mantissa
-    // codes: the table of query multiples [D][NP][2^KB] x 8 bytes
+    // PoT-4: the shifted packed query pairs [D][8][NP]; mantissa codes: the table of query multiples [D][NP][2^KB] x 8 bytes
     static constexpr int kQpOff = (kMbarOff + 256 + 255) & ~255;   // the table datapaths want 256-byte alignment
     // (the prologue's scratch for the unpacked queries, D x GT words, uses the same space first)
-    static constexpr int kQpData = kTable ? D * NP * (8 << KB) : KB == 0 ? D * 8 * NP * 4 : D * NP * 4;
+    static constexpr int kQpData = kTable ? D * NP * (8 << KB) : D * 8 * NP * 4;
     static constexpr int kQpBytes = kQpData > D * GT * 4 ? kQpData : D * GT * 4;
     static constexpr int kQscaleOff = kQpOff + kQpBytes;
     // (The softmax weights of a tile need no space of their own: they overwrite the tile's key
     // codes in the stage buffer, which are dead by then.)
     static constexpr int kBytes = kQscaleOff + 128;
-    static constexpr int kBlocksPerSM = decode_shape(D, KB).blocks_per_sm;
+    static constexpr int kBlocksPerSM = shift_shape(D, KB).blocks_per_sm;
     static_assert(NW * GT * (D + 2) * 4 <= NW * NS * Stage::kBytes && NW * NS * 8 <= 256, "merge scratch must fit in the stage buffers");
     static_assert(Stage::kCodeBytes >= 32 * 8 * 4, "the weights of a tile must fit in its code area");
     static_assert(NW * NS * Stage::kBytes >= kPlanScratchInts * 4, "the block plan's scratch must fit in the stage buffers");
     static_assert(Stage::kBytes == half_block_bytes(D, KB, NIB), "a stage buffer is a verbatim copy of half a page block");
 };
 
-template <int D, int KB, bool NIB, int GT, int MODE = 0>
+template <int D, int KB, bool NIB, int GT, bool SP>
 #ifdef SA_ABLATE_NO_MIN_BLOCKS
-__global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW)) decode_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW)) shift_kernel(DecodeArgs a) {
 #else
-__global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (DecodeSmem<D, KB, NIB, GT>::kBlocksPerSM)) decode_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (DecodeSmem<D, KB, NIB, GT>::kBlocksPerSM)) shift_kernel(DecodeArgs a) {
 #endif
-    // MODE 0: the decode kernel; 1: the same with SA_FLAG_SHIFT_BY_MULTIPLY; 2: the score pass of the shift-based
-    // A.V option (a.zr set: rounded logits and statistics instead of softmax and A.V), kept out of the other two
-    // 3: the same with SA_FLAG_ADD_ON_ALU; 4: the test hook that never issues one chosen tile's copy (sa_debug_decode_lost_copy)
-    constexpr bool MUL = (MODE == 1), SP = (MODE == 2), ALUO = (MODE == 3), LOST = (MODE == 4);
-    constexpr uint32_t kPolls = LOST ? (1u << 10) : kWaitLimit;
-    // KB = 0: PoT-4 (packed shift datapath); KB = 1, 2, 4: mantissa codes (table datapath);
-    // KB = 8: uniform INT8 comparison code (dp4a).  MUL: the shifts run on the integer multiplier
-    // (SA_FLAG_SHIFT_BY_MULTIPLY; same scores, reported separately from the shift kernels).
+    // KB = 0: PoT-4 (packed datapath); KB = 1, 2, 4: mantissa codes (table datapath); no multiply-add in either (the
+    // score pass: sign flip and add as one multiply-add by +1 / -1, see sa_datapath.cuh).
+    // SP: the score pass of the shift-based A.V option (rounded logits and statistics instead of softmax and A.V).
     using SM = DecodeSmem<D, KB, NIB, GT>;
     using Stage = typename SM::Stage;
     constexpr int EPL = D / 32;
@@ -109,7 +105,7 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
     BlockPlan bp{(int)blockIdx.z, (int)blockIdx.x, a.n_splits, 0};
     if (a.wait_first) pdl_wait();
     if (__builtin_expect(ranked, 0))
-        bp = plan_block(plan_args(a), LOST ? (blockIdx.z + 1) % a.batch : blockIdx.z, blockIdx.x, false, a.wait_first != 0, bp, plan_scratch);
+        bp = plan_block(plan_args(a), blockIdx.z, blockIdx.x, false, a.wait_first != 0, bp, plan_scratch);
     int b = bp.b;
     const uint32_t mbar0 = smem_addr(smem + SM::kMbarOff) + warp * NS * 8;
     const uint32_t stage0 = smem_addr(smem + SM::kStageOff) + warp * NS * Stage::kBytes;
@@ -196,7 +192,7 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
                     }
                 }
             }
-        } else if constexpr (KB != 8) {
+        } else {
             uint32_t qp_reg[(D * NP + NT - 1) / NT];
 #pragma unroll
             for (int k = 0; k < (D * NP + NT - 1) / NT; ++k) {
@@ -220,25 +216,6 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
                     }
                 }
             }
-        } else {
-            // four consecutive elements of one query per word, in the byte order of the key words
-            uint32_t* q4_s = reinterpret_cast<uint32_t*>(smem + SM::kQpOff);
-            uint32_t q4_reg[(D / 4 * GT + NT - 1) / NT];
-#pragma unroll
-            for (int k = 0; k < (D / 4 * GT + NT - 1) / NT; ++k) {
-                const int idx = threadIdx.x + k * NT;
-                const int w = idx / GT, g = idx % GT;
-                q4_reg[k] = 0u;
-                if (idx < D / 4 * GT)
-                    q4_reg[k] = (uint32_t)(q_s[4 * w][g] & 0xff) | ((uint32_t)(q_s[4 * w + 1][g] & 0xff) << 8) |
-                                ((uint32_t)(q_s[4 * w + 2][g] & 0xff) << 16) | ((uint32_t)(q_s[4 * w + 3][g] & 0xff) << 24);
-            }
-            __syncthreads();                                       // q_s is about to be overwritten
-#pragma unroll
-            for (int k = 0; k < (D / 4 * GT + NT - 1) / NT; ++k) {
-                const int idx = threadIdx.x + k * NT;
-                if (idx < D / 4 * GT) q4_s[idx] = q4_reg[k];
-            }
         }
         __syncthreads();
 
@@ -257,8 +234,7 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
         if (lane == 0 && tile_g >= 0) pidx_g = a.page_table[(size_t)bq * a.max_pages + (tile_g >> 1)];
         again = false;
         if (__builtin_expect(ranked && !a.wait_first, 0)) {       // the plan that counts; wait_first made it after the wait already
-            // (the test hook's guess was made for another block's coordinates: it never stands)
-            bp = plan_block(plan_args(a), blockIdx.z, blockIdx.x, !LOST, true, bp, plan_scratch);
+            bp = plan_block(plan_args(a), blockIdx.z, blockIdx.x, true, true, bp, plan_scratch);
             again = bp.b != bq && bp.b >= 0;
             if (bp.split != split_g || bp.n_splits != nsp_g) tile_g = -1;     // the hint was for other tiles
             b = bp.b;
@@ -288,7 +264,7 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
     const int n_my = first < tile1 ? (tile1 - first + NW - 1) / NW : 0;
     if (tile_new >= first && tile_new < tile1 && (tile_new - first) % NW == 0) {      // warp-uniform: this warp owns that tile
         // encode / quantise the token and write it into its page before the tile is copied to shared memory
-        constexpr int WMODE = (KB == 8) ? 32 : (NIB ? 8 + KB : KB);
+        constexpr int WMODE = NIB ? 8 + KB : KB;
         CacheArgs ca{};
         ca.page_bytes = a.page_bytes;
         ca.kcode_off = a.kcode_off;
@@ -309,7 +285,6 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
         const int tile = first + NW * i;
         const int pidx = (tile == tile_g) ? pidx_g : a.page_table[(size_t)b * a.max_pages + (tile >> 1)];
         const int s = i % NS;
-        if (LOST && tile == a.lost_tile && b == a.lost_b && kvh == a.lost_kvh) return;   // test hook: this copy never starts
         if (pidx < 0 || pidx >= a.n_pages) {
             mbar_arrive(mbar0 + s * 8);
         } else {
@@ -363,11 +338,11 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
         const int s = i % NS;
         const uint32_t parity = (uint32_t)(i / NS) & 1u;
         // the decision is made warp-uniform: a lane must never leave the loop alone
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar0 + s * 8, parity, kPolls))) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar0 + s * 8, parity))) {
             failed = true;
             // give the other stage's copy (already issued) a bounded chance to land before this
             // warp's buffers are re-used by the block merge
-            if (NS > 1 && i + 1 < n_my) (void)mbar_wait_bounded(mbar0 + ((i + 1) % NS) * 8, (uint32_t)((i + 1) / NS) & 1u, kPolls);
+            if (NS > 1 && i + 1 < n_my) (void)mbar_wait_bounded(mbar0 + ((i + 1) % NS) * 8, (uint32_t)((i + 1) / NS) & 1u);
             break;
         }
         const int pidx = a.page_table[(size_t)b * a.max_pages + (tile >> 1)];
@@ -381,7 +356,7 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
             int32_t A[GT];
             const uint32_t* cw = reinterpret_cast<const uint32_t*>(st) + lane * 4;
             if constexpr (SM::kTable) {
-                using TS = TableScore<KB, NP, MUL, ALUO>;
+                using TS = TableScore<KB, NP, false, !SP>;
                 uint32_t grp = smem_addr(smem + SM::kQpOff);    // table of the next 16 elements (256-byte aligned)
                 TS ts;
                 ts.begin(a.one);
@@ -423,10 +398,10 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
                 }
 #pragma unroll
                 for (int g = 0; g < GT; ++g) A[g] = (int32_t)((uint32_t)ts.score(g) << a.f_extra);   // exact: the true sum fits INT32
-            } else if constexpr (KB != 8) {
+            } else {
                 // PoT-4: the packed pairs, shifted ahead of the loop, are looked up by the key's exponent field
                 using ST = ShiftTable<NP>;
-                PackedShift<NP, ALUO> pl;
+                PackedShift<NP, !SP> pl;
                 pl.begin(a.one);
                 uint32_t grp = smem_addr(smem + SM::kQpOff);     // rows of the next group of elements (256-byte aligned)
                 if constexpr (!NIB) {
@@ -450,19 +425,6 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
                 }
 #pragma unroll
                 for (int g = 0; g < GT; ++g) A[g] = (int32_t)((uint32_t)pl.score(g) << a.f_extra);   // exact: the true sum fits INT32
-            } else {
-                // comparison datapath: four INT8 multiply-accumulates per instruction
-                const uint32_t* q4_s = reinterpret_cast<const uint32_t*>(smem + SM::kQpOff);
-#pragma unroll
-                for (int g = 0; g < GT; ++g) A[g] = 0;
-#pragma unroll 4
-                for (int wq = 0; wq < D / 4; ++wq) {
-                    const uint32_t w = cw[(wq >> 2) * 128 + (wq & 3)];
-                    uint32_t q4[GT];
-                    load_np<GT>(q4_s + wq * GT, q4);
-#pragma unroll
-                    for (int g = 0; g < GT; ++g) A[g] = __dp4a((int)q4[g], (int)w, A[g]);
-                }
             }
             const uint32_t meta = reinterpret_cast<const uint32_t*>(st + Stage::kMetaOff)[lane];
 
@@ -633,54 +595,38 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
     block_merge_and_store<D, GT, NW>(a, red_s, M, l, acc, lane, warp, slot, h0, failed);
 }
 
-template <int D, int KB, bool NIB, int GT, int MODE>
+template <int D, int KB, bool NIB, int GT, bool SP>
 static void launch_one(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     constexpr int bytes = DecodeSmem<D, KB, NIB, GT>::kBytes;
     if (bytes > 48 * 1024) {
         // opt in to more than 48 KB of dynamic shared memory (an attribute of the function; no allocation)
-        static const cudaError_t once = cudaFuncSetAttribute(decode_kernel<D, KB, NIB, GT, MODE>,
+        static const cudaError_t once = cudaFuncSetAttribute(shift_kernel<D, KB, NIB, GT, SP>,
                                                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         (void)once;
     }
-    (void)launch_pdl(decode_kernel<D, KB, NIB, GT, MODE>, grid, dim3(32 * DecodeSmem<D, KB, NIB, GT>::NW), (size_t)bytes, s, a);
+    (void)launch_pdl(shift_kernel<D, KB, NIB, GT, SP>, grid, dim3(32 * DecodeSmem<D, KB, NIB, GT>::NW), (size_t)bytes, s, a);
 }
 
-template <int D, int KB, bool NIB, int MODE>
+template <int D, int KB, bool NIB, bool SP>
 static void launch_gt(const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
     switch (GT) {
-        case 8: launch_one<D, KB, NIB, 8, MODE>(a, grid, s); break;
-        case 4: launch_one<D, KB, NIB, 4, MODE>(a, grid, s); break;
-        case 2: launch_one<D, KB, NIB, 2, MODE>(a, grid, s); break;
-        default: launch_one<D, KB, NIB, 1, MODE>(a, grid, s); break;
+        case 8: launch_one<D, KB, NIB, 8, SP>(a, grid, s); break;
+        case 4: launch_one<D, KB, NIB, 4, SP>(a, grid, s); break;
+        case 2: launch_one<D, KB, NIB, 2, SP>(a, grid, s); break;
+        default: launch_one<D, KB, NIB, 1, SP>(a, grid, s); break;
     }
 }
 
-// All instantiations of one key code and container: head_dim 64 / 128, the queries per block, and the
-// kernel's mode (0 decode; 1 the same with the shifts on the integer multiplier, mantissa codes only;
-// 2 the score pass of the shift-based A.V option, 3 sign flips and adds on the ALU pipe: power-of-two codes only).
+// All instantiations of one key code and container: head_dim 64 / 128, the queries per block, decode or score pass.
 template <int KB, bool NIB>
-static void launch_code(int d, int mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
-    constexpr bool kPot = (KB != 8);
-    constexpr bool kMul = (KB == 1 || KB == 2 || KB == 4);
+static void launch_code(int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
     if (d == 64) {
-        if (kPot && mode == 2) launch_gt<64, KB, NIB, kPot ? 2 : 0>(a, GT, grid, s);
-        else if (kPot && mode == 3) launch_gt<64, KB, NIB, kPot ? 3 : 0>(a, GT, grid, s);
-        else if (kMul && mode == 1) launch_gt<64, KB, NIB, kMul ? 1 : 0>(a, GT, grid, s);
-        else launch_gt<64, KB, NIB, 0>(a, GT, grid, s);
+        if (score_pass) launch_gt<64, KB, NIB, true>(a, GT, grid, s);
+        else launch_gt<64, KB, NIB, false>(a, GT, grid, s);
     } else {
-        if (kPot && mode == 2) launch_gt<128, KB, NIB, kPot ? 2 : 0>(a, GT, grid, s);
-        else if (kPot && mode == 3) launch_gt<128, KB, NIB, kPot ? 3 : 0>(a, GT, grid, s);
-        else if (kMul && mode == 1) launch_gt<128, KB, NIB, kMul ? 1 : 0>(a, GT, grid, s);
-        else launch_gt<128, KB, NIB, 0>(a, GT, grid, s);
+        if (score_pass) launch_gt<128, KB, NIB, true>(a, GT, grid, s);
+        else launch_gt<128, KB, NIB, false>(a, GT, grid, s);
     }
 }
-
-// One translation unit per key code (they compile in parallel); nib: the sub-byte container of the code.
-void launch_decode_pot4(bool nib, int d, int mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
-void launch_decode_potm1(bool nib, int d, int mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
-void launch_decode_potm2(bool nib, int d, int mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
-void launch_decode_potm4(int d, int mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
-void launch_decode_potm4_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s);   // test hook: head_dim 64, 8 queries per block
-void launch_decode_int8(int d, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
 
 }  // namespace sa

@@ -1,0 +1,393 @@
+// The decode kernel: attention of one query group over a quantised key cache.
+//
+// Grid (split, KV head x query chunk, sequence).  Every warp prepares the block's (up to 8) query heads as matrix
+// fragments in its own registers (ahead of the wait on the preceding kernel), then walks its own 32-key tiles with a
+// private online-softmax state: no block-wide barrier in the main loop.  Per tile, on fragments throughout:
+//   scores   exact integer products of the decoded key codes and the queries (sa_score_mma.cuh): keys x queries;
+//   softmax  lane (r, c): keys r, r + 8, r + 16, r + 24 of queries 2 c, 2 c + 1.  The weight of a value row is
+//            w = 2^(z - g - R) with an integer reference R per query that bounds z - g from above to within two bits
+//            (z: logit in the log2 domain, 2^-g: the value's scale); the normaliser sums 2^(z - R).  R moves (and the
+//            state is rescaled by the exact power of two) only when a weight would leave the range of binary16;
+//   A.V      O^T[dims][queries] += V^T[dims][keys] w[keys][queries] as m16n8k16 products: INT8 values are exact in
+//            binary16, every weight enters as the sum of two binary16 terms (22 significant bits for weights within
+//            2^-17 of the largest, an absolute 2^-38 of it below), accumulation in FP32.  The weights reach the operand layout
+//            through movmatrix, without shared memory.
+// The warps' states and then the blocks' partial results are merged with exact power-of-two factors.  For
+// sa_decode_step the warp that owns the new token's tile writes the token first.
+#pragma once
+#include "sa_cache_write.cuh"
+#include "sa_common.cuh"
+#include "sa_decode_common.cuh"
+#include "sa_mma.cuh"
+#include "sa_score_mma.cuh"
+#include "sa_stage.cuh"
+
+namespace sa {
+
+constexpr int kWeightShift = 14;          // weights are scaled by 2^14: the largest (2^1.98 above R) stays below 65504
+constexpr float kWeightLimit = 65000.0f;  // a weight above this moves R
+constexpr float kRefMax = 268435456.0f;   // |R| <= 2^28
+
+template <int FMT>
+constexpr int format_kb() { return FMT == FMT_PLANAR1 ? 1 : FMT == FMT_PLANAR2 ? 2 : FMT == FMT_INT8 ? 8 : 0; }
+
+// Shared-memory plan of one block: [NW warps x NS stage buffers][mbarriers][R of every warp and query]; the block
+// merge's rows re-use the stage buffers once every warp has left its tile loop.
+template <int D, int FMT, int NW, int NS>
+struct MmaSmem {
+    using SC = ScoreMma<D, FMT>;
+    static constexpr int PLANES = FMT == FMT_PLANAR1 ? 1 : FMT == FMT_PLANAR2 ? 2 : 0;
+    using Stage = TileStage<SC::CH, true, D, PLANES, D / 8>;
+    static constexpr int kMbarOff = NW * NS * Stage::kBytes;
+    static constexpr int kRefOff = kMbarOff + ((NW * NS * 8 + 127) & ~127);
+    static constexpr int kBytes = kRefOff + NW * 8 * 4;
+    static_assert(NW * 8 * (D + 2) * 4 <= NW * NS * Stage::kBytes, "merge rows must fit in the stage buffers");
+    static_assert(NW * NS * Stage::kBytes >= kPlanScratchInts * 4, "the block plan's scratch must fit in the stage buffers");
+    static_assert(Stage::kBytes == half_block_bytes(D, format_kb<FMT>(), SC::kDense), "a stage buffer is a verbatim copy of half a page block");
+};
+
+// CODE: the cache-write mode of the fused append (see write_token).  LOST: the test hook that never issues one chosen
+// tile's copy and makes its first plan for another block's coordinates (sa_debug_decode_lost_copy).
+template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST>
+__global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(DecodeArgs a) {
+    using SM = MmaSmem<D, FMT, NW, NS>;
+    using SC = typename SM::SC;
+    using Stage = typename SM::Stage;
+    constexpr int MT = D / 16;                     // 16-dim row tiles of O^T
+    constexpr uint32_t kPolls = LOST ? (1u << 10) : kWaitLimit;
+    extern __shared__ __align__(1024) uint8_t smem[];
+
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r = lane >> 2, c = lane & 3;
+    const int GT = a.gt;                           // query heads of this block (1 .. 8)
+    const int chunks = a.G / GT;
+    const int kvh = blockIdx.y / chunks;
+    const int h0 = kvh * a.G + (blockIdx.y % chunks) * GT;
+    // What this block works on: sequence z and split x of the host's n_splits, or (batches of 2 .. 128 sequences) what
+    // plan_block deals it from the cached lengths.  The plan made here, from lengths the preceding kernel may be about
+    // to change, is a guess that lets the query preparation run ahead of the dependency wait; the plan made after the
+    // wait decides, and the preparation is repeated in the rare case that it names another sequence.
+    const bool ranked = batch_is_ranked(a.batch);
+    int* plan_scratch = reinterpret_cast<int*>(smem);
+    BlockPlan bp{(int)blockIdx.z, (int)blockIdx.x, a.n_splits, 0};
+    if (a.wait_first) pdl_wait();
+    if (ranked)
+        bp = plan_block(plan_args(a), LOST ? (blockIdx.z + 1) % a.batch : blockIdx.z, blockIdx.x, false, a.wait_first != 0, bp, plan_scratch);
+    const uint32_t mbar0 = smem_addr(smem + SM::kMbarOff) + warp * NS * 8;
+    const uint32_t stage0 = smem_addr(smem) + warp * NS * Stage::kBytes;
+
+    if (lane == 0) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) mbar_init(mbar0 + s * 8, 1u);
+        fence_mbar_init();
+        fence_proxy_async();
+    }
+    __syncwarp();
+    pdl_launch_dependents();    // the split-K merge may be scheduled as soon as blocks of this grid retire
+
+    SC q;
+    float qs0, qs1;             // logit scale (Delta * log2(e) / sqrt(d) * unit of the scores) of queries 2 c, 2 c + 1
+    int b = bp.b, tile_g, pidx_g;
+    bool again;
+#pragma unroll 1
+    do {
+        const int split_g = bp.split, nsp_g = bp.n_splits;         // what the hint below is computed for
+        const int bq = b < 0 ? 0 : b;                              // (a block without work so far prepares sequence 0)
+        const int len_g = (ranked ? bp.len : __ldcg(a.seq_lens + bq)) + (a.Knew ? 1 : 0);
+        // ---- queries: reads only Q, which no kernel of a decode step writes, so it runs before the wait ----
+        const float qs = q.load(r < GT ? a.Q + ((size_t)bq * a.Hq + h0 + r) * D : nullptr, lane, a.hadamard != 0) * a.zscale;
+        qs0 = __shfl_sync(0xffffffffu, qs, 8 * c);
+        qs1 = __shfl_sync(0xffffffffu, qs, 8 * c + 4);
+        // A guess at this warp's first tile, only to ask L2 for it while the preceding kernel drains (loads that bypass
+        // L1, so nothing stale can be read back later).
+        const int n_tiles_g = (min(max(len_g, 0), a.max_pages * kPageTokens) + 31) >> 5;
+        tile_g = split_begin(n_tiles_g, bp.split, bp.n_splits) + warp;
+        if (tile_g >= split_begin(n_tiles_g, bp.split + 1, bp.n_splits)) tile_g = -1;
+        if (tile_g >= 0) {
+            const int p_g = __ldcg(a.page_table + (size_t)bq * a.max_pages + (tile_g >> 1));
+            if (lane == 0 && p_g >= 0 && p_g < a.n_pages)
+                Stage::prefetch(a.pages + ((size_t)p_g * a.Hkv + kvh) * a.page_bytes, (tile_g & 1) * 32, true);
+        }
+        pdl_wait();                 // everything below reads what the preceding kernels in the stream wrote (the cache)
+        // the page of the guessed first tile, read again now that it is valid, at the same time as the length(s)
+        pidx_g = tile_g >= 0 ? a.page_table[(size_t)bq * a.max_pages + (tile_g >> 1)] : -1;
+        again = false;
+        if (ranked && !a.wait_first) {                            // the plan that counts; wait_first made it after the wait already
+            bp = plan_block(plan_args(a), blockIdx.z, blockIdx.x, !LOST, true, bp, plan_scratch);
+            again = bp.b != bq && bp.b >= 0;
+            if (bp.split != split_g || bp.n_splits != nsp_g) tile_g = -1;     // the hint was for other tiles
+            b = bp.b;
+        }
+    } while (again);
+    if (ranked && b < 0) return;                                  // more blocks than (sequence, split) pairs
+
+    // ---- this warp's tiles ----
+    int len = ranked ? bp.len : a.seq_lens[b];
+    const int32_t* table = a.page_table + (size_t)b * a.max_pages;
+    int tile_new = -1, pidx_new = -1;
+    if (a.Knew) {
+        // Fused append: the step's new token goes to position len (if its page is mapped) and is part of this step's
+        // attention.  Every block takes the same decision; the split-K merge kernel bumps seq_lens once all have read it.
+        const int lp = len / kPageTokens;
+        pidx_new = (len >= 0 && lp < a.max_pages) ? table[lp] : -1;
+        if (pidx_new >= 0 && pidx_new < a.n_pages) {
+            tile_new = len >> 5;
+            len += 1;
+        }
+    }
+    const int n_tiles = (min(len, a.max_pages * kPageTokens) + 31) >> 5;
+    const int first = split_begin(n_tiles, bp.split, bp.n_splits) + warp;
+    const int tile1 = split_begin(n_tiles, bp.split + 1, bp.n_splits);
+    const int n_my = first < tile1 ? (tile1 - first + NW - 1) / NW : 0;
+    if (tile_new >= first && tile_new < tile1 && (tile_new - first) % NW == 0) {      // warp-uniform: this warp owns that tile
+        CacheArgs ca{};
+        ca.page_bytes = a.page_bytes;
+        ca.kcode_off = a.kcode_off;
+        ca.meta_off = a.meta_off;
+        ca.v_off = a.v_off;
+        ca.plane_off = a.plane_off;
+        ca.hadamard = a.hadamard;
+        ca.k = a.k;
+        uint8_t* block = const_cast<uint8_t*>(a.pages) + ((size_t)pidx_new * a.Hkv + kvh) * a.page_bytes;
+        const size_t row = ((size_t)b * a.Hkv + kvh) * D;
+        write_token<D, CODE>(block, ca, (len - 1) % kPageTokens, lane, a.Knew + row, a.Vnew + row);
+        fence_proxy_async_global();
+        __syncwarp();
+    }
+    // Start the copy of my i-th tile, whose page is `pidx`, into stage i % NS; lane 0 keeps which stages hold a mapped
+    // tile (one whose page is not mapped gets a plain arrival: the phase completes, the tile is skipped).
+    uint32_t mapped = 0u;
+    auto issue = [&](int i, int pidx) {
+        const int tile = first + NW * i, s = i % NS;
+        if (LOST && tile == a.lost_tile && b == a.lost_b && kvh == a.lost_kvh) return;   // test hook: this copy never starts
+        if (pidx < 0 || pidx >= a.n_pages) {
+            mapped &= ~(1u << s);
+            mbar_arrive(mbar0 + s * 8);
+        } else {
+            mapped |= 1u << s;
+            Stage::issue(stage0 + s * Stage::kBytes, a.pages + ((size_t)pidx * a.Hkv + kvh) * a.page_bytes, (tile & 1) * 32, mbar0 + s * 8);
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+        if (i < n_my) {
+            const int tile = first + NW * i;
+            const int pidx = (tile == tile_g) ? pidx_g : table[tile >> 1];
+            if (lane == 0) issue(i, pidx);
+        }
+
+    float R0 = 0.0f, R1 = 0.0f;                    // references of queries 2 c, 2 c + 1 (integers)
+    bool seen = false;                             // no key yet: R is not set
+    float l0 = 0.0f, l1 = 0.0f;                    // this lane's share of the normalisers
+    float acc[MT][4];                              // O^T tiles: dims 16 mt + 2 r (c0, c1), + 1 (c2, c3) of queries 2 c, 2 c + 1
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[mt][e] = 0.0f;
+    bool failed = false;
+
+    for (int i = 0; i < n_my; ++i) {
+        const int tile = first + NW * i;
+        const int s = i % NS;
+        // the page of the tile that will take this stage over, fetched while this one is worked on
+        const int pidx_next = (i + NS < n_my) ? table[(tile + NW * NS) >> 1] : -1;
+        // the decision is made warp-uniform: a lane must never leave the loop alone
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar0 + s * 8, (uint32_t)(i / NS) & 1u, kPolls))) {
+            failed = true;
+            // give the other stages' copies (already issued) a bounded chance to land before this warp's buffers are
+            // re-used by the block merge
+            for (int k = 1; k < NS && i + k < n_my; ++k)
+                (void)mbar_wait_bounded(mbar0 + ((i + k) % NS) * 8, (uint32_t)((i + k) / NS) & 1u, kPolls);
+            break;
+        }
+        if ((__shfl_sync(0xffffffffu, mapped, 0) >> s) & 1u) {
+            const uint32_t st = stage0 + s * Stage::kBytes;
+            const int n_valid = len - tile * 32;
+
+            // ---- scores ----
+            float z[4][2], zh[SC::NACC == 2 ? 4 : 1][2];
+            q.tile(st, st + Stage::kPlaneOff, lane, z, zh);
+            if (a.dbg_scores) {                               // parity tests only
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        if (8 * j + r < n_valid && 2 * c + e < GT) {
+                            int A = (int)(z[j][e] * a.score_unit);
+                            if constexpr (SC::NACC == 2) A += (int)(zh[j][e] * a.score_unit);
+                            a.dbg_scores[((size_t)b * a.Hq + h0 + 2 * c + e) * a.dbg_stride + (size_t)tile * 32 + 8 * j + r] =
+                                (int)((uint32_t)A << a.f_extra);
+                        }
+            }
+            // ---- logits and weights ----
+            float zq[4][2], vs[4], g[4];                      // logit per score unit; 2^(14 - g_j); g_j
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t meta = lds_u32(st + Stage::kMetaOff + (8 * j + r) * 4);
+                const float sj = half_bits_to_float(meta & 0xffffu);
+                const int gi = (int)(meta << 8) >> 24;        // in [-10, 30] for written tokens
+                g[j] = (float)gi;
+                vs[j] = __int_as_float((127 + kWeightShift - gi) << 23);
+                zq[j][0] = qs0 * sj;
+                zq[j][1] = qs1 * sj;
+                if constexpr (SC::NACC == 2) {                // rounded once, like the conversion of one integer sum
+                    z[j][0] += zh[j][0];
+                    z[j][1] += zh[j][1];
+                }
+            }
+            float p[4][2], w[4][2];
+            auto weights = [&]() {                            // returns the largest of this lane
+                float top = 0.0f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        p[j][e] = ex2_approx(fmaf(z[j][e], zq[j][e], e ? -R1 : -R0));
+                        w[j][e] = p[j][e] * vs[j];
+                    }
+                if (n_valid < 32) {                           // the sequence's last tile: slots past its end may hold anything
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (8 * j + r >= n_valid) p[j][0] = p[j][1] = w[j][0] = w[j][1] = 0.0f;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) top = fmaxf(top, fmaxf(w[j][0], w[j][1]));
+                return top;
+            };
+            bool move = !seen;
+            if (seen) move = weights() > kWeightLimit;
+            if (__any_sync(0xffffffffu, move)) {              // rare after the first tile
+                float y0 = -INFINITY, y1 = -INFINITY;         // largest z - g of the tile
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (8 * j + r < n_valid) {
+                        y0 = fmaxf(y0, fmaf(z[j][0], zq[j][0], -g[j]));
+                        y1 = fmaxf(y1, fmaf(z[j][1], zq[j][1], -g[j]));
+                    }
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) {
+                    y0 = fmaxf(y0, __shfl_xor_sync(0xffffffffu, y0, o));
+                    y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
+                }
+                y0 = fminf(fmaxf(ceilf(y0), -kRefMax), kRefMax);
+                y1 = fminf(fmaxf(ceilf(y1), -kRefMax), kRefMax);
+                if (seen) {
+                    y0 = fmaxf(R0, y0);
+                    y1 = fmaxf(R1, y1);
+                    const float f0 = pow2i_neg(__float2int_rn(R0 - y0)), f1 = pow2i_neg(__float2int_rn(R1 - y1));
+                    l0 *= f0;
+                    l1 *= f1;
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) {
+                        acc[mt][0] *= f0;
+                        acc[mt][1] *= f1;
+                        acc[mt][2] *= f0;
+                        acc[mt][3] *= f1;
+                    }
+                }
+                R0 = y0;
+                R1 = y1;
+                seen = true;
+                (void)weights();
+            }
+            uint32_t bh[4], bl[4];                            // operand fragments: keys 8 j + 2 c, + 1 of query r
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                l0 += p[j][0];
+                l1 += p[j][1];
+                const __half2 h = __floats2half2_rn(w[j][0], w[j][1]);
+                const float2 hf = __half22float2(h);
+                const __half2 lo = __floats2half2_rn(w[j][0] - hf.x, w[j][1] - hf.y);
+                bh[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&h));
+                bl[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&lo));
+            }
+            // ---- A.V: an 8 x 8 block of 16-bit pairs (8 keys x 16 dims of INT8), transposed by ldmatrix: row r of
+            // the operand is dim 2 r (bytes 0, 2), row r + 8 dim 2 r + 1 (bytes 1, 3), columns the keys 2 c, 2 c + 1 ----
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                uint32_t x[4];
+                ldmatrix_x4_trans(x, st + Stage::kVOff + mt * 512 + lane * 16);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const uint32_t a0 = int8_to_half2<false>(x[2 * k]), a1 = int8_to_half2<true>(x[2 * k]);
+                    const uint32_t a2 = int8_to_half2<false>(x[2 * k + 1]), a3 = int8_to_half2<true>(x[2 * k + 1]);
+                    mma_f16_16816(acc[mt], a0, a1, a2, a3, bh[2 * k], bh[2 * k + 1]);
+                    mma_f16_16816(acc[mt], a0, a1, a2, a3, bl[2 * k], bl[2 * k + 1]);
+                }
+            }
+        }
+        __syncwarp();                                         // every lane is done with this stage
+        if (lane == 0 && i + NS < n_my) {
+            fence_proxy_async();
+            issue(i + NS, pidx_next);
+        }
+    }
+
+    // ---- merge the warps of the block, write the block's partial ----
+    // R of every warp and query goes to shared memory; every warp scales its state by the exact 2^(R - Rb), Rb the
+    // block's largest, and writes it out; the rows are added in a fixed order.
+    float* ref_s = reinterpret_cast<float*>(smem + SM::kRefOff);                   // [NW][8]
+    float (*red_s)[8][D + 2] = reinterpret_cast<float (*)[8][D + 2]>(smem);        // {unused, l, O[D]}
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+        l0 += __shfl_xor_sync(0xffffffffu, l0, o);
+        l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+    }
+    if (r == 0) {
+        ref_s[warp * 8 + 2 * c] = seen ? R0 : (float)kMNone;
+        ref_s[warp * 8 + 2 * c + 1] = seen ? R1 : (float)kMNone;
+    }
+    // A warp whose bounded wait for a copy expired makes the block's whole partial a marked one: l = NaN is written
+    // below from a register, not through the rows, which alias the stage buffers — a copy that was merely late could
+    // still land in them.
+    const bool poisoned = __syncthreads_or(failed ? 1 : 0) != 0;
+    float Rb0 = (float)kMNone, Rb1 = (float)kMNone;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        Rb0 = fmaxf(Rb0, ref_s[w * 8 + 2 * c]);
+        Rb1 = fmaxf(Rb1, ref_s[w * 8 + 2 * c + 1]);
+    }
+    const float f0 = seen ? pow2i_neg(__float2int_rn(R0 - Rb0)) : 0.0f, f1 = seen ? pow2i_neg(__float2int_rn(R1 - Rb1)) : 0.0f;
+    if (r == 0) {
+        red_s[warp][2 * c][1] = l0 * f0;
+        red_s[warp][2 * c + 1][1] = l1 * f1;
+    }
+    const float v0 = f0 * (1.0f / (1 << kWeightShift)), v1 = f1 * (1.0f / (1 << kWeightShift));
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+        const int dim = 16 * mt + 2 * r;
+        *reinterpret_cast<float2*>(&red_s[warp][2 * c][2 + dim]) = make_float2(acc[mt][0] * v0, acc[mt][2] * v0);
+        *reinterpret_cast<float2*>(&red_s[warp][2 * c + 1][2 + dim]) = make_float2(acc[mt][1] * v1, acc[mt][3] * v1);
+    }
+    __syncthreads();
+    const int slot = ranked ? blockIdx.z * a.n_splits + blockIdx.x : blockIdx.x * a.batch + blockIdx.z;
+    float* out = a.partials + ((size_t)slot * a.Hq + h0) * (D + 2);
+    for (int idx = threadIdx.x; idx < GT * (D + 2); idx += 32 * NW) {
+        const int g = idx / (D + 2), col = idx % (D + 2);                          // 0: R, 1: l, 2 ..: O
+        float v = 0.0f;
+        if (col == 0) {
+            v = (float)kMNone;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) v = fmaxf(v, ref_s[w * 8 + g]);
+            v = __int_as_float(__float2int_rn(v));
+        } else {
+#pragma unroll
+            for (int w = 0; w < NW; ++w) v += red_s[w][g][col];
+        }
+        if (poisoned && col <= 1) v = (col == 0) ? __int_as_float(0) : __int_as_float(0x7fc00000);   // R = 0, l = NaN
+        out[idx] = v;
+    }
+}
+
+template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST = false>
+static void launch_mma(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
+    constexpr int bytes = MmaSmem<D, FMT, NW, NS>::kBytes;
+    if (bytes > 48 * 1024) {
+        static const cudaError_t once = cudaFuncSetAttribute(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST>,
+                                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        (void)once;
+    }
+    (void)launch_pdl(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST>, grid, dim3(32 * NW), (size_t)bytes, s, a);
+}
+
+}  // namespace sa

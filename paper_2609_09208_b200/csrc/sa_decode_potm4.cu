@@ -1,11 +1,8 @@
-// Instantiations of the decode kernel for one key code (see sa_decode_kernel.cuh).
+// Instantiations of the shift-and-add kernel for one key code (see sa_decode_kernel.cuh).
 #include "sa_decode_kernel.cuh"
 
 namespace sa {
-void launch_decode_potm4(int d, int mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
-    launch_code<4, false>(d, mode, a, GT, grid, s);
-}
-void launch_decode_potm4_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
-    launch_one<64, 4, false, 8, 4>(a, grid, s);
+void launch_shift_potm4(int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
+    launch_code<4, false>(d, score_pass, a, GT, grid, s);
 }
 }  // namespace sa

@@ -28,6 +28,7 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
     if (p.fp16) {
         if (cfg->klayout != SA_KLAYOUT_BYTE) return SA_ERR_UNSUPPORTED;
         if (p.hadamard) return SA_ERR_UNSUPPORTED;   // the rotation is a pre-quantisation transform
+        p.shape = kFp16Shape;
         p.k = 0;
         p.nibble = false;
         p.F = 0;
@@ -44,6 +45,7 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
     if (cfg->code == SA_INT8) {
         if (cfg->klayout != SA_KLAYOUT_BYTE || cfg->headroom_F != 0) return SA_ERR_UNSUPPORTED;
         p.int8 = true;
+        p.shape = mma_shape(p.d, 8);
         p.k = 0;
         p.F = 0;
         p.f_extra = 0;
@@ -59,6 +61,7 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
     if (cfg->code != SA_POT4 && cfg->code != SA_POTM1 && cfg->code != SA_POTM2 && cfg->code != SA_POTM4)
         return SA_ERR_UNSUPPORTED;
     p.k = cfg->code;
+    p.shape = p.addalu ? shift_shape(p.d, p.k) : mma_shape(p.d, p.k);
     if (cfg->klayout == SA_KLAYOUT_NIBBLE) {
         if (p.k != 0) return SA_ERR_UNSUPPORTED;
         p.nibble = true;
@@ -121,8 +124,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt)
     //     (an SM's throughput falls almost in proportion to its resident warps).
     // The sequence lengths live on the device, so the model uses the cache's capacity.
     const long long units = (long long)batch * p.Hkv * (p.G / GT);
-    const KernelShape shape = p.fp16 ? kFp16Shape : decode_shape(p.d, p.int8 ? 8 : p.k);
-    const int bps = shape.blocks_per_sm, nw = shape.warps;
+    const int bps = p.shape.blocks_per_sm, nw = p.shape.warps;
     const int n_sms = sm_count();
     const long long slots = (long long)n_sms * bps;
     const long long tiles = (long long)max_pages * (kPageTokens / 32);

@@ -7,7 +7,7 @@ namespace sa {
 
 // D(16x8, f32) += A(16x16, f16, row) * B(16x8, f16, col)
 SA_D void mma_f16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile(
+    asm(
         "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
@@ -21,6 +21,38 @@ SA_D void mma_tf32_1688(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, ui
         "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// D(16x8, s32) += A(16x32, s8, row) * B(32x8, s8, col).  Lane (g, t): a0 = A[g][4t ..], a1 = A[g + 8][4t ..],
+// a2 = A[g][16 + 4t ..], a3 = A[g + 8][16 + 4t ..] (four consecutive bytes each); b0 = B[4t ..][g], b1 = B[16 + 4t ..][g].
+SA_D void mma_s8_16832(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// Four 8 x 8 matrices of 16-bit elements as they lie: lane i supplies the address of row i % 8 of matrix i / 8; lane
+// (g, t) receives M_j[g][2t], M_j[g][2t + 1] (the t-th 32-bit word of row g).
+SA_D void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+SA_D uint32_t lds_u32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+SA_D uint2 lds_u32x2(uint32_t addr) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+// Transpose of an 8 x 8 matrix of 16-bit elements held by the warp: in lane (g, t) M[g][2t], M[g][2t + 1];
+// out M[2t][g], M[2t + 1][g].
+SA_D uint32_t movmatrix_trans(uint32_t x) {
+    uint32_t d;
+    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(x));
+    return d;
 }
 // Four 8 x 8 matrices of 16-bit elements, transposed on the way: lane i supplies the address of
 // row i % 8 of matrix i / 8 (16 bytes); lane (g, t) receives from matrix j the two elements

@@ -35,9 +35,9 @@ SA_D void store_bytes(uint8_t* dst, const uint8_t (&c)[N]) {
 }
 
 // Key vector -> canonical code bytes; returns the scale's binary16 bits (the largest magnitude).
-// Section II-A: per-key-vector scale; section II-D: nearest-in-log2 codeword.
+// Section II-A: per-key-vector scale; section II-D: nearest-in-log2 codeword.  K: mantissa bits, or -1 (then k).
 template <int EPL, int K>
-SA_D uint32_t encode_key_vec(uint32_t (&bits)[EPL], int lane, bool hadamard, uint8_t (&codes)[EPL]) {
+SA_D uint32_t encode_key_vec(uint32_t (&bits)[EPL], int lane, bool hadamard, uint8_t (&codes)[EPL], int k = K) {
     if (hadamard) {
         float x[EPL];
 #pragma unroll
@@ -49,7 +49,7 @@ SA_D uint32_t encode_key_vec(uint32_t (&bits)[EPL], int lane, bool hadamard, uin
     for (int i = 0; i < EPL; ++i) smax = max(smax, bits[i] & 0x7fffu);   // binary16 magnitudes order like their bits
     smax = warp_max_u32(smax);
 #pragma unroll
-    for (int i = 0; i < EPL; ++i) codes[i] = encode_element<K>(bits[i], smax);
+    for (int i = 0; i < EPL; ++i) codes[i] = encode_element_k(K >= 0 ? K : k, bits[i], smax);
     return smax;
 }
 

@@ -1,0 +1,281 @@
+// Integer scores of a 32-key tile as exact matrix products (the contraction of eq. (3) / (5) over head_dim).
+//
+// A tile's key codes are the A operand (rows = keys) and the block's up to 8 quantised queries the B operand of
+// warp-level products; each code is decoded once, for all queries, into the small number it stands for:
+//   byte / planar containers  (1 + j/2^k) * 2^(g - 15) with its sign, as a binary16 value (g = 7 - e; 0 for the zero
+//                             code): sign, exponent field and mantissa field only change places.  Query integers are
+//                             binary16 values too, so every product is exact in FP32, and so is the sum: it is a whole
+//                             number of units 2^-(14 + k) below 2^24 (64 * 127 * 31 * 2^6 = 16 128 000 < 2^24 for PoT-M4).
+//                             At head_dim 128 PoT-M4 could reach 2^25: its two halves are accumulated apart.
+//   nibble container          2^(g - 1) <= 64 as an INT8 value: one byte permute looks four of them up, the sign bit of
+//                             the nibble (the permute's replicate-sign mode over non-negative bytes) turning the
+//                             others into 0; a second lookup with the signs flipped is multiplied by -q.  INT32 sums.
+//   INT8 keys                 as stored.  INT32 sums.
+// So the INT32 scores are those of the shift-and-add datapath (sa_datapath.cuh) bit for bit.
+//
+// Fragments: lane (r, c) = (lane / 4, lane % 4) holds the c-th 32-bit word of a 16-byte code chunk of keys r, r + 8,
+// r + 16, r + 24 (one ldmatrix.x4 per chunk: 8 keys x 16 bytes are 128 contiguous bytes, no bank conflict).  The order of
+// the elements along the contraction is free as long as the queries are packed in the same order.
+#pragma once
+#include "sa_common.cuh"
+#include "sa_mma.cuh"
+#include "sa_quant.cuh"
+
+namespace sa {
+
+enum ScoreFormat { FMT_BYTE = 0, FMT_NIBBLE = 1, FMT_PLANAR1 = 2, FMT_PLANAR2 = 3, FMT_INT8 = 4 };
+
+// Bytes 0 and 2 (ODD: 1 and 3) of a word of the byte container as a pair of binary16 values:
+// sign 7 -> 15, mantissa 6..3 -> 9..6, g 2..0 -> 12..10 of each half.
+template <bool ODD>
+SA_HD uint32_t byte_codes_to_half2(uint32_t w) {
+    return ODD ? ((w & 0x80008000u) | ((w >> 5) & 0x03c003c0u) | ((w << 2) & 0x1c001c00u))
+               : (((w << 8) & 0x80008000u) | ((w << 3) & 0x03c003c0u) | ((w << 10) & 0x1c001c00u));
+}
+// Nibble N (0 .. 3) of both halves of t as a pair of binary16 powers of two with their signs.
+template <int N>
+SA_HD uint32_t nibble_codes_to_half2(uint32_t t) {
+    const uint32_t s = N == 3 ? t : t << (12 - 4 * N), g = N == 3 ? t >> 2 : t << (10 - 4 * N);
+    return (s & 0x80008000u) | (g & 0x1c001c00u);
+}
+// INT8 values of two keys of one dimension (bytes 0 and 2, ODD: 1 and 3) as a pair of binary16 values: the biased byte
+// v + 128 in the low mantissa bits of 1024, minus 1152 (exact).
+template <bool ODD>
+SA_D uint32_t int8_to_half2(uint32_t x) {
+    const uint32_t y = ODD ? x >> 8 : x;
+    uint32_t h = (y & 0x00ff00ffu) ^ 0x64806480u;
+    asm("add.rn.f16x2 %0, %0, %1;" : "+r"(h) : "r"(0xe480e480u));
+    return h;
+}
+
+// The quantised queries of a block as B fragments in registers of every warp: lane (r, c) prepares query r.
+// E consecutive elements per lane and chunk: 4 (16-element chunks) or 8 (32-element chunks).
+template <int D, int FMT>
+struct ScoreMma {
+    static constexpr bool kInt = (FMT == FMT_NIBBLE || FMT == FMT_INT8);
+    static constexpr bool kDense = (FMT == FMT_NIBBLE || FMT == FMT_PLANAR1 || FMT == FMT_PLANAR2);
+    static constexpr int E = kDense ? 8 : 4;
+    static constexpr int CH = D / (4 * E);                        // code chunks
+    static constexpr int NACC = (FMT == FMT_BYTE && D == 128) ? 2 : 1;
+    static constexpr int NB = kInt ? D / 16 : D / 8;              // registers of B fragments
+    uint32_t q[NB];
+    uint32_t qn[FMT == FMT_NIBBLE ? NB : 1];                      // -q
+
+    // Quantises query r of this lane's fragment row (row: its D binary16 elements; null: a zero query).  Same
+    // arithmetic, in the same order, as quantise_query_vec: rotation with strides 1, 2, ..., largest magnitude,
+    // IEEE divide, round half to even.  Returns Delta.
+    SA_D float load(const uint16_t* row, int lane, bool hadamard) {
+        const int c = lane & 3;
+        float x[CH][E];
+#pragma unroll
+        for (int k = 0; k < CH; ++k)
+#pragma unroll
+            for (int i = 0; i < E; i += 4) {
+                uint2 w = make_uint2(0u, 0u);
+                if (row) w = *reinterpret_cast<const uint2*>(row + k * 4 * E + c * E + i);
+                x[k][i] = half_bits_to_float(w.x & 0xffffu);
+                x[k][i + 1] = half_bits_to_float(w.x >> 16);
+                x[k][i + 2] = half_bits_to_float(w.y & 0xffffu);
+                x[k][i + 3] = half_bits_to_float(w.y >> 16);
+            }
+        if (hadamard) rotate(x, c);
+        float amax = 0.0f;
+#pragma unroll
+        for (int k = 0; k < CH; ++k)
+#pragma unroll
+            for (int i = 0; i < E; ++i) amax = fmaxf(amax, fabsf(x[k][i]));
+        amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
+        amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
+        const float inv = amax == 0.0f ? 0.0f : __fdiv_rn(127.0f, amax);
+        int v[CH][E];
+#pragma unroll
+        for (int k = 0; k < CH; ++k)
+#pragma unroll
+            for (int i = 0; i < E; ++i) v[k][i] = max(-127, min(127, __float2int_rn(__fmul_rn(x[k][i], inv))));
+        pack(v);
+        return __fdiv_rn(amax, 127.0f);
+    }
+
+    // D-element Walsh-Hadamard transform of the quad's four lanes (element k * 4E + c * E + i), rounded to binary16.
+    SA_D static void rotate(float (&x)[CH][E], int c) {
+#pragma unroll
+        for (int h = 1; h < E; h <<= 1)
+#pragma unroll
+            for (int k = 0; k < CH; ++k)
+#pragma unroll
+                for (int i = 0; i < E; ++i)
+                    if ((i & h) == 0) {
+                        const float a = x[k][i], b = x[k][i + h];
+                        x[k][i] = __fadd_rn(a, b);
+                        x[k][i + h] = __fsub_rn(a, b);
+                    }
+#pragma unroll
+        for (int h = 1; h < 4; h <<= 1)
+#pragma unroll
+            for (int k = 0; k < CH; ++k)
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    const float o = __shfl_xor_sync(0xffffffffu, x[k][i], h);
+                    x[k][i] = (c & h) ? __fsub_rn(o, x[k][i]) : __fadd_rn(x[k][i], o);
+                }
+#pragma unroll
+        for (int h = 1; h < CH; h <<= 1)
+#pragma unroll
+            for (int k = 0; k < CH; ++k)
+                if ((k & h) == 0)
+#pragma unroll
+                    for (int i = 0; i < E; ++i) {
+                        const float a = x[k][i], b = x[k + h][i];
+                        x[k][i] = __fadd_rn(a, b);
+                        x[k + h][i] = __fsub_rn(a, b);
+                    }
+        const float scale = (D == 64) ? 0.125f : 0.088388346f;    // 1/sqrt(64), 1/sqrt(128)
+#pragma unroll
+        for (int k = 0; k < CH; ++k)
+#pragma unroll
+            for (int i = 0; i < E; ++i) x[k][i] = __half2float(__float2half_rn(__fmul_rn(x[k][i], scale)));
+    }
+
+    SA_D static uint32_t h2(int lo, int hi) {                     // |integers| <= 127: exact
+        const __half2 h = __floats2half2_rn((float)lo, (float)hi);
+        return *reinterpret_cast<const uint32_t*>(&h);
+    }
+    SA_D static uint32_t b4(int a, int b, int c, int d) {
+        return (uint32_t)(a & 0xff) | ((uint32_t)(b & 0xff) << 8) | ((uint32_t)(c & 0xff) << 16) | ((uint32_t)d << 24);
+    }
+    // The order of the elements along the contraction: that of tile() below.
+    SA_D void pack(const int (&v)[CH][E]) {
+        if constexpr (FMT == FMT_BYTE) {
+#pragma unroll
+            for (int k = 0; k < CH; ++k) {
+                q[2 * k] = h2(v[k][0], v[k][2]);
+                q[2 * k + 1] = h2(v[k][1], v[k][3]);
+            }
+        } else if constexpr (FMT == FMT_INT8) {
+#pragma unroll
+            for (int k = 0; k < CH; ++k) q[k] = b4(v[k][0], v[k][1], v[k][2], v[k][3]);
+        } else if constexpr (FMT == FMT_NIBBLE) {
+#pragma unroll
+            for (int k = 0; k < CH; ++k)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    q[2 * k + i] = b4(v[k][4 * i], v[k][4 * i + 1], v[k][4 * i + 2], v[k][4 * i + 3]);
+                    qn[2 * k + i] = b4(-v[k][4 * i], -v[k][4 * i + 1], -v[k][4 * i + 2], -v[k][4 * i + 3]);
+                }
+        } else {                                                  // planar: the same element of two chunks side by side
+#pragma unroll
+            for (int k = 0; k < CH; k += 2)
+#pragma unroll
+                for (int n = 0; n < 8; ++n) q[k * 4 + n] = h2(v[k][n], v[k + 1][n]);
+        }
+    }
+
+    // Scores of the 32 keys of a staged tile: sc[j][e], j = 2 t + h: key 16 t + 8 h + r, query 2 c + e, in units of
+    // 2^-(14 + k) (integer formats: 1).  st: shared address of the tile's codes; planes: its mantissa bit planes.
+    // hi[][]: the part of dimensions 64 .. 127 of NACC == 2 (not yet added).
+    SA_D void tile(uint32_t st, uint32_t planes, int lane, float (&sc)[4][2], float (&hi)[NACC == 2 ? 4 : 1][2]) const {
+        const uint32_t row = st + lane * 16;
+        if constexpr (kInt) {
+            int d[2][4] = {};
+            if constexpr (FMT == FMT_INT8) {
+#pragma unroll
+                for (int k = 0; k < CH; k += 2) {
+                    uint32_t a[4], b[4];
+                    ldmatrix_x4(a, row + k * 512);
+                    ldmatrix_x4(b, row + (k + 1) * 512);
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) mma_s8_16832(d[t], a[2 * t], a[2 * t + 1], b[2 * t], b[2 * t + 1], q[k], q[k + 1]);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < CH; ++k) {
+                    uint32_t w[4];
+                    ldmatrix_x4(w, row + k * 512);
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const uint32_t w0 = w[2 * t], w1 = w[2 * t + 1], n0 = w0 ^ 0x88888888u, n1 = w1 ^ 0x88888888u;
+                        mma_s8_16832(d[t], lookup(w0), lookup(w1), lookup(w0 >> 16), lookup(w1 >> 16), q[2 * k], q[2 * k + 1]);
+                        mma_s8_16832(d[t], lookup(n0), lookup(n1), lookup(n0 >> 16), lookup(n1 >> 16), qn[2 * k], qn[2 * k + 1]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sc[2 * t + (e >> 1)][e & 1] = (float)d[t][e];      // below 2^24: exact
+        } else {
+            float d[2 * NACC][4] = {};
+            if constexpr (FMT == FMT_BYTE) {
+#pragma unroll
+                for (int k = 0; k < CH; ++k) {
+                    uint32_t w[4];
+                    ldmatrix_x4(w, row + k * 512);
+#pragma unroll
+                    for (int t = 0; t < 2; ++t)
+                        mma_f16_16816(d[(NACC == 2 && k >= CH / 2 ? 2 : 0) + t], byte_codes_to_half2<false>(w[2 * t]),
+                                      byte_codes_to_half2<false>(w[2 * t + 1]), byte_codes_to_half2<true>(w[2 * t]),
+                                      byte_codes_to_half2<true>(w[2 * t + 1]), q[2 * k], q[2 * k + 1]);
+                }
+            } else {
+                constexpr int KB = FMT == FMT_PLANAR1 ? 1 : 2;
+                const int c = lane & 3;
+                const uint32_t psel = (uint32_t)c | ((uint32_t)(4 + c) << 8);
+#pragma unroll
+                for (int k = 0; k < CH; k += 2) {
+                    uint32_t w0[4], w1[4];
+                    ldmatrix_x4(w0, row + k * 512);
+                    ldmatrix_x4(w1, row + (k + 1) * 512);
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        uint32_t f[2][8];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int j = 2 * t + h;
+                            uint32_t pl[KB];
+#pragma unroll
+                            for (int b = 0; b < KB; ++b) {
+                                const uint2 p = lds_u32x2(planes + (b * 32 + 8 * j + (lane >> 2)) * (D / 8) + k * 4);
+                                pl[b] = __byte_perm(p.x, p.y, psel);           // bit n: element n of the two chunks
+                            }
+                            planar(f[h], __byte_perm(w0[j], w1[j], 0x5410), __byte_perm(w0[j], w1[j], 0x7632), pl);
+                        }
+#pragma unroll
+                        for (int n = 0; n < 8; n += 2)
+                            mma_f16_16816(d[t], f[0][n], f[1][n], f[0][n + 1], f[1][n + 1], q[k * 4 + n], q[k * 4 + n + 1]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    sc[2 * t + (e >> 1)][e & 1] = d[t][e];
+                    if constexpr (NACC == 2) hi[2 * t + (e >> 1)][e & 1] = d[2 + t][e];
+                }
+        }
+    }
+
+private:
+    SA_D static uint32_t lookup(uint32_t w) {                     // 2^(g - 1) of four nibbles, 0 where the sign bit is set
+        uint32_t d;
+        asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(0x04020100u), "r"(0x40201008u), "r"(w));
+        return d;
+    }
+    template <int KB>
+    SA_D static void planar(uint32_t (&f)[8], uint32_t lo, uint32_t hi, const uint32_t (&pl)[KB]) {
+        f[0] = nibble_codes_to_half2<0>(lo);
+        f[1] = nibble_codes_to_half2<1>(lo);
+        f[2] = nibble_codes_to_half2<2>(lo);
+        f[3] = nibble_codes_to_half2<3>(lo);
+        f[4] = nibble_codes_to_half2<0>(hi);
+        f[5] = nibble_codes_to_half2<1>(hi);
+        f[6] = nibble_codes_to_half2<2>(hi);
+        f[7] = nibble_codes_to_half2<3>(hi);
+#pragma unroll
+        for (int n = 0; n < 8; ++n)
+#pragma unroll
+            for (int b = 0; b < KB; ++b) f[n] |= (pl[b] << (10 - KB + b - n)) & (0x02000200u >> (KB - 1 - b));
+    }
+};
+
+}  // namespace sa

@@ -257,6 +257,7 @@ extern "C" sa_status sa_shiftav_workspace_bytes(const sa_config* cfg, int batch,
     const sa_status st = make_plan(cfg, &p);
     if (st != SA_OK) return st;
     if (p.fp16 || p.int8) return SA_ERR_UNSUPPORTED;
+    p.shape = shift_shape(p.d, p.k);                             // the score pass is the shift-and-add kernel's
     int S, GT;
     split_plan(p, batch, max_pages_per_seq, &S, &GT);
     size_t zo, mo, go;
@@ -272,6 +273,7 @@ extern "C" sa_status sa_decode_attention_shiftav(const sa_config* cfg, const sa_
     sa_status st = make_plan(cfg, &p);
     if (st != SA_OK) return st;
     if (p.fp16 || p.int8) return SA_ERR_UNSUPPORTED;
+    p.shape = shift_shape(p.d, p.k);                             // the score pass is the shift-and-add kernel's
     // INT32 tile accumulator: 32 keys x 128 x 2^N < 2^31
     if (n_bits < 1 || n_bits > 18 || k_max < 0 || k_max > n_bits) return SA_ERR_INVALID_ARG;
     DecodeArgs a;
@@ -291,7 +293,7 @@ extern "C" sa_status sa_decode_attention_shiftav(const sa_config* cfg, const sa_
     a.stat_g = reinterpret_cast<int32_t*>(ws + go);
     a.n_bits = n_bits;
     a.k_max = k_max;
-    a.zscale = (float)(1.4426950408889634 / sqrt((double)p.d) / (double)(1LL << p.F));
+    set_scales(p, false, &a);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     launch_decode_main(p, a, GT, s);                             // pass 1: scores, rounded logits, statistics
     if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;

@@ -1,0 +1,74 @@
+"""The matrix-product decode kernel at the edges of its arithmetic: integer sums next to the accumulator's 2^24, weights
+whose reference has to move with nearly every tile, value scales spread over many binades; every container."""
+import numpy as np
+import pytest
+
+from oracle import sa_oracle as ora
+from paper_2609_09208_b200 import binding as sa
+from paper_2609_09208_b200 import build as sa_build
+from paper_2609_09208_b200 import synth
+
+pytestmark = pytest.mark.gpu
+CONTAINERS = [(0, False), (0, True), (1, False), (1, True), (2, True), (4, False), (8, False)]
+
+
+def decode(case):
+    import torch
+    sa_build.build()
+    dev = torch.device("cuda:0")
+    up = lambda x: torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).to(dev)
+    cfg = sa.make_config(case.head_dim, case.n_q_heads, case.n_kv_heads, case.code_k, nibble=case.nibble)
+    cache = sa.PagedCache(cfg, case.lens, dev)
+    cache.fill(up(case.K), up(case.V), case.cu_lens)
+    O = torch.full((case.batch, case.n_q_heads, case.head_dim), float("nan"), dtype=torch.float32, device=dev)
+    dbg = torch.full((case.batch, case.n_q_heads, cache.max_pages * 64), -7, dtype=torch.int32, device=dev)
+    sa.decode_attention(cfg, cache.handle, up(case.Q), O, cache.workspace, dbg)
+    torch.cuda.synchronize()
+    ref = ora.decode_attention(case.Q, case.K, case.V, case.cu_lens, case.code_k, 6 + (case.code_k if case.code_k != 8 else 0),
+                               want_scores=True, n_threads=8)
+    return O.cpu().numpy(), dbg.cpu().numpy(), ref
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("k,nibble", CONTAINERS)
+def test_scores_exact_next_to_the_accumulator_limit(d, k, nibble):
+    """Sums of terms of the largest magnitude with a few smallest ones in any position: every INT32 score as the oracle's."""
+    rng = np.random.default_rng(100 + d + k)
+    case = synth.make_case("limit", [333], 16, 2, d, k, nibble=nibble, seed=1)
+    mags = np.array([1.0, 1.0, 1.0, 31 / 32, 2.0 ** -6, 17 / 16 * 2.0 ** -6, 0.0])
+    K = rng.choice(mags, size=case.K.shape, p=[0.3, 0.3, 0.2, 0.1, 0.04, 0.03, 0.03])
+    K[..., 0] = 1.0
+    signs = rng.choice([-1.0, 1.0], size=case.K.shape)
+    signs[::2] = 1.0                                          # half of the keys: all terms of one sign
+    case.K[:] = (K * signs).astype(np.float16)
+    Q = rng.choice([127.0, 126.0, 1.0], size=case.Q.shape, p=[0.9, 0.06, 0.04])
+    Q[..., 1] = 127.0
+    Q[:, 1::2] *= rng.choice([-1.0, 1.0], size=Q[:, 1::2].shape)
+    case.Q[:] = Q.astype(np.float16)
+    O, dbg, ref = decode(case)
+    assert np.array_equal(dbg[0, :, :333].astype(np.int64), ref["A"][0])
+    assert np.max(np.abs(O - ref["O"])) <= 1e-3
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("k,nibble", CONTAINERS)
+@pytest.mark.parametrize("spread", [0, 6])
+def test_outputs_with_a_moving_reference_and_spread_value_scales(d, k, nibble, spread):
+    """Logits that grow along the sequence (the reference of the weights moves again and again) and value rows whose
+    scales differ by up to 2^(2 * spread): outputs within 1e-5 of the oracle's in the 2-norm of every head."""
+    rng = np.random.default_rng(200 + d + k)
+    case = synth.make_case("moving", [700, 65], 8, 1, d, k, nibble=nibble, seed=3)
+    q = case.Q[:, :1].astype(np.float32)
+    case.Q[:] = (q * np.linspace(0.2, 1.0, 8)[None, :, None]).astype(np.float16)       # all heads look the same way
+    for b in range(2):
+        n = int(case.lens[b])
+        ramp = np.linspace(-1.0, 3.0, n)[:, None, None]
+        rows = slice(int(case.cu_lens[b]), int(case.cu_lens[b + 1]))
+        case.K[rows] = (ramp * q[b][None] + 0.1 * case.K[rows]).astype(np.float16)
+    case.V[:] = (case.V * np.exp2(rng.uniform(-spread, spread, (len(case.V), 1, 1)))).astype(np.float16)
+    O, dbg, ref = decode(case)
+    for b in range(2):
+        assert np.array_equal(dbg[b, :, :case.lens[b]].astype(np.int64), ref["A"][b][:, :case.lens[b]])
+        for h in range(8):
+            err = np.linalg.norm(O[b, h] - ref["O"][b, h]) / np.linalg.norm(ref["O"][b, h])
+            assert err <= 1e-5, (b, h, err)
