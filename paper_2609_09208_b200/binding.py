@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the C-ABI library (``include/sa.h``): argument marshalling only.
+"""Thin binding of the C-ABI library (``include/sa.h``): argument marshalling only, by ctypes or, for the calls of a
+decode loop, by the extension module ``_native`` (``csrc/sa_python.cpp``).
 
 Every function takes torch CUDA tensors (device memory, owned by the caller), passes their
 ``data_ptr()`` and the current torch CUDA stream to the library and raises ``SaError`` on a
@@ -8,10 +9,13 @@ shared object is missing, ``lib()`` raises.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsa.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 SA_POT4, SA_POTM1, SA_POTM2, SA_POTM4, SA_INT8, SA_KV_FP16 = 0, 1, 2, 4, 8, 16
 SA_KLAYOUT_BYTE, SA_KLAYOUT_NIBBLE, SA_KLAYOUT_PLANAR = 0, 1, 2
@@ -52,6 +56,7 @@ class SaError(RuntimeError):
 
 
 _lib = None
+_nat = None
 
 
 def lib():
@@ -66,6 +71,21 @@ def lib():
         _lib.sa_status_string.argtypes = [C.c_int]
         _lib.sa_version.restype = C.c_int
     return _lib
+
+
+def native():
+    """Load the extension module ``_native.so`` (built beside ``libsa.so``, which it calls)."""
+    global _nat
+    if _nat is None:
+        lib()
+        if not os.path.exists(NATIVE_PATH):
+            raise RuntimeError("%s is missing: run `python -m paper_2609_09208_b200.build`" % NATIVE_PATH)
+        name = __package__ + "._native"
+        loader = importlib.machinery.ExtensionFileLoader(name, NATIVE_PATH)
+        spec = importlib.util.spec_from_loader(name, loader)
+        _nat = importlib.util.module_from_spec(spec)
+        loader.exec_module(_nat)
+    return _nat
 
 
 def status_string(status: int) -> str:
@@ -113,7 +133,7 @@ def staging_bytes(cfg: SaConfig, batch: int) -> int:
 
 def _stream():
     import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
 
 
 def _ptr(t):
@@ -143,8 +163,9 @@ def quantise_values(cfg, V, v_hat, g):
 
 
 def append_kv(cfg, cache: SaCache, K_new, V_new, bump_lens: bool = True):
-    _check(lib().sa_append_kv(C.byref(cfg), C.byref(cache), _ptr(K_new), _ptr(V_new),
-                              C.c_int(1 if bump_lens else 0), _stream()), "sa_append_kv")
+    st = (_nat or native()).append_kv(cfg, cache, K_new, V_new, 1 if bump_lens else 0)
+    if st:
+        raise SaError(st, "sa_append_kv")
 
 
 def fill_kv(cfg, cache: SaCache, K, V, cu_lens_host):
@@ -157,33 +178,22 @@ def fill_kv(cfg, cache: SaCache, K, V, cu_lens_host):
 
 def decode_attention(cfg, cache: SaCache, Q, O, workspace, dbg_scores=None, stages: int = 3):
     """stages: 3 = whole call; 1 = main kernel only; 2 = split-K merge only."""
-    if stages == 3:
-        st = lib().sa_decode_attention(C.byref(cfg), C.byref(cache), _ptr(Q), _ptr(O), _ptr(workspace),
-                                       C.c_size_t(workspace.numel() * workspace.element_size()),
-                                       _ptr(dbg_scores), _stream())
-    else:
-        st = lib().sa_decode_attention_stages(C.byref(cfg), C.byref(cache), _ptr(Q), _ptr(O), _ptr(workspace),
-                                              C.c_size_t(workspace.numel() * workspace.element_size()),
-                                              _ptr(dbg_scores), C.c_int(stages), _stream())
-    _check(st, "sa_decode_attention")
+    st = (_nat or native()).decode_attention(cfg, cache, Q, O, workspace, dbg_scores, stages)
+    if st:
+        raise SaError(st, "sa_decode_attention")
 
 
 def decode_attention_fp16(cfg, cache: SaCache, Q, O, workspace, stages: int = 3):
-    if stages == 3:
-        st = lib().sa_decode_attention_fp16(C.byref(cfg), C.byref(cache), _ptr(Q), _ptr(O), _ptr(workspace),
-                                            C.c_size_t(workspace.numel() * workspace.element_size()), _stream())
-    else:
-        st = lib().sa_decode_attention_fp16_stages(C.byref(cfg), C.byref(cache), _ptr(Q), _ptr(O), _ptr(workspace),
-                                                   C.c_size_t(workspace.numel() * workspace.element_size()),
-                                                   C.c_int(stages), _stream())
-    _check(st, "sa_decode_attention_fp16")
+    st = (_nat or native()).decode_attention_fp16(cfg, cache, Q, O, workspace, stages)
+    if st:
+        raise SaError(st, "sa_decode_attention_fp16")
 
 
 def decode_step(cfg, cache: SaCache, Q, K_new, V_new, O, workspace):
     """Append the step's token and attend over the extended cache in one pass (sa_decode_step)."""
-    _check(lib().sa_decode_step(C.byref(cfg), C.byref(cache), _ptr(Q), _ptr(K_new), _ptr(V_new), _ptr(O),
-                                _ptr(workspace), C.c_size_t(workspace.numel() * workspace.element_size()),
-                                _stream()), "sa_decode_step")
+    st = (_nat or native()).decode_step(cfg, cache, Q, K_new, V_new, O, workspace)
+    if st:
+        raise SaError(st, "sa_decode_step")
 
 
 def shiftav_workspace_bytes(cfg: SaConfig, batch: int, max_pages_per_seq: int) -> int:
@@ -240,10 +250,9 @@ def debug_unpack(cfg, cache: SaCache, b: int, n_tokens: int, codes=None, scales=
 
 def decode_step_host(cfg, cache: SaCache, Q_host, K_new_host, V_new_host, O_host, staging, workspace):
     """Host (pinned) tensors in and out; device scratch `staging` and `workspace`."""
-    _check(lib().sa_decode_step_host(
-        C.byref(cfg), C.byref(cache), _ptr(Q_host), _ptr(K_new_host), _ptr(V_new_host), _ptr(O_host),
-        _ptr(staging), C.c_size_t(staging.numel() * staging.element_size()), _ptr(workspace),
-        C.c_size_t(workspace.numel() * workspace.element_size()), _stream()), "sa_decode_step_host")
+    st = (_nat or native()).decode_step_host(cfg, cache, Q_host, K_new_host, V_new_host, O_host, staging, workspace)
+    if st:
+        raise SaError(st, "sa_decode_step_host")
 
 
 class PagedCache:

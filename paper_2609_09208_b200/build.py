@@ -1,4 +1,5 @@
-"""Build step: compiles the CUDA sources in ``csrc/`` into ``libsa.so`` next to this file.
+"""Build step: compiles the CUDA sources in ``csrc/`` into ``libsa.so`` and ``csrc/sa_python.cpp`` (the native half of
+``binding.py``) into ``_native.so``, next to this file.
 
 nvcc cross-compiles for sm_100a without a GPU.  Every ``.cu`` file is compiled to an object of its
 own (in parallel, under ``build/``) and re-compiled only when it, a header or the flags changed;
@@ -12,11 +13,13 @@ import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libsa.so")
+NATIVE = os.path.join(_HERE, "_native.so")
 OBJ_DIR = os.path.join(_HERE, "build")
 
 NVCC_FLAGS = [
@@ -49,6 +52,17 @@ def _compile_one(src, obj, defines, verbose):
     os.replace(tmp, obj)
 
 
+def build_native(force: bool = False) -> str:
+    """The CPython extension that marshals the per-layer calls; it links to ``libsa.so`` beside it."""
+    src, hdr = os.path.join(CSRC, "sa_python.cpp"), os.path.join(_HERE, "..", "include", "sa.h")
+    if force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < max(os.path.getmtime(src), os.path.getmtime(hdr)):
+        tmp = NATIVE + ".%d.tmp" % os.getpid()
+        subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"], src,
+                               "-o", tmp, "-L" + _HERE, "-l:libsa.so", "-Wl,-rpath,$ORIGIN"])
+        os.replace(tmp, NATIVE)
+    return NATIVE
+
+
 def build(force: bool = False, verbose: bool = False, defines=(), out: str = LIB) -> str:
     """Compile what is stale and link ``out``.  ``defines``: extra ``-D...`` flags (a distinct object cache per set)."""
     tag = _tag(defines)
@@ -57,6 +71,8 @@ def build(force: bool = False, verbose: bool = False, defines=(), out: str = LIB
     hdr_time = max(os.path.getmtime(h) for h in _headers())
     src_time = max(hdr_time, max(os.path.getmtime(s) for s in sources()))
     if not force and os.path.exists(out) and os.path.getmtime(out) >= src_time and linked in (tag, None if not defines else tag):
+        if out == LIB:
+            build_native()
         return out                                  # up to date (a library shipped without its objects is trusted by its date)
     os.makedirs(OBJ_DIR, exist_ok=True)
     jobs, objs = [], []
@@ -75,6 +91,8 @@ def build(force: bool = False, verbose: bool = False, defines=(), out: str = LIB
         os.replace(tmp, out)
         with open(stamp, "w") as f:
             f.write(tag)
+    if out == LIB:
+        build_native(force)
     return out
 
 

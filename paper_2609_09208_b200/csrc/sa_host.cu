@@ -128,6 +128,20 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt)
     const int n_sms = sm_count();
     const long long slots = (long long)n_sms * bps;
     const long long tiles = (long long)max_pages * (kPageTokens / 32);
+    // Searching S takes 1 - 9 us, as long as a decode call on the GPU, and a program asks for the same few shapes over and
+    // over: every thread keeps its last answers.
+    struct Kept {
+        long long units, tiles;
+        int nw, bps, sms, S;
+    };
+    static thread_local Kept kept[8] = {};
+    static thread_local unsigned turn = 0;
+    for (const Kept& k : kept)
+        if (k.units == units && k.tiles == tiles && k.nw == nw && k.bps == bps && k.sms == n_sms) {
+            *n_splits = k.S;
+            *gt = GT;
+            return;
+        }
     long long cap = tiles / 2;                      // at least two tiles per block (short caches: spread them over the SMs)
     if (cap < 1) cap = 1;
     if (cap > 512) cap = 512;
@@ -151,6 +165,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt)
         }
         if (blocks > 16 * slots) break;             // more waves than this never pay
     }
+    kept[turn++ % 8] = Kept{units, tiles, nw, bps, n_sms, (int)best_S};
     *n_splits = (int)best_S;
     *gt = GT;
 }
