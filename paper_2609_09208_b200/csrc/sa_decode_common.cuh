@@ -500,7 +500,7 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
 }
 
 // Logit scale (the queries' Delta and the keys' s_j still to be multiplied in) of the kernel that serves the plan.
-// matrix: the products of sa_score_mma.cuh, whose sums come in units of 2^-(14 + k) (INT8, nibbles: 1) whatever F is.
+// matrix: the products of sa_score_mma.cuh, whose sums come in units of 2^-(6 + k) (PoT-M4: 2^-18; INT8, nibbles: 1) whatever F is.
 inline void set_scales(const Plan& p, bool matrix, DecodeArgs* a) {
     const double base = 1.4426950408889634 / sqrt((double)p.d);
     if (p.fp16) a->zscale = (float)base;
@@ -508,8 +508,8 @@ inline void set_scales(const Plan& p, bool matrix, DecodeArgs* a) {
     else if (!matrix) a->zscale = (float)(base / (double)(1LL << p.F));
     else if (p.nibble && p.k == 0) a->zscale = (float)(base / 64.0);
     else {
-        a->zscale = (float)(base * 256.0);
-        a->score_unit = (float)(1 << (14 + p.k));
+        a->zscale = (float)(p.k == 4 ? base * 256.0 : base);
+        a->score_unit = (float)(p.k == 4 ? 1 << 18 : 1 << (6 + p.k));
     }
 }
 

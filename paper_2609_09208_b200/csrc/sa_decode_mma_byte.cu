@@ -8,10 +8,12 @@ static void launch(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     launch_mma<D, FMT, CODE, sh.warps, sh.blocks_per_sm, sh.stages>(a, grid, s);
 }
 void launch_mma_byte(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t s) {
-    const bool fine = k == 1 || k == 2;                        // the shape is all that differs (mma_shape)
-    if (d == 128) launch<128, FMT_BYTE, 7, 4>(a, grid, s);
-    else if (fine) launch<64, FMT_BYTE, 7, 1>(a, grid, s);
-    else launch<64, FMT_BYTE, 7, 4>(a, grid, s);
+    if (d == 128) {
+        if (k == 4) launch<128, FMT_BYTE, 7, 4>(a, grid, s);
+        else launch<128, FMT_BYTE3, 7, 2>(a, grid, s);
+    } else if (k == 4) launch<64, FMT_BYTE, 7, 4>(a, grid, s);
+    else if (k == 0) launch<64, FMT_BYTE3, 7, 0>(a, grid, s);
+    else launch<64, FMT_BYTE3, 7, 2>(a, grid, s);
 }
 void launch_mma_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     constexpr KernelShape sh = mma_shape(64, 4);

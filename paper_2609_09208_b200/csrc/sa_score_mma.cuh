@@ -2,41 +2,65 @@
 //
 // A tile's key codes are the A operand (rows = keys) and the block's up to 8 quantised queries the B operand of
 // warp-level products; each code is decoded once, for all queries, into the small number it stands for:
-//   byte / planar containers  (1 + j/2^k) * 2^(g - 15) with its sign, as a binary16 value (g = 7 - e; 0 for the zero
-//                             code): sign, exponent field and mantissa field only change places.  Query integers are
-//                             binary16 values too, so every product is exact in FP32, and so is the sum: it is a whole
-//                             number of units 2^-(14 + k) below 2^24 (64 * 127 * 31 * 2^6 = 16 128 000 < 2^24 for PoT-M4).
+//   byte / planar containers  (1 + j/2^k) * 2^(g - c) with its sign, as a binary16 value (g = 7 - e; 0 for the zero
+//                             code).  Up to three mantissa bits (c = 7): sign, exponent field and mantissa field change
+//                             places within the byte, four codes at a time, which makes it an FP8 (e4m3) value, and one
+//                             conversion instruction turns two of those into binary16.  PoT-M4 (c = 15): the fields are
+//                             moved to their places in binary16 directly.  Query integers are binary16 values too, so
+//                             every product is exact in FP32, and so is the sum: it is a whole number of units
+//                             2^-(c - 1 + k) below 2^24 (64 * 127 * 31 * 2^6 = 16 128 000 < 2^24 for PoT-M4).
 //                             At head_dim 128 PoT-M4 could reach 2^25: its two halves are accumulated apart.
 //   nibble container          2^(g - 1) <= 64 as an INT8 value: one byte permute looks four of them up, the sign bit of
 //                             the nibble (the permute's replicate-sign mode over non-negative bytes) turning the
 //                             others into 0; a second lookup with the signs flipped is multiplied by -q.  INT32 sums.
 //   INT8 keys                 as stored.  INT32 sums.
-// So the INT32 scores are those of the shift-and-add datapath (sa_datapath.cuh) bit for bit.
+// So the INT32 scores are those of the shift-and-add datapath (sa_datapath.cuh) bit for bit.  (The decode is what a tile
+// costs most: for four codes 11 instructions in the direct form, 7 by way of FP8.  FP8 operands of the product itself
+// cost more: mma.sync expands them into conversions, again for every product they enter.)
 //
 // Fragments: lane (r, c) = (lane / 4, lane % 4) holds the c-th 32-bit word of a 16-byte code chunk of keys r, r + 8,
 // r + 16, r + 24 (one ldmatrix.x4 per chunk: 8 keys x 16 bytes are 128 contiguous bytes, no bank conflict).  The order of
 // the elements along the contraction is free as long as the queries are packed in the same order.
 #pragma once
 #include "sa_common.cuh"
+#include "sa_datapath.cuh"
 #include "sa_mma.cuh"
 #include "sa_quant.cuh"
 
 namespace sa {
 
-enum ScoreFormat { FMT_BYTE = 0, FMT_NIBBLE = 1, FMT_PLANAR1 = 2, FMT_PLANAR2 = 3, FMT_INT8 = 4 };
+// FMT_BYTE3: the byte container of the codes with at most three mantissa bits (all but PoT-M4)
+enum ScoreFormat { FMT_BYTE = 0, FMT_NIBBLE = 1, FMT_PLANAR1 = 2, FMT_PLANAR2 = 3, FMT_INT8 = 4, FMT_BYTE3 = 5 };
 
-// Bytes 0 and 2 (ODD: 1 and 3) of a word of the byte container as a pair of binary16 values:
+// Bytes 0 and 2 (ODD: 1 and 3) of a word of the byte container (sign << 7 | mantissa << 3 | g) as a pair of binary16 values:
 // sign 7 -> 15, mantissa 6..3 -> 9..6, g 2..0 -> 12..10 of each half.
 template <bool ODD>
 SA_HD uint32_t byte_codes_to_half2(uint32_t w) {
     return ODD ? ((w & 0x80008000u) | ((w >> 5) & 0x03c003c0u) | ((w << 2) & 0x1c001c00u))
                : (((w << 8) & 0x80008000u) | ((w << 3) & 0x03c003c0u) | ((w << 10) & 0x1c001c00u));
 }
-// Nibble N (0 .. 3) of both halves of t as a pair of binary16 powers of two with their signs.
-template <int N>
-SA_HD uint32_t nibble_codes_to_half2(uint32_t t) {
-    const uint32_t s = N == 3 ? t : t << (12 - 4 * N), g = N == 3 ? t >> 2 : t << (10 - 4 * N);
-    return (s & 0x80008000u) | (g & 0x1c001c00u);
+// Four codes of the byte container with at most three mantissa bits as FP8 values (sign << 7 | g << 3 | mantissa >> 1).
+SA_HD uint32_t byte_codes_to_fp8(uint32_t w) {
+    return (w & 0x80808080u) | ((w << 3) & 0x38383838u) | ((w >> 4) & 0x07070707u);
+}
+// FP8 values 0 and 1 (HIGH: 2 and 3) of a word as a pair of binary16 values.
+template <bool HIGH>
+SA_D uint32_t fp8_to_half2(uint32_t f) {
+    uint32_t h;
+    if constexpr (HIGH) asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; cvt.rn.f16x2.e4m3x2 %0, h;}" : "=r"(h) : "r"(f));
+    else asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; cvt.rn.f16x2.e4m3x2 %0, l;}" : "=r"(h) : "r"(f));
+    return h;
+}
+// Even (ODD: odd) elements of a word of nibbles (sign << 3 | g) as FP8 powers of two with their signs.
+template <bool ODD>
+SA_HD uint32_t nibble_codes_to_fp8(uint32_t w) {
+    return ODD ? ((w & 0x80808080u) | ((w >> 1) & 0x38383838u)) : (((w << 4) & 0x80808080u) | ((w << 3) & 0x38383838u));
+}
+// The mantissa bits of the even elements in a byte of a bit plane (odd ones: of the byte >> 1), bit 2 i to bit AT of byte
+// i: the product places copies of the byte at offsets 6 apart, the mask keeps the wanted bit of each.
+template <int AT>
+SA_HD uint32_t plane_bits(uint32_t p) {
+    return ((p & 0x55u) * (0x00041041u << AT)) & (0x01010101u << AT);
 }
 // INT8 values of two keys of one dimension (bytes 0 and 2, ODD: 1 and 3) as a pair of binary16 values: the biased byte
 // v + 128 in the low mantissa bits of 1024, minus 1152 (exact).
@@ -136,42 +160,43 @@ struct ScoreMma {
             for (int i = 0; i < E; ++i) x[k][i] = __half2float(__float2half_rn(__fmul_rn(x[k][i], scale)));
     }
 
+    SA_D static uint32_t b4(int a, int b, int c, int d) {
+        return (uint32_t)(a & 0xff) | ((uint32_t)(b & 0xff) << 8) | ((uint32_t)(c & 0xff) << 16) | ((uint32_t)d << 24);
+    }
     SA_D static uint32_t h2(int lo, int hi) {                     // |integers| <= 127: exact
         const __half2 h = __floats2half2_rn((float)lo, (float)hi);
         return *reinterpret_cast<const uint32_t*>(&h);
     }
-    SA_D static uint32_t b4(int a, int b, int c, int d) {
-        return (uint32_t)(a & 0xff) | ((uint32_t)(b & 0xff) << 8) | ((uint32_t)(c & 0xff) << 16) | ((uint32_t)d << 24);
-    }
     // The order of the elements along the contraction: that of tile() below.
     SA_D void pack(const int (&v)[CH][E]) {
-        if constexpr (FMT == FMT_BYTE) {
 #pragma unroll
-            for (int k = 0; k < CH; ++k) {
+        for (int k = 0; k < CH; ++k) {
+            if constexpr (FMT == FMT_BYTE) {
                 q[2 * k] = h2(v[k][0], v[k][2]);
                 q[2 * k + 1] = h2(v[k][1], v[k][3]);
-            }
-        } else if constexpr (FMT == FMT_INT8) {
-#pragma unroll
-            for (int k = 0; k < CH; ++k) q[k] = b4(v[k][0], v[k][1], v[k][2], v[k][3]);
-        } else if constexpr (FMT == FMT_NIBBLE) {
-#pragma unroll
-            for (int k = 0; k < CH; ++k)
+            } else if constexpr (FMT == FMT_BYTE3) {
+                q[2 * k] = h2(v[k][0], v[k][1]);
+                q[2 * k + 1] = h2(v[k][2], v[k][3]);
+            } else if constexpr (FMT == FMT_INT8) {
+                q[k] = b4(v[k][0], v[k][1], v[k][2], v[k][3]);
+            } else if constexpr (FMT == FMT_NIBBLE) {
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
                     q[2 * k + i] = b4(v[k][4 * i], v[k][4 * i + 1], v[k][4 * i + 2], v[k][4 * i + 3]);
                     qn[2 * k + i] = b4(-v[k][4 * i], -v[k][4 * i + 1], -v[k][4 * i + 2], -v[k][4 * i + 3]);
                 }
-        } else {                                                  // planar: the same element of two chunks side by side
+            } else {
 #pragma unroll
-            for (int k = 0; k < CH; k += 2)
-#pragma unroll
-                for (int n = 0; n < 8; ++n) q[k * 4 + n] = h2(v[k][n], v[k + 1][n]);
+                for (int i = 0; i < 2; ++i) {                     // even, then odd elements
+                    q[4 * k + 2 * i] = h2(v[k][i], v[k][2 + i]);
+                    q[4 * k + 2 * i + 1] = h2(v[k][4 + i], v[k][6 + i]);
+                }
+            }
         }
     }
 
     // Scores of the 32 keys of a staged tile: sc[j][e], j = 2 t + h: key 16 t + 8 h + r, query 2 c + e, in units of
-    // 2^-(14 + k) (integer formats: 1).  st: shared address of the tile's codes; planes: its mantissa bit planes.
+    // 2^-(6 + k) (PoT-M4: 2^-18; integer formats: 1).  st: shared address of the tile's codes; planes: its mantissa bit planes.
     // hi[][]: the part of dimensions 64 .. 127 of NACC == 2 (not yet added).
     SA_D void tile(uint32_t st, uint32_t planes, int lane, float (&sc)[4][2], float (&hi)[NACC == 2 ? 4 : 1][2]) const {
         const uint32_t row = st + lane * 16;
@@ -205,43 +230,51 @@ struct ScoreMma {
                 for (int e = 0; e < 4; ++e) sc[2 * t + (e >> 1)][e & 1] = (float)d[t][e];      // below 2^24: exact
         } else {
             float d[2 * NACC][4] = {};
-            if constexpr (FMT == FMT_BYTE) {
+            if constexpr (!kDense) {
 #pragma unroll
                 for (int k = 0; k < CH; ++k) {
                     uint32_t w[4];
                     ldmatrix_x4(w, row + k * 512);
 #pragma unroll
-                    for (int t = 0; t < 2; ++t)
-                        mma_f16_16816(d[(NACC == 2 && k >= CH / 2 ? 2 : 0) + t], byte_codes_to_half2<false>(w[2 * t]),
-                                      byte_codes_to_half2<false>(w[2 * t + 1]), byte_codes_to_half2<true>(w[2 * t]),
-                                      byte_codes_to_half2<true>(w[2 * t + 1]), q[2 * k], q[2 * k + 1]);
+                    for (int t = 0; t < 2; ++t) {
+                        float(&acc)[4] = d[(NACC == 2 && k >= CH / 2 ? 2 : 0) + t];
+                        if constexpr (FMT == FMT_BYTE) {
+                            mma_f16_16816(acc, byte_codes_to_half2<false>(w[2 * t]), byte_codes_to_half2<false>(w[2 * t + 1]),
+                                          byte_codes_to_half2<true>(w[2 * t]), byte_codes_to_half2<true>(w[2 * t + 1]), q[2 * k], q[2 * k + 1]);
+                        } else {
+                            const uint32_t f0 = byte_codes_to_fp8(w[2 * t]), f1 = byte_codes_to_fp8(w[2 * t + 1]);
+                            mma_f16_16816(acc, fp8_to_half2<false>(f0), fp8_to_half2<false>(f1), fp8_to_half2<true>(f0), fp8_to_half2<true>(f1),
+                                          q[2 * k], q[2 * k + 1]);
+                        }
+                    }
                 }
             } else {
-                constexpr int KB = FMT == FMT_PLANAR1 ? 1 : 2;
-                const int c = lane & 3;
-                const uint32_t psel = (uint32_t)c | ((uint32_t)(4 + c) << 8);
 #pragma unroll
-                for (int k = 0; k < CH; k += 2) {
-                    uint32_t w0[4], w1[4];
-                    ldmatrix_x4(w0, row + k * 512);
-                    ldmatrix_x4(w1, row + (k + 1) * 512);
+                for (int k = 0; k < CH; ++k) {
+                    uint32_t w[4];
+                    ldmatrix_x4(w, row + k * 512);
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
-                        uint32_t f[2][8];
+                        uint32_t f[2][2];                                      // [key r / r + 8 of the half][even / odd elements]
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const int j = 2 * t + h;
-                            uint32_t pl[KB];
-#pragma unroll
-                            for (int b = 0; b < KB; ++b) {
-                                const uint2 p = lds_u32x2(planes + (b * 32 + 8 * j + (lane >> 2)) * (D / 8) + k * 4);
-                                pl[b] = __byte_perm(p.x, p.y, psel);           // bit n: element n of the two chunks
+                            f[h][0] = nibble_codes_to_fp8<false>(w[j]);
+                            f[h][1] = nibble_codes_to_fp8<true>(w[j]);
+                            const uint32_t pa = planes + (8 * j + (lane >> 2)) * (D / 8) + 4 * k + (lane & 3);
+                            uint32_t p = lds_u8(pa);
+                            f[h][0] |= plane_bits<FMT == FMT_PLANAR1 ? 2 : 1>(p);
+                            f[h][1] |= plane_bits<FMT == FMT_PLANAR1 ? 2 : 1>(p >> 1);
+                            if constexpr (FMT == FMT_PLANAR2) {
+                                p = lds_u8(pa + 32 * (D / 8));
+                                f[h][0] |= plane_bits<2>(p);
+                                f[h][1] |= plane_bits<2>(p >> 1);
                             }
-                            planar(f[h], __byte_perm(w0[j], w1[j], 0x5410), __byte_perm(w0[j], w1[j], 0x7632), pl);
                         }
 #pragma unroll
-                        for (int n = 0; n < 8; n += 2)
-                            mma_f16_16816(d[t], f[0][n], f[1][n], f[0][n + 1], f[1][n + 1], q[k * 4 + n], q[k * 4 + n + 1]);
+                        for (int i = 0; i < 2; ++i)
+                            mma_f16_16816(d[t], fp8_to_half2<false>(f[0][i]), fp8_to_half2<false>(f[1][i]), fp8_to_half2<true>(f[0][i]),
+                                          fp8_to_half2<true>(f[1][i]), q[4 * k + 2 * i], q[4 * k + 2 * i + 1]);
                     }
                 }
             }
@@ -260,21 +293,6 @@ private:
         uint32_t d;
         asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(0x04020100u), "r"(0x40201008u), "r"(w));
         return d;
-    }
-    template <int KB>
-    SA_D static void planar(uint32_t (&f)[8], uint32_t lo, uint32_t hi, const uint32_t (&pl)[KB]) {
-        f[0] = nibble_codes_to_half2<0>(lo);
-        f[1] = nibble_codes_to_half2<1>(lo);
-        f[2] = nibble_codes_to_half2<2>(lo);
-        f[3] = nibble_codes_to_half2<3>(lo);
-        f[4] = nibble_codes_to_half2<0>(hi);
-        f[5] = nibble_codes_to_half2<1>(hi);
-        f[6] = nibble_codes_to_half2<2>(hi);
-        f[7] = nibble_codes_to_half2<3>(hi);
-#pragma unroll
-        for (int n = 0; n < 8; ++n)
-#pragma unroll
-            for (int b = 0; b < KB; ++b) f[n] |= (pl[b] << (10 - KB + b - n)) & (0x02000200u >> (KB - 1 - b));
     }
 };
 
