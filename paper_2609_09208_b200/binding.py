@@ -171,9 +171,9 @@ def append_kv(cfg, cache: SaCache, K_new, V_new, bump_lens: bool = True):
 def fill_kv(cfg, cache: SaCache, K, V, cu_lens_host):
     """cu_lens_host: numpy int64 array of batch + 1 entries (host memory)."""
     import numpy as np
-    cu = np.ascontiguousarray(cu_lens_host, dtype=np.int64)
-    _check(lib().sa_fill_kv(C.byref(cfg), C.byref(cache), _ptr(K), _ptr(V),
-                            cu.ctypes.data_as(C.c_void_p), _stream()), "sa_fill_kv")
+    st = (_nat or native()).fill_kv(cfg, cache, K, V, np.ascontiguousarray(cu_lens_host, dtype=np.int64))
+    if st:
+        raise SaError(st, "sa_fill_kv")
 
 
 def decode_attention(cfg, cache: SaCache, Q, O, workspace, dbg_scores=None, stages: int = 3):

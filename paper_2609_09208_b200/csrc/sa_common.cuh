@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/sa.h"
 
@@ -103,35 +104,55 @@ SA_HD void half_normalise(uint32_t mag_bits, int* M, int* X) {
     }
 }
 
-// Code of one key element (section II-A, II-D): `a_bits` the element's binary16 bits, `s_bits`
-// the magnitude bits of the vector's scale (the largest magnitude in the vector), K the number of
-// mantissa bits.  Returns the canonical byte.  Integer arithmetic only, hence exact:
+SA_HD uint32_t float_bits(float x) {
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    uint32_t u;
+    memcpy(&u, &x, 4);
+    return u;
+#endif
+}
+// A key vector's scale (binary16 bits of its largest magnitude) as the encoder uses it.
+struct KeyScale {
+    uint32_t M, MM;           // s = M * 2^X with M in [1024, 2047]; M^2
+    float inv;                // 1 / s (0 for an all-zero vector)
+};
+SA_HD KeyScale key_scale(uint32_t s_bits) {
+    const float s = __half2float(__ushort_as_half((unsigned short)(s_bits & 0x7fffu)));      // exact, normalised
+    KeyScale k;
+    k.M = ((float_bits(s) >> 13) & 0x3ffu) | 0x400u;
+    k.MM = k.M * k.M;
+    k.inv = s > 0.0f ? 1.0f / s : 0.0f;
+    return k;
+}
+// Code of one key element (section II-A, II-D), `a_bits` the element's binary16 bits, K the number of mantissa bits, as
+// the magnitude's place on the grid: g 2^K + j (g = 7 - e) for the codeword (1 + j/2^K) 2^-e, below 2^K: the zero code.
 //   u = a/s = rho * 2^-e0 with rho in [1, 2);  j = floor((rho - 1) 2^K);  with n = 2^K + j the
 //   neighbours on the grid are n and n + 1 (in units of 2^(-K-e0)), and the upper one is nearer
 //   in log2 exactly when rho^2 4^K >= n (n + 1).
-SA_HD uint8_t encode_element_k(int K, uint32_t a_bits, uint32_t s_bits) {
-    const uint32_t mag = a_bits & 0x7fffu;
-    if (mag == 0) return 0x70;
-    int Ma, Xa, Ms, Xs;
-    half_normalise(mag, &Ma, &Xa);
-    half_normalise(s_bits & 0x7fffu, &Ms, &Xs);
-    int e0 = Xs - Xa;
-    uint32_t num = (uint32_t)Ma;
-    if (Ma < Ms) { e0 += 1; num <<= 1; }
-    if (e0 > 8) return 0x70;                       // far below the grid; also keeps e0 small
-    uint32_t j = ((num - (uint32_t)Ms) << K) / (uint32_t)Ms;
-    const unsigned long long n = (1u << K) + j;
-    const unsigned long long lhs = (unsigned long long)num * num << (2 * K);
-    const unsigned long long rhs = n * (n + 1) * (unsigned long long)Ms * (unsigned long long)Ms;
-    if (lhs >= rhs) {
-        ++j;
-        if (j == (1u << K)) { j = 0; --e0; }
-    }
-    if (e0 >= 7) return 0x70;
-    return (uint8_t)(((a_bits >> 15) << 7) | ((uint32_t)e0 << 4) | (j << (4 - K)));
+// e0 and j are the exponent field and the leading mantissa bits of an FP32 quotient: rho 2^K is a whole number or at least
+// 1 / 2047 (relative 2^-16) from one, the quotient is within two units in the last place, so raising it by sixteen (2^-19)
+// decides both cases.  The comparison is exact: rho = num / M with num = Ma or 2 Ma, num < 2^12, and both sides fit 32 bits
+// (n (n + 1) <= 992, M^2 < 2^22).
+SA_HD uint32_t encode_place(int K, uint32_t a_bits, const KeyScale& s) {
+    const float a = __half2float(__ushort_as_half((unsigned short)(a_bits & 0x7fffu)));
+    const uint32_t rb = float_bits(a * s.inv) + 16u;
+    const uint32_t place = rb >> (23 - K);                    // (exponent field, j)
+    const uint32_t n = (place & ((1u << K) - 1u)) | (1u << K);
+    const uint32_t Ma = ((float_bits(a) >> 13) & 0x3ffu) | 0x400u;
+    const uint32_t num = Ma < s.M ? 2u * Ma : Ma;
+    const int p = (int)place - (120 << K) + (num * num << (2 * K) >= (n * n + n) * s.MM ? 1 : 0);
+    return (uint32_t)(p < 0 ? 0 : p);
+}
+// ... as the canonical byte.
+SA_HD uint8_t encode_element_k(int K, uint32_t a_bits, const KeyScale& s) {
+    const uint32_t p = encode_place(K, a_bits, s);
+    if (p < (1u << K)) return 0x70;
+    return (uint8_t)(((a_bits >> 8) & 0x80u) | ((7u - (p >> K)) << 4) | ((p & ((1u << K) - 1u)) << (4 - K)));
 }
 template <int K>
-SA_HD uint8_t encode_element(uint32_t a_bits, uint32_t s_bits) { return encode_element_k(K, a_bits, s_bits); }
+SA_HD uint8_t encode_element(uint32_t a_bits, uint32_t s_bits) { return encode_element_k(K, a_bits, key_scale(s_bits)); }
 
 // Power-of-two exponent g of the value scale: the largest g with amax * 2^g <= 127
 // (section II-E).  amax = M * 2^X, so amax * 2^g <= 127  <=>  M * 2^(X + g + 4) <= 2032.

@@ -90,19 +90,167 @@ __global__ void __launch_bounds__(128) append_kernel(CacheArgs a, const uint16_t
     if (ok && bump && threadIdx.x == 0) a.seq_lens[b] = len + 1;
 }
 
-// sa_fill_kv: tokens row0 .. row0 + T - 1 of the flat K/V arrays are sequence b's tokens 0 .. T-1.
-template <int D, int MODE>
-__global__ void __launch_bounds__(128) fill_kernel(CacheArgs a, const uint16_t* __restrict__ Kin,
-                                                   const uint16_t* __restrict__ Vin, int b, int64_t row0,
-                                                   int T) {
+// sa_fill_kv.  One warp takes the keys or the values of one KV head for the 32 tokens of half a page, lane = token: a
+// thread has its whole head vector in registers (no shuffles for the largest magnitude or the rotation), and as the chunks of
+// the 32 tokens follow one another in the page, the warp's stores are 512 contiguous bytes per chunk.  (A warp per
+// vector wrote two bytes per lane and encoded with 64-bit products and a division: 41 us for the four prompts of
+// 18 384 tokens x 4 heads, now bound by the instructions of the encoder.)  All sequences of a call go in one launch.
+constexpr int kFillBatch = 64;            // sequences per launch
+struct FillSeqs {
+    int64_t row0[kFillBatch];             // first row of the sequence in K / V
+    int tiles[kFillBatch + 1];            // 32-token tiles ahead of it
+    int len[kFillBatch];
+    int b0, n;                            // sequences b0 .. b0 + n - 1
+};
+
+// Walsh-Hadamard rotation of a whole head vector in one thread, as hadamard_warp (the same butterflies in the same order).
+template <int D>
+SA_D void hadamard_thread(uint32_t (&h)[D / 2]) {
+    float x[D];
+#pragma unroll
+    for (int i = 0; i < D / 2; ++i) {
+        x[2 * i] = half_bits_to_float(h[i] & 0xffffu);
+        x[2 * i + 1] = half_bits_to_float(h[i] >> 16);
+    }
+#pragma unroll
+    for (int st = 1; st < D; st <<= 1)
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+            if ((i & st) == 0) {
+                const float a = x[i], b = x[i + st];
+                x[i] = __fadd_rn(a, b);
+                x[i + st] = __fsub_rn(a, b);
+            }
+    const float scale = (D == 64) ? 0.125f : 0.088388346f;
+#pragma unroll
+    for (int i = 0; i < D / 2; ++i)
+        h[i] = (uint32_t)__half_as_ushort(__float2half_rn(__fmul_rn(x[2 * i], scale))) |
+               ((uint32_t)__half_as_ushort(__float2half_rn(__fmul_rn(x[2 * i + 1], scale))) << 16);
+}
+
+// The vector of one token -> its place in the half page `half` (t: token within it).
+template <int D, int MODE, bool HAD>
+SA_D void fill_keys(uint8_t* half, const CacheArgs& a, int t, uint32_t (&h)[D / 2]) {
+    constexpr bool NIB = MODE >= 8 && MODE <= 10;
+    constexpr int K = MODE == 32 ? 8 : NIB ? MODE - 8 : MODE;
+    if constexpr (HAD) hadamard_thread<D>(h);
+    uint32_t top = 0;                                         // two magnitudes at a time; they order like their bits
+#pragma unroll
+    for (int i = 0; i < D / 2; ++i) top = __vmaxu2(top, h[i] & 0x7fff7fffu);
+    const uint32_t smax = max(top & 0xffffu, top >> 16);
+    const KeyScale ks = key_scale(smax);
+    const float amax = half_bits_to_float(smax);
+    const float inv8 = (K == 8 && amax != 0.0f) ? __fdiv_rn(127.0f, amax) : 0.0f;
+    auto code = [&](int m) -> uint32_t {                      // physical byte (sub-byte containers: canonical byte ^ 0x70)
+        const uint32_t bits = (m & 1) ? h[m >> 1] >> 16 : h[m >> 1] & 0xffffu;
+        if constexpr (K == 8) {
+            const int r = __float2int_rn(__fmul_rn(half_bits_to_float(bits), inv8));
+            return (uint32_t)max(-127, min(127, r)) & 0xffu;
+        } else {
+            const uint32_t p = encode_place(K, bits, ks), sign = (bits >> 8) & 0x80u, j = p & ((1u << K) - 1u);
+            const uint32_t c = NIB ? sign | ((p >> K) << 4) | (j << (4 - K)) : sign | (j << (7 - K)) | (p >> K);
+            return p < (1u << K) ? 0u : c;
+        }
+    };
+    if constexpr (!NIB) {
+#pragma unroll
+        for (int c = 0; c < D / 16; ++c) {
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                w[i] = code(16 * c + 4 * i) | (code(16 * c + 4 * i + 1) << 8) | (code(16 * c + 4 * i + 2) << 16) | (code(16 * c + 4 * i + 3) << 24);
+            *reinterpret_cast<uint4*>(half + a.kcode_off + (size_t)(c * kTileTokens + t) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    } else {
+        uint32_t plane[K > 0 && K < 8 ? K : 1][D / 32] = {};
+#pragma unroll
+        for (int c = 0; c < D / 32; ++c) {
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                w[i] = 0u;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t x = code(32 * c + 8 * i + e);
+                    w[i] |= (x >> 4) << (4 * e);
+                    if constexpr (K > 0)
+#pragma unroll
+                        for (int bit = 0; bit < K; ++bit) plane[bit][c] |= ((x >> (4 - K + bit)) & 1u) << (8 * i + e);
+                }
+            }
+            *reinterpret_cast<uint4*>(half + a.kcode_off + (size_t)(c * kTileTokens + t) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        if constexpr (K > 0)
+#pragma unroll
+            for (int bit = 0; bit < K; ++bit)
+#pragma unroll
+                for (int c = 0; c < D / 32; c += 2)
+                    *reinterpret_cast<uint2*>(half + a.plane_off + (size_t)(bit * kTileTokens + t) * (D / 8) + 4 * c) = make_uint2(plane[bit][c], plane[bit][c + 1]);
+    }
+    *reinterpret_cast<uint16_t*>(half + a.meta_off + (size_t)t * 4) = (uint16_t)smax;
+}
+template <int D>
+SA_D void fill_values(uint8_t* half, const CacheArgs& a, int t, const uint32_t (&h)[D / 2]) {
+    uint32_t top = 0;
+#pragma unroll
+    for (int i = 0; i < D / 2; ++i) top = __vmaxu2(top, h[i] & 0x7fff7fffu);
+    const int g = value_exponent(max(top & 0xffffu, top >> 16));
+    const float f = pow2i(g);
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c) {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            w[i] = 0u;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const uint32_t x = h[8 * c + 2 * i + (e >> 1)], bits = (e & 1) ? x >> 16 : x & 0xffffu;
+                w[i] |= ((uint32_t)__float2int_rn(__fmul_rn(half_bits_to_float(bits), f)) & 0xffu) << (8 * e);
+            }
+        }
+        *reinterpret_cast<uint4*>(half + a.v_off + (size_t)(c * kTileTokens + t) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    *reinterpret_cast<uint16_t*>(half + a.meta_off + (size_t)t * 4 + 2) = (uint16_t)(g & 0xff);
+}
+
+template <int D, int MODE, bool HAD>                          // HAD on its own: the rotation needs twice the registers
+__global__ void __launch_bounds__(128) fill_kernel(CacheArgs a, const uint16_t* __restrict__ Kin, const uint16_t* __restrict__ Vin,
+                                                   const __grid_constant__ FillSeqs seqs) {
     const int lane = threadIdx.x & 31;
-    const int64_t v = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);   // (token, head) vector index
-    if (v >= (int64_t)T * a.Hkv) return;
-    const int t = (int)(v / a.Hkv), h = (int)(v % a.Hkv);
-    uint8_t* block = page_block(a, b, t / kPageTokens, h);
-    if (!block) return;
-    const size_t row = ((size_t)(row0 + t) * a.Hkv + h) * D;
-    write_token<D, MODE>(block, a, t % kPageTokens, lane, Kin + row, Vin + row);
+    const int64_t unit = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);        // (tile, head, keys or values)
+    const int tile = (int)(unit / (2 * a.Hkv)), rest = (int)(unit % (2 * a.Hkv));
+    const int head = rest >> 1;
+    if (tile >= seqs.tiles[seqs.n]) return;
+    int i = 0;                                                                // the sequence: the last one that starts at or before the tile
+    for (int j0 = 0; j0 < seqs.n; j0 += 32) {
+        const int j = j0 + lane;
+        i += __popc(__ballot_sync(0xffffffffu, j < seqs.n && seqs.tiles[j + 1] <= tile));
+    }
+    const int t = (tile - seqs.tiles[i]) * kTileTokens;                       // first token
+    pdl_wait();                                                               // earlier kernels may read this cache or write the inputs
+    pdl_launch_dependents();
+    uint8_t* block = page_block(a, seqs.b0 + i, t / kPageTokens, head);
+    if (!block || t + lane >= seqs.len[i]) return;
+    uint8_t* half = block + (size_t)((t % kPageTokens) >> 5) * (a.page_bytes >> 1);
+    const uint4* src = reinterpret_cast<const uint4*>(((rest & 1) ? Vin : Kin) + ((size_t)(seqs.row0[i] + t + lane) * a.Hkv + head) * D);
+    uint32_t h[D / 2];
+#pragma unroll
+    for (int k = 0; k < D / 8; ++k) {
+        const uint4 v = __ldg(src + k);
+        h[4 * k] = v.x;
+        h[4 * k + 1] = v.y;
+        h[4 * k + 2] = v.z;
+        h[4 * k + 3] = v.w;
+    }
+    if constexpr (MODE == 16) {                                               // unquantised: 16-byte chunks of 8 elements
+        uint8_t* dst = half + ((rest & 1) ? a.v_off : a.kcode_off);
+#pragma unroll
+        for (int k = 0; k < D / 8; ++k)
+            *reinterpret_cast<uint4*>(dst + (size_t)(k * kTileTokens + lane) * 16) = make_uint4(h[4 * k], h[4 * k + 1], h[4 * k + 2], h[4 * k + 3]);
+    } else {
+        if (rest & 1) fill_values<D>(half, a, lane, h);
+        else fill_keys<D, MODE, HAD>(half, a, lane, h);
+    }
 }
 
 // sa_debug_unpack
@@ -316,12 +464,22 @@ sa_status sa_fill_kv(const sa_config* cfg, const sa_cache* cache, const uint16_t
     if (!K || !V) return SA_ERR_INVALID_ARG;
     if (!aligned(K, 16) || !aligned(V, 16)) return SA_ERR_ALIGNMENT;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    for (int b = 0; b < a.batch; ++b) {
-        const int64_t row0 = cu_lens_host[b];
-        const int T = (int)(cu_lens_host[b + 1] - row0);
-        if (T == 0) continue;
-        const unsigned grid = (unsigned)(((int64_t)T * a.Hkv + 3) / 4);
-#define CALL(D, M) fill_kernel<D, M><<<grid, 128, 0, s>>>(a, K, V, b, row0, T)
+    for (int b0 = 0; b0 < a.batch; b0 += kFillBatch) {
+        FillSeqs seqs{};
+        seqs.b0 = b0;
+        seqs.n = a.batch - b0 < kFillBatch ? a.batch - b0 : kFillBatch;
+        for (int i = 0; i < seqs.n; ++i) {
+            seqs.row0[i] = cu_lens_host[b0 + i];
+            seqs.len[i] = (int)(cu_lens_host[b0 + i + 1] - cu_lens_host[b0 + i]);
+            seqs.tiles[i + 1] = seqs.tiles[i] + (seqs.len[i] + kTileTokens - 1) / kTileTokens;
+        }
+        const int64_t units = (int64_t)seqs.tiles[seqs.n] * 2 * a.Hkv;
+        if (units == 0) continue;
+        if ((units + 3) / 4 > 0x7fffffffLL) return SA_ERR_CAPACITY;
+        const unsigned grid = (unsigned)((units + 3) / 4);
+#define CALL(D, M)                                                                               \
+    if (M != 16 && a.hadamard) (void)launch_pdl(fill_kernel<D, M, M != 16>, dim3(grid), dim3(128), 0, s, a, K, V, seqs);        \
+    else (void)launch_pdl(fill_kernel<D, M, false>, dim3(grid), dim3(128), 0, s, a, K, V, seqs)
         SA_DISPATCH_D_MODE(p, CALL);
 #undef CALL
         if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;

@@ -171,7 +171,27 @@ PyObject* append_kv(PyObject*, PyObject* const* v, Py_ssize_t n) {
     SA_RETURN(sa_append_kv(cfg, cache, K, V, bump, s));
 }
 
+// (cfg, cache, K, V, cu_lens): cu_lens a contiguous host array of 64-bit integers
+PyObject* fill_kv(PyObject*, PyObject* const* v, Py_ssize_t n) {
+    Args a{v, n};
+    const sa_config* cfg = a.structure<sa_config>();
+    const sa_cache* cache = a.structure<sa_cache>();
+    const uint16_t* K = a.tensor<uint16_t>();
+    const uint16_t* V = a.tensor<uint16_t>();
+    PyObject* o = a.bad ? nullptr : a.next();
+    const sa_stream s = a.stream();
+    Py_buffer cu;
+    if (a.bad || PyObject_GetBuffer(o, &cu, PyBUF_SIMPLE) != 0) return nullptr;
+    sa_status st;
+    Py_BEGIN_ALLOW_THREADS
+    st = sa_fill_kv(cfg, cache, K, V, static_cast<const int64_t*>(cu.buf), s);
+    Py_END_ALLOW_THREADS
+    PyBuffer_Release(&cu);
+    return PyLong_FromLong(st);
+}
+
 PyMethodDef kMethods[] = {
+    {"fill_kv", (PyCFunction)(void (*)(void))fill_kv, METH_FASTCALL, nullptr},
     {"decode_attention", (PyCFunction)(void (*)(void))decode_attention, METH_FASTCALL, nullptr},
     {"decode_attention_fp16", (PyCFunction)(void (*)(void))decode_attention_fp16, METH_FASTCALL, nullptr},
     {"decode_step", (PyCFunction)(void (*)(void))decode_step, METH_FASTCALL, nullptr},

@@ -48,8 +48,9 @@ SA_D uint32_t encode_key_vec(uint32_t (&bits)[EPL], int lane, bool hadamard, uin
 #pragma unroll
     for (int i = 0; i < EPL; ++i) smax = max(smax, bits[i] & 0x7fffu);   // binary16 magnitudes order like their bits
     smax = warp_max_u32(smax);
+    const KeyScale s = key_scale(smax);
 #pragma unroll
-    for (int i = 0; i < EPL; ++i) codes[i] = encode_element_k(K >= 0 ? K : k, bits[i], smax);
+    for (int i = 0; i < EPL; ++i) codes[i] = encode_element_k(K >= 0 ? K : k, bits[i], s);
     return smax;
 }
 
