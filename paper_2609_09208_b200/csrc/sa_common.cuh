@@ -36,6 +36,7 @@ struct KernelShape {
 constexpr KernelShape mma_shape(int d, int kb) {
     return d == 128 ? KernelShape{6, 2, 2} : (kb == 1 || kb == 2) ? KernelShape{4, 4, 2} : KernelShape{8, 2, 2};
 }
+constexpr int kClusterMost = 8;           // blocks of a thread-block cluster
 // Shift-and-add kernels (sa_decode_kernel.cuh): one stage buffer per warp where a second one would cost resident warps
 // (d = 128, where a tile is 8 KB, and PoT-M4 with its 32 KB table of query multiples).
 constexpr KernelShape shift_shape(int d, int kb) {
@@ -61,14 +62,16 @@ struct Plan {
     sa_layout lay;
     size_t plane_off;         // dense planar container: offset of the mantissa bit planes inside a block
     KernelShape shape;        // of the decode kernel that serves this configuration
+    bool matrix;              // that kernel is the one of sa_decode_mma.cuh
 };
 
 sa_status make_plan(const sa_config* cfg, Plan* out);
 // Streaming multiprocessors of the current device (cudaDevAttrMultiProcessorCount, asked once per device; 148,
 // a B200, where no device answers, so that the size queries also work on a machine without a GPU).
 int sm_count();
-// number of splits of the key axis for a cache of this shape, and queries handled per block
-void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt);
+// Number of splits of the key axis for a cache of this shape, and queries handled per block.  cluster (matrix kernel): the
+// splits form one thread-block cluster.
+void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster = nullptr);
 
 // ---------------------------------------------------------------------------------------------
 // Exact helpers (usable on host for unit tests of the arithmetic, and on device).
@@ -265,20 +268,27 @@ SA_D float half_bits_to_float(uint32_t b) { return __half2float(__ushort_as_half
 #endif  // __CUDACC__
 
 #ifdef __CUDACC__
-// Launch with programmatic stream serialisation allowed (see pdl_wait above).
+// Launch with programmatic stream serialisation allowed (see pdl_wait above), in clusters of `cluster` blocks along x.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, unsigned cluster, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+    return launch_pdl_cluster(kernel, grid, block, smem, s, 1u, args...);
 }
 #endif
 

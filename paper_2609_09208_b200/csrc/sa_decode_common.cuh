@@ -44,6 +44,11 @@ struct DecodeArgs {
     // of unequal lengths is cut into (0: every sequence keeps n_splits).  Null / 0 elsewhere.
     int32_t* plan;
     int bal_target;
+    // Matrix kernel, whole: all splits of a sequence form a thread-block cluster (of `cluster` blocks; 1 otherwise), which
+    // merges them into O, and no merge kernel runs.  `counter` (zero between calls) then counts the blocks that have read the
+    // lengths, if the call appends tokens.
+    int cluster, whole;
+    unsigned* counter;
 };
 
 // Batches of 2 .. kRankedBatchMax sequences: which (sequence, split) a block of the grid works on is decided on the
@@ -422,6 +427,15 @@ __global__ void __launch_bounds__(kMergeThreads, 2048 / kMergeThreads) merge_ker
     }
 }
 
+// A counter for calls with this workspace that append tokens and have no merge kernel, or null.
+unsigned* step_counter(const void* workspace, cudaStream_t s);
+// Takes back the one-launch form of a call that appends tokens where no counter is to be had.
+inline void settle_whole(const void* workspace, cudaStream_t s, DecodeArgs* a) {
+    if (a->whole && a->Knew) a->counter = step_counter(workspace, s);
+    if (a->whole && a->Knew && !a->counter) a->whole = 0;
+    if (!a->whole) a->cluster = 1;
+}
+
 sa_status decode_step_impl(const sa_config* cfg, const sa_cache* cache, const uint16_t* Q, const uint16_t* K_new,
                            const uint16_t* V_new, float* O, void* workspace, size_t workspace_bytes, sa_stream stream,
                            bool q_after_wait);
@@ -442,7 +456,8 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     if (mis(c->pages, p.lay.align) || mis(c->page_table, 4) || mis(c->seq_lens, 4) || mis(Q, 16) || mis(O, 16))
         return SA_ERR_ALIGNMENT;
     int S, GT;
-    split_plan(p, c->batch, c->max_pages_per_seq, &S, &GT);
+    bool cluster;
+    split_plan(p, c->batch, c->max_pages_per_seq, &S, &GT, &cluster);
     // the kernels place the splits with 32-bit arithmetic: tiles * (splits + 1) must stay below 2^31
     if ((long long)c->max_pages_per_seq * (kPageTokens / kTileTokens) * (S + 1) >= (1LL << 31)) return SA_ERR_CAPACITY;
     const size_t need = decode_workspace_bytes(p, c->batch, S, with_plan);
@@ -486,6 +501,9 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     a->wait_first = 0;
     a->plan = nullptr;
     a->bal_target = 0;
+    a->cluster = cluster ? S : 1;
+    a->whole = p.matrix && S == a->cluster ? 1 : 0;
+    a->counter = nullptr;
     if (with_plan && batch_is_ranked(c->batch)) {
         a->plan = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)S * c->batch * p.Hq * (p.d + 2) * sizeof(float));
         // blocks per grid row that a batch of unequal lengths is cut into: the grid, rounded down to whole waves of
@@ -500,12 +518,12 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
 }
 
 // Logit scale (the queries' Delta and the keys' s_j still to be multiplied in) of the kernel that serves the plan.
-// matrix: the products of sa_score_mma.cuh, whose sums come in units of 2^-(6 + k) (PoT-M4: 2^-18; INT8, nibbles: 1) whatever F is.
-inline void set_scales(const Plan& p, bool matrix, DecodeArgs* a) {
+// The sums of sa_score_mma.cuh come in units of 2^-(6 + k) (PoT-M4: 2^-18; INT8, nibbles: 1) whatever F is.
+inline void set_scales(const Plan& p, DecodeArgs* a) {
     const double base = 1.4426950408889634 / sqrt((double)p.d);
     if (p.fp16) a->zscale = (float)base;
     else if (p.int8) a->zscale = (float)(base / 127.0);                       // key unit = scale / 127
-    else if (!matrix) a->zscale = (float)(base / (double)(1LL << p.F));
+    else if (!p.matrix) a->zscale = (float)(base / (double)(1LL << p.F));
     else if (p.nibble && p.k == 0) a->zscale = (float)(base / 64.0);
     else {
         a->zscale = (float)(p.k == 4 ? base * 256.0 : base);

@@ -348,7 +348,7 @@ extern "C" sa_status sa_decode_attention_fp16_stages(const sa_config* cfg, const
     int GT;
     st = make_decode_args(p, cache, Q, O, workspace, workspace_bytes, &a, &GT);
     if (st != SA_OK) return st;
-    set_scales(p, false, &a);
+    set_scales(p, &a);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (stages & 1) {
         launch_decode_fp16_main(p, a, GT, s);

@@ -41,15 +41,68 @@ struct MmaSmem {
     static constexpr int kMbarOff = NW * NS * Stage::kBytes;
     static constexpr int kRefOff = kMbarOff + ((NW * NS * 8 + 127) & ~127);
     static constexpr int kBytes = kRefOff + NW * 8 * 4;
-    static_assert(NW * 8 * (D + 2) * 4 <= NW * NS * Stage::kBytes, "merge rows must fit in the stage buffers");
+    static constexpr int kSumOff = NW * 8 * (D + 2) * 4;      // the block's sums, behind the merge rows (within the stage buffers)
+    static_assert(kSumOff + 8 * (D + 2) * 4 <= NW * NS * Stage::kBytes, "merge rows and sums must fit in the stage buffers");
     static_assert(NW * NS * Stage::kBytes >= kPlanScratchInts * 4, "the block plan's scratch must fit in the stage buffers");
     static_assert(Stage::kBytes == half_block_bytes(D, format_kb<FMT>(), SC::kDense), "a stage buffer is a verbatim copy of half a page block");
 };
 
+// The lengths grow by one when the kernel appends the step's tokens and no merge kernel follows: by the hand of the last
+// block to get here, every block having read what it needs of them.  One warp per block.
+SA_D void bump_lengths(const DecodeArgs& a, int lane) {
+    unsigned old = 0;
+    if (lane == 0) old = atomicAdd(a.counter, 1u);
+    if (__shfl_sync(0xffffffffu, old, 0) + 1 != gridDim.x * gridDim.y * gridDim.z) return;
+    if (lane == 0) *a.counter = 0u;
+    for (int b = lane; b < a.batch; b += 32) {
+        const int len = __ldcg(a.seq_lens + b), lp = len / kPageTokens;
+        const int page = (len >= 0 && lp < a.max_pages) ? a.page_table[(size_t)b * a.max_pages + lp] : -1;
+        if (page >= 0 && page < a.n_pages) const_cast<int32_t*>(a.seq_lens)[b] = len + 1;
+    }
+}
+
+// This block's share of the outputs of a cluster (a.cluster blocks, each with its sums {R, l, O[D]} of the query heads at
+// shared address `sums`) -> O.  All loads of an output are in flight together; the blocks are
+// added in order.
+template <int D, int NT>
+SA_D void merge_cluster(const DecodeArgs& a, uint32_t sums, float* O) {
+    constexpr int kMost = kClusterMost;
+    const int C = a.cluster, items = a.gt * (D / 2), per = (items + C - 1) / C, rank = blockIdx.x % C;
+    for (int i = rank * per + threadIdx.x; i < min(items, (rank + 1) * per); i += NT) {
+        const int g = i / (D / 2), col = i % (D / 2);
+        float2 h[kMost], v[kMost];
+        int Rm = kMNone;
+#pragma unroll
+        for (int k = 0; k < kMost; ++k) {
+            h[k] = v[k] = make_float2(0.0f, 0.0f);
+            if (k < C) {
+                const uint32_t row = C > 1 ? cluster_map(sums, k) : sums;
+                h[k] = C > 1 ? lds_cluster_f2(row + g * (D + 2) * 4) : lds_f2(row + g * (D + 2) * 4);
+                v[k] = C > 1 ? lds_cluster_f2(row + (g * (D + 2) + 2 + 2 * col) * 4) : lds_f2(row + (g * (D + 2) + 2 + 2 * col) * 4);
+                Rm = max(Rm, __float_as_int(h[k].x));
+            }
+        }
+        float l = 0.0f, x = 0.0f, y = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kMost; ++k)
+            if (k < C) {
+                const float f = pow2i_neg(__float_as_int(h[k].x) - Rm);            // (a block without a key carries zeros)
+                l += h[k].y * f;
+                x += v[k].x * f;
+                y += v[k].y * f;
+            }
+        // no key at all: zeros; a marked sum (a bounded wait gave up) stays visible as NaN
+        const float inv = l == 0.0f ? 0.0f : 1.0f / l;
+        *reinterpret_cast<float2*>(O + (size_t)g * D + 2 * col) = make_float2(x * inv, y * inv);
+    }
+}
+
 // CODE: the cache-write mode of the fused append (see write_token).  LOST: the test hook that never issues one chosen
 // tile's copy and makes its first plan for another block's coordinates (sa_debug_decode_lost_copy).
-template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST>
-__global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(DecodeArgs a) {
+// WHOLE: the splits of a sequence form one cluster (or there is one split), which merges them (merge_cluster); an
+// instantiation of its own, as the code at the end costs the others 0.1 - 0.3 us.
+template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST, bool WHOLE>
+__global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_constant__ DecodeArgs a) {
     using SM = MmaSmem<D, FMT, NW, NS>;
     using SC = typename SM::SC;
     using Stage = typename SM::Stage;
@@ -119,7 +172,10 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(DecodeArgs a) 
             b = bp.b;
         }
     } while (again);
-    if (ranked && b < 0) return;                                  // more blocks than (sequence, split) pairs
+    if (ranked && b < 0) {                                        // more blocks than (sequence, split) pairs
+        if (WHOLE && a.counter && warp == 0) bump_lengths(a, lane);
+        return;
+    }
 
     // ---- this warp's tiles ----
     int len = ranked ? bp.len : a.seq_lens[b];
@@ -341,6 +397,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(DecodeArgs a) 
     // below from a register, not through the rows, which alias the stage buffers — a copy that was merely late could
     // still land in them.
     const bool poisoned = __syncthreads_or(failed ? 1 : 0) != 0;
+    if (WHOLE && a.counter && warp == 0) bump_lengths(a, lane);   // every warp of the block has read the lengths
     float Rb0 = (float)kMNone, Rb1 = (float)kMNone;
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
@@ -361,7 +418,8 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(DecodeArgs a) 
     }
     __syncthreads();
     const int slot = ranked ? blockIdx.z * a.n_splits + blockIdx.x : blockIdx.x * a.batch + blockIdx.z;
-    float* out = a.partials + ((size_t)slot * a.Hq + h0) * (D + 2);
+    float* sum_s = reinterpret_cast<float*>(smem + SM::kSumOff);                   // [8][D + 2]
+    float* out = WHOLE ? sum_s : a.partials + ((size_t)slot * a.Hq + h0) * (D + 2);
     for (int idx = threadIdx.x; idx < GT * (D + 2); idx += 32 * NW) {
         const int g = idx / (D + 2), col = idx % (D + 2);                          // 0: R, 1: l, 2 ..: O
         float v = 0.0f;
@@ -377,17 +435,29 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(DecodeArgs a) 
         if (poisoned && col <= 1) v = (col == 0) ? __int_as_float(0) : __int_as_float(0x7fc00000);   // R = 0, l = NaN
         out[idx] = v;
     }
+    if constexpr (WHOLE) {
+        if (a.cluster > 1) cluster_sync();
+        else __syncthreads();
+        merge_cluster<D, 32 * NW>(a, smem_addr(sum_s), a.O + ((size_t)b * a.Hq + h0) * D);
+        if (a.cluster > 1) cluster_sync();                                         // no block may leave while others read its sums
+    }
 }
 
-template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST = false>
-static void launch_mma(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
+template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST, bool WHOLE>
+static void launch_mma_as(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     constexpr int bytes = MmaSmem<D, FMT, NW, NS>::kBytes;
     if (bytes > 48 * 1024) {
-        static const cudaError_t once = cudaFuncSetAttribute(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST>,
+        static const cudaError_t once = cudaFuncSetAttribute(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST, WHOLE>,
                                                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         (void)once;
     }
-    (void)launch_pdl(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST>, grid, dim3(32 * NW), (size_t)bytes, s, a);
+    (void)launch_pdl_cluster(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST, WHOLE>, grid, dim3(32 * NW), (size_t)bytes, s,
+                             (unsigned)a.cluster, a);
+}
+template <int D, int FMT, int CODE, int NW, int BPS, int NS>
+static void launch_mma(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
+    if (a.whole) launch_mma_as<D, FMT, CODE, NW, BPS, NS, false, true>(a, grid, s);
+    else launch_mma_as<D, FMT, CODE, NW, BPS, NS, false, false>(a, grid, s);
 }
 
 }  // namespace sa

@@ -17,6 +17,6 @@ void launch_mma_byte(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t 
 }
 void launch_mma_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     constexpr KernelShape sh = mma_shape(64, 4);
-    launch_mma<64, FMT_BYTE, 7, sh.warps, sh.blocks_per_sm, sh.stages, true>(a, grid, s);
+    launch_mma_as<64, FMT_BYTE, 7, sh.warps, sh.blocks_per_sm, sh.stages, true, false>(a, grid, s);
 }
 }  // namespace sa

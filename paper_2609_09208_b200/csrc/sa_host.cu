@@ -45,6 +45,7 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
     if (cfg->code == SA_INT8) {
         if (cfg->klayout != SA_KLAYOUT_BYTE || cfg->headroom_F != 0) return SA_ERR_UNSUPPORTED;
         p.int8 = true;
+        p.matrix = true;
         p.shape = mma_shape(p.d, 8);
         p.k = 0;
         p.F = 0;
@@ -61,7 +62,8 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
     if (cfg->code != SA_POT4 && cfg->code != SA_POTM1 && cfg->code != SA_POTM2 && cfg->code != SA_POTM4)
         return SA_ERR_UNSUPPORTED;
     p.k = cfg->code;
-    p.shape = p.addalu ? shift_shape(p.d, p.k) : mma_shape(p.d, p.k);
+    p.matrix = !p.addalu;
+    p.shape = p.matrix ? mma_shape(p.d, p.k) : shift_shape(p.d, p.k);
     if (cfg->klayout == SA_KLAYOUT_NIBBLE) {
         if (p.k != 0) return SA_ERR_UNSUPPORTED;
         p.nibble = true;
@@ -109,7 +111,7 @@ int sm_count() {
     return cached[dev];
 }
 
-void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt) {
+void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster) {
     int GT = 1;
     for (int c = 8; c >= 1; c >>= 1)
         if (p.G % c == 0) { GT = c; break; }
@@ -118,7 +120,8 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt)
     // launch, fitted to measured sweeps over S, in units of one tile per warp on a full SM:
     //   * a block lasts about  r + c_fix  with r between tiles / (warps S) and its ceiling (warps that
     //     run out of tiles leave their issue slots to the others, but not all of the time), and
-    //     c_fix for the prologue (query quantisation, table) and the block merge;
+    //     c_fix for the prologue (query quantisation, table) and the block merge (the matrix kernel spends 4.4 us on
+    //     them and 1.8 us on a tile per warp: 2.5; 32 x 4096 tokens, d = 128: 76.3 -> 57.2 us against 0.5);
     //   * blocks run in waves of (SMs of the current device) x resident-blocks-per-SM; a last wave whose SMs hold only the
     //     fraction f of that takes 0.1 + 0.9 f of a full wave's time, a single partial wave f^0.2
     //     (an SM's throughput falls almost in proportion to its resident warps).
@@ -128,6 +131,17 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt)
     const int n_sms = sm_count();
     const long long slots = (long long)n_sms * bps;
     const long long tiles = (long long)max_pages * (kPageTokens / 32);
+    // A single sequence that is short: a cluster of 8 blocks per query group, which merges its splits itself.  One launch
+    // instead of two (2.0 us of host time) and no trip of the partials through L2: 1024 tokens of one head 9.4 -> 5.3 us a
+    // call from Python, of 32 / 4 heads 6.2 -> 5.8.  The line is a tile per warp: longer sequences are done sooner on all
+    // SMs and with the merge kernel (PoT-4, 8192 tokens: 8.1 us in clusters, 5.8 without).
+    if (cluster) *cluster = false;
+    if (p.matrix && batch == 1 && tiles <= kClusterMost * nw) {
+        if (cluster) *cluster = true;
+        *n_splits = (int)(tiles / 2 < 1 ? 1 : tiles / 2 > kClusterMost ? kClusterMost : tiles / 2);
+        *gt = GT;
+        return;
+    }
     // Searching S takes 1 - 9 us, as long as a decode call on the GPU, and a program asks for the same few shapes over and
     // over: every thread keeps its last answers.
     struct Kept {
@@ -145,7 +159,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt)
     long long cap = tiles / 2;                      // at least two tiles per block (short caches: spread them over the SMs)
     if (cap < 1) cap = 1;
     if (cap > 512) cap = 512;
-    const double c_fix = 0.5;
+    const double c_fix = p.matrix ? 2.5 : 0.5;
     double best = 0.0;
     long long best_S = 1;
     for (long long S = 1; S <= cap; ++S) {

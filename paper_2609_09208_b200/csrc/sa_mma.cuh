@@ -47,6 +47,25 @@ SA_D uint32_t lds_u8(uint32_t addr) {
     asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
+SA_D float2 lds_f2(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+// Thread-block clusters: barrier over the cluster, shared address of block `rank`, a load from such an address.
+SA_D void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+SA_D uint32_t cluster_map(uint32_t addr, int rank) {
+    uint32_t d;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+    return d;
+}
+SA_D float2 lds_cluster_f2(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
+}
 // Transpose of an 8 x 8 matrix of 16-bit elements held by the warp: in lane (g, t) M[g][2t], M[g][2t + 1];
 // out M[2t][g], M[2t + 1][g].
 SA_D uint32_t movmatrix_trans(uint32_t x) {

@@ -257,6 +257,7 @@ extern "C" sa_status sa_shiftav_workspace_bytes(const sa_config* cfg, int batch,
     const sa_status st = make_plan(cfg, &p);
     if (st != SA_OK) return st;
     if (p.fp16 || p.int8) return SA_ERR_UNSUPPORTED;
+    p.matrix = false;
     p.shape = shift_shape(p.d, p.k);                             // the score pass is the shift-and-add kernel's
     int S, GT;
     split_plan(p, batch, max_pages_per_seq, &S, &GT);
@@ -273,6 +274,7 @@ extern "C" sa_status sa_decode_attention_shiftav(const sa_config* cfg, const sa_
     sa_status st = make_plan(cfg, &p);
     if (st != SA_OK) return st;
     if (p.fp16 || p.int8) return SA_ERR_UNSUPPORTED;
+    p.matrix = false;
     p.shape = shift_shape(p.d, p.k);                             // the score pass is the shift-and-add kernel's
     // INT32 tile accumulator: 32 keys x 128 x 2^N < 2^31
     if (n_bits < 1 || n_bits > 18 || k_max < 0 || k_max > n_bits) return SA_ERR_INVALID_ARG;
@@ -293,7 +295,7 @@ extern "C" sa_status sa_decode_attention_shiftav(const sa_config* cfg, const sa_
     a.stat_g = reinterpret_cast<int32_t*>(ws + go);
     a.n_bits = n_bits;
     a.k_max = k_max;
-    set_scales(p, false, &a);
+    set_scales(p, &a);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     launch_decode_main(p, a, GT, s);                             // pass 1: scores, rounded logits, statistics
     if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;

@@ -72,3 +72,52 @@ def test_outputs_with_a_moving_reference_and_spread_value_scales(d, k, nibble, s
         for h in range(8):
             err = np.linalg.norm(O[b, h] - ref["O"][b, h]) / np.linalg.norm(ref["O"][b, h])
             assert err <= 1e-5, (b, h, err)
+
+
+@pytest.mark.parametrize("d,Hq,Hkv,lens", [(64, 32, 4, [0]), (64, 8, 1, [63]), (64, 32, 4, [1000]), (64, 1, 1, [2046]), (128, 8, 2, [1500]),
+                                           (128, 16, 16, [200 + 7 * i for i in range(40)]), (64, 4, 4, [33] * 130)])
+@pytest.mark.parametrize("k,nibble", [(0, True), (1, False), (4, False)])
+def test_steps_without_a_merge_kernel(d, Hq, Hkv, lens, k, nibble):
+    """Short single sequences (merged by a thread-block cluster) and batches with one split per sequence: several steps in
+    a row without a synchronisation, the lengths counted up by the decode kernel itself; outputs as the oracle's on the
+    extended cache, and as the same steps replayed from a CUDA graph."""
+    import torch
+    sa_build.build()
+    dev = torch.device("cuda:0")
+    up = lambda x: torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).to(dev)
+    lens, n_steps = np.asarray(lens), 3
+    B = len(lens)
+    full = synth.make_case("whole", lens + n_steps, Hq, Hkv, d, k, nibble=nibble, outliers=True, seed=300 + d + k)
+    cfg = sa.make_config(d, Hq, Hkv, k, nibble=nibble)
+    cache = sa.PagedCache(cfg, lens, dev, extra_tokens=n_steps)
+    old = np.concatenate([np.arange(full.cu_lens[b], full.cu_lens[b] + lens[b]) for b in range(B)]).astype(np.int64)
+    cache.fill(up(full.K[old]), up(full.V[old]), np.concatenate([[0], np.cumsum(lens)]))
+    new = [np.array([full.cu_lens[b] + lens[b] + i for b in range(B)]) for i in range(n_steps)]
+    Kn, Vn, Q = [up(full.K[n]) for n in new], [up(full.V[n]) for n in new], up(full.Q)
+    O = [torch.full((B, Hq, d), float("nan"), dtype=torch.float32, device=dev) for _ in range(n_steps)]
+
+    def steps():
+        for i in range(n_steps):
+            sa.decode_step(cfg, cache.handle, Q, Kn[i], Vn[i], O[i], cache.workspace)
+
+    steps()
+    torch.cuda.synchronize()
+    assert cache.seq_lens.cpu().numpy().tolist() == (lens + n_steps).tolist()
+    first = [o.clone() for o in O]
+    for i in range(n_steps):
+        rows = np.concatenate([np.arange(full.cu_lens[b], full.cu_lens[b] + lens[b] + i + 1) for b in range(B)])
+        ref = ora.decode_attention(full.Q, full.K[rows], full.V[rows], np.concatenate([[0], np.cumsum(lens + i + 1)]), k, 6 + k,
+                                   n_threads=8)["O"]
+        assert np.max(np.abs(first[i].cpu().numpy() - ref)) <= 1e-3
+    lens0 = torch.from_numpy(lens.astype(np.int32)).to(dev)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        cache.seq_lens.copy_(lens0)
+        steps()
+    for _ in range(2):
+        for o in O:
+            o.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert cache.seq_lens.cpu().numpy().tolist() == (lens + n_steps).tolist()
+        assert all(torch.equal(a, b) for a, b in zip(O, first))
