@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
 
     SC q;
     float qs0, qs1;             // logit scale (Delta * log2(e) / sqrt(d) * unit of the scores) of queries 2 c, 2 c + 1
-    int b = bp.b, tile_g, pidx_g;
+    int b = bp.b, n_tiles_g, first_g, tile1_g, pidx_g, lp_g, pnew_g;
     bool again;
 #pragma unroll 1
     do {
@@ -153,22 +153,34 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         qs1 = __shfl_sync(0xffffffffu, qs, 8 * c + 4);
         // A guess at this warp's first tile, only to ask L2 for it while the preceding kernel drains (loads that bypass
         // L1, so nothing stale can be read back later).
-        const int n_tiles_g = (min(max(len_g, 0), a.max_pages * kPageTokens) + 31) >> 5;
-        tile_g = split_begin(n_tiles_g, bp.split, bp.n_splits) + warp;
-        if (tile_g >= split_begin(n_tiles_g, bp.split + 1, bp.n_splits)) tile_g = -1;
-        if (tile_g >= 0) {
-            const int p_g = __ldcg(a.page_table + (size_t)bq * a.max_pages + (tile_g >> 1));
+        n_tiles_g = (min(max(len_g, 0), a.max_pages * kPageTokens) + 31) >> 5;
+        first_g = split_begin(n_tiles_g, bp.split, bp.n_splits) + warp;
+        tile1_g = split_begin(n_tiles_g, bp.split + 1, bp.n_splits);
+        lp_g = a.Knew && len_g > 0 ? (len_g - 1) / kPageTokens : -1;          // the new token's page
+        if (lp_g >= a.max_pages) lp_g = -1;
+        if (first_g < tile1_g) {
+            const int p_g = __ldcg(a.page_table + (size_t)bq * a.max_pages + (first_g >> 1));
             if (lane == 0 && p_g >= 0 && p_g < a.n_pages)
-                Stage::prefetch(a.pages + ((size_t)p_g * a.Hkv + kvh) * a.page_bytes, (tile_g & 1) * 32, true);
+                Stage::prefetch(a.pages + ((size_t)p_g * a.Hkv + kvh) * a.page_bytes, (first_g & 1) * 32, true);
         }
         pdl_wait();                 // everything below reads what the preceding kernels in the stream wrote (the cache)
-        // the page of the guessed first tile, read again now that it is valid, at the same time as the length(s)
-        pidx_g = tile_g >= 0 ? a.page_table[(size_t)bq * a.max_pages + (tile_g >> 1)] : -1;
+        // The pages of the guessed first tile and of the new token, read again now that they are valid, at the same time as
+        // the length(s): one round trip where the guess holds, which it does unless a length crossed a tile boundary.  The
+        // warp that is to write the new token asks for its rows as well.
+        const int32_t* table_g = a.page_table + (size_t)bq * a.max_pages;
+        pidx_g = first_g < tile1_g ? table_g[first_g >> 1] : -1;
+        pnew_g = lp_g >= 0 ? table_g[lp_g] : -1;
+        if (lp_g >= 0 && n_tiles_g - 1 >= first_g && n_tiles_g == tile1_g && (n_tiles_g - 1 - first_g) % NW == 0) {
+            const size_t row = ((size_t)bq * a.Hkv + kvh) * D;
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(a.Knew + row + lane * (D / 32)));
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(a.Vnew + row + lane * (D / 32)));
+        }
         again = false;
         if (ranked && !a.wait_first) {                            // the plan that counts; wait_first made it after the wait already
             bp = plan_block(plan_args(a), blockIdx.z, blockIdx.x, !LOST, true, bp, plan_scratch);
             again = bp.b != bq && bp.b >= 0;
-            if (bp.split != split_g || bp.n_splits != nsp_g) tile_g = -1;     // the hint was for other tiles
+            if (bp.split != split_g || bp.n_splits != nsp_g) n_tiles_g = -1;  // the guess was for other tiles
+            if (bp.b != bq) n_tiles_g = lp_g = -1;
             b = bp.b;
         }
     } while (again);
@@ -185,31 +197,19 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         // Fused append: the step's new token goes to position len (if its page is mapped) and is part of this step's
         // attention.  Every block takes the same decision; the split-K merge kernel bumps seq_lens once all have read it.
         const int lp = len / kPageTokens;
-        pidx_new = (len >= 0 && lp < a.max_pages) ? table[lp] : -1;
+        pidx_new = (len >= 0 && lp < a.max_pages) ? (lp == lp_g ? pnew_g : table[lp]) : -1;
         if (pidx_new >= 0 && pidx_new < a.n_pages) {
             tile_new = len >> 5;
             len += 1;
         }
     }
     const int n_tiles = (min(len, a.max_pages * kPageTokens) + 31) >> 5;
-    const int first = split_begin(n_tiles, bp.split, bp.n_splits) + warp;
-    const int tile1 = split_begin(n_tiles, bp.split + 1, bp.n_splits);
+    const bool same = n_tiles == n_tiles_g;                       // the divisions of the guess stand
+    const int first = same ? first_g : split_begin(n_tiles, bp.split, bp.n_splits) + warp;
+    const int tile1 = same ? tile1_g : split_begin(n_tiles, bp.split + 1, bp.n_splits);
     const int n_my = first < tile1 ? (tile1 - first + NW - 1) / NW : 0;
-    if (tile_new >= first && tile_new < tile1 && (tile_new - first) % NW == 0) {      // warp-uniform: this warp owns that tile
-        CacheArgs ca{};
-        ca.page_bytes = a.page_bytes;
-        ca.kcode_off = a.kcode_off;
-        ca.meta_off = a.meta_off;
-        ca.v_off = a.v_off;
-        ca.plane_off = a.plane_off;
-        ca.hadamard = a.hadamard;
-        ca.k = a.k;
-        uint8_t* block = const_cast<uint8_t*>(a.pages) + ((size_t)pidx_new * a.Hkv + kvh) * a.page_bytes;
-        const size_t row = ((size_t)b * a.Hkv + kvh) * D;
-        write_token<D, CODE>(block, ca, (len - 1) % kPageTokens, lane, a.Knew + row, a.Vnew + row);
-        fence_proxy_async_global();
-        __syncwarp();
-    }
+    // which of my tiles is the new token's (warp-uniform; the others' copies start before the token is encoded)
+    const int i_new = (tile_new >= first && tile_new < tile1 && (tile_new - first) % NW == 0) ? (tile_new - first) / NW : -1;
     // Start the copy of my i-th tile, whose page is `pidx`, into stage i % NS; lane 0 keeps which stages hold a mapped
     // tile (one whose page is not mapped gets a plain arrival: the phase completes, the tile is skipped).
     uint32_t mapped = 0u;
@@ -226,11 +226,26 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     };
 #pragma unroll
     for (int i = 0; i < NS; ++i)
-        if (i < n_my) {
-            const int tile = first + NW * i;
-            const int pidx = (tile == tile_g) ? pidx_g : table[tile >> 1];
+        if (i < n_my && i != i_new) {
+            const int pidx = (same && i == 0) ? pidx_g : table[(first + NW * i) >> 1];
             if (lane == 0) issue(i, pidx);
         }
+    if (i_new >= 0) {                                             // encode / quantise the token, write it into its page, copy its tile
+        CacheArgs ca{};
+        ca.page_bytes = a.page_bytes;
+        ca.kcode_off = a.kcode_off;
+        ca.meta_off = a.meta_off;
+        ca.v_off = a.v_off;
+        ca.plane_off = a.plane_off;
+        ca.hadamard = a.hadamard;
+        ca.k = a.k;
+        uint8_t* block = const_cast<uint8_t*>(a.pages) + ((size_t)pidx_new * a.Hkv + kvh) * a.page_bytes;
+        const size_t row = ((size_t)b * a.Hkv + kvh) * D;
+        write_token<D, CODE>(block, ca, (len - 1) % kPageTokens, lane, a.Knew + row, a.Vnew + row);
+        fence_proxy_async_global();
+        __syncwarp();
+        if (lane == 0 && i_new < NS) issue(i_new, pidx_new);
+    }
 
     float R0 = 0.0f, R1 = 0.0f;                    // references of queries 2 c, 2 c + 1 (integers)
     bool seen = false;                             // no key yet: R is not set
@@ -420,20 +435,27 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     const int slot = ranked ? blockIdx.z * a.n_splits + blockIdx.x : blockIdx.x * a.batch + blockIdx.z;
     float* sum_s = reinterpret_cast<float*>(smem + SM::kSumOff);                   // [8][D + 2]
     float* out = WHOLE ? sum_s : a.partials + ((size_t)slot * a.Hq + h0) * (D + 2);
-    for (int idx = threadIdx.x; idx < GT * (D + 2); idx += 32 * NW) {
-        const int g = idx / (D + 2), col = idx % (D + 2);                          // 0: R, 1: l, 2 ..: O
-        float v = 0.0f;
-        if (col == 0) {
-            v = (float)kMNone;
+    for (int idx = threadIdx.x; idx < GT * (D / 2); idx += 32 * NW) {              // two dims of one head
+        const int g = idx / (D / 2), col = idx % (D / 2);
+        float2 v = make_float2(0.0f, 0.0f);
 #pragma unroll
-            for (int w = 0; w < NW; ++w) v = fmaxf(v, ref_s[w * 8 + g]);
-            v = __int_as_float(__float2int_rn(v));
-        } else {
-#pragma unroll
-            for (int w = 0; w < NW; ++w) v += red_s[w][g][col];
+        for (int w = 0; w < NW; ++w) {
+            const float2 x = *reinterpret_cast<const float2*>(&red_s[w][g][2 + 2 * col]);
+            v.x += x.x;
+            v.y += x.y;
         }
-        if (poisoned && col <= 1) v = (col == 0) ? __int_as_float(0) : __int_as_float(0x7fc00000);   // R = 0, l = NaN
-        out[idx] = v;
+        *reinterpret_cast<float2*>(out + g * (D + 2) + 2 + 2 * col) = v;
+    }
+    if (threadIdx.x >= 32 * NW - 8 && 8 - (32 * NW - (int)threadIdx.x) < GT) {     // R and l (by the last warp: it has no more dims than the others)
+        const int g = 8 - (32 * NW - (int)threadIdx.x);
+        float Rm = (float)kMNone, l = 0.0f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            Rm = fmaxf(Rm, ref_s[w * 8 + g]);
+            l += red_s[w][g][1];
+        }
+        *reinterpret_cast<float2*>(out + g * (D + 2)) = poisoned ? make_float2(__int_as_float(0), __int_as_float(0x7fc00000))      // R = 0, l = NaN
+                                                               : make_float2(__int_as_float(__float2int_rn(Rm)), l);
     }
     if constexpr (WHOLE) {
         if (a.cluster > 1) cluster_sync();
