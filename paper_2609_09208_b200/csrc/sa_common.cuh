@@ -36,6 +36,8 @@ struct KernelShape {
 constexpr KernelShape mma_shape(int d, int kb) {
     return d == 128 ? KernelShape{6, 2, 2} : (kb == 1 || kb == 2) ? KernelShape{4, 4, 2} : KernelShape{8, 2, 2};
 }
+// ... over the binary16 cache (tiles of 8 and 16 KB).
+constexpr KernelShape fp16_shape(int d) { return d == 128 ? KernelShape{6, 2, 1} : KernelShape{5, 2, 2}; }
 constexpr int kClusterMost = 8;           // blocks of a thread-block cluster
 // Shift-and-add kernels (sa_decode_kernel.cuh): one stage buffer per warp where a second one would cost resident warps
 // (d = 128, where a tile is 8 KB, and PoT-M4 with its 32 KB table of query multiples).
@@ -46,7 +48,6 @@ constexpr KernelShape shift_shape(int d, int kb) {
            : (kb == 4)          ? KernelShape{8, 2, ns}
                                 : KernelShape{4, 5, ns};
 }
-constexpr KernelShape kFp16Shape{4, 3, 2};
 
 // ---------------------------------------------------------------------------------------------
 // Host-side description of a validated configuration.

@@ -6,11 +6,11 @@
 using namespace sa;
 
 namespace sa {
-void launch_decode_fp16_main(const Plan& p, const DecodeArgs& a, int GT, cudaStream_t s);   // sa_decode_fp16.cu
 void launch_mma_byte(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t s);         // sa_decode_mma_*.cu
 void launch_mma_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_mma_dense(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_mma_int8(int d, const DecodeArgs& a, dim3 grid, cudaStream_t s);
+void launch_mma_fp16(int d, const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_shift_pot4(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);   // sa_decode_pot*.cu
 void launch_shift_potm1(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
 void launch_shift_potm2(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
@@ -21,7 +21,8 @@ void launch_decode_main(const Plan& p, const DecodeArgs& a, int GT, cudaStream_t
     const dim3 grid((unsigned)a.n_splits, (unsigned)(p.Hkv * (p.G / GT)), (unsigned)a.batch);
     const bool sp = a.zr != nullptr;
     if (p.matrix) {
-        if (p.int8) launch_mma_int8(p.d, a, grid, s);
+        if (p.fp16) launch_mma_fp16(p.d, a, grid, s);
+        else if (p.int8) launch_mma_int8(p.d, a, grid, s);
         else if (p.nibble) launch_mma_dense(p.d, p.k, a, grid, s);
         else launch_mma_byte(p.d, p.k, a, grid, s);
     } else if (p.k == 0) launch_shift_pot4(p.nibble, p.d, sp, a, GT, grid, s);
@@ -31,18 +32,13 @@ void launch_decode_main(const Plan& p, const DecodeArgs& a, int GT, cudaStream_t
 }
 }  // namespace sa
 
-extern "C" sa_status sa_decode_attention_stages(const sa_config* cfg, const sa_cache* cache,
-                                                const uint16_t* Q, float* O, void* workspace,
-                                                size_t workspace_bytes, int32_t* dbg_scores, int stages,
-                                                sa_stream stream) {
-    Plan p;
-    sa_status st = make_plan(cfg, &p);
-    if (st != SA_OK) return st;
-    if (p.fp16) return SA_ERR_UNSUPPORTED;
+// Both decode entries: stages 1 = the decode kernel, 2 = the merge of its partials, 3 = a whole call.
+static sa_status decode_stages(const Plan& p, const sa_cache* cache, const uint16_t* Q, float* O, void* workspace,
+                               size_t workspace_bytes, int32_t* dbg_scores, int stages, sa_stream stream) {
     if ((stages & ~3) || stages == 0) return SA_ERR_INVALID_ARG;
     DecodeArgs a;
     int GT;
-    st = make_decode_args(p, cache, Q, O, workspace, workspace_bytes, &a, &GT);
+    const sa_status st = make_decode_args(p, cache, Q, O, workspace, workspace_bytes, &a, &GT);
     if (st != SA_OK) return st;
     if (dbg_scores && (reinterpret_cast<uintptr_t>(dbg_scores) & 3)) return SA_ERR_ALIGNMENT;
     a.dbg_scores = dbg_scores;
@@ -55,6 +51,33 @@ extern "C" sa_status sa_decode_attention_stages(const sa_config* cfg, const sa_c
         if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
     }
     return (stages & 2) && !a.whole ? launch_merge(p, a, s) : SA_OK;
+}
+
+extern "C" sa_status sa_decode_attention_stages(const sa_config* cfg, const sa_cache* cache,
+                                                const uint16_t* Q, float* O, void* workspace,
+                                                size_t workspace_bytes, int32_t* dbg_scores, int stages,
+                                                sa_stream stream) {
+    Plan p;
+    const sa_status st = make_plan(cfg, &p);
+    if (st != SA_OK) return st;
+    if (p.fp16) return SA_ERR_UNSUPPORTED;
+    return decode_stages(p, cache, Q, O, workspace, workspace_bytes, dbg_scores, stages, stream);
+}
+
+extern "C" sa_status sa_decode_attention_fp16_stages(const sa_config* cfg, const sa_cache* cache,
+                                                     const uint16_t* Q, float* O, void* workspace,
+                                                     size_t workspace_bytes, int stages, sa_stream stream) {
+    Plan p;
+    const sa_status st = make_plan(cfg, &p);
+    if (st != SA_OK) return st;
+    if (!p.fp16) return SA_ERR_UNSUPPORTED;
+    return decode_stages(p, cache, Q, O, workspace, workspace_bytes, nullptr, stages, stream);
+}
+
+extern "C" sa_status sa_decode_attention_fp16(const sa_config* cfg, const sa_cache* cache, const uint16_t* Q,
+                                              float* O, void* workspace, size_t workspace_bytes,
+                                              sa_stream stream) {
+    return sa_decode_attention_fp16_stages(cfg, cache, Q, O, workspace, workspace_bytes, 3, stream);
 }
 
 extern "C" sa_status sa_debug_decode_lost_copy(const sa_config* cfg, const sa_cache* cache, const uint16_t* Q, float* O,
@@ -121,8 +144,7 @@ sa_status sa::decode_step_impl(const sa_config* cfg, const sa_cache* cache, cons
     set_scales(p, &a);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     settle_whole(workspace, s, &a);
-    if (p.fp16) launch_decode_fp16_main(p, a, GT, s);
-    else launch_decode_main(p, a, GT, s);
+    launch_decode_main(p, a, GT, s);
     if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
     return a.whole ? SA_OK : launch_merge(p, a, s);
 }

@@ -1,4 +1,4 @@
-// The decode kernel: attention of one query group over a quantised key cache.
+// The decode kernel: attention of one query group over a quantised key cache, or over binary16 keys and values.
 //
 // Grid (split, KV head x query chunk, sequence).  Every warp prepares the block's (up to 8) query heads as matrix
 // fragments in its own registers (ahead of the wait on the preceding kernel), then walks its own 32-key tiles with a
@@ -11,7 +11,7 @@
 //   A.V      O^T[dims][queries] += V^T[dims][keys] w[keys][queries] as m16n8k16 products: INT8 values are exact in
 //            binary16, every weight enters as the sum of two binary16 terms (22 significant bits for weights within
 //            2^-17 of the largest, an absolute 2^-38 of it below), accumulation in FP32.  The weights reach the operand layout
-//            through movmatrix, without shared memory.
+//            through movmatrix, without shared memory.  (Binary16 values: one term, the weights rounded to binary16.)
 // The warps' states and then the blocks' partial results are merged with exact power-of-two factors.  For
 // sa_decode_step the warp that owns the new token's tile writes the token first.
 #pragma once
@@ -37,14 +37,14 @@ template <int D, int FMT, int NW, int NS>
 struct MmaSmem {
     using SC = ScoreMma<D, FMT>;
     static constexpr int PLANES = FMT == FMT_PLANAR1 ? 1 : FMT == FMT_PLANAR2 ? 2 : 0;
-    using Stage = TileStage<SC::CH, true, D, PLANES, D / 8>;
+    using Stage = TileStage<SC::CH, FMT != FMT_FP16, FMT == FMT_FP16 ? 2 * D : D, PLANES, D / 8>;
     static constexpr int kMbarOff = NW * NS * Stage::kBytes;
     static constexpr int kRefOff = kMbarOff + ((NW * NS * 8 + 127) & ~127);
     static constexpr int kBytes = kRefOff + NW * 8 * 4;
     static constexpr int kSumOff = NW * 8 * (D + 2) * 4;      // the block's sums, behind the merge rows (within the stage buffers)
     static_assert(kSumOff + 8 * (D + 2) * 4 <= NW * NS * Stage::kBytes, "merge rows and sums must fit in the stage buffers");
     static_assert(NW * NS * Stage::kBytes >= kPlanScratchInts * 4, "the block plan's scratch must fit in the stage buffers");
-    static_assert(Stage::kBytes == half_block_bytes(D, format_kb<FMT>(), SC::kDense), "a stage buffer is a verbatim copy of half a page block");
+    static_assert(Stage::kBytes == (FMT == FMT_FP16 ? half_block_bytes_fp16(D) : half_block_bytes(D, format_kb<FMT>(), SC::kDense)), "a stage buffer is a verbatim copy of half a page block");
 };
 
 // The lengths grow by one when the kernel appends the step's tokens and no merge kernel follows: by the hand of the last
@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     using SC = typename SM::SC;
     using Stage = typename SM::Stage;
     constexpr int MT = D / 16;                     // 16-dim row tiles of O^T
+    constexpr bool kFp16 = FMT == FMT_FP16;
     constexpr uint32_t kPolls = LOST ? (1u << 10) : kWaitLimit;
     extern __shared__ __align__(1024) uint8_t smem[];
 
@@ -294,6 +295,13 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
             float zq[4][2], vs[4], g[4];                      // logit per score unit; 2^(14 - g_j); g_j
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
+                if constexpr (kFp16) {                        // no scales
+                    g[j] = 0.0f;
+                    vs[j] = (float)(1 << kWeightShift);
+                    zq[j][0] = qs0;
+                    zq[j][1] = qs1;
+                    continue;
+                }
                 const uint32_t meta = lds_u32(st + Stage::kMetaOff + (8 * j + r) * 4);
                 const float sj = half_bits_to_float(meta & 0xffffu);
                 const int gi = (int)(meta << 8) >> 24;        // in [-10, 30] for written tokens
@@ -364,19 +372,43 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
             uint32_t bh[4], bl[4];                            // operand fragments: keys 8 j + 2 c, + 1 of query r
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                l0 += p[j][0];
-                l1 += p[j][1];
                 const __half2 h = __floats2half2_rn(w[j][0], w[j][1]);
                 const float2 hf = __half22float2(h);
-                const __half2 lo = __floats2half2_rn(w[j][0] - hf.x, w[j][1] - hf.y);
                 bh[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&h));
-                bl[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&lo));
+                if constexpr (kFp16) {
+                    // one term; the normaliser sums the same rounded weights, so the result is an exact weighted mean
+                    l0 += hf.x;
+                    l1 += hf.y;
+                } else {
+                    l0 += p[j][0];
+                    l1 += p[j][1];
+                    const __half2 lo = __floats2half2_rn(w[j][0] - hf.x, w[j][1] - hf.y);
+                    bl[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&lo));
+                }
             }
             // ---- A.V: an 8 x 8 block of 16-bit pairs (8 keys x 16 dims of INT8), transposed by ldmatrix: row r of
             // the operand is dim 2 r (bytes 0, 2), row r + 8 dim 2 r + 1 (bytes 1, 3), columns the keys 2 c, 2 c + 1 ----
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt) {
                 uint32_t x[4];
+                if constexpr (kFp16) {                        // binary16 values: chunk 2 mt is rows r (dims 16 mt + r), chunk 2 mt + 1 rows r + 8
+                    uint32_t y[4];
+                    ldmatrix_x4_trans(x, st + Stage::kVOff + 2 * mt * 512 + lane * 16);
+                    ldmatrix_x4_trans(y, st + Stage::kVOff + (2 * mt + 1) * 512 + lane * 16);
+                    if (n_valid < 32) {
+                        // slots past the end may hold anything (even NaN patterns): their weight is zero, but 0 * NaN is not
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int key = 8 * j + 2 * c;
+                            const uint32_t keep = key >= n_valid ? 0u : key + 1 >= n_valid ? 0x0000ffffu : 0xffffffffu;
+                            x[j] &= keep;
+                            y[j] &= keep;
+                        }
+                    }
+                    mma_f16_16816(acc[mt], x[0], y[0], x[1], y[1], bh[0], bh[1]);
+                    mma_f16_16816(acc[mt], x[2], y[2], x[3], y[3], bh[2], bh[3]);
+                    continue;
+                }
                 ldmatrix_x4_trans(x, st + Stage::kVOff + mt * 512 + lane * 16);
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
@@ -420,13 +452,21 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         Rb1 = fmaxf(Rb1, ref_s[w * 8 + 2 * c + 1]);
     }
     const float f0 = seen ? pow2i_neg(__float2int_rn(R0 - Rb0)) : 0.0f, f1 = seen ? pow2i_neg(__float2int_rn(R1 - Rb1)) : 0.0f;
-    if (r == 0) {
-        red_s[warp][2 * c][1] = l0 * f0;
-        red_s[warp][2 * c + 1][1] = l1 * f1;
-    }
     const float v0 = f0 * (1.0f / (1 << kWeightShift)), v1 = f1 * (1.0f / (1 << kWeightShift));
+    if (r == 0) {
+        red_s[warp][2 * c][1] = l0 * (kFp16 ? v0 : f0);
+        red_s[warp][2 * c + 1][1] = l1 * (kFp16 ? v1 : f1);
+    }
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
+        if constexpr (kFp16) {
+            const int dim = 16 * mt + r;
+            red_s[warp][2 * c][2 + dim] = acc[mt][0] * v0;
+            red_s[warp][2 * c][2 + dim + 8] = acc[mt][2] * v0;
+            red_s[warp][2 * c + 1][2 + dim] = acc[mt][1] * v1;
+            red_s[warp][2 * c + 1][2 + dim + 8] = acc[mt][3] * v1;
+            continue;
+        }
         const int dim = 16 * mt + 2 * r;
         *reinterpret_cast<float2*>(&red_s[warp][2 * c][2 + dim]) = make_float2(acc[mt][0] * v0, acc[mt][2] * v0);
         *reinterpret_cast<float2*>(&red_s[warp][2 * c + 1][2 + dim]) = make_float2(acc[mt][1] * v1, acc[mt][3] * v1);

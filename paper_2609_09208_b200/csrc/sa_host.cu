@@ -28,7 +28,8 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
     if (p.fp16) {
         if (cfg->klayout != SA_KLAYOUT_BYTE) return SA_ERR_UNSUPPORTED;
         if (p.hadamard) return SA_ERR_UNSUPPORTED;   // the rotation is a pre-quantisation transform
-        p.shape = kFp16Shape;
+        p.matrix = true;
+        p.shape = fp16_shape(p.d);
         p.k = 0;
         p.nibble = false;
         p.F = 0;

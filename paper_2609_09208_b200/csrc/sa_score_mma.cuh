@@ -14,6 +14,7 @@
 //                             the nibble (the permute's replicate-sign mode over non-negative bytes) turning the
 //                             others into 0; a second lookup with the signs flipped is multiplied by -q.  INT32 sums.
 //   INT8 keys                 as stored.  INT32 sums.
+//   binary16 keys             as stored, with the binary16 query; the sums are rounded like any FP32 sum.
 // So the INT32 scores are those of the shift-and-add datapath (sa_datapath.cuh) bit for bit.  (The decode is what a tile
 // costs most: for four codes 11 instructions in the direct form, 7 by way of FP8.  FP8 operands of the product itself
 // cost more: mma.sync expands them into conversions, again for every product they enter.)
@@ -29,8 +30,8 @@
 
 namespace sa {
 
-// FMT_BYTE3: the byte container of the codes with at most three mantissa bits (all but PoT-M4)
-enum ScoreFormat { FMT_BYTE = 0, FMT_NIBBLE = 1, FMT_PLANAR1 = 2, FMT_PLANAR2 = 3, FMT_INT8 = 4, FMT_BYTE3 = 5 };
+// FMT_FP16: the unquantised cache; FMT_BYTE3: the byte container of the codes with at most three mantissa bits (all but PoT-M4)
+enum ScoreFormat { FMT_BYTE = 0, FMT_NIBBLE = 1, FMT_PLANAR1 = 2, FMT_PLANAR2 = 3, FMT_INT8 = 4, FMT_BYTE3 = 5, FMT_FP16 = 6 };
 
 // Bytes 0 and 2 (ODD: 1 and 3) of a word of the byte container (sign << 7 | mantissa << 3 | g) as a pair of binary16 values:
 // sign 7 -> 15, mantissa 6..3 -> 9..6, g 2..0 -> 12..10 of each half.
@@ -73,12 +74,12 @@ SA_D uint32_t int8_to_half2(uint32_t x) {
 }
 
 // The quantised queries of a block as B fragments in registers of every warp: lane (r, c) prepares query r.
-// E consecutive elements per lane and chunk: 4 (16-element chunks) or 8 (32-element chunks).
+// E consecutive elements per lane and chunk: 2, 4 or 8 (chunks of 8, 16 or 32 elements).
 template <int D, int FMT>
 struct ScoreMma {
     static constexpr bool kInt = (FMT == FMT_NIBBLE || FMT == FMT_INT8);
     static constexpr bool kDense = (FMT == FMT_NIBBLE || FMT == FMT_PLANAR1 || FMT == FMT_PLANAR2);
-    static constexpr int E = kDense ? 8 : 4;
+    static constexpr int E = FMT == FMT_FP16 ? 2 : kDense ? 8 : 4;
     static constexpr int CH = D / (4 * E);                        // code chunks
     static constexpr int NACC = (FMT == FMT_BYTE && D == 128) ? 2 : 1;
     static constexpr int NB = kInt ? D / 16 : D / 8;              // registers of B fragments
@@ -90,6 +91,15 @@ struct ScoreMma {
     // IEEE divide, round half to even.  Returns Delta.
     SA_D float load(const uint16_t* row, int lane, bool hadamard) {
         const int c = lane & 3;
+        if constexpr (FMT == FMT_FP16) {                          // nothing to quantise
+#pragma unroll
+            for (int k = 0; k < CH; ++k) q[k] = row ? *reinterpret_cast<const uint32_t*>(row + k * 8 + c * 2) : 0u;
+            return 1.0f;
+        } else {
+            return quantise(row, c, hadamard);
+        }
+    }
+    SA_D float quantise(const uint16_t* row, int c, bool hadamard) {
         float x[CH][E];
 #pragma unroll
         for (int k = 0; k < CH; ++k)
@@ -230,7 +240,16 @@ struct ScoreMma {
                 for (int e = 0; e < 4; ++e) sc[2 * t + (e >> 1)][e & 1] = (float)d[t][e];      // below 2^24: exact
         } else {
             float d[2 * NACC][4] = {};
-            if constexpr (!kDense) {
+            if constexpr (FMT == FMT_FP16) {
+#pragma unroll
+                for (int k = 0; k < CH; k += 2) {
+                    uint32_t w0[4], w1[4];
+                    ldmatrix_x4(w0, row + k * 512);
+                    ldmatrix_x4(w1, row + (k + 1) * 512);
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) mma_f16_16816(d[t], w0[2 * t], w0[2 * t + 1], w1[2 * t], w1[2 * t + 1], q[k], q[k + 1]);
+                }
+            } else if constexpr (!kDense) {
 #pragma unroll
                 for (int k = 0; k < CH; ++k) {
                     uint32_t w[4];
