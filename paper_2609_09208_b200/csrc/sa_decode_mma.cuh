@@ -25,7 +25,6 @@
 namespace sa {
 
 constexpr int kWeightShift = 14;          // weights are scaled by 2^14: the largest (2^1.98 above R) stays below 65504
-constexpr float kWeightLimit = 65000.0f;  // a weight above this moves R
 constexpr float kRefMax = 268435456.0f;   // |R| <= 2^28
 
 template <int FMT>
@@ -211,25 +210,25 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     const int n_my = first < tile1 ? (tile1 - first + NW - 1) / NW : 0;
     // which of my tiles is the new token's (warp-uniform; the others' copies start before the token is encoded)
     const int i_new = (tile_new >= first && tile_new < tile1 && (tile_new - first) % NW == 0) ? (tile_new - first) / NW : -1;
-    // Start the copy of my i-th tile, whose page is `pidx`, into stage i % NS; lane 0 keeps which stages hold a mapped
-    // tile (one whose page is not mapped gets a plain arrival: the phase completes, the tile is skipped).
-    uint32_t mapped = 0u;
+    // Start the copy of my i-th tile, whose page is `pidx`, into stage i % NS; returns how many of its keys count (32 or more:
+    // all).  A tile whose page is not mapped gets a plain arrival instead, which completes the phase, and counts for none.
+    const uint8_t* pool = a.pages + (size_t)kvh * a.page_bytes;
+    const size_t page_step = (size_t)a.Hkv * a.page_bytes;
     auto issue = [&](int i, int pidx) {
         const int tile = first + NW * i, s = i % NS;
-        if (LOST && tile == a.lost_tile && b == a.lost_b && kvh == a.lost_kvh) return;   // test hook: this copy never starts
-        if (pidx < 0 || pidx >= a.n_pages) {
-            mapped &= ~(1u << s);
-            mbar_arrive(mbar0 + s * 8);
-        } else {
-            mapped |= 1u << s;
-            Stage::issue(stage0 + s * Stage::kBytes, a.pages + ((size_t)pidx * a.Hkv + kvh) * a.page_bytes, (tile & 1) * 32, mbar0 + s * 8);
+        const bool mapped = pidx >= 0 && pidx < a.n_pages;
+        if (lane == 0 && !(LOST && tile == a.lost_tile && b == a.lost_b && kvh == a.lost_kvh)) {     // test hook: that copy never starts
+            if (mapped) Stage::issue(stage0 + s * Stage::kBytes, pool + pidx * page_step, (tile & 1) * 32, mbar0 + s * 8);
+            else mbar_arrive(mbar0 + s * 8);
         }
+        return mapped ? len - tile * 32 : 0;
     };
+    int n_keys[NS];                                               // of the tiles in flight, the next one first
 #pragma unroll
     for (int i = 0; i < NS; ++i)
         if (i < n_my && i != i_new) {
             const int pidx = (same && i == 0) ? pidx_g : table[(first + NW * i) >> 1];
-            if (lane == 0) issue(i, pidx);
+            n_keys[i] = issue(i, pidx);
         }
     if (i_new >= 0) {                                             // encode / quantise the token, write it into its page, copy its tile
         CacheArgs ca{};
@@ -245,7 +244,9 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         write_token<D, CODE>(block, ca, (len - 1) % kPageTokens, lane, a.Knew + row, a.Vnew + row);
         fence_proxy_async_global();
         __syncwarp();
-        if (lane == 0 && i_new < NS) issue(i_new, pidx_new);
+#pragma unroll
+        for (int i = 0; i < NS; ++i)
+            if (i == i_new) n_keys[i] = issue(i, pidx_new);
     }
 
     float R0 = 0.0f, R1 = 0.0f;                    // references of queries 2 c, 2 c + 1 (integers)
@@ -272,9 +273,9 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
                 (void)mbar_wait_bounded(mbar0 + ((i + k) % NS) * 8, (uint32_t)((i + k) / NS) & 1u, kPolls);
             break;
         }
-        if ((__shfl_sync(0xffffffffu, mapped, 0) >> s) & 1u) {
+        {
             const uint32_t st = stage0 + s * Stage::kBytes;
-            const int n_valid = len - tile * 32;
+            const int n_valid = n_keys[0];
 
             // ---- scores ----
             float z[4][2], zh[SC::NACC == 2 ? 4 : 1][2];
@@ -292,31 +293,66 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
                         }
             }
             // ---- logits and weights ----
-            float zq[4][2], vs[4], g[4];                      // logit per score unit; 2^(14 - g_j); g_j
+            float zq[4][2], vs[4];                            // logit per score unit; 2^(14 - g_j)
+            uint32_t meta[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 if constexpr (kFp16) {                        // no scales
-                    g[j] = 0.0f;
+                    meta[j] = 0u;
                     vs[j] = (float)(1 << kWeightShift);
                     zq[j][0] = qs0;
                     zq[j][1] = qs1;
-                    continue;
+                } else {
+                    meta[j] = lds_u32(st + Stage::kMetaOff + (8 * j + r) * 4);
+                    const float sj = half_bits_to_float(meta[j] & 0xffffu);
+                    // byte 2 is g_j, in [-10, 30] for written tokens; byte 3 is zero: (g_j << 24) >> 1 = g_j << 23
+                    vs[j] = __int_as_float(((127 + kWeightShift) << 23) - ((int)__byte_perm(meta[j], 0u, 0x2444u) >> 1));
+                    zq[j][0] = qs0 * sj;
+                    zq[j][1] = qs1 * sj;
                 }
-                const uint32_t meta = lds_u32(st + Stage::kMetaOff + (8 * j + r) * 4);
-                const float sj = half_bits_to_float(meta & 0xffffu);
-                const int gi = (int)(meta << 8) >> 24;        // in [-10, 30] for written tokens
-                g[j] = (float)gi;
-                vs[j] = __int_as_float((127 + kWeightShift - gi) << 23);
-                zq[j][0] = qs0 * sj;
-                zq[j][1] = qs1 * sj;
                 if constexpr (SC::NACC == 2) {                // rounded once, like the conversion of one integer sum
                     z[j][0] += zh[j][0];
                     z[j][1] += zh[j][1];
                 }
             }
             float p[4][2], w[4][2];
-            auto weights = [&]() {                            // returns the largest of this lane
-                float top = 0.0f;
+            __half2 h[4];
+            bool move = !seen;                                // warp-uniform; rare after the first tile
+            for (int turn = 0; turn < 2; ++turn) {            // (a reference that has moved fits)
+                if (move) {
+                    float y0 = -INFINITY, y1 = -INFINITY;     // largest z - g of the tile
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (8 * j + r < n_valid) {
+                            const float g = (float)((int)(meta[j] << 8) >> 24);
+                            y0 = fmaxf(y0, fmaf(z[j][0], zq[j][0], -g));
+                            y1 = fmaxf(y1, fmaf(z[j][1], zq[j][1], -g));
+                        }
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) {
+                        y0 = fmaxf(y0, __shfl_xor_sync(0xffffffffu, y0, o));
+                        y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
+                    }
+                    y0 = fminf(fmaxf(ceilf(y0), -kRefMax), kRefMax);
+                    y1 = fminf(fmaxf(ceilf(y1), -kRefMax), kRefMax);
+                    if (seen) {
+                        y0 = fmaxf(R0, y0);
+                        y1 = fmaxf(R1, y1);
+                        const float f0 = pow2i_neg(__float2int_rn(R0 - y0)), f1 = pow2i_neg(__float2int_rn(R1 - y1));
+                        l0 *= f0;
+                        l1 *= f1;
+#pragma unroll
+                        for (int mt = 0; mt < MT; ++mt) {
+                            acc[mt][0] *= f0;
+                            acc[mt][1] *= f1;
+                            acc[mt][2] *= f0;
+                            acc[mt][3] *= f1;
+                        }
+                    }
+                    R0 = y0;
+                    R1 = y1;
+                    seen = true;
+                }
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
 #pragma unroll
@@ -330,51 +366,17 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
                         if (8 * j + r >= n_valid) p[j][0] = p[j][1] = w[j][0] = w[j][1] = 0.0f;
                 }
 #pragma unroll
-                for (int j = 0; j < 4; ++j) top = fmaxf(top, fmaxf(w[j][0], w[j][1]));
-                return top;
-            };
-            bool move = !seen;
-            if (seen) move = weights() > kWeightLimit;
-            if (__any_sync(0xffffffffu, move)) {              // rare after the first tile
-                float y0 = -INFINITY, y1 = -INFINITY;         // largest z - g of the tile
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (8 * j + r < n_valid) {
-                        y0 = fmaxf(y0, fmaf(z[j][0], zq[j][0], -g[j]));
-                        y1 = fmaxf(y1, fmaf(z[j][1], zq[j][1], -g[j]));
-                    }
-#pragma unroll
-                for (int o = 4; o < 32; o <<= 1) {
-                    y0 = fmaxf(y0, __shfl_xor_sync(0xffffffffu, y0, o));
-                    y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
-                }
-                y0 = fminf(fmaxf(ceilf(y0), -kRefMax), kRefMax);
-                y1 = fminf(fmaxf(ceilf(y1), -kRefMax), kRefMax);
-                if (seen) {
-                    y0 = fmaxf(R0, y0);
-                    y1 = fmaxf(R1, y1);
-                    const float f0 = pow2i_neg(__float2int_rn(R0 - y0)), f1 = pow2i_neg(__float2int_rn(R1 - y1));
-                    l0 *= f0;
-                    l1 *= f1;
-#pragma unroll
-                    for (int mt = 0; mt < MT; ++mt) {
-                        acc[mt][0] *= f0;
-                        acc[mt][1] *= f1;
-                        acc[mt][2] *= f0;
-                        acc[mt][3] *= f1;
-                    }
-                }
-                R0 = y0;
-                R1 = y1;
-                seen = true;
-                (void)weights();
+                for (int j = 0; j < 4; ++j) h[j] = __floats2half2_rn(w[j][0], w[j][1]);
+                // a weight beyond binary16 has become infinite: 0x7c00, the only value that 0x0400 carries into the sign bit
+                const __half2 top = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
+                move = __any_sync(0xffffffffu, ((*reinterpret_cast<const uint32_t*>(&top) + 0x04000400u) & 0x80008000u) != 0u);
+                if (__builtin_expect(!move, 1)) break;
             }
             uint32_t bh[4], bl[4];                            // operand fragments: keys 8 j + 2 c, + 1 of query r
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const __half2 h = __floats2half2_rn(w[j][0], w[j][1]);
-                const float2 hf = __half22float2(h);
-                bh[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&h));
+                const float2 hf = __half22float2(h[j]);
+                bh[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&h[j]));
                 if constexpr (kFp16) {
                     // one term; the normaliser sums the same rounded weights, so the result is an exact weighted mean
                     l0 += hf.x;
@@ -420,9 +422,11 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
             }
         }
         __syncwarp();                                         // every lane is done with this stage
-        if (lane == 0 && i + NS < n_my) {
-            fence_proxy_async();
-            issue(i + NS, pidx_next);
+#pragma unroll
+        for (int k = 0; k + 1 < NS; ++k) n_keys[k] = n_keys[k + 1];
+        if (i + NS < n_my) {
+            if (lane == 0) fence_proxy_async();
+            n_keys[NS - 1] = issue(i + NS, pidx_next);
         }
     }
 

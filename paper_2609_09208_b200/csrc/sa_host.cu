@@ -160,7 +160,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     long long cap = tiles / 2;                      // at least two tiles per block (short caches: spread them over the SMs)
     if (cap < 1) cap = 1;
     if (cap > 512) cap = 512;
-    const double c_fix = p.matrix ? 2.5 : 0.5;
+    const double c_fix = !p.matrix ? 0.5 : p.int8 ? 3.5 : 2.5;        // (INT8 keys need no decoding: a shorter round)
     double best = 0.0;
     long long best_S = 1;
     for (long long S = 1; S <= cap; ++S) {
