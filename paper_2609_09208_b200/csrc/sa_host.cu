@@ -147,12 +147,14 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     // over: every thread keeps its last answers.
     struct Kept {
         long long units, tiles;
+        double c_fix;
         int nw, bps, sms, S;
     };
+    const double c_fix = !p.matrix ? 0.5 : p.int8 ? 3.5 : 2.5;        // (INT8 keys need no decoding: a shorter round)
     static thread_local Kept kept[8] = {};
     static thread_local unsigned turn = 0;
     for (const Kept& k : kept)
-        if (k.units == units && k.tiles == tiles && k.nw == nw && k.bps == bps && k.sms == n_sms) {
+        if (k.units == units && k.tiles == tiles && k.c_fix == c_fix && k.nw == nw && k.bps == bps && k.sms == n_sms) {
             *n_splits = k.S;
             *gt = GT;
             return;
@@ -160,7 +162,6 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     long long cap = tiles / 2;                      // at least two tiles per block (short caches: spread them over the SMs)
     if (cap < 1) cap = 1;
     if (cap > 512) cap = 512;
-    const double c_fix = !p.matrix ? 0.5 : p.int8 ? 3.5 : 2.5;        // (INT8 keys need no decoding: a shorter round)
     double best = 0.0;
     long long best_S = 1;
     for (long long S = 1; S <= cap; ++S) {
@@ -180,7 +181,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
         }
         if (blocks > 16 * slots) break;             // more waves than this never pay
     }
-    kept[turn++ % 8] = Kept{units, tiles, nw, bps, n_sms, (int)best_S};
+    kept[turn++ % 8] = Kept{units, tiles, c_fix, nw, bps, n_sms, (int)best_S};
     *n_splits = (int)best_S;
     *gt = GT;
 }
