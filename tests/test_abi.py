@@ -214,12 +214,3 @@ def test_shiftav_entry_validates_on_the_host():
     assert call(0, 0) == 1 and call(19, 3) == 1 and call(15, 16) == 1 and call(15, -1) == 1
     assert call(15, 15, one, C.c_size_t(full - 1)) == 4
     assert call(15, 15, C.c_void_p(256 + 16), big) == 3
-
-
-def test_workspace_size_does_not_depend_on_what_was_asked_before():
-    """Split plans are kept per shape: configurations that share the shape but not the kernel must not share the plan."""
-    def sizes(order):
-        return {c: [sa.workspace_bytes(sa.make_config(64, 32, 4, c[0], add_on_alu=c[1]), b, p) for b in (1, 3, 32) for p in (40, 512)]
-                for c in order}
-    configs = [(sa.SA_POTM4, False), (sa.SA_POTM1, True), (sa.SA_INT8, False), (sa.SA_POTM1, False), (sa.SA_KV_FP16, False), (sa.SA_POTM4, True)]
-    assert sizes(configs) == sizes(configs[::-1])
