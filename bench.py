@@ -9,8 +9,8 @@ Workload (N = 1 and every N: one replica per GPU, weak scaling): the Llama-1.1B-
 step at T = 32768 with the PoT-M4 8-bit key code — batch 1, 32 query heads sharing 4 KV heads,
 head_dim 64, 22 decoder layers each with its own paged KV cache (64-token pages, shuffled page
 table).  One step = for every layer: append the new token's K, V to the cache (key encode, value
-quantise, cache write) and run decode attention (query quantise, integer shift-accumulate scores,
-integer-maximum online softmax, A.V, split-K merge).  The 22 caches total ~380 MB, three times the
+quantise, cache write) and run decode attention (query quantise, exact integer scores, online softmax
+with integer references, A.V, split-K merge).  The 22 caches total ~380 MB, three times the
 126 MB L2, so no layer's cache survives in L2 until the next step.
 
 Timed with CUDA events on the launching stream, barrier + synchronize on both sides, maximum over
@@ -55,11 +55,11 @@ VARIANTS = {
     "potm1_planar": (1, True, False, False),  # dense 5-bit container: sign/exponent nibbles + one mantissa bit plane
     "potm2_planar": (2, True, False, False),  # dense 6-bit container
     "fp16": (0, False, False, True),
-    "int8mac": (8, False, False, False),      # uniform INT8 keys, dp4a scores: the paper's multiply-native comparison
+    "int8mac": (8, False, False, False),      # uniform INT8 keys: the paper's multiply-native comparison
 }
-# the same codes with the shifts executed by the integer multiplier (SA_FLAG_SHIFT_BY_MULTIPLY; not the default)
+# the same codes with SA_FLAG_SHIFT_BY_MULTIPLY, which today selects the default kernels
 MULSHIFT = {"potm4_mulshift": "potm4", "potm1_mulshift": "potm1", "potm2_mulshift": "potm2"}
-# ... and with every sign flip and add on the ALU pipe, no multiply-add at all (SA_FLAG_ADD_ON_ALU; not the default)
+# ... and with scores by shifts, sign flips and adds on the ALU pipe, no multiplier at all (SA_FLAG_ADD_ON_ALU; not the default)
 ADDALU = {"potm4_alu": "potm4", "pot4_nibble_alu": "pot4_nibble", "potm1_alu": "potm1"}
 for _name, _base in list(MULSHIFT.items()) + list(ADDALU.items()):
     VARIANTS[_name] = VARIANTS[_base]
@@ -131,7 +131,7 @@ class Workload:
             self.O.append(torch.zeros((batch, Hq, d), dtype=torch.float32, device=dev))
         torch.cuda.synchronize()
         self.keys_per_step = layers * batch * T * Hkv
-        self.launches_per_step = layers * 2          # main kernel (appends the new token), merge
+        self.launches_per_step = layers * 2          # main kernel (appends the new token), merge (short sequences: the first alone)
 
     def decode(self, l, stages=3):
         sa = self.sa
@@ -659,8 +659,7 @@ def run_ours(args):
     }
     pipes = line["pipe_utilisation"]
     if pipes and pipes.get("rows"):
-        # The resource that actually binds the shift kernels is the integer ALU pipe (shift, logic, permute):
-        # 64 lanes per SM and clock.  Fraction from the recorded capture of the nearest batch size.
+        # The integer ALU pipe (shift, logic, permute): 64 lanes per SM and clock.  Fraction from the recorded capture of the nearest batch size.
         row = min(pipes["rows"], key=lambda r: abs(r["batch"] - wl.batch))
         n_sms = torch.cuda.get_device_properties(dev).multi_processor_count
         alu_peak = n_sms * 64 * (clocks.get("sm_mhz") or 1965.0) * 1e6    # no clock sample in a very short run: the maximum
@@ -668,20 +667,6 @@ def run_ours(args):
                                 "achieved": alu_peak * row["alu_pipe_pct"] / 100.0, "issue_slots_frac": row["issue_slots_pct"] / 100.0,
                                 "source": "ncu sm__inst_executed_pipe_alu of the capture at batch %d, kernel sources %s (profiles/); "
                                           "not measured by this run" % (row["batch"], pipes.get("kernel_source_hash"))}
-    code_k = VARIANTS[args.variant][0]
-    if code_k in (1, 2, 4) and not wl.fp16:
-        # The floor of the table datapath of the mantissa codes, measured live: every (key, element, query pair) update
-        # gathers one 8-byte table entry from shared memory, and an SM's shared-memory pipe moves 128 bytes per clock
-        # (profiles/instruction_throughput_b200.md: a 64-bit gather is two wavefronts wherever its lanes point).
-        pairs = (group + 1) // 2
-        table_bytes = wl.batch * wl.T * wl.Hkv * wl.d * pairs * 8.0      # per launch: one layer's cached keys
-        sms = torch.cuda.get_device_properties(dev).multi_processor_count
-        smem_peak = sms * 128.0 * (clocks.get("sm_mhz") or 1965.0) * 1e6
-        line["roofline_shared"] = {"bound": "shared-memory pipe", "unit": "B/s", "peak": smem_peak,
-                                   "achieved": table_bytes / (main_us * 1e-6), "frac": table_bytes / (main_us * 1e-6) / smem_peak,
-                                   "what": "table entries gathered per launch (keys x head_dim x query pairs x 8 B) / main kernel "
-                                           "time, against SMs x 128 B/clk x sampled SM clock; the kernel's other shared-memory "
-                                           "traffic (key codes, values, weights) is not counted"}
     if rank == 0 and args.gpus == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(args.variant, args.seq_len, args.batch)
     if rank == 0 and args.gpus == 1 and not args.no_context:
@@ -902,7 +887,7 @@ def run_sweep(args):
             cell("cfg3 T=32768 B=%d %s%s shift-based A.V (N = k_max = 15)" % (B, names[code], "_nibble" if nib else ""),
                  [32768] * B, 32, 4, 64, code, nibble=nib, outliers=False, shiftav=True, oracle=False)
         for code, nib in ([] if quick else [(1, False), (4, False)]):
-            cell("cfg3 T=32768 B=%d %s%s shifts on the integer multiplier" % (B, names[code], "_nibble" if nib else ""),
+            cell("cfg3 T=32768 B=%d %s%s SA_FLAG_SHIFT_BY_MULTIPLY (the default kernels)" % (B, names[code], "_nibble" if nib else ""),
                  [32768] * B, 32, 4, 64, code, nibble=nib, outliers=False, shift_by_multiply=True, oracle=False)
         for code, nib in ([] if quick else [(0, True), (4, False)]):
             cell("cfg3 T=32768 B=%d %s%s adds on the ALU pipe" % (B, names[code], "_nibble" if nib else ""),

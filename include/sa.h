@@ -71,7 +71,7 @@ enum { SA_POT4 = 0, SA_POTM1 = 1, SA_POTM2 = 2, SA_POTM4 = 4, SA_INT8 = 8, SA_KV
 /* SA_INT8 is the comparison code of section III / VI (an INT8 multiply-accumulate kernel built on the
  * same skeleton as the shift kernels): uniform INT8 keys, khat = round(K * 127 / amax) with the row maximum as
  * scale, stored one byte per element in the byte container (132 bytes per key at d = 64, the same
- * as PoT-M4); scores are integer dot products evaluated with dp4a.  Everything else (query and
+ * as PoT-M4); scores are integer dot products with INT32 sums.  Everything else (query and
  * value quantisers, softmax, A.V, merge, cache layout) is shared with the power-of-two codes. */
 /* How key codes are stored in a page.
  * SA_KLAYOUT_BYTE: one byte per element (any code).
@@ -216,11 +216,15 @@ sa_status sa_decode_attention_fp16(const sa_config* cfg, const sa_cache* cache, 
  *   sa_append_kv(cfg, cache, K_new, V_new, 1, stream); sa_decode_attention(cfg, cache, Q, O, ...);
  * The warp of the decode kernel that owns the new token's 32-key tile encodes and writes the token
  * before it stages that tile, so the separate append kernel and its launch disappear from the
- * step; seq_lens[b] is incremented by the split-K merge kernel, after every block has read it.
+ * step; seq_lens[b] is incremented after every block has read it: by the split-K merge kernel, or, where the
+ * plan needs no merge kernel (a short single sequence, whose splits form a thread-block cluster, or one split per
+ * sequence), by the last block of the decode kernel itself.  The blocks then meet at a counter in device memory:
+ * the library keeps 16 KB of them on every GPU, gives each workspace its own, and falls back to two kernels once
+ * they are all taken.
  * As with sa_append_kv the token's page must already be mapped; if it is not, the token is not
  * written, the length stays, and the step attends over the old cache.
  * With more than 8 query heads per KV head the call runs the two kernels separately.  A binary16
- * cache (SA_KV_FP16) is served the same way by the binary16 decode kernel.  Same buffers,
+ * cache (SA_KV_FP16) is served the same way.  Same buffers,
  * alignment and workspace as sa_decode_attention; K_new, V_new [batch, n_kv_heads, head_dim]
  * binary16, 16-byte aligned. */
 sa_status sa_decode_step(const sa_config* cfg, const sa_cache* cache, const uint16_t* Q,
@@ -298,8 +302,8 @@ sa_status sa_decode_attention_static(const sa_config* cfg, const sa_cache* cache
 /* Test hook for the failure path of the staged copies (the paper has no counterpart).  sa_decode_attention
  * in which the bulk copy of ONE tile — 32-token tile `tile` of sequence `b`, KV head `kv_head` — is never
  * issued and every wait for a copy gives up after 2^10 polls instead of 2^18.  The warp that owns that tile
- * finds its wait exhausted, abandons its remaining tiles and marks its block's partial result; the split-K
- * merge carries the mark into O: the rows of the query heads of `kv_head` in sequence `b` come out as NaN,
+ * finds its wait exhausted, abandons its remaining tiles and marks its block's partial result; the merge of the
+ * splits (in a kernel or in a cluster) carries the mark into O: the rows of the query heads of `kv_head` in sequence `b` come out as NaN,
  * every other row is the ordinary result, and the call returns like any other (nothing is left in flight,
  * nothing waits without a bound).  Only head_dim 64, SA_POTM4 in the byte container, 8 query heads per KV
  * head, no flags: anything else is SA_ERR_UNSUPPORTED. */

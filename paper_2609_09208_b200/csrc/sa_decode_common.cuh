@@ -287,7 +287,7 @@ SA_D void block_merge_and_store(const DecodeArgs& a, float (*red_s)[GT][D + 2], 
 // two resident blocks of the decode kernel: the next decode kernel is launched while this one runs
 // (programmatic dependent launch), and a merge block that took the place of one of its blocks would make
 // that block, and with it the whole grid, finish late.
-// With more than 96 splits (the FP16 kernel at batch 1: 111) the block has 256 threads = 64 groups instead, so that
+// With more than 96 splits (a binary16 cache at batch 1: 111) the block has 256 threads = 64 groups instead, so that
 // the partials are still fetched in one round trip; it then no longer fits beside the quantised kernels' two blocks,
 // whose split counts stay below that.
 constexpr int kMergeDims = 16;                                // output dims per block
