@@ -130,28 +130,28 @@ SA_HD KeyScale key_scale(uint32_t s_bits) {
     k.inv = s > 0.0f ? 1.0f / s : 0.0f;
     return k;
 }
-// Code of one key element (section II-A, II-D), `a_bits` the element's binary16 bits, K the number of mantissa bits, as
-// the magnitude's place on the grid: g 2^K + j (g = 7 - e) for the codeword (1 + j/2^K) 2^-e, below 2^K: the zero code.
+// Code of one key element (section II-A, II-D), `a` the element's binary16 value (its sign does not matter), K the number of
+// mantissa bits, as the magnitude's place on the grid: g 2^K + j (g = 7 - e) for the codeword (1 + j/2^K) 2^-e, below 2^K: the
+// zero code.
 //   u = a/s = rho * 2^-e0 with rho in [1, 2);  j = floor((rho - 1) 2^K);  with n = 2^K + j the
 //   neighbours on the grid are n and n + 1 (in units of 2^(-K-e0)), and the upper one is nearer
 //   in log2 exactly when rho^2 4^K >= n (n + 1).
 // e0 and j are the exponent field and the leading mantissa bits of an FP32 quotient: rho 2^K is a whole number or at least
 // 1 / 2047 (relative 2^-16) from one, the quotient is within two units in the last place, so raising it by sixteen (2^-19)
-// decides both cases.  The comparison is exact: rho = num / M with num = Ma or 2 Ma, num < 2^12, and both sides fit 32 bits
-// (n (n + 1) <= 992, M^2 < 2^22).
-SA_HD uint32_t encode_place(int K, uint32_t a_bits, const KeyScale& s) {
-    const float a = __half2float(__ushort_as_half((unsigned short)(a_bits & 0x7fffu)));
-    const uint32_t rb = float_bits(a * s.inv) + 16u;
+// decides both cases.  The comparison is exact: rho = num / M with num = Ma or 2 Ma, num 2^K < 2^16, and both sides fit 32
+// bits (n (n + 1) <= 992, M^2 < 2^22).
+SA_HD uint32_t encode_place(int K, float a, const KeyScale& s) {
+    const uint32_t rb = float_bits(fabsf(a) * s.inv) + 16u;
     const uint32_t place = rb >> (23 - K);                    // (exponent field, j)
     const uint32_t n = (place & ((1u << K) - 1u)) | (1u << K);
-    const uint32_t Ma = ((float_bits(a) >> 13) & 0x3ffu) | 0x400u;
-    const uint32_t num = Ma < s.M ? 2u * Ma : Ma;
-    const int p = (int)place - (120 << K) + (num * num << (2 * K) >= (n * n + n) * s.MM ? 1 : 0);
+    const uint32_t Ma = ((float_bits(a) >> (13 - K)) & (0x3ffu << K)) | (0x400u << K);       // times 2^K
+    const uint32_t num = Ma < s.M << K ? 2u * Ma : Ma;
+    const int p = (int)place - (120 << K) + (num * num >= (n * n + n) * s.MM ? 1 : 0);
     return (uint32_t)(p < 0 ? 0 : p);
 }
 // ... as the canonical byte.
 SA_HD uint8_t encode_element_k(int K, uint32_t a_bits, const KeyScale& s) {
-    const uint32_t p = encode_place(K, a_bits, s);
+    const uint32_t p = encode_place(K, __half2float(__ushort_as_half((unsigned short)a_bits)), s);
     if (p < (1u << K)) return 0x70;
     return (uint8_t)(((a_bits >> 8) & 0x80u) | ((7u - (p >> K)) << 4) | ((p & ((1u << K) - 1u)) << (4 - K)));
 }

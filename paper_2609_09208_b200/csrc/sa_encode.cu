@@ -90,11 +90,15 @@ __global__ void __launch_bounds__(128) append_kernel(CacheArgs a, const uint16_t
     if (ok && bump && threadIdx.x == 0) a.seq_lens[b] = len + 1;
 }
 
-// sa_fill_kv.  One warp takes the keys or the values of one KV head for the 32 tokens of half a page, lane = token: a
-// thread has its whole head vector in registers (no shuffles for the largest magnitude or the rotation), and as the chunks of
-// the 32 tokens follow one another in the page, the warp's stores are 512 contiguous bytes per chunk.  (A warp per
-// vector wrote two bytes per lane and encoded with 64-bit products and a division: 41 us for the four prompts of
-// 18 384 tokens x 4 heads, now bound by the instructions of the encoder.)  All sequences of a call go in one launch.
+// sa_fill_kv.  One warp takes the keys or the values of one KV head for the 32 tokens of half a page.  It loads whole 128-byte
+// lines and turns them in shared memory, so that lane = token: a thread has its whole head vector (no shuffles for the largest
+// magnitude or the rotation), and as the chunks of the 32 tokens follow one another in the page, the warp's stores are
+// 512 contiguous bytes per chunk.  (Each thread loading its own row meant 32 lines per load instruction.)  All sequences of a
+// call go in one launch.  Large calls are bound by the encoder on the ALU pipe (82 % before signs and value bytes were handled
+// four at a time), binary16 by memory; the smallest by the fetch of code that every warp runs once, hence rolled loops where
+// 64 unrolled elements are tens of kilobytes (PoT-4's short code is better off with 32 at a time).  Measured on PoT-M4 /
+// PoT-4 / binary16, us: 32 tokens of 4 heads 4.7 / 3.5 / 2.0 -> 3.0 / 2.5 / 1.8, four prompts of 18 384 tokens 12.3 / 10.0 / 8.4
+// -> 9.1 / 7.4 / 7.5, 8 x 32768 tokens 109 / 90 / 91 -> 102 / 89 / 81 (81 us are the copy rate).
 constexpr int kFillBatch = 64;            // sequences per launch
 struct FillSeqs {
     int64_t row0[kFillBatch];             // first row of the sequence in K / V
@@ -129,84 +133,136 @@ SA_D void hadamard_thread(uint32_t (&h)[D / 2]) {
 }
 
 // The vector of one token -> its place in the half page `half` (t: token within it).
+SA_D float2 half2_bits_to_float2(uint32_t x) { return __half22float2(*reinterpret_cast<const __half2*>(&x)); }
+
+// One thread's vector in the warp's shared buffer (16-byte chunk i of row t at chunk i ^ (t & 7), so that neither the rows'
+// owners nor the coalesced writes meet a bank conflict): its largest magnitude, then its elements 8 at a time.  KEEP: rotated,
+// in registers.
+template <int D, bool KEEP>
+struct VecRow {
+    const uint4* row;
+    int x7;
+    uint32_t h[KEEP ? D / 2 : 1];
+    uint32_t top = 0;
+    SA_D VecRow(const uint4* buffer, int t) : row(buffer + t * (D / 8)), x7(t & 7) {
+        if constexpr (KEEP) {
+#pragma unroll
+            for (int i = 0; i < D / 8; ++i) {
+                const uint4 v = row[i ^ x7];
+                h[4 * i] = v.x, h[4 * i + 1] = v.y, h[4 * i + 2] = v.z, h[4 * i + 3] = v.w;
+            }
+            hadamard_thread<D>(h);
+#pragma unroll
+            for (int i = 0; i < D / 2; ++i) top = __vmaxu2(top, h[i] & 0x7fff7fffu);      // two magnitudes at a time; they order like their bits
+        } else {
+#pragma unroll
+            for (int i = 0; i < D / 8; ++i) {
+                const uint4 v = row[i ^ x7];
+                top = __vmaxu2(__vmaxu2(top, __vmaxu2(v.x & 0x7fff7fffu, v.y & 0x7fff7fffu)), __vmaxu2(v.z & 0x7fff7fffu, v.w & 0x7fff7fffu));
+            }
+        }
+    }
+    SA_D uint32_t max_bits() const { return max(top & 0xffffu, top >> 16); }
+    SA_D void get(int i, uint32_t* x) const {
+        if constexpr (KEEP) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = h[4 * i + e];
+        } else {
+            const uint4 v = row[i ^ x7];
+            x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+        }
+    }
+};
 template <int D, int MODE, bool HAD>
-SA_D void fill_keys(uint8_t* half, const CacheArgs& a, int t, uint32_t (&h)[D / 2]) {
+SA_D void fill_keys(uint8_t* half, const CacheArgs& a, int t, const uint4* src) {
     constexpr bool NIB = MODE >= 8 && MODE <= 10;
     constexpr int K = MODE == 32 ? 8 : NIB ? MODE - 8 : MODE;
-    if constexpr (HAD) hadamard_thread<D>(h);
-    uint32_t top = 0;                                         // two magnitudes at a time; they order like their bits
-#pragma unroll
-    for (int i = 0; i < D / 2; ++i) top = __vmaxu2(top, h[i] & 0x7fff7fffu);
-    const uint32_t smax = max(top & 0xffffu, top >> 16);
+    VecRow<D, HAD> row(src, t);
+    const uint32_t smax = row.max_bits();
     const KeyScale ks = key_scale(smax);
     const float amax = half_bits_to_float(smax);
     const float inv8 = (K == 8 && amax != 0.0f) ? __fdiv_rn(127.0f, amax) : 0.0f;
-    auto code = [&](int m) -> uint32_t {                      // physical byte (sub-byte containers: canonical byte ^ 0x70)
-        const uint32_t bits = (m & 1) ? h[m >> 1] >> 16 : h[m >> 1] & 0xffffu;
-        if constexpr (K == 8) {
-            const int r = __float2int_rn(__fmul_rn(half_bits_to_float(bits), inv8));
-            return (uint32_t)max(-127, min(127, r)) & 0xffu;
-        } else {
-            const uint32_t p = encode_place(K, bits, ks), sign = (bits >> 8) & 0x80u, j = p & ((1u << K) - 1u);
-            const uint32_t c = NIB ? sign | ((p >> K) << 4) | (j << (4 - K)) : sign | (j << (7 - K)) | (p >> K);
-            return p < (1u << K) ? 0u : c;
-        }
+    auto place = [&](float x) -> uint32_t {                   // 0 for the zero code
+        const uint32_t p = encode_place(K, x, ks);
+        return p < (1u << K) ? 0u : p;
     };
+    uint8_t* dst = half + a.kcode_off + (size_t)t * 16;
     if constexpr (!NIB) {
-#pragma unroll
+#pragma unroll(HAD ? D / 16 : 1)
         for (int c = 0; c < D / 16; ++c) {
-            uint32_t w[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                w[i] = code(16 * c + 4 * i) | (code(16 * c + 4 * i + 1) << 8) | (code(16 * c + 4 * i + 2) << 16) | (code(16 * c + 4 * i + 3) << 24);
-            *reinterpret_cast<uint4*>(half + a.kcode_off + (size_t)(c * kTileTokens + t) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    } else {
-        uint32_t plane[K > 0 && K < 8 ? K : 1][D / 32] = {};
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-            uint32_t w[4];
+            uint32_t x[8], w[4];
+            row.get(2 * c, x);
+            row.get(2 * c + 1, x + 4);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
+                const float2 f[2] = {half2_bits_to_float2(x[2 * i]), half2_bits_to_float2(x[2 * i + 1])};
+                const float e[4] = {f[0].x, f[0].y, f[1].x, f[1].y};
                 w[i] = 0u;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const uint32_t x = code(32 * c + 8 * i + e);
-                    w[i] |= (x >> 4) << (4 * e);
-                    if constexpr (K > 0)
-#pragma unroll
-                        for (int bit = 0; bit < K; ++bit) plane[bit][c] |= ((x >> (4 - K + bit)) & 1u) << (8 * i + e);
+                for (int k = 0; k < 4; ++k) {
+                    if constexpr (K == 8) {
+                        const int q = __float2int_rn(__fmul_rn(e[k], inv8));
+                        w[i] |= ((uint32_t)max(-127, min(127, q)) & 0xffu) << (8 * k);
+                    } else {
+                        const uint32_t p = place(e[k]);       // -> mantissa field << 3 | g
+                        w[i] |= (((p << (7 - K)) & (0x7fu & (0x7fu << (7 - K)))) | (p >> K)) << (8 * k);
+                    }
                 }
+                // the four signs at once, kept beside nonzero bytes only
+                if constexpr (K != 8) w[i] |= __byte_perm(x[2 * i], x[2 * i + 1], 0x7531) & 0x80808080u & (w[i] + 0x7f7f7f7fu);
             }
-            *reinterpret_cast<uint4*>(half + a.kcode_off + (size_t)(c * kTileTokens + t) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4*>(dst + (size_t)(c * kTileTokens) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        if constexpr (K > 0)
+    } else {
+        constexpr int P = K > 0 && K < 8 ? K : 1;
+        uint32_t w[4] = {}, plane[P] = {};                    // the chunk and the mantissa bits of its 32 elements, filled from the top
+#pragma unroll(HAD ? D / 8 : K == 0 ? 4 : 1)
+        for (int i = 0; i < D / 8; ++i) {
+            uint32_t x[4], next = 0u;
+            row.get(i, x);
 #pragma unroll
-            for (int bit = 0; bit < K; ++bit)
+            for (int bit = 0; bit < P; ++bit) plane[bit] >>= 8;
 #pragma unroll
-                for (int c = 0; c < D / 32; c += 2)
-                    *reinterpret_cast<uint2*>(half + a.plane_off + (size_t)(bit * kTileTokens + t) * (D / 8) + 4 * c) = make_uint2(plane[bit][c], plane[bit][c + 1]);
+            for (int e = 0; e < 8; ++e) {
+                const float2 f = half2_bits_to_float2(x[e >> 1]);
+                const uint32_t p = place((e & 1) ? f.y : f.x);
+                next |= (p >> K) << (4 * e);
+                if constexpr (K > 0)
+#pragma unroll
+                    for (int bit = 0; bit < K; ++bit) plane[bit] |= ((p >> bit) & 1u) << (24 + e);
+            }
+            const uint32_t lo = __byte_perm(x[0], x[1], 0x7351), hi = __byte_perm(x[2], x[3], 0x7351);      // the bytes with the signs
+            const uint32_t even = __byte_perm(lo, hi, 0x5410), odd = __byte_perm(lo, hi, 0x7632);
+            next |= (((even >> 4) & 0x08080808u) | (odd & 0x80808080u)) & (next + 0x77777777u);
+            w[0] = w[1], w[1] = w[2], w[2] = w[3], w[3] = next;
+            if ((i & 3) == 3) {
+                *reinterpret_cast<uint4*>(dst + (size_t)((i >> 2) * kTileTokens) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+                if constexpr (K > 0)
+#pragma unroll
+                    for (int bit = 0; bit < K; ++bit)
+                        *reinterpret_cast<uint32_t*>(half + a.plane_off + (size_t)(bit * kTileTokens + t) * (D / 8) + (i & ~3)) = plane[bit];
+            }
+        }
     }
     *reinterpret_cast<uint16_t*>(half + a.meta_off + (size_t)t * 4) = (uint16_t)smax;
 }
 template <int D>
-SA_D void fill_values(uint8_t* half, const CacheArgs& a, int t, const uint32_t (&h)[D / 2]) {
-    uint32_t top = 0;
-#pragma unroll
-    for (int i = 0; i < D / 2; ++i) top = __vmaxu2(top, h[i] & 0x7fff7fffu);
-    const int g = value_exponent(max(top & 0xffffu, top >> 16));
+SA_D void fill_values(uint8_t* half, const CacheArgs& a, int t, const uint4* src) {
+    VecRow<D, false> row(src, t);
+    const int g = value_exponent(row.max_bits());
     const float f = pow2i(g);
-#pragma unroll
+#pragma unroll 1
     for (int c = 0; c < D / 16; ++c) {
-        uint32_t w[4];
+        uint32_t h[8], w[4];
+        row.get(2 * c, h);
+        row.get(2 * c + 1, h + 4);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            w[i] = 0u;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const uint32_t x = h[8 * c + 2 * i + (e >> 1)], bits = (e & 1) ? x >> 16 : x & 0xffffu;
-                w[i] |= ((uint32_t)__float2int_rn(__fmul_rn(half_bits_to_float(bits), f)) & 0xffu) << (8 * e);
-            }
+            // scaling by 2^g is exact, so adding 1.5 * 2^23 rounds to the nearest integer (ties to even), the low byte of the bits
+            const float2 x = half2_bits_to_float2(h[2 * i]), y = half2_bits_to_float2(h[2 * i + 1]);
+            const uint32_t lo = __byte_perm(__float_as_uint(__fmaf_rn(x.x, f, 12582912.0f)), __float_as_uint(__fmaf_rn(x.y, f, 12582912.0f)), 0x0040);
+            const uint32_t hi = __byte_perm(__float_as_uint(__fmaf_rn(y.x, f, 12582912.0f)), __float_as_uint(__fmaf_rn(y.y, f, 12582912.0f)), 0x0040);
+            w[i] = __byte_perm(lo, hi, 0x5410);
         }
         *reinterpret_cast<uint4*>(half + a.v_off + (size_t)(c * kTileTokens + t) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
     }
@@ -230,26 +286,33 @@ __global__ void __launch_bounds__(128) fill_kernel(CacheArgs a, const uint16_t* 
     pdl_wait();                                                               // earlier kernels may read this cache or write the inputs
     pdl_launch_dependents();
     uint8_t* block = page_block(a, seqs.b0 + i, t / kPageTokens, head);
-    if (!block || t + lane >= seqs.len[i]) return;
+    if (!block) return;
     uint8_t* half = block + (size_t)((t % kPageTokens) >> 5) * (a.page_bytes >> 1);
-    const uint4* src = reinterpret_cast<const uint4*>(((rest & 1) ? Vin : Kin) + ((size_t)(seqs.row0[i] + t + lane) * a.Hkv + head) * D);
-    uint32_t h[D / 2];
+    // the tile's rows, a 16-byte chunk per lane: whole 128-byte lines per load
+    constexpr int C = D / 8, R = 32 / C;
+    __shared__ uint4 buffers[4][32 * C];
+    uint4* src = buffers[threadIdx.x >> 5];
+    const int n = seqs.len[i] - t, ch = lane % C;
+    const uint4* in = reinterpret_cast<const uint4*>(((rest & 1) ? Vin : Kin) + ((size_t)(seqs.row0[i] + t) * a.Hkv + head) * D) + ch;
+    const size_t pitch = (size_t)a.Hkv * C;
+    uint4 v[C];
 #pragma unroll
-    for (int k = 0; k < D / 8; ++k) {
-        const uint4 v = __ldg(src + k);
-        h[4 * k] = v.x;
-        h[4 * k + 1] = v.y;
-        h[4 * k + 2] = v.z;
-        h[4 * k + 3] = v.w;
+    for (int k = 0; k < C; ++k)
+        if (k * R + lane / C < n) v[k] = __ldg(in + (size_t)(k * R + lane / C) * pitch);
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+        const int row = k * R + lane / C;
+        if (row < n) src[row * C + (ch ^ (row & 7))] = v[k];
     }
+    __syncwarp();
+    if (lane >= n) return;
     if constexpr (MODE == 16) {                                               // unquantised: 16-byte chunks of 8 elements
         uint8_t* dst = half + ((rest & 1) ? a.v_off : a.kcode_off);
 #pragma unroll
-        for (int k = 0; k < D / 8; ++k)
-            *reinterpret_cast<uint4*>(dst + (size_t)(k * kTileTokens + lane) * 16) = make_uint4(h[4 * k], h[4 * k + 1], h[4 * k + 2], h[4 * k + 3]);
+        for (int k = 0; k < D / 8; ++k) *reinterpret_cast<uint4*>(dst + (size_t)(k * kTileTokens + lane) * 16) = src[lane * C + (k ^ (lane & 7))];
     } else {
-        if (rest & 1) fill_values<D>(half, a, lane, h);
-        else fill_keys<D, MODE, HAD>(half, a, lane, h);
+        if (rest & 1) fill_values<D>(half, a, lane, src);
+        else fill_keys<D, MODE, HAD>(half, a, lane, src);
     }
 }
 
