@@ -171,7 +171,8 @@ PyObject* append_kv(PyObject*, PyObject* const* v, Py_ssize_t n) {
     SA_RETURN(sa_append_kv(cfg, cache, K, V, bump, s));
 }
 
-// (cfg, cache, K, V, cu_lens): cu_lens a contiguous host array of 64-bit integers
+// (cfg, cache, K, V, cu_lens): cu_lens a contiguous host array of at least batch + 1 64-bit integers, which the library
+// reads on the host
 PyObject* fill_kv(PyObject*, PyObject* const* v, Py_ssize_t n) {
     Args a{v, n};
     const sa_config* cfg = a.structure<sa_config>();
@@ -179,9 +180,17 @@ PyObject* fill_kv(PyObject*, PyObject* const* v, Py_ssize_t n) {
     const uint16_t* K = a.tensor<uint16_t>();
     const uint16_t* V = a.tensor<uint16_t>();
     PyObject* o = a.bad ? nullptr : a.next();
-    const sa_stream s = a.stream();
     Py_buffer cu;
     if (a.bad || PyObject_GetBuffer(o, &cu, PyBUF_SIMPLE) != 0) return nullptr;
+    if (cu.len / (Py_ssize_t)sizeof(int64_t) <= (Py_ssize_t)cache->batch) {
+        a.bad = true;
+        PyErr_Format(PyExc_ValueError, "cu_lens holds %zd bytes, not the batch + 1 = %zd numbers of 8", cu.len, (Py_ssize_t)cache->batch + 1);
+    }
+    const sa_stream s = a.stream();
+    if (a.bad) {
+        PyBuffer_Release(&cu);
+        return nullptr;
+    }
     sa_status st;
     Py_BEGIN_ALLOW_THREADS
     st = sa_fill_kv(cfg, cache, K, V, static_cast<const int64_t*>(cu.buf), s);

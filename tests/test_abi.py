@@ -4,6 +4,7 @@ import ctypes as C
 import os
 import re
 
+import numpy as np
 import pytest
 
 from paper_2609_09208_b200 import binding as sa
@@ -214,3 +215,12 @@ def test_shiftav_entry_validates_on_the_host():
     assert call(0, 0) == 1 and call(19, 3) == 1 and call(15, 16) == 1 and call(15, -1) == 1
     assert call(15, 15, one, C.c_size_t(full - 1)) == 4
     assert call(15, 15, C.c_void_p(256 + 16), big) == 3
+
+
+@pytest.mark.parametrize("entries", [0, 1, 2, 3])
+def test_fill_refuses_fewer_sequence_starts_than_the_batch_has(entries):
+    """sa_fill_kv reads batch + 1 starts from host memory: an array that holds fewer is refused before the call."""
+    cfg = sa.make_config(64, 32, 4, sa.SA_POTM4)
+    cache = sa.SaCache(256, 256, 256, 3, 4, 12)
+    with pytest.raises(ValueError, match="batch"):
+        sa.fill_kv(cfg, cache, None, None, np.zeros(entries, dtype=np.int64))
