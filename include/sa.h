@@ -218,9 +218,8 @@ sa_status sa_decode_attention_fp16(const sa_config* cfg, const sa_cache* cache, 
  * before it stages that tile, so the separate append kernel and its launch disappear from the
  * step; seq_lens[b] is incremented after every block has read it: by the split-K merge kernel, or, where the
  * plan needs no merge kernel (a short single sequence, whose splits form a thread-block cluster, or one split per
- * sequence), by the last block of the decode kernel itself.  The blocks then meet at a counter in device memory:
- * the library keeps 16 KB of them on every GPU, gives each workspace its own, and falls back to two kernels once
- * they are all taken.
+ * sequence), by the last block of the decode kernel itself (the blocks are counted in the workspace, which such a
+ * step needs for nothing else and which needs no initialisation for it).
  * As with sa_append_kv the token's page must already be mapped; if it is not, the token is not
  * written, the length stays, and the step attends over the old cache.
  * With more than 8 query heads per KV head the call runs the two kernels separately.  A binary16

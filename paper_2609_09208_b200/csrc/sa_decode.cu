@@ -45,7 +45,7 @@ static sa_status decode_stages(const Plan& p, const sa_cache* cache, const uint1
     set_scales(p, &a);   // logits in the log2 domain: A * Delta * s * 2^-F * log2(e) / sqrt(d)
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (stages != 3) a.whole = 0;
-    settle_whole(workspace, s, &a);
+    settle_whole(workspace, p, &a);
     if (stages & 1) {
         launch_decode_main(p, a, GT, s);
         if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
@@ -98,7 +98,7 @@ extern "C" sa_status sa_debug_decode_lost_copy(const sa_config* cfg, const sa_ca
     a.lost_tile = tile;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     a.whole = 0;
-    settle_whole(workspace, s, &a);
+    settle_whole(workspace, p, &a);
     launch_mma_lost_copy(a, dim3((unsigned)a.n_splits, (unsigned)p.Hkv, (unsigned)a.batch), s);
     if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
     return launch_merge(p, a, s);
@@ -143,7 +143,7 @@ sa_status sa::decode_step_impl(const sa_config* cfg, const sa_cache* cache, cons
     a.wait_first = q_after_wait ? 1 : 0;
     set_scales(p, &a);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    settle_whole(workspace, s, &a);
+    settle_whole(workspace, p, &a);
     launch_decode_main(p, a, GT, s);
     if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
     return a.whole ? SA_OK : launch_merge(p, a, s);
@@ -171,51 +171,6 @@ extern "C" sa_status sa_decode_attention(const sa_config* cfg, const sa_cache* c
 #include <mutex>
 
 static __device__ __align__(256) unsigned char sa_static_scratch[SA_STATIC_SCRATCH_BYTES];
-
-// ---------------------------------------------------------------------------------------------
-// Counters of the steps that are one launch (settle_whole).  A counter has to be zero when a call starts and every call
-// leaves it zero, so it cannot live in the caller's workspace, which needs no initialisation; but as calls that share a
-// workspace never overlap on the GPU, one for each workspace address is enough.  They are a fixed array of the library
-// image, handed out to the first kCounters addresses seen on a device; a call beyond those, or one that would have to look
-// the array's address up in the middle of a stream capture, uses the separate merge kernel instead.
-// ---------------------------------------------------------------------------------------------
-constexpr int kCounters = 4096;
-static __device__ unsigned sa_step_counters[kCounters];
-
-unsigned* sa::step_counter(const void* workspace, cudaStream_t s) {
-    struct Table {
-        unsigned* base = nullptr;
-        int n = 0;
-        const void* owner[2 * kCounters] = {};                  // open addressing
-        int index[2 * kCounters] = {};
-    };
-    constexpr int kDevices = 64;
-    static std::mutex mutex;
-    static Table* tables[kDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return nullptr;
-    std::lock_guard<std::mutex> lock(mutex);
-    if (!tables[dev]) {
-        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-        void* base = nullptr;
-        if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone ||
-            cudaGetSymbolAddress(&base, sa_step_counters) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return nullptr;
-        }
-        tables[dev] = new Table;
-        tables[dev]->base = static_cast<unsigned*>(base);
-    }
-    Table& t = *tables[dev];
-    unsigned i = ((unsigned)(reinterpret_cast<uintptr_t>(workspace) >> 4) * 2654435761u >> 8) % (2 * kCounters);
-    while (t.owner[i] && t.owner[i] != workspace) i = (i + 1) % (2 * kCounters);
-    if (!t.owner[i]) {
-        if (t.n == kCounters) return nullptr;
-        t.owner[i] = workspace;
-        t.index[i] = t.n++;
-    }
-    return t.base + t.index[i];
-}
 
 namespace {
 constexpr int kMaxScratchDevices = 64;

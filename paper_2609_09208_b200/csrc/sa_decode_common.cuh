@@ -45,10 +45,10 @@ struct DecodeArgs {
     int32_t* plan;
     int bal_target;
     // Matrix kernel, whole: all splits of a sequence form a thread-block cluster (of `cluster` blocks; 1 otherwise), which
-    // merges them into O, and no merge kernel runs.  `counter` (zero between calls) then counts the blocks that have read the
-    // lengths, if the call appends tokens.
+    // merges them into O, and no merge kernel runs.  If the call appends tokens, `arrivals` then counts the blocks that have
+    // read the lengths (last_to_arrive).
     int cluster, whole;
-    unsigned* counter;
+    unsigned long long* arrivals;
 };
 
 // Batches of 2 .. kRankedBatchMax sequences: which (sequence, split) a block of the grid works on is decided on the
@@ -427,12 +427,30 @@ __global__ void __launch_bounds__(kMergeThreads, 2048 / kMergeThreads) merge_ker
     }
 }
 
-// A counter for calls with this workspace that append tokens and have no merge kernel, or null.
-unsigned* step_counter(const void* workspace, cudaStream_t s);
-// Takes back the one-launch form of a call that appends tokens where no counter is to be had.
-inline void settle_whole(const void* workspace, cudaStream_t s, DecodeArgs* a) {
-    if (a->whole && a->Knew) a->counter = step_counter(workspace, s);
-    if (a->whole && a->Knew && !a->counter) a->whole = 0;
+// The blocks of a call that appends tokens and has no merge kernel meet at the first word of the workspace, which such a
+// call needs for nothing else (it writes no partials).  The workspace arrives with any contents: the word counts only while
+// its upper 40 bits are this mark, and the first block that finds anything else there sets it to the mark and one arrival.
+// Every call leaves the mark and no arrivals.  Nothing that this library writes into a workspace looks like the mark: its
+// upper half is a NaN that no arithmetic produces (where a partial has l or an output), and larger than any integer of a
+// plan, a maximum or a rounded logit.  Other contents would have to hit 40 chosen bits.
+constexpr int kArrivalBits = 24;
+constexpr unsigned long long kArrivalMark = 0x7fa5c3d296ull << kArrivalBits;
+// Whether this is the last of `blocks` (< 2^24) blocks to call it with `word`.  One thread per block.
+SA_D bool last_to_arrive(unsigned long long* word, unsigned blocks) {
+    unsigned long long seen;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(word) : "memory");
+    unsigned arrived = 0;
+    if ((seen >> kArrivalBits) == (kArrivalMark >> kArrivalBits) || atomicCAS(word, seen, kArrivalMark + 1) != seen)
+        arrived = (unsigned)atomicAdd(word, 1ull) & ((1u << kArrivalBits) - 1u);      // (if the exchange failed, another block has set the mark)
+    if (arrived + 1 != blocks) return false;
+    *word = kArrivalMark;
+    return true;
+}
+// Settles the form of the call: one launch, unless it appends tokens with more blocks than the word can count.
+inline void settle_whole(void* workspace, const Plan& p, DecodeArgs* a) {
+    const long long blocks = (long long)a->n_splits * p.Hkv * (p.G / a->gt) * a->batch;
+    if (a->whole && a->Knew && blocks >= (1LL << kArrivalBits)) a->whole = 0;
+    if (a->whole && a->Knew) a->arrivals = static_cast<unsigned long long*>(workspace);
     if (!a->whole) a->cluster = 1;
 }
 
@@ -503,7 +521,7 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     a->bal_target = 0;
     a->cluster = cluster ? S : 1;
     a->whole = p.matrix && S == a->cluster ? 1 : 0;
-    a->counter = nullptr;
+    a->arrivals = nullptr;
     if (with_plan && batch_is_ranked(c->batch)) {
         a->plan = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)S * c->batch * p.Hq * (p.d + 2) * sizeof(float));
         // blocks per grid row that a batch of unequal lengths is cut into: the grid, rounded down to whole waves of

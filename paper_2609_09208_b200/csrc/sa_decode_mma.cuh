@@ -49,10 +49,9 @@ struct MmaSmem {
 // The lengths grow by one when the kernel appends the step's tokens and no merge kernel follows: by the hand of the last
 // block to get here, every block having read what it needs of them.  One warp per block.
 SA_D void bump_lengths(const DecodeArgs& a, int lane) {
-    unsigned old = 0;
-    if (lane == 0) old = atomicAdd(a.counter, 1u);
-    if (__shfl_sync(0xffffffffu, old, 0) + 1 != gridDim.x * gridDim.y * gridDim.z) return;
-    if (lane == 0) *a.counter = 0u;
+    bool last = false;
+    if (lane == 0) last = last_to_arrive(a.arrivals, gridDim.x * gridDim.y * gridDim.z);
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
     for (int b = lane; b < a.batch; b += 32) {
         const int len = __ldcg(a.seq_lens + b), lp = len / kPageTokens;
         const int page = (len >= 0 && lp < a.max_pages) ? a.page_table[(size_t)b * a.max_pages + lp] : -1;
@@ -185,7 +184,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         }
     } while (again);
     if (ranked && b < 0) {                                        // more blocks than (sequence, split) pairs
-        if (WHOLE && a.counter && warp == 0) bump_lengths(a, lane);
+        if (WHOLE && a.arrivals && warp == 0) bump_lengths(a, lane);
         return;
     }
 
@@ -448,7 +447,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     // below from a register, not through the rows, which alias the stage buffers — a copy that was merely late could
     // still land in them.
     const bool poisoned = __syncthreads_or(failed ? 1 : 0) != 0;
-    if (WHOLE && a.counter && warp == 0) bump_lengths(a, lane);   // every warp of the block has read the lengths
+    if (WHOLE && a.arrivals && warp == 0) bump_lengths(a, lane);  // every warp of the block has read the lengths
     float Rb0 = (float)kMNone, Rb1 = (float)kMNone;
 #pragma unroll
     for (int w = 0; w < NW; ++w) {

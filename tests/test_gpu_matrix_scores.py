@@ -121,3 +121,75 @@ def test_steps_without_a_merge_kernel(d, Hq, Hkv, lens, k, nibble):
         torch.cuda.synchronize()
         assert cache.seq_lens.cpu().numpy().tolist() == (lens + n_steps).tolist()
         assert all(torch.equal(a, b) for a, b in zip(O, first))
+
+
+def one_launch_setup(lens, Hq, Hkv, d=64, k=4):
+    import torch
+    sa_build.build()
+    dev = torch.device("cuda:0")
+    up = lambda x: torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).to(dev)
+    lens = np.asarray(lens)
+    B = len(lens)
+    full = synth.make_case("arrive", lens + 1, Hq, Hkv, d, k, outliers=True, seed=330 + B)
+    cfg = sa.make_config(d, Hq, Hkv, k)
+    cache = sa.PagedCache(cfg, lens, dev, extra_tokens=1)
+    old = np.concatenate([np.arange(full.cu_lens[b], full.cu_lens[b] + lens[b]) for b in range(B)]).astype(np.int64)
+    cache.fill(up(full.K[old]), up(full.V[old]), np.concatenate([[0], np.cumsum(lens)]))
+    new = np.array([full.cu_lens[b + 1] - 1 for b in range(B)])
+    O = torch.full((B, Hq, d), float("nan"), dtype=torch.float32, device=dev)
+    want = ora.decode_attention(full.Q, full.K, full.V, full.cu_lens, k, 6 + k, n_threads=8)["O"]
+    return cfg, cache, up(full.Q), up(full.K[new]), up(full.V[new]), O, want
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv", [([1000], 32, 4), ([17], 1, 1), ([33] * 130, 4, 4)])
+@pytest.mark.parametrize("contents", ["zeros", "ones", "random", "partials", "nearly the mark"])
+def test_step_of_one_launch_takes_a_workspace_with_any_contents(lens, Hq, Hkv, contents):
+    """A step without a merge kernel counts its blocks in the workspace: the lengths grow by one whatever was there, and
+    nothing behind the counting word is written (a step of two launches would leave its partials there)."""
+    import torch
+    cfg, cache, Q, K, V, O, want = one_launch_setup(lens, Hq, Hkv)
+    ws, lens0 = cache.workspace, cache.seq_lens.clone()
+    if contents == "zeros":
+        ws.zero_()
+    elif contents == "ones":
+        ws.fill_(255)
+    elif contents == "partials":
+        sa.decode_attention(cfg, cache.handle, Q, O, ws, stages=1)
+    else:
+        ws.copy_(torch.randint(0, 256, ws.shape, generator=torch.Generator().manual_seed(5), dtype=torch.uint8))
+        if contents == "nearly the mark":                    # its upper half, with other bits below
+            ws[:8].view(torch.int64).copy_(torch.tensor([(0x7fa5c3d2 << 32) | (0x95 << 24) | 3]))
+    before = ws.clone()
+    for i in range(3):
+        cache.seq_lens.copy_(lens0)
+        sa.decode_step(cfg, cache.handle, Q, K, V, O, ws)
+        torch.cuda.synchronize()
+        assert torch.equal(cache.seq_lens, lens0 + 1), i
+        assert np.max(np.abs(O.cpu().numpy() - want)) <= 1e-3
+    end = len(ws) - (16 if 2 <= len(lens) <= 128 else 0)
+    assert torch.equal(ws[16:end], before[16:end])
+
+
+def test_any_number_of_workspaces_serves_steps_of_one_launch():
+    """A program with a workspace for every request, more than 4096 of them over its life: the last step is one launch as
+    the first was, from a side stream and recorded in a graph before any other call too."""
+    import torch
+    cfg, cache, Q, K, V, O, want = one_launch_setup([300], 8, 1)
+    lens0 = cache.seq_lens.clone()
+    size = (len(cache.workspace) + 255) // 256 * 256
+    pool = torch.full((4200, size), 255, dtype=torch.uint8, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        cache.seq_lens.copy_(lens0)
+        sa.decode_step(cfg, cache.handle, Q, K, V, O, pool[0])
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(cache.seq_lens, lens0 + 1)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for ws in pool[1:]:
+            cache.seq_lens.copy_(lens0)
+            sa.decode_step(cfg, cache.handle, Q, K, V, O, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(cache.seq_lens, lens0 + 1)
+    assert np.max(np.abs(O.cpu().numpy() - want)) <= 1e-3
+    assert bool((pool[:, 16:] == 255).all())
