@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
+#include <atomic>
 
 #include "../../include/sa.h"
 
@@ -64,6 +65,20 @@ struct Plan {
     size_t plane_off;         // dense planar container: offset of the mantissa bit planes inside a block
     KernelShape shape;        // of the decode kernel that serves this configuration
     bool matrix;              // that kernel is the one of sa_decode_mma.cuh
+};
+
+// Does something once for every device (an attribute of a kernel belongs to a device's context): set() is called until it has
+// returned true for the device, by several threads at once if they come together, and for devices beyond 63 each time.
+struct OncePerDevice {
+    std::atomic<uint64_t> done{0};
+    template <typename Set>
+    bool operator()(int dev, Set set) {
+        const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+        if (done.load(std::memory_order_acquire) & bit) return true;
+        if (!set()) return false;
+        done.fetch_or(bit, std::memory_order_release);
+        return true;
+    }
 };
 
 sa_status make_plan(const sa_config* cfg, Plan* out);
@@ -290,6 +305,15 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
     return launch_pdl_cluster(kernel, grid, block, smem, s, 1u, args...);
+}
+// Opts a kernel in to `bytes` of dynamic shared memory on the current device where that is more than the 48 KB every kernel
+// may have; `once` is the kernel's own.  False: the attribute was refused (the runtime's last error says why).
+template <typename... KArgs>
+inline bool allow_shared(void (*kernel)(KArgs...), int bytes, OncePerDevice& once) {
+    int dev = -1;
+    if (bytes <= 48 * 1024) return true;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    return once(dev, [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; });
 }
 #endif
 

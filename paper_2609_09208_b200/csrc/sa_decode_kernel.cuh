@@ -598,12 +598,8 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
 template <int D, int KB, bool NIB, int GT, bool SP>
 static void launch_one(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     constexpr int bytes = DecodeSmem<D, KB, NIB, GT>::kBytes;
-    if (bytes > 48 * 1024) {
-        // opt in to more than 48 KB of dynamic shared memory (an attribute of the function; no allocation)
-        static const cudaError_t once = cudaFuncSetAttribute(shift_kernel<D, KB, NIB, GT, SP>,
-                                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        (void)once;
-    }
+    static OncePerDevice once;
+    if (!allow_shared(shift_kernel<D, KB, NIB, GT, SP>, bytes, once)) return;      // (the caller asks for the last error)
     (void)launch_pdl(shift_kernel<D, KB, NIB, GT, SP>, grid, dim3(32 * DecodeSmem<D, KB, NIB, GT>::NW), (size_t)bytes, s, a);
 }
 

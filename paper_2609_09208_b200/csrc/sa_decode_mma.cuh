@@ -511,11 +511,8 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
 template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST, bool WHOLE>
 static void launch_mma_as(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     constexpr int bytes = MmaSmem<D, FMT, NW, NS>::kBytes;
-    if (bytes > 48 * 1024) {
-        static const cudaError_t once = cudaFuncSetAttribute(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST, WHOLE>,
-                                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        (void)once;
-    }
+    static OncePerDevice once;
+    if (!allow_shared(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST, WHOLE>, bytes, once)) return;      // (the caller asks for the last error)
     (void)launch_pdl_cluster(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST, WHOLE>, grid, dim3(32 * NW), (size_t)bytes, s,
                              (unsigned)a.cluster, a);
 }

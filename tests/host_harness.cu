@@ -120,6 +120,13 @@ int hh_encode_element(int k, unsigned a_bits, unsigned s_bits) {
 void hh_encode_many(int k, const uint16_t* a_bits, int64_t n, unsigned s_bits, uint8_t* out) {
     for (int64_t i = 0; i < n; ++i) out[i] = (uint8_t)hh_encode_element(k, a_bits[i], s_bits);
 }
+// OncePerDevice: the devices asked in turn, set() succeeding except at the positions in `fails`; returns the calls of set()
+int hh_once_per_device(const int* devs, const int* fails, int n, int* ok) {
+    OncePerDevice once;
+    int calls = 0;
+    for (int i = 0; i < n; ++i) ok[i] = once(devs[i], [&] { return ++calls, !fails[i]; });
+    return calls;
+}
 int hh_value_exponent(unsigned amax_bits) { return value_exponent(amax_bits); }
 void hh_score8(int k, const uint8_t* canon, const int8_t* q8, int d, int nibble_path, int32_t* out) {
     score8_any<0>(k, canon, q8, d, k == 0 ? nibble_path : 0, out);

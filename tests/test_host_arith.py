@@ -120,3 +120,14 @@ def test_score_datapaths_equal_oracle_scores(hh, k, d):
             hh.hh_score8_alu(C.c_int(k), codes.ctypes.data_as(C.c_void_p), q.ctypes.data_as(C.c_void_p), C.c_int(d),
                              C.c_int(path), out.ctypes.data_as(C.c_void_p))
             assert np.array_equal(out.astype(np.int64), want[:, 0]), ("adds on the ALU pipe", path, trial, out, want[:, 0])
+
+
+@pytest.mark.parametrize("devs,fails,calls", [
+    ([0, 0, 1, 0, 1, 1], [0] * 6, 2),                    # once on each device, not once in the process
+    ([0, 0, 0], [1, 0, 0], 2),                           # what was refused is asked for again
+    ([63, 63, 64, 64, 70], [0] * 5, 4)])                 # beyond the table: each time
+def test_kernel_attributes_are_set_once_per_device(hh, devs, fails, calls):
+    n = len(devs)
+    ok = (C.c_int * n)()
+    assert hh.hh_once_per_device((C.c_int * n)(*devs), (C.c_int * n)(*fails), C.c_int(n), ok) == calls
+    assert list(ok) == [1 - f for f in fails]
