@@ -30,8 +30,10 @@ constexpr float kRefMax = 268435456.0f;   // |R| <= 2^28
 template <int FMT>
 constexpr int format_kb() { return FMT == FMT_PLANAR1 ? 1 : FMT == FMT_PLANAR2 ? 2 : FMT == FMT_INT8 ? 8 : 0; }
 
-// Shared-memory plan of one block: [NW warps x NS stage buffers][mbarriers][R of every warp and query]; the block
-// merge's rows re-use the stage buffers once every warp has left its tile loop.
+// Shared-memory plan of one block: [NW warps x NS stage buffers][mbarriers][R of every warp and query][{R, l} of the block
+// for every query]; the block merge's rows and the block's sums re-use the stage buffers once every warp has left its tile
+// loop.  {R, l} has a place of its own because l carries the mark of a copy that never came: a copy that was merely late
+// may still land in its stage buffer.
 template <int D, int FMT, int NW, int NS>
 struct MmaSmem {
     using SC = ScoreMma<D, FMT>;
@@ -39,9 +41,11 @@ struct MmaSmem {
     using Stage = TileStage<SC::CH, FMT != FMT_FP16, FMT == FMT_FP16 ? 2 * D : D, PLANES, D / 8>;
     static constexpr int kMbarOff = NW * NS * Stage::kBytes;
     static constexpr int kRefOff = kMbarOff + ((NW * NS * 8 + 127) & ~127);
-    static constexpr int kBytes = kRefOff + NW * 8 * 4;
-    static constexpr int kSumOff = NW * 8 * (D + 2) * 4;      // the block's sums, behind the merge rows (within the stage buffers)
-    static_assert(kSumOff + 8 * (D + 2) * 4 <= NW * NS * Stage::kBytes, "merge rows and sums must fit in the stage buffers");
+    static constexpr int kHeadOff = kRefOff + NW * 8 * 4;
+    static constexpr int kBytes = kHeadOff + 8 * 8;
+    static constexpr int kSumOff = NW * 8 * (D + 2) * 4;      // the block's O, behind the merge rows (within the stage buffers)
+    static_assert(kSumOff + 8 * D * 4 <= NW * NS * Stage::kBytes, "merge rows and sums must fit in the stage buffers");
+    static_assert(kHeadOff >= NW * NS * Stage::kBytes, "no copy may land on the marks");
     static_assert(NW * NS * Stage::kBytes >= kPlanScratchInts * 4, "the block plan's scratch must fit in the stage buffers");
     static_assert(Stage::kBytes == (FMT == FMT_FP16 ? half_block_bytes_fp16(D) : half_block_bytes(D, format_kb<FMT>(), SC::kDense)), "a stage buffer is a verbatim copy of half a page block");
 };
@@ -59,11 +63,11 @@ SA_D void bump_lengths(const DecodeArgs& a, int lane) {
     }
 }
 
-// This block's share of the outputs of a cluster (a.cluster blocks, each with its sums {R, l, O[D]} of the query heads at
-// shared address `sums`) -> O.  All loads of an output are in flight together; the blocks are
+// This block's share of the outputs of a cluster (a.cluster blocks, each with {R, l} of the query heads at shared address
+// `heads` and their O[D] at `sums`) -> O.  All loads of an output are in flight together; the blocks are
 // added in order.
 template <int D, int NT>
-SA_D void merge_cluster(const DecodeArgs& a, uint32_t sums, float* O) {
+SA_D void merge_cluster(const DecodeArgs& a, uint32_t heads, uint32_t sums, float* O) {
     constexpr int kMost = kClusterMost;
     const int C = a.cluster, items = a.gt * (D / 2), per = (items + C - 1) / C, rank = blockIdx.x % C;
     for (int i = rank * per + threadIdx.x; i < min(items, (rank + 1) * per); i += NT) {
@@ -74,9 +78,9 @@ SA_D void merge_cluster(const DecodeArgs& a, uint32_t sums, float* O) {
         for (int k = 0; k < kMost; ++k) {
             h[k] = v[k] = make_float2(0.0f, 0.0f);
             if (k < C) {
-                const uint32_t row = C > 1 ? cluster_map(sums, k) : sums;
-                h[k] = C > 1 ? lds_cluster_f2(row + g * (D + 2) * 4) : lds_f2(row + g * (D + 2) * 4);
-                v[k] = C > 1 ? lds_cluster_f2(row + (g * (D + 2) + 2 + 2 * col) * 4) : lds_f2(row + (g * (D + 2) + 2 + 2 * col) * 4);
+                const uint32_t head = heads + g * 8, dims = sums + (g * D + 2 * col) * 4;
+                h[k] = C > 1 ? lds_cluster_f2(cluster_map(head, k)) : lds_f2(head);
+                v[k] = C > 1 ? lds_cluster_f2(cluster_map(dims, k)) : lds_f2(dims);
                 Rm = max(Rm, __float_as_int(h[k].x));
             }
         }
@@ -476,8 +480,10 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     }
     __syncthreads();
     const int slot = ranked ? blockIdx.z * a.n_splits + blockIdx.x : blockIdx.x * a.batch + blockIdx.z;
-    float* sum_s = reinterpret_cast<float*>(smem + SM::kSumOff);                   // [8][D + 2]
-    float* out = WHOLE ? sum_s : a.partials + ((size_t)slot * a.Hq + h0) * (D + 2);
+    // the block's {R, l} and O of every head: the partial, or for the merge within the cluster
+    float* head_out = WHOLE ? reinterpret_cast<float*>(smem + SM::kHeadOff) : a.partials + ((size_t)slot * a.Hq + h0) * (D + 2);
+    float* sum_out = WHOLE ? reinterpret_cast<float*>(smem + SM::kSumOff) : head_out + 2;
+    constexpr int kHeadStep = WHOLE ? 2 : D + 2, kSumStep = WHOLE ? D : D + 2;
     for (int idx = threadIdx.x; idx < GT * (D / 2); idx += 32 * NW) {              // two dims of one head
         const int g = idx / (D / 2), col = idx % (D / 2);
         float2 v = make_float2(0.0f, 0.0f);
@@ -487,7 +493,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
             v.x += x.x;
             v.y += x.y;
         }
-        *reinterpret_cast<float2*>(out + g * (D + 2) + 2 + 2 * col) = v;
+        *reinterpret_cast<float2*>(sum_out + g * kSumStep + 2 * col) = v;
     }
     if (threadIdx.x >= 32 * NW - 8 && 8 - (32 * NW - (int)threadIdx.x) < GT) {     // R and l (by the last warp: it has no more dims than the others)
         const int g = 8 - (32 * NW - (int)threadIdx.x);
@@ -497,13 +503,13 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
             Rm = fmaxf(Rm, ref_s[w * 8 + g]);
             l += red_s[w][g][1];
         }
-        *reinterpret_cast<float2*>(out + g * (D + 2)) = poisoned ? make_float2(__int_as_float(0), __int_as_float(0x7fc00000))      // R = 0, l = NaN
-                                                               : make_float2(__int_as_float(__float2int_rn(Rm)), l);
+        *reinterpret_cast<float2*>(head_out + g * kHeadStep) = poisoned ? make_float2(__int_as_float(0), __int_as_float(0x7fc00000))      // R = 0, l = NaN
+                                                                        : make_float2(__int_as_float(__float2int_rn(Rm)), l);
     }
     if constexpr (WHOLE) {
         if (a.cluster > 1) cluster_sync();
         else __syncthreads();
-        merge_cluster<D, 32 * NW>(a, smem_addr(sum_s), a.O + ((size_t)b * a.Hq + h0) * D);
+        merge_cluster<D, 32 * NW>(a, smem_addr(smem + SM::kHeadOff), smem_addr(smem + SM::kSumOff), a.O + ((size_t)b * a.Hq + h0) * D);
         if (a.cluster > 1) cluster_sync();                                         // no block may leave while others read its sums
     }
 }
