@@ -302,7 +302,8 @@ sa_status sa_decode_attention_static(const sa_config* cfg, const sa_cache* cache
  * in which the bulk copy of ONE tile — 32-token tile `tile` of sequence `b`, KV head `kv_head` — is never
  * issued and every wait for a copy gives up after 2^10 polls instead of 2^18.  The warp that owns that tile
  * finds its wait exhausted, abandons its remaining tiles and marks its block's partial result; the merge of the
- * splits (in a kernel or in a cluster) carries the mark into O: the rows of the query heads of `kv_head` in sequence `b` come out as NaN,
+ * splits (in a kernel, in a cluster or, with one split, in the block: as sa_decode_attention would do it for this
+ * cache) carries the mark into O: the rows of the query heads of `kv_head` in sequence `b` come out as NaN,
  * every other row is the ordinary result, and the call returns like any other (nothing is left in flight,
  * nothing waits without a bound).  Only head_dim 64, SA_POTM4 in the byte container, 8 query heads per KV
  * head, no flags: anything else is SA_ERR_UNSUPPORTED. */

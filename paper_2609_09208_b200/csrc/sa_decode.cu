@@ -97,11 +97,10 @@ extern "C" sa_status sa_debug_decode_lost_copy(const sa_config* cfg, const sa_ca
     a.lost_kvh = kv_head;
     a.lost_tile = tile;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    a.whole = 0;
-    settle_whole(workspace, p, &a);
+    settle_whole(workspace, p, &a);                              // the form that sa_decode_attention takes
     launch_mma_lost_copy(a, dim3((unsigned)a.n_splits, (unsigned)p.Hkv, (unsigned)a.batch), s);
     if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
-    return launch_merge(p, a, s);
+    return a.whole ? SA_OK : launch_merge(p, a, s);
 }
 
 extern "C" sa_status sa_decode_step(const sa_config* cfg, const sa_cache* cache, const uint16_t* Q,

@@ -17,6 +17,7 @@ void launch_mma_byte(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t 
 }
 void launch_mma_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     constexpr KernelShape sh = mma_shape(64, 4);
-    launch_mma_as<64, FMT_BYTE, 7, sh.warps, sh.blocks_per_sm, sh.stages, true, false>(a, grid, s);
+    if (a.whole) launch_mma_as<64, FMT_BYTE, 7, sh.warps, sh.blocks_per_sm, sh.stages, true, true>(a, grid, s);
+    else launch_mma_as<64, FMT_BYTE, 7, sh.warps, sh.blocks_per_sm, sh.stages, true, false>(a, grid, s);
 }
 }  // namespace sa

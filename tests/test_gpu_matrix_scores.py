@@ -193,3 +193,31 @@ def test_any_number_of_workspaces_serves_steps_of_one_launch():
     assert torch.equal(cache.seq_lens, lens0 + 1)
     assert np.max(np.abs(O.cpu().numpy() - want)) <= 1e-3
     assert bool((pool[:, 16:] == 255).all())
+
+
+@pytest.mark.parametrize("lens,lost", [([2000], (0, 1, 40)), ([2000], (0, 3, 62)), ([70], (0, 0, 2)), ([20], (0, 2, 0)), ([33, 64, 0, 5], (1, 2, 1))])
+def test_lost_copy_is_marked_where_no_merge_kernel_runs(lens, lost):
+    """The bounded wait of a copy made to run out (test hook, 2^10 polls) where the splits of a sequence are merged in their
+    thread-block cluster or the sequence has one split: exactly the rows of that (sequence, KV head) are NaN, the others
+    ordinary, and the call was one launch (no partials behind)."""
+    import torch
+    sa_build.build()
+    dev = torch.device("cuda:0")
+    up = lambda x: torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).to(dev)
+    b, kvh, tile = lost
+    case = synth.make_case("lost", lens, 32, 4, 64, 4, outliers=True, seed=5200)
+    cfg = sa.make_config(64, 32, 4, sa.SA_POTM4)
+    cache = sa.PagedCache(cfg, case.lens, dev)
+    cache.fill(up(case.K), up(case.V), case.cu_lens)
+    O = torch.zeros((case.batch, 32, 64), dtype=torch.float32, device=dev)
+    cache.workspace.fill_(255)
+    sa.debug_decode_lost_copy(cfg, cache.handle, up(case.Q), O, cache.workspace, b, kvh, tile)
+    torch.cuda.synchronize()
+    got = O.cpu().numpy()
+    ref = ora.decode_attention(case.Q, case.K, case.V, case.cu_lens, 4, 10, n_threads=8)["O"]
+    hit = np.zeros((case.batch, 32), dtype=bool)
+    hit[b, kvh * 8:(kvh + 1) * 8] = True
+    assert np.isnan(got[hit]).all()
+    assert np.max(np.abs(got[~hit] - ref[~hit])) <= 1e-3
+    end = len(cache.workspace) - (16 * ((8 * case.batch + 15) // 16) if case.batch > 1 else 0)
+    assert bool((cache.workspace[:end] == 255).all())
