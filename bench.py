@@ -57,7 +57,7 @@ VARIANTS = {
     "fp16": (0, False, False, True),
     "int8mac": (8, False, False, False),      # uniform INT8 keys: the paper's multiply-native comparison
 }
-# the same codes with SA_FLAG_SHIFT_BY_MULTIPLY, which today selects the default kernels
+# the same codes on the CUDA cores with the shifts executed by the integer multiplier (SA_FLAG_SHIFT_BY_MULTIPLY; not the default)
 MULSHIFT = {"potm4_mulshift": "potm4", "potm1_mulshift": "potm1", "potm2_mulshift": "potm2"}
 # ... and with scores by shifts, sign flips and adds on the ALU pipe, no multiplier at all (SA_FLAG_ADD_ON_ALU; not the default)
 ADDALU = {"potm4_alu": "potm4", "pot4_nibble_alu": "pot4_nibble", "potm1_alu": "potm1"}
@@ -654,7 +654,7 @@ def run_ours(args):
         "scores_per_s": value * group,                      # (query, key) scores: keys/s x query heads per KV head
         "cold_call_us": {"median": sorted(cold)[len(cold) // 2], "best": min(cold),
                          "what": "one sa_decode_step call (one layer), L2 flushed before each of 5 calls"},
-        "pipe_utilisation": recorded_pipes(BASE_OF.get(args.variant, args.variant) if args.variant in MULSHIFT else args.variant),
+        "pipe_utilisation": recorded_pipes(args.variant),
         "kernel_source_hash": source_hash(),
     }
     pipes = line["pipe_utilisation"]
@@ -887,7 +887,7 @@ def run_sweep(args):
             cell("cfg3 T=32768 B=%d %s%s shift-based A.V (N = k_max = 15)" % (B, names[code], "_nibble" if nib else ""),
                  [32768] * B, 32, 4, 64, code, nibble=nib, outliers=False, shiftav=True, oracle=False)
         for code, nib in ([] if quick else [(1, False), (4, False)]):
-            cell("cfg3 T=32768 B=%d %s%s SA_FLAG_SHIFT_BY_MULTIPLY (the default kernels)" % (B, names[code], "_nibble" if nib else ""),
+            cell("cfg3 T=32768 B=%d %s%s shifts on the integer multiplier" % (B, names[code], "_nibble" if nib else ""),
                  [32768] * B, 32, 4, 64, code, nibble=nib, outliers=False, shift_by_multiply=True, oracle=False)
         for code, nib in ([] if quick else [(0, True), (4, False)]):
             cell("cfg3 T=32768 B=%d %s%s adds on the ALU pipe" % (B, names[code], "_nibble" if nib else ""),

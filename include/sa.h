@@ -84,10 +84,12 @@ enum { SA_POT4 = 0, SA_POTM1 = 1, SA_POTM2 = 2, SA_POTM4 = 4, SA_INT8 = 8, SA_KV
 enum { SA_KLAYOUT_BYTE = 0, SA_KLAYOUT_NIBBLE = 1, SA_KLAYOUT_PLANAR = 2 };
 /* flags */
 #define SA_FLAG_HADAMARD 1u /* rotate Q and K by the normalised Walsh-Hadamard matrix before quantising */
-/* Decode kernels only, mantissa codes (PoT-M1 / M2 / M4) only: the caller asks for scores formed on multipliers.  The
- * default kernels do that already (each key element is decoded once, for the whole query group, and the scores are
- * exact matrix products), so the flag selects the same kernels; it is kept for programs that set it.  (PoT-4:
- * SA_ERR_UNSUPPORTED.) */
+/* Decode kernels only, mantissa codes (PoT-M1 / M2 / M4) only, off by default: the shift-and-add datapath on the CUDA
+ * cores with the left shift of eq. (3), (4) executed on the integer multiplier.  Each key element is decoded once, for the
+ * whole query group, to sigma * 2^(F - k - e) (0 for the zero code) and every (query, element) update is one integer
+ * multiply-add by that power of two.  The INT32 scores are the same bit for bit.  It uses the multiplier array as a
+ * barrel shifter, so it is not the paper's multiplier-free datapath; it exists to be measured beside that and beside the
+ * default, which is 2 - 3 times faster on this GPU.  (PoT-4 has no shift left in its key loop: SA_ERR_UNSUPPORTED.) */
 #define SA_FLAG_SHIFT_BY_MULTIPLY 2u
 /* Decode kernels only, power-of-two codes only, off by default: the paper's multiplier-free datapath.  Every shift, sign
  * flip and add of the integer score (eq. (3)) is a shift, logic or add instruction on the CUDA cores; no instruction of

@@ -1,6 +1,6 @@
 // Entry points of the decode path: argument checks, the split plan, and the dispatch to the decode kernels — matrix
-// scores (sa_decode_mma.cuh) or, for SA_FLAG_ADD_ON_ALU and the score pass of the shift-based A.V option, shifts and adds
-// (sa_decode_kernel.cuh) — and the split-K merge.
+// scores (sa_decode_mma.cuh) or, for SA_FLAG_ADD_ON_ALU, SA_FLAG_SHIFT_BY_MULTIPLY and the score pass of the shift-based
+// A.V option, shifts and adds (sa_decode_kernel.cuh) — and the split-K merge.
 #include "sa_decode_common.cuh"
 
 using namespace sa;
@@ -11,24 +11,24 @@ void launch_mma_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_mma_dense(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_mma_int8(int d, const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_mma_fp16(int d, const DecodeArgs& a, dim3 grid, cudaStream_t s);
-void launch_shift_pot4(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);   // sa_decode_pot*.cu
-void launch_shift_potm1(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
-void launch_shift_potm2(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
-void launch_shift_potm4(int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
+void launch_shift_pot4(bool nib, int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);   // sa_decode_pot*.cu
+void launch_shift_potm1(bool nib, int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
+void launch_shift_potm2(bool nib, int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
+void launch_shift_potm4(int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
 
 // The decode kernel for these arguments (the score pass of the shift-A.V option when a.zr is set).
 void launch_decode_main(const Plan& p, const DecodeArgs& a, int GT, cudaStream_t s) {
     const dim3 grid((unsigned)a.n_splits, (unsigned)(p.Hkv * (p.G / GT)), (unsigned)a.batch);
-    const bool sp = a.zr != nullptr;
+    const ShiftMode mode = a.zr ? SHIFT_SCORE_PASS : p.mulshift ? SHIFT_MUL : SHIFT_ALU;
     if (p.matrix) {
         if (p.fp16) launch_mma_fp16(p.d, a, grid, s);
         else if (p.int8) launch_mma_int8(p.d, a, grid, s);
         else if (p.nibble) launch_mma_dense(p.d, p.k, a, grid, s);
         else launch_mma_byte(p.d, p.k, a, grid, s);
-    } else if (p.k == 0) launch_shift_pot4(p.nibble, p.d, sp, a, GT, grid, s);
-    else if (p.k == 1) launch_shift_potm1(p.nibble, p.d, sp, a, GT, grid, s);
-    else if (p.k == 2) launch_shift_potm2(p.nibble, p.d, sp, a, GT, grid, s);
-    else launch_shift_potm4(p.d, sp, a, GT, grid, s);
+    } else if (p.k == 0) launch_shift_pot4(p.nibble, p.d, mode, a, GT, grid, s);
+    else if (p.k == 1) launch_shift_potm1(p.nibble, p.d, mode, a, GT, grid, s);
+    else if (p.k == 2) launch_shift_potm2(p.nibble, p.d, mode, a, GT, grid, s);
+    else launch_shift_potm4(p.d, mode, a, GT, grid, s);
 }
 }  // namespace sa
 

@@ -10,6 +10,11 @@
 
 namespace sa {
 
+// What a shift-and-add kernel (sa_decode_kernel.cuh) does beside looking queries up and adding them: sign flips and adds as
+// logic and add instructions (SA_FLAG_ADD_ON_ALU); the score pass of the shift-based A.V option, sign flip and add as one
+// multiply-add by +1 / -1; the shift and the sign as one multiply-add by sigma * 2^r (SA_FLAG_SHIFT_BY_MULTIPLY).
+enum ShiftMode { SHIFT_ALU, SHIFT_SCORE_PASS, SHIFT_MUL };
+
 struct DecodeArgs {
     const uint8_t* pages;
     const int32_t* page_table;

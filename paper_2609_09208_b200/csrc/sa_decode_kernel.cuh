@@ -2,7 +2,8 @@
 // (sa_decode_pot*.cu, one per key code so that they compile in parallel).
 #pragma once
 // Decode attention whose integer scores are formed by shifts, sign flips and adds alone, as the paper writes them
-// (section II-B eq. (3), II-D eq. (5)).  It serves SA_FLAG_ADD_ON_ALU and the score pass of the shift-based A.V option;
+// (section II-B eq. (3), II-D eq. (5)), on the CUDA cores.  It serves SA_FLAG_ADD_ON_ALU, SA_FLAG_SHIFT_BY_MULTIPLY (whose
+// shifts are multiplications by powers of two) and the score pass of the shift-based A.V option;
 // the default kernel (sa_decode_mma.cuh) forms the same integers as matrix products, at 2 - 5 times the rate.
 //
 // Grid (split, KV head x query chunk, sequence); 4, 8 or 10 warps per block (shift_shape).  A block
@@ -68,15 +69,15 @@ struct DecodeSmem {
     static_assert(Stage::kBytes == half_block_bytes(D, KB, NIB), "a stage buffer is a verbatim copy of half a page block");
 };
 
-template <int D, int KB, bool NIB, int GT, bool SP>
+template <int D, int KB, bool NIB, int GT, ShiftMode MODE>
 #ifdef SA_ABLATE_NO_MIN_BLOCKS
 __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW)) shift_kernel(DecodeArgs a) {
 #else
 __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (DecodeSmem<D, KB, NIB, GT>::kBlocksPerSM)) shift_kernel(DecodeArgs a) {
 #endif
-    // KB = 0: PoT-4 (packed datapath); KB = 1, 2, 4: mantissa codes (table datapath); no multiply-add in either (the
-    // score pass: sign flip and add as one multiply-add by +1 / -1, see sa_datapath.cuh).
+    // KB = 0: PoT-4 (packed datapath); KB = 1, 2, 4: mantissa codes (table datapath).
     // SP: the score pass of the shift-based A.V option (rounded logits and statistics instead of softmax and A.V).
+    constexpr bool SP = MODE == SHIFT_SCORE_PASS;
     using SM = DecodeSmem<D, KB, NIB, GT>;
     using Stage = typename SM::Stage;
     constexpr int EPL = D / 32;
@@ -356,7 +357,7 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
             int32_t A[GT];
             const uint32_t* cw = reinterpret_cast<const uint32_t*>(st) + lane * 4;
             if constexpr (SM::kTable) {
-                using TS = TableScore<KB, NP, false, !SP>;
+                using TS = TableScore<KB, NP, MODE == SHIFT_MUL, MODE == SHIFT_ALU>;
                 uint32_t grp = smem_addr(smem + SM::kQpOff);    // table of the next 16 elements (256-byte aligned)
                 TS ts;
                 ts.begin(a.one);
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
             } else {
                 // PoT-4: the packed pairs, shifted ahead of the loop, are looked up by the key's exponent field
                 using ST = ShiftTable<NP>;
-                PackedShift<NP, !SP> pl;
+                PackedShift<NP, MODE == SHIFT_ALU> pl;
                 pl.begin(a.one);
                 uint32_t grp = smem_addr(smem + SM::kQpOff);     // rows of the next group of elements (256-byte aligned)
                 if constexpr (!NIB) {
@@ -595,34 +596,35 @@ __global__ void __launch_bounds__((32 * DecodeSmem<D, KB, NIB, GT>::NW), (Decode
     block_merge_and_store<D, GT, NW>(a, red_s, M, l, acc, lane, warp, slot, h0, failed);
 }
 
-template <int D, int KB, bool NIB, int GT, bool SP>
+template <int D, int KB, bool NIB, int GT, ShiftMode MODE>
 static void launch_one(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
     constexpr int bytes = DecodeSmem<D, KB, NIB, GT>::kBytes;
     static OncePerDevice once;
-    if (!allow_shared(shift_kernel<D, KB, NIB, GT, SP>, bytes, once)) return;      // (the caller asks for the last error)
-    (void)launch_pdl(shift_kernel<D, KB, NIB, GT, SP>, grid, dim3(32 * DecodeSmem<D, KB, NIB, GT>::NW), (size_t)bytes, s, a);
+    if (!allow_shared(shift_kernel<D, KB, NIB, GT, MODE>, bytes, once)) return;      // (the caller asks for the last error)
+    (void)launch_pdl(shift_kernel<D, KB, NIB, GT, MODE>, grid, dim3(32 * DecodeSmem<D, KB, NIB, GT>::NW), (size_t)bytes, s, a);
 }
 
-template <int D, int KB, bool NIB, bool SP>
+template <int D, int KB, bool NIB, ShiftMode MODE>
 static void launch_gt(const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
     switch (GT) {
-        case 8: launch_one<D, KB, NIB, 8, SP>(a, grid, s); break;
-        case 4: launch_one<D, KB, NIB, 4, SP>(a, grid, s); break;
-        case 2: launch_one<D, KB, NIB, 2, SP>(a, grid, s); break;
-        default: launch_one<D, KB, NIB, 1, SP>(a, grid, s); break;
+        case 8: launch_one<D, KB, NIB, 8, MODE>(a, grid, s); break;
+        case 4: launch_one<D, KB, NIB, 4, MODE>(a, grid, s); break;
+        case 2: launch_one<D, KB, NIB, 2, MODE>(a, grid, s); break;
+        default: launch_one<D, KB, NIB, 1, MODE>(a, grid, s); break;
     }
 }
 
-// All instantiations of one key code and container: head_dim 64 / 128, the queries per block, decode or score pass.
+// All instantiations of one key code and container: head_dim 64 / 128, the queries per block, the mode.
+template <int D, int KB, bool NIB>
+static void launch_mode(ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
+    if (mode == SHIFT_SCORE_PASS) launch_gt<D, KB, NIB, SHIFT_SCORE_PASS>(a, GT, grid, s);
+    else if (mode == SHIFT_ALU) launch_gt<D, KB, NIB, SHIFT_ALU>(a, GT, grid, s);
+    else if constexpr (KB != 0) launch_gt<D, KB, NIB, SHIFT_MUL>(a, GT, grid, s);      // (PoT-4: refused by make_plan)
+}
 template <int KB, bool NIB>
-static void launch_code(int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
-    if (d == 64) {
-        if (score_pass) launch_gt<64, KB, NIB, true>(a, GT, grid, s);
-        else launch_gt<64, KB, NIB, false>(a, GT, grid, s);
-    } else {
-        if (score_pass) launch_gt<128, KB, NIB, true>(a, GT, grid, s);
-        else launch_gt<128, KB, NIB, false>(a, GT, grid, s);
-    }
+static void launch_code(int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
+    if (d == 64) launch_mode<64, KB, NIB>(mode, a, GT, grid, s);
+    else launch_mode<128, KB, NIB>(mode, a, GT, grid, s);
 }
 
 }  // namespace sa

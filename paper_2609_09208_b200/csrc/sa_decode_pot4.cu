@@ -2,8 +2,8 @@
 #include "sa_decode_kernel.cuh"
 
 namespace sa {
-void launch_shift_pot4(bool nib, int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
-    if (nib) launch_code<0, true>(d, score_pass, a, GT, grid, s);
-    else launch_code<0, false>(d, score_pass, a, GT, grid, s);
+void launch_shift_pot4(bool nib, int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
+    if (nib) launch_code<0, true>(d, mode, a, GT, grid, s);
+    else launch_code<0, false>(d, mode, a, GT, grid, s);
 }
 }  // namespace sa

@@ -2,7 +2,7 @@
 #include "sa_decode_kernel.cuh"
 
 namespace sa {
-void launch_shift_potm4(int d, bool score_pass, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
-    launch_code<4, false>(d, score_pass, a, GT, grid, s);
+void launch_shift_potm4(int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
+    launch_code<4, false>(d, mode, a, GT, grid, s);
 }
 }  // namespace sa

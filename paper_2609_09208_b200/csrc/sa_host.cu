@@ -63,7 +63,7 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
     if (cfg->code != SA_POT4 && cfg->code != SA_POTM1 && cfg->code != SA_POTM2 && cfg->code != SA_POTM4)
         return SA_ERR_UNSUPPORTED;
     p.k = cfg->code;
-    p.matrix = !p.addalu;
+    p.matrix = !p.addalu && !p.mulshift;
     p.shape = p.matrix ? mma_shape(p.d, p.k) : shift_shape(p.d, p.k);
     if (cfg->klayout == SA_KLAYOUT_NIBBLE) {
         if (p.k != 0) return SA_ERR_UNSUPPORTED;
