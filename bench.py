@@ -61,7 +61,9 @@ VARIANTS = {
 MULSHIFT = {"potm4_mulshift": "potm4", "potm1_mulshift": "potm1", "potm2_mulshift": "potm2"}
 # ... and with scores by shifts, sign flips and adds on the ALU pipe, no multiplier at all (SA_FLAG_ADD_ON_ALU; not the default)
 ADDALU = {"potm4_alu": "potm4", "pot4_nibble_alu": "pot4_nibble", "potm1_alu": "potm1"}
-for _name, _base in list(MULSHIFT.items()) + list(ADDALU.items()):
+# ... and with shifts, and every sign flip and add as one multiply-add by +1 / -1 (SA_FLAG_SHIFT_ADD; not the default)
+SHIFTADD = {"potm4_shift": "potm4", "pot4_nibble_shift": "pot4_nibble", "potm1_shift": "potm1"}
+for _name, _base in list(MULSHIFT.items()) + list(ADDALU.items()) + list(SHIFTADD.items()):
     VARIANTS[_name] = VARIANTS[_base]
 
 
@@ -101,7 +103,8 @@ class Workload:
         self.fp16, self.code_k, self.hadamard, self.seed = fp16, code_k, hadamard, seed
         self.bpk = bytes_per_key(d, code_k, nibble, fp16)
         self.cfg = sa.make_config(d, Hq, Hkv, sa.SA_KV_FP16 if fp16 else code_k, nibble=nibble, hadamard=hadamard,
-                                  shift_by_multiply=variant in MULSHIFT, add_on_alu=variant in ADDALU)
+                                  shift_by_multiply=variant in MULSHIFT, add_on_alu=variant in ADDALU,
+                                  shift_add=variant in SHIFTADD)
         self.caches, self.Q, self.Kn, self.Vn, self.O = [], [], [], [], []
         cu = np.arange(batch + 1, dtype=np.int64) * T
         pages_per_seq = (T + room_tokens + 63) // 64
@@ -679,7 +682,7 @@ def run_ours(args):
 
 
 # the recorded captures are of the default kernels; a labelled variant reads its base code's DRAM traffic
-BASE_OF = dict(list(MULSHIFT.items()) + list(ADDALU.items()))
+BASE_OF = dict(list(MULSHIFT.items()) + list(ADDALU.items()) + list(SHIFTADD.items()))
 
 
 def context_rows(args, dev):
@@ -688,8 +691,8 @@ def context_rows(args, dev):
     import torch
     variants = ["fp16", "int8mac", "pot4_nibble", "potm4"]
     cells = [(v, b) for b in (1, 8, 32) for v in variants]
-    cells += [("potm4_alu", 1), ("potm4_mulshift", 1), ("potm4_alu", 32), ("potm4_mulshift", 32),
-              ("pot4_nibble_alu", 32), ("potm1", 1), ("potm1", 32)]
+    cells += [("potm4_shift", 1), ("potm4_alu", 1), ("potm4_mulshift", 1), ("potm4_shift", 32), ("potm4_alu", 32),
+              ("potm4_mulshift", 32), ("pot4_nibble_shift", 32), ("pot4_nibble_alu", 32), ("potm1", 1), ("potm1", 32)]
     rows, us_of = [], {}
     for variant, batch in cells:
         code_k, nibble, _, fp16 = VARIANTS[variant]
@@ -740,12 +743,12 @@ class SweepCell:
     """Seeded synthetic caches of one cell on the device, enough distinct copies that one pass reads more than L2."""
 
     def __init__(self, dev, lens, Hq, Hkv, d, code, nibble=False, hadamard=False, outliers=True, seed=1, min_bytes=400e6,
-                 shiftav=False, shift_by_multiply=False, add_on_alu=False):
+                 shiftav=False, shift_by_multiply=False, add_on_alu=False, shift_add=False):
         import torch
         from paper_2609_09208_b200 import binding as sa
         self.sa, self.torch = sa, torch
         self.cfg = sa.make_config(d, Hq, Hkv, code, nibble=nibble, hadamard=hadamard and code != 16,
-                                  shift_by_multiply=shift_by_multiply, add_on_alu=add_on_alu)
+                                  shift_by_multiply=shift_by_multiply, add_on_alu=add_on_alu, shift_add=shift_add)
         self.fp16 = code == 16
         self.shiftav = shiftav                                # eq. (6), (7) option: N = k_max = 15
         lens = np.asarray(lens, dtype=np.int64)
@@ -889,6 +892,9 @@ def run_sweep(args):
         for code, nib in ([] if quick else [(1, False), (4, False)]):
             cell("cfg3 T=32768 B=%d %s%s shifts on the integer multiplier" % (B, names[code], "_nibble" if nib else ""),
                  [32768] * B, 32, 4, 64, code, nibble=nib, outliers=False, shift_by_multiply=True, oracle=False)
+        for code, nib in ([] if quick else [(0, True), (4, False)]):
+            cell("cfg3 T=32768 B=%d %s%s shifts and adds on both integer pipes" % (B, names[code], "_nibble" if nib else ""),
+                 [32768] * B, 32, 4, 64, code, nibble=nib, outliers=False, shift_add=True, oracle=False)
         for code, nib in ([] if quick else [(0, True), (4, False)]):
             cell("cfg3 T=32768 B=%d %s%s adds on the ALU pipe" % (B, names[code], "_nibble" if nib else ""),
                  [32768] * B, 32, 4, 64, code, nibble=nib, outliers=False, add_on_alu=True, oracle=False)

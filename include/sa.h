@@ -96,6 +96,11 @@ enum { SA_KLAYOUT_BYTE = 0, SA_KLAYOUT_NIBBLE = 1, SA_KLAYOUT_PLANAR = 2 };
  * the score datapath touches a multiplier or a tensor core.  The INT32 scores are the same bit for bit.  It is 2 - 5
  * times slower than the default on this GPU and exists to be measured beside it.  Excludes SA_FLAG_SHIFT_BY_MULTIPLY. */
 #define SA_FLAG_ADD_ON_ALU 4u
+/* Decode kernels only, power-of-two codes only, off by default: the scores on the integer datapath of the CUDA cores, split
+ * over its two pipes.  Every magnitude is shifted by a shift instruction; the sign flip and the add are one integer
+ * multiply-add by +1 or -1, which issues beside the shifts.  Same INT32 scores bit for bit, 1.3 - 1.6 times the rate of
+ * SA_FLAG_ADD_ON_ALU.  Excludes the two flags above.  (8u is not a flag.) */
+#define SA_FLAG_SHIFT_ADD 16u
 
 typedef struct {
     int head_dim;    /* 64 or 128 */
@@ -107,7 +112,7 @@ typedef struct {
                         Must satisfy F >= 6 + k (eq. (4): every shift is a left shift) and
                         head_dim * 127 * (2^(k+1) - 1) * 2^(F - k) < 2^31 (INT32 accumulator) */
     int page_tokens; /* 64 */
-    unsigned flags;  /* SA_FLAG_HADAMARD | SA_FLAG_SHIFT_BY_MULTIPLY | SA_FLAG_ADD_ON_ALU */
+    unsigned flags;  /* SA_FLAG_HADAMARD and at most one of SA_FLAG_SHIFT_BY_MULTIPLY, SA_FLAG_ADD_ON_ALU, SA_FLAG_SHIFT_ADD */
 } sa_config;
 
 typedef struct {
@@ -186,7 +191,8 @@ sa_status sa_fill_kv(const sa_config* cfg, const sa_cache* cache, const uint16_t
  *   The scores are matrix products on the tensor cores, over the whole query group of a KV head: a decoded
  *   key element is a 5-bit magnitude times a power of two, the queries are 8-bit integers, and binary16
  *   operands with FP32 sums below 2^24 units (or INT8 operands with INT32 sums) give the integer of eq. (3)
- *   without rounding.  SA_FLAG_ADD_ON_ALU forms the same integers by shifts and adds alone.
+ *   without rounding.  SA_FLAG_SHIFT_ADD and SA_FLAG_ADD_ON_ALU form the same integers by shifts, sign flips and adds on
+ *   the CUDA cores.
  *   The A.V products run on the tensor cores with FP32 accumulation: the INT8 values are exact in binary16,
  *   and every weight enters as the sum of two binary16 terms (22 significant bits down to 2^-17 of the
  *   largest weight, an absolute 2^-38 of it below that); measured |dO| against the CPU oracle: 1e-6 relative.

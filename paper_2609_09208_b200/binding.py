@@ -22,6 +22,7 @@ SA_KLAYOUT_BYTE, SA_KLAYOUT_NIBBLE, SA_KLAYOUT_PLANAR = 0, 1, 2
 SA_FLAG_HADAMARD = 1
 SA_FLAG_SHIFT_BY_MULTIPLY = 2
 SA_FLAG_ADD_ON_ALU = 4
+SA_FLAG_SHIFT_ADD = 16
 PAGE_TOKENS = 64
 
 EXPORTS = [
@@ -99,17 +100,18 @@ def _check(st: int, where: str):
 
 def make_config(head_dim: int, n_q_heads: int, n_kv_heads: int, code: int, *, nibble: bool = False,
                 headroom_F: int = 0, hadamard: bool = False, shift_by_multiply: bool = False,
-                add_on_alu: bool = False) -> SaConfig:
+                add_on_alu: bool = False, shift_add: bool = False) -> SaConfig:
     """nibble=True selects the dense sub-byte container of the code: two 4-bit codes per byte for PoT-4,
-    nibbles plus mantissa bit planes (5 / 6 bits per element) for PoT-M1 / PoT-M2.  shift_by_multiply=True
-    selects the non-default decode kernels whose shifts run on the integer multiplier, add_on_alu=True the
-    non-default ones without any multiply-add in the score datapath (same scores either way)."""
+    nibbles plus mantissa bit planes (5 / 6 bits per element) for PoT-M1 / PoT-M2.  At most one of the next three
+    selects non-default decode kernels with the scores on the CUDA cores (the same scores): shift_add=True shifts and
+    adds (a sign flip and add is a multiply-add by +1 or -1), add_on_alu=True the same without any multiply-add,
+    shift_by_multiply=True with the shifts on the integer multiplier."""
     klayout = SA_KLAYOUT_BYTE
     if nibble:
         klayout = SA_KLAYOUT_NIBBLE if code == SA_POT4 else SA_KLAYOUT_PLANAR
     return SaConfig(head_dim, n_q_heads, n_kv_heads, code, klayout, headroom_F, PAGE_TOKENS,
                     (SA_FLAG_HADAMARD if hadamard else 0) | (SA_FLAG_SHIFT_BY_MULTIPLY if shift_by_multiply else 0) |
-                    (SA_FLAG_ADD_ON_ALU if add_on_alu else 0))
+                    (SA_FLAG_ADD_ON_ALU if add_on_alu else 0) | (SA_FLAG_SHIFT_ADD if shift_add else 0))
 
 
 def get_layout(cfg: SaConfig) -> SaLayout:

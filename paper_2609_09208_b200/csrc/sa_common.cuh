@@ -57,6 +57,7 @@ struct Plan {
     int d, Hq, Hkv, G, k;     // k = mantissa bits (0 for SA_KV_FP16)
     bool mulshift;            // SA_FLAG_SHIFT_BY_MULTIPLY: the scores' shifts run on the integer multiplier
     bool addalu;              // SA_FLAG_ADD_ON_ALU: sign flips and adds as logic/add instructions, no multiply-add
+    bool shiftadd;            // SA_FLAG_SHIFT_ADD: shifts, and sign flip and add as one multiply-add by +1 / -1
     bool fp16, nibble, hadamard, int8;   // nibble: 4-bit sign/exponent codes (PoT-4 nibble container, or with k = 1, 2
                                          // the dense planar container); int8: the uniform INT8 comparison code
     int F;                    // head-room actually used

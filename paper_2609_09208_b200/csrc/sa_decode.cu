@@ -1,5 +1,5 @@
 // Entry points of the decode path: argument checks, the split plan, and the dispatch to the decode kernels — matrix
-// scores (sa_decode_mma.cuh) or, for SA_FLAG_ADD_ON_ALU, SA_FLAG_SHIFT_BY_MULTIPLY and the score pass of the shift-based
+// scores (sa_decode_mma.cuh) or, for the flags that ask for the CUDA cores and the score pass of the shift-based
 // A.V option, shifts and adds (sa_decode_kernel.cuh) — and the split-K merge.
 #include "sa_decode_common.cuh"
 
@@ -19,7 +19,7 @@ void launch_shift_potm4(int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3
 // The decode kernel for these arguments (the score pass of the shift-A.V option when a.zr is set).
 void launch_decode_main(const Plan& p, const DecodeArgs& a, int GT, cudaStream_t s) {
     const dim3 grid((unsigned)a.n_splits, (unsigned)(p.Hkv * (p.G / GT)), (unsigned)a.batch);
-    const ShiftMode mode = a.zr ? SHIFT_SCORE_PASS : p.mulshift ? SHIFT_MUL : SHIFT_ALU;
+    const ShiftMode mode = a.zr ? SHIFT_SCORE_PASS : p.mulshift ? SHIFT_MUL : p.addalu ? SHIFT_ALU : SHIFT_FMA;
     if (p.matrix) {
         if (p.fp16) launch_mma_fp16(p.d, a, grid, s);
         else if (p.int8) launch_mma_int8(p.d, a, grid, s);
@@ -86,7 +86,7 @@ extern "C" sa_status sa_debug_decode_lost_copy(const sa_config* cfg, const sa_ca
     Plan p;
     sa_status st = make_plan(cfg, &p);
     if (st != SA_OK) return st;
-    if (p.fp16 || p.int8 || p.nibble || p.d != 64 || p.k != 4 || p.G != 8 || p.mulshift || p.addalu) return SA_ERR_UNSUPPORTED;
+    if (p.fp16 || p.int8 || p.nibble || p.d != 64 || p.k != 4 || p.G != 8 || !p.matrix) return SA_ERR_UNSUPPORTED;
     DecodeArgs a;
     int GT;
     st = make_decode_args(p, cache, Q, O, workspace, workspace_bytes, &a, &GT);

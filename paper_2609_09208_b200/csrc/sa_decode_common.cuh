@@ -10,10 +10,10 @@
 
 namespace sa {
 
-// What a shift-and-add kernel (sa_decode_kernel.cuh) does beside looking queries up and adding them: sign flips and adds as
-// logic and add instructions (SA_FLAG_ADD_ON_ALU); the score pass of the shift-based A.V option, sign flip and add as one
-// multiply-add by +1 / -1; the shift and the sign as one multiply-add by sigma * 2^r (SA_FLAG_SHIFT_BY_MULTIPLY).
-enum ShiftMode { SHIFT_ALU, SHIFT_SCORE_PASS, SHIFT_MUL };
+// What a shift-and-add kernel (sa_decode_kernel.cuh) does with a looked-up query: sign flip and add as logic and add
+// instructions (SA_FLAG_ADD_ON_ALU) or as one multiply-add by +1 / -1 (SA_FLAG_SHIFT_ADD, and the score pass of the
+// shift-based A.V option); the shift too, as one multiply-add by sigma * 2^r (SA_FLAG_SHIFT_BY_MULTIPLY).
+enum ShiftMode { SHIFT_ALU, SHIFT_FMA, SHIFT_MUL, SHIFT_SCORE_PASS };
 
 struct DecodeArgs {
     const uint8_t* pages;

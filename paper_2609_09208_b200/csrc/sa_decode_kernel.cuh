@@ -2,9 +2,9 @@
 // (sa_decode_pot*.cu, one per key code so that they compile in parallel).
 #pragma once
 // Decode attention whose integer scores are formed by shifts, sign flips and adds alone, as the paper writes them
-// (section II-B eq. (3), II-D eq. (5)), on the CUDA cores.  It serves SA_FLAG_ADD_ON_ALU, SA_FLAG_SHIFT_BY_MULTIPLY (whose
-// shifts are multiplications by powers of two) and the score pass of the shift-based A.V option;
-// the default kernel (sa_decode_mma.cuh) forms the same integers as matrix products, at 2 - 5 times the rate.
+// (section II-B eq. (3), II-D eq. (5)), on the CUDA cores.  It serves SA_FLAG_SHIFT_ADD, SA_FLAG_ADD_ON_ALU,
+// SA_FLAG_SHIFT_BY_MULTIPLY (whose shifts are multiplications by powers of two) and the score pass of the shift-based A.V
+// option; the default kernel (sa_decode_mma.cuh) forms the same integers as matrix products, at 2 - 5 times the rate.
 //
 // Grid (split, KV head x query chunk, sequence); 4, 8 or 10 warps per block (shift_shape).  A block
 // quantises its GT query heads into shared memory (ahead of its wait on the preceding kernel),
@@ -619,6 +619,7 @@ template <int D, int KB, bool NIB>
 static void launch_mode(ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s) {
     if (mode == SHIFT_SCORE_PASS) launch_gt<D, KB, NIB, SHIFT_SCORE_PASS>(a, GT, grid, s);
     else if (mode == SHIFT_ALU) launch_gt<D, KB, NIB, SHIFT_ALU>(a, GT, grid, s);
+    else if (mode == SHIFT_FMA) launch_gt<D, KB, NIB, SHIFT_FMA>(a, GT, grid, s);
     else if constexpr (KB != 0) launch_gt<D, KB, NIB, SHIFT_MUL>(a, GT, grid, s);      // (PoT-4: refused by make_plan)
 }
 template <int KB, bool NIB>

@@ -12,11 +12,12 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
         return SA_ERR_INVALID_ARG;
     if (cfg->head_dim != 64 && cfg->head_dim != 128) return SA_ERR_UNSUPPORTED;
     if (cfg->page_tokens != kPageTokens) return SA_ERR_UNSUPPORTED;
-    if (cfg->flags & ~(SA_FLAG_HADAMARD | SA_FLAG_SHIFT_BY_MULTIPLY | SA_FLAG_ADD_ON_ALU)) return SA_ERR_INVALID_ARG;
+    if (cfg->flags & ~(SA_FLAG_HADAMARD | SA_FLAG_SHIFT_BY_MULTIPLY | SA_FLAG_ADD_ON_ALU | SA_FLAG_SHIFT_ADD)) return SA_ERR_INVALID_ARG;
     p.mulshift = (cfg->flags & SA_FLAG_SHIFT_BY_MULTIPLY) != 0;
     p.addalu = (cfg->flags & SA_FLAG_ADD_ON_ALU) != 0;
-    if (p.mulshift && p.addalu) return SA_ERR_INVALID_ARG;
-    if (p.addalu && (cfg->code == SA_KV_FP16 || cfg->code == SA_INT8)) return SA_ERR_UNSUPPORTED;   // no shift-and-add datapath there
+    p.shiftadd = (cfg->flags & SA_FLAG_SHIFT_ADD) != 0;
+    if (p.mulshift + p.addalu + p.shiftadd > 1) return SA_ERR_INVALID_ARG;
+    if ((p.addalu || p.shiftadd) && (cfg->code == SA_KV_FP16 || cfg->code == SA_INT8)) return SA_ERR_UNSUPPORTED;   // no shift-and-add datapath there
     // no shift in the key loop to move: FP16 and INT8 have none, PoT-4 looks its shifted queries up
     if (p.mulshift && (cfg->code == SA_KV_FP16 || cfg->code == SA_INT8 || cfg->code == SA_POT4)) return SA_ERR_UNSUPPORTED;
     p.d = cfg->head_dim;
@@ -63,7 +64,7 @@ sa_status make_plan(const sa_config* cfg, Plan* out) {
     if (cfg->code != SA_POT4 && cfg->code != SA_POTM1 && cfg->code != SA_POTM2 && cfg->code != SA_POTM4)
         return SA_ERR_UNSUPPORTED;
     p.k = cfg->code;
-    p.matrix = !p.addalu && !p.mulshift;
+    p.matrix = !p.addalu && !p.mulshift && !p.shiftadd;
     p.shape = p.matrix ? mma_shape(p.d, p.k) : shift_shape(p.d, p.k);
     if (cfg->klayout == SA_KLAYOUT_NIBBLE) {
         if (p.k != 0) return SA_ERR_UNSUPPORTED;

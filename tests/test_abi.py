@@ -171,6 +171,14 @@ def test_flag_combinations():
     assert _status(sa.get_layout, sa.make_config(64, 32, 4, sa.SA_POTM4, add_on_alu=True, shift_by_multiply=True)) == 1
     assert _status(sa.get_layout, sa.make_config(64, 32, 4, sa.SA_INT8, add_on_alu=True)) == 2
     assert _status(sa.get_layout, sa.make_config(64, 32, 4, sa.SA_KV_FP16, add_on_alu=True)) == 2
+    # shifts and adds over both integer pipes: the power-of-two codes, and no other datapath beside it
+    for code, nib in [(sa.SA_POT4, False), (sa.SA_POT4, True), (sa.SA_POTM1, True), (sa.SA_POTM2, False), (sa.SA_POTM4, False)]:
+        assert _status(sa.get_layout, sa.make_config(64, 32, 4, code, nibble=nib, shift_add=True)) == 0
+    assert _status(sa.get_layout, sa.make_config(64, 32, 4, sa.SA_POTM4, shift_add=True, hadamard=True)) == 0
+    for other in ("add_on_alu", "shift_by_multiply"):
+        assert _status(sa.get_layout, sa.make_config(64, 32, 4, sa.SA_POTM4, shift_add=True, **{other: True})) == 1
+    for code in (sa.SA_INT8, sa.SA_KV_FP16):
+        assert _status(sa.get_layout, sa.make_config(64, 32, 4, code, shift_add=True)) == 2
 
 
 def test_lost_copy_hook_validates_on_the_host():

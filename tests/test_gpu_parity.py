@@ -693,6 +693,26 @@ def test_add_on_alu_excludes_shift_by_multiply(dev):
         sa.get_layout(cfg)
 
 
+# ---------------------------------- shifts, and sign flip and add as one multiply-add by +-1 (non-default option)
+@pytest.mark.parametrize("d,Hq,Hkv", [(64, 32, 4), (128, 8, 2), (64, 6, 2)])
+@pytest.mark.parametrize("k,nibble", [(0, False), (0, True), (1, False), (1, True), (2, True), (4, False)])
+def test_shift_add_gives_the_same_scores_and_outputs(dev, d, Hq, Hkv, k, nibble):
+    """SA_FLAG_SHIFT_ADD: INT32 scores bit-exact against the oracle, and the outputs those of SA_FLAG_ADD_ON_ALU bit for
+    bit (the same kernel but for the instructions of the sum); ragged batch, head-room above the default."""
+    import torch
+    F = 6 + k + (2 if d == 64 else 0)
+    case = synth.make_case("shiftadd", [700, 0, 33, 129], Hq, Hkv, d, k, outliers=True, seed=5000 + 10 * k + d, nibble=nibble)
+    alu, _, _ = run_decode(case, dev, F=F, permute_seed=11, add_on_alu=True)
+    cfg = sa.make_config(d, Hq, Hkv, k, nibble=nibble, headroom_F=F, shift_add=True)
+    cfg, cache = build_cache(case, dev, cfg=cfg, permute_seed=11)
+    O = torch.full((case.batch, Hq, d), float("nan"), dtype=torch.float32, device=dev)
+    dbg = torch.full((case.batch, Hq, cache.max_pages * 64), -7, dtype=torch.int32, device=dev)
+    sa.decode_attention(cfg, cache.handle, t16(case.Q, dev), O, cache.workspace, dbg)
+    torch.cuda.synchronize()
+    check_against_oracle(case, O.cpu().numpy(), dbg.cpu().numpy(), F=F)
+    assert np.array_equal(O.cpu().numpy().view(np.uint32), alu.view(np.uint32))
+
+
 # ------------------------------------------------------------------ a staged copy that never arrives
 @pytest.mark.parametrize("lost", [(1, 2, 3), (0, 0, 0), (2, 3, 9)])
 def test_lost_copy_marks_exactly_its_rows_and_returns(dev, lost):
