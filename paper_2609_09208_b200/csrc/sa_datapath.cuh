@@ -1,6 +1,7 @@
-// The integer score datapath of the decode kernel (section II-B eq. (3), II-C eq. (4), II-D
+// The integer score datapath of the shift-and-add kernels (sa_decode_kernel.cuh; section II-B eq. (3), II-C eq. (4), II-D
 // eq. (5)): shifts, sign flips and adds only.  Everything here also compiles for the host so
-// that the unit tests can run the very same arithmetic against the CPU oracle without a GPU.
+// that the unit tests can run the very same arithmetic against the CPU oracle without a GPU.  Described is the form of
+// SA_FLAG_SHIFT_ADD; the template parameters ALU and MUL are those of SA_FLAG_ADD_ON_ALU and SA_FLAG_SHIFT_BY_MULTIPLY.
 //
 // Term of element m at head-room F0 = 6 + KB:  sigma * (qhat << r) * (2^KB + j),  r = 6 - e >= 0.
 //
@@ -138,7 +139,7 @@ SA_HD uint32_t pack_pair(int q_lo, int q_hi) { return ((uint32_t)q_hi << 16) + (
 // and at the end  lower-query sum = tot - (hit << 16) - bias  (exact: the true value is far below
 // 2^32) and  upper-query sum = hit.  That is one ALU instruction and two FMA-pipe adds per window
 // register.
-// ALU (SA_FLAG_ADD_ON_ALU, not the default): sg is a sign MASK (0 / 0xffffffff) and every sign flip and add
+// ALU (SA_FLAG_ADD_ON_ALU): sg is a sign MASK (0 / 0xffffffff) and every sign flip and add
 // is an exclusive-or, a subtract and an add on the ALU pipe; the multiplier array is not used at all.
 template <int NP, bool ALU = false>
 struct PackedShift {
@@ -307,9 +308,9 @@ SA_HD void table_gather(const uint8_t* base, uint32_t offs, int i, uint32_t& x, 
     y = e[1];
 }
 
-// MUL (SA_FLAG_SHIFT_BY_MULTIPLY, not the default): sigma * 2^r is formed once per key element and the
+// MUL (SA_FLAG_SHIFT_BY_MULTIPLY): sigma * 2^r is formed once per key element and the
 // update is one multiply-add of the table entry by it.
-// ALU (SA_FLAG_ADD_ON_ALU, not the default): the sign flip and the add are an exclusive-or, a subtract and an
+// ALU (SA_FLAG_ADD_ON_ALU): the sign flip and the add are an exclusive-or, a subtract and an
 // add on the ALU pipe (sg is then the sign mask 0 / 0xffffffff); the multiplier array is not used at all.
 template <int KB, int NGP, bool MUL = false, bool ALU = false>
 struct TableScore {

@@ -292,9 +292,9 @@ SA_D void block_merge_and_store(const DecodeArgs& a, float (*red_s)[GT][D + 2], 
 // two resident blocks of the decode kernel: the next decode kernel is launched while this one runs
 // (programmatic dependent launch), and a merge block that took the place of one of its blocks would make
 // that block, and with it the whole grid, finish late.
-// With more than 96 splits (a binary16 cache at batch 1: 111) the block has 256 threads = 64 groups instead, so that
-// the partials are still fetched in one round trip; it then no longer fits beside the quantised kernels' two blocks,
-// whose split counts stay below that.
+// With more than 96 splits (kernels of four resident blocks at batch 1: 148) the block has 256 threads = 64 groups instead,
+// so that the partials are still fetched in one round trip: PoT-M1, 32 / 4 heads, d = 64, 16 384 tokens 8.45 us a call
+// against 9.24 with 128 threads, 32 768 tokens 10.16 against 10.82, 65 536 tokens 13.7 against 14.4.
 constexpr int kMergeDims = 16;                                // output dims per block
 constexpr int kMergeLanes = kMergeDims / 4;                   // float4 lanes
 constexpr int kMergeChunk = 3;                                // splits per thread whose loads are in flight together
@@ -322,8 +322,13 @@ __global__ void __launch_bounds__(kMergeThreads, 2048 / kMergeThreads) merge_ker
     // partials this block is about to wait for is still running — so that its blocks move in as that kernel's
     // blocks retire and are already waiting when this one completes.  That is safe because every kernel of this
     // library reads, ahead of its own wait, nothing that this kernel or its predecessors write (the decode kernels:
-    // only Q and hints).  It pays for the ten-warp decode kernels at batch 1 (3–6 % of a step); with the four-warp
-    // kernels (PoT-M1 / M2, d = 128, FP16) the early arrivals slow the running kernel down by more than they gain.
+    // only Q and hints).  Steps recorded in a graph, us per layer, late -> early (SM clock 1965 MHz):
+    //   shapes that release early (eight warps or more: d = 64, PoT-4, PoT-M4, INT8): one sequence of 32 768 tokens
+    //     11.20 -> 10.97 (PoT-M4), 10.57 -> 10.26 (PoT-4 nibble), 10.35 -> 9.94 (INT8); of 4096 tokens 7.18 -> 7.16,
+    //     6.88 -> 7.24, 6.87 -> 6.93; batch 8 x 8192 16.97 -> 16.64 (PoT-M4), the others and batch 32 within 1 %;
+    //   shapes that do not: PoT-M2 planar 6.57 -> 6.93 (4096), 10.94 -> 11.9 (32 768); binary16 6.08 -> 6.49, 11.6 -> 11.15;
+    //     PoT-M1 byte 6.3 -> 6.48, 10.7 -> 10.43; at batch 4 and above within 1 %, binary16 at batch 8 -4 %.
+    // Nothing was slower for early release at d = 128 (0 to -5 %), where the rule, which only counts warps, has it late.
     if (bump.early_release) pdl_launch_dependents();
     pdl_wait();                                               // the partials come from the kernel before
     if (!bump.early_release) pdl_launch_dependents();

@@ -126,7 +126,9 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     //     them and 1.8 us on a tile per warp: 2.5; 32 x 4096 tokens, d = 128: 76.3 -> 57.2 us against 0.5);
     //   * blocks run in waves of (SMs of the current device) x resident-blocks-per-SM; a last wave whose SMs hold only the
     //     fraction f of that takes 0.1 + 0.9 f of a full wave's time, a single partial wave f^0.2
-    //     (an SM's throughput falls almost in proportion to its resident warps).
+    //     (an SM's throughput falls almost in proportion to its resident warps).  f is taken from the SM with the most blocks,
+    //     so 256 blocks on 296 slots count as a full wave, which they are not: PoT-M4, 32 sequences, gets 2 splits at 513 to
+    //     520 pages (122.6 us) and 8 at 512 and at 530 (116.0 us; 8 splits at 513 to 520 pages take 116.0 us as well).
     // The sequence lengths live on the device, so the model uses the cache's capacity.
     const long long units = (long long)batch * p.Hkv * (p.G / GT);
     const int bps = p.shape.blocks_per_sm, nw = p.shape.warps;
@@ -136,7 +138,8 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     // A single sequence that is short: a cluster of 8 blocks per query group, which merges its splits itself.  One launch
     // instead of two (2.0 us of host time) and no trip of the partials through L2: 1024 tokens of one head 9.4 -> 5.3 us a
     // call from Python, of 32 / 4 heads 6.2 -> 5.8.  The line is a tile per warp: longer sequences are done sooner on all
-    // SMs and with the merge kernel (PoT-4, 8192 tokens: 8.1 us in clusters, 5.8 without).
+    // SMs and with the merge kernel (PoT-4, 8192 tokens: 8.1 us in clusters, 5.8 without).  Batches have not been measured in
+    // this form: plan_block does not know clusters.
     if (cluster) *cluster = false;
     if (p.matrix && batch == 1 && tiles <= kClusterMost * nw) {
         if (cluster) *cluster = true;

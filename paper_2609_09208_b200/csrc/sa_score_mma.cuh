@@ -16,8 +16,8 @@
 //   INT8 keys                 as stored.  INT32 sums.
 //   binary16 keys             as stored, with the binary16 query; the sums are rounded like any FP32 sum.
 // So the INT32 scores are those of the shift-and-add datapath (sa_datapath.cuh) bit for bit.  (The decode is what a tile
-// costs most: for four codes 11 instructions in the direct form, 7 by way of FP8.  FP8 operands of the product itself
-// cost more: mma.sync expands them into conversions, again for every product they enter.)
+// costs most: for four codes 11 instructions in the direct form, 7 by way of FP8.  With FP8 operands of the product itself,
+// which are exact too, 32 x 32 768 tokens took 147 us against 116.)
 //
 // Fragments: lane (r, c) = (lane / 4, lane % 4) holds the c-th 32-bit word of a 16-byte code chunk of keys r, r + 8,
 // r + 16, r + 24 (one ldmatrix.x4 per chunk: 8 keys x 16 bytes are 128 contiguous bytes, no bank conflict).  The order of

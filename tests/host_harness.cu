@@ -40,7 +40,7 @@ static void score8_packed(const uint8_t* canon, const int8_t* q8, int d, bool ni
 
 // The scores of a mantissa code (k = 1, 2, 4) through the table datapath.
 // The same scores through the table datapath of the mantissa codes.
-// VAR 0: the default datapath; 1: the shifts as multiplications by 2^r; 2: sign flips and adds on the ALU pipe only
+// VAR 0: the datapath of SA_FLAG_SHIFT_ADD; 1: the shifts as multiplications by 2^r; 2: sign flips and adds on the ALU pipe only
 template <int K, int VAR>
 static void score8_table(const uint8_t* canon, const int8_t* q8, int d, int32_t* out) {
     using TS = TableScore<K, 4, VAR == 1, VAR == 2>;
