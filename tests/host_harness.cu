@@ -2,6 +2,7 @@
 // (which are also compiled for the host) through a C interface, so that they can be checked
 // against the CPU oracle without a GPU.  Built by tests/test_host_arith.py; not part of the library.
 #include "../paper_2609_09208_b200/csrc/sa_datapath.cuh"
+#include "../paper_2609_09208_b200/csrc/sa_decode_common.cuh"
 
 using namespace sa;
 
@@ -126,6 +127,21 @@ int hh_once_per_device(const int* devs, const int* fails, int n, int* ok) {
     int calls = 0;
     for (int i = 0; i < n; ++i) ok[i] = once(devs[i], [&] { return ++calls, !fails[i]; });
     return calls;
+}
+// settle_whole for a plan that needs no merge kernel; returns whole | (arrivals set) << 1
+int hh_settle_whole(int n_splits, int Hkv, int G, int gt, int batch, int appends) {
+    Plan p{};
+    p.Hkv = Hkv;
+    p.G = G;
+    DecodeArgs a{};
+    a.n_splits = a.cluster = n_splits;
+    a.gt = gt;
+    a.batch = batch;
+    a.whole = 1;
+    alignas(16) static unsigned char workspace[16];
+    if (appends) a.Knew = reinterpret_cast<const uint16_t*>(workspace);
+    settle_whole(workspace, p, &a);
+    return a.whole | (a.arrivals ? 2 : 0) | (a.cluster == n_splits ? 4 : 0);
 }
 int hh_value_exponent(unsigned amax_bits) { return value_exponent(amax_bits); }
 void hh_score8(int k, const uint8_t* canon, const int8_t* q8, int d, int nibble_path, int32_t* out) {

@@ -23,8 +23,8 @@ def hh():
     os.makedirs(os.path.dirname(LIB), exist_ok=True)
     deps = [SRC] + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")]
     if not os.path.exists(LIB) or any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps):
-        subprocess.check_call(["/usr/local/cuda/bin/nvcc", "-std=c++17", "-O2", "-shared", "-Xcompiler", "-fPIC",
-                               "-Wno-deprecated-gpu-targets", "-o", LIB, SRC])
+        subprocess.check_call(["/usr/local/cuda/bin/nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-O2", "-shared",
+                               "-Xcompiler", "-fPIC", "-o", LIB, SRC])
     lib = C.CDLL(LIB)
     return lib
 
@@ -131,3 +131,12 @@ def test_kernel_attributes_are_set_once_per_device(hh, devs, fails, calls):
     ok = (C.c_int * n)()
     assert hh.hh_once_per_device((C.c_int * n)(*devs), (C.c_int * n)(*fails), C.c_int(n), ok) == calls
     assert list(ok) == [1 - f for f in fails]
+
+
+@pytest.mark.parametrize("shape,appends,want", [
+    ((8, 4, 8, 8, 1), 1, 7), ((8, 4, 8, 8, 1), 0, 5),                      # a cluster of eight; nothing to count without an append
+    ((1, 256, 8, 8, 65535), 1, 7), ((1, 256, 8, 4, 65535), 1, 4),          # 2^24 - 256 blocks are counted, twice as many are not
+    ((1, 256, 1, 1, 65536), 1, 4), ((1, 256, 8, 4, 65535), 0, 5)])
+def test_steps_of_one_launch_have_at_most_as_many_blocks_as_the_word_counts(hh, shape, appends, want):
+    """settle_whole(splits, KV heads, group, queries per block, batch): one launch (1), counting word (2), cluster kept (4)."""
+    assert hh.hh_settle_whole(*[C.c_int(x) for x in shape], C.c_int(appends)) == want
