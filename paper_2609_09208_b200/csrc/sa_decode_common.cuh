@@ -439,20 +439,25 @@ __global__ void __launch_bounds__(kMergeThreads, 2048 / kMergeThreads) merge_ker
 
 // The blocks of a call that appends tokens and has no merge kernel meet at the first word of the workspace, which such a
 // call needs for nothing else (it writes no partials).  The workspace arrives with any contents: the word counts only while
-// its upper 40 bits are this mark, and the first block that finds anything else there sets it to the mark and one arrival.
-// Every call leaves the mark and no arrivals.  Nothing that this library writes into a workspace looks like the mark: its
-// upper half is a NaN that no arithmetic produces (where a partial has l or an output), and larger than any integer of a
-// plan, a maximum or a rounded logit.  Other contents would have to hit 40 chosen bits.
+// its upper 40 bits are this mark.  A block adds one to the word whatever it holds; if it did not hold the mark, the block
+// arrives once more, as the one that replaces the word, stray additions included, by the mark and one arrival, or behind it.
+// Every call leaves the mark and no arrivals, so that the next one takes a single addition per block (with a look at the word
+// ahead of it a step of one sequence of 1000 tokens took 6.65 us instead of 6.29, of 400 x 500 tokens 63.0 instead of 61.1).
+// Nothing that this library writes into a workspace looks like the mark: its upper half is a NaN that no arithmetic produces
+// (where a partial has l or an output), and larger than any integer of a plan, a maximum or a rounded logit.  Other contents
+// would have to hit 40 chosen bits.
 constexpr int kArrivalBits = 24;
 constexpr unsigned long long kArrivalMark = 0x7fa5c3d296ull << kArrivalBits;
 // Whether this is the last of `blocks` (< 2^24) blocks to call it with `word`.  One thread per block.
 SA_D bool last_to_arrive(unsigned long long* word, unsigned blocks) {
-    unsigned long long seen;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(word) : "memory");
-    unsigned arrived = 0;
-    if ((seen >> kArrivalBits) == (kArrivalMark >> kArrivalBits) || atomicCAS(word, seen, kArrivalMark + 1) != seen)
-        arrived = (unsigned)atomicAdd(word, 1ull) & ((1u << kArrivalBits) - 1u);      // (if the exchange failed, another block has set the mark)
-    if (arrived + 1 != blocks) return false;
+    unsigned long long old = atomicAdd(word, 1ull);
+    while ((old >> kArrivalBits) != (kArrivalMark >> kArrivalBits)) {
+        // (an exchange fails only because another block has changed the word, which every block does at most three times)
+        const unsigned long long seen = atomicAdd(word, 0ull);
+        if ((seen >> kArrivalBits) == (kArrivalMark >> kArrivalBits)) old = atomicAdd(word, 1ull);
+        else if (atomicCAS(word, seen, kArrivalMark + 1) == seen) old = kArrivalMark;
+    }
+    if ((unsigned)(old - kArrivalMark) + 1 != blocks) return false;
     *word = kArrivalMark;
     return true;
 }

@@ -142,7 +142,7 @@ def one_launch_setup(lens, Hq, Hkv, d=64, k=4):
 
 
 @pytest.mark.parametrize("lens,Hq,Hkv", [([1000], 32, 4), ([17], 1, 1), ([33] * 130, 4, 4)])
-@pytest.mark.parametrize("contents", ["zeros", "ones", "random", "partials", "nearly the mark"])
+@pytest.mark.parametrize("contents", ["zeros", "ones", "random", "partials", "nearly the mark", "one below the mark"])
 def test_step_of_one_launch_takes_a_workspace_with_any_contents(lens, Hq, Hkv, contents):
     """A step without a merge kernel counts its blocks in the workspace: the lengths grow by one whatever was there, and
     nothing behind the counting word is written (a step of two launches would leave its partials there)."""
@@ -159,6 +159,8 @@ def test_step_of_one_launch_takes_a_workspace_with_any_contents(lens, Hq, Hkv, c
         ws.copy_(torch.randint(0, 256, ws.shape, generator=torch.Generator().manual_seed(5), dtype=torch.uint8))
         if contents == "nearly the mark":                    # its upper half, with other bits below
             ws[:8].view(torch.int64).copy_(torch.tensor([(0x7fa5c3d2 << 32) | (0x95 << 24) | 3]))
+        if contents == "one below the mark":                 # the first block's addition makes the mark
+            ws[:8].view(torch.int64).copy_(torch.tensor([(0x7fa5c3d296 << 24) - 1]))
     before = ws.clone()
     for i in range(3):
         cache.seq_lens.copy_(lens0)
