@@ -63,11 +63,11 @@ SA_D void bump_lengths(const DecodeArgs& a, int lane) {
     }
 }
 
-// This block's share of the outputs of a cluster (a.cluster blocks, each with {R, l} of the query heads at shared address
-// `heads` and their O[D] at `sums`) -> O.  All loads of an output are in flight together; the blocks are
+// This block's share of the outputs of a cluster (a.cluster blocks, each with the O[D] of its query heads at shared address
+// `sums` and their {R, l} HEADS bytes behind that) -> O.  All loads of an output are in flight together; the blocks are
 // added in order.
-template <int D, int NT>
-SA_D void merge_cluster(const DecodeArgs& a, uint32_t heads, uint32_t sums, float* O) {
+template <int D, int NT, int HEADS>
+SA_D void merge_cluster(const DecodeArgs& a, uint32_t sums, float* O) {
     constexpr int kMost = kClusterMost;
     const int C = a.cluster, items = a.gt * (D / 2), per = (items + C - 1) / C, rank = blockIdx.x % C;
     for (int i = rank * per + threadIdx.x; i < min(items, (rank + 1) * per); i += NT) {
@@ -78,9 +78,9 @@ SA_D void merge_cluster(const DecodeArgs& a, uint32_t heads, uint32_t sums, floa
         for (int k = 0; k < kMost; ++k) {
             h[k] = v[k] = make_float2(0.0f, 0.0f);
             if (k < C) {
-                const uint32_t head = heads + g * 8, dims = sums + (g * D + 2 * col) * 4;
-                h[k] = C > 1 ? lds_cluster_f2(cluster_map(head, k)) : lds_f2(head);
-                v[k] = C > 1 ? lds_cluster_f2(cluster_map(dims, k)) : lds_f2(dims);
+                const uint32_t row = C > 1 ? cluster_map(sums, k) : sums;
+                h[k] = C > 1 ? lds_cluster_f2(row + HEADS + g * 8) : lds_f2(row + HEADS + g * 8);
+                v[k] = C > 1 ? lds_cluster_f2(row + (g * D + 2 * col) * 4) : lds_f2(row + (g * D + 2 * col) * 4);
                 Rm = max(Rm, __float_as_int(h[k].x));
             }
         }
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     if constexpr (WHOLE) {
         if (a.cluster > 1) cluster_sync();
         else __syncthreads();
-        merge_cluster<D, 32 * NW>(a, smem_addr(smem + SM::kHeadOff), smem_addr(smem + SM::kSumOff), a.O + ((size_t)b * a.Hq + h0) * D);
+        merge_cluster<D, 32 * NW, SM::kHeadOff - SM::kSumOff>(a, smem_addr(smem + SM::kSumOff), a.O + ((size_t)b * a.Hq + h0) * D);
         if (a.cluster > 1) cluster_sync();                                         // no block may leave while others read its sums
     }
 }
