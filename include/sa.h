@@ -14,7 +14,8 @@
  *     synchronises.  Arguments are validated on the host before anything is launched; a call
  *     that returns an error has launched nothing.
  *   - Half-precision data is passed as IEEE binary16 bit patterns in `uint16_t`.
- *   - Inputs must be finite.
+ *   - Inputs must be finite.  In the decode calls a logit q.k / sqrt(d) is to stay below 1.8e8 (2^28 in the log2 domain):
+ *     a row with a larger one comes out as NaN.
  *   - Query head h reads KV head h / (n_q_heads / n_kv_heads).
  *
  * Number formats (section II-A, II-D, II-E)

@@ -25,7 +25,11 @@
 namespace sa {
 
 constexpr int kWeightShift = 14;          // weights are scaled by 2^14: the largest (2^1.98 above R) stays below 65504
-constexpr float kRefMax = 268435456.0f;   // |R| <= 2^28
+// |R| <= 2^28.  R is a float, so from 2^24 on it lies on a grid, of 16 at the limit.  It is rounded up (the reference must not
+// lie below z - g by more than the 1.98 that the weights have to spare), which leaves the largest weight at 2^-3 at least:
+// 21 bits in two binary16 terms.  A row with a larger logit comes out as NaN; a small integer beside R, right up to
+// 1.6e9, cost 0 - 2 % of every call in a loop of its own and 2 - 6 % in the loop of the others.
+constexpr float kRefMax = 268435456.0f;
 
 template <int FMT>
 constexpr int format_kb() { return FMT == FMT_PLANAR1 ? 1 : FMT == FMT_PLANAR2 ? 2 : FMT == FMT_INT8 ? 8 : 0; }
@@ -323,13 +327,13 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
             bool move = !seen;                                // warp-uniform; rare after the first tile
             for (int turn = 0; turn < 2; ++turn) {            // (a reference that has moved fits)
                 if (move) {
-                    float y0 = -INFINITY, y1 = -INFINITY;     // largest z - g of the tile
+                    float y0 = -INFINITY, y1 = -INFINITY;     // largest z - g of the tile, not rounded down
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
                         if (8 * j + r < n_valid) {
                             const float g = (float)((int)(meta[j] << 8) >> 24);
-                            y0 = fmaxf(y0, fmaf(z[j][0], zq[j][0], -g));
-                            y1 = fmaxf(y1, fmaf(z[j][1], zq[j][1], -g));
+                            y0 = fmaxf(y0, __fmaf_ru(z[j][0], zq[j][0], -g));
+                            y1 = fmaxf(y1, __fmaf_ru(z[j][1], zq[j][1], -g));
                         }
 #pragma unroll
                     for (int o = 4; o < 32; o <<= 1) {

@@ -223,3 +223,45 @@ def test_lost_copy_is_marked_where_no_merge_kernel_runs(lens, lost):
     assert np.max(np.abs(got[~hit] - ref[~hit])) <= 1e-3
     end = len(cache.workspace) - (16 * ((8 * case.batch + 15) // 16) if case.batch > 1 else 0)
     assert bool((cache.workspace[:end] == 255).all())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("k,nibble", CONTAINERS + [(16, False)])
+@pytest.mark.parametrize("size,sign", [(2000, 1), (3000, 1), (4000, 1), (6000, -1)])
+def test_logits_beyond_the_integers_of_a_float(d, k, nibble, size, sign):
+    """Keys and queries whose logits reach 2^25.4 .. 2^27.9 in the log2 domain, where a float near the reference is off by
+    more than the weights have to spare, growing along the sequence so that the reference moves often, or all of them far below zero:
+    every row is the value row of its best key (the next best is 1024 or more below), with scales 2^-8 .. 2^8."""
+    import torch
+    sa_build.build()
+    dev = torch.device("cuda:0")
+    up = lambda x: torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).to(dev)
+    rng = np.random.default_rng(400 + d + k + size)
+    lens = [900] if size == 3000 else [900, 65]  # one sequence: merged in a cluster
+    case = synth.make_case("large", lens, 8, 1, d, 0 if k == 16 else k, nibble=nibble, seed=5)
+    pattern = rng.choice([-1.0, 1.0], size=d)
+    case.Q[:] = (size * np.linspace(0.5, 1.0, 8)[None, :, None] * pattern).astype(np.float16)
+    for b in range(len(lens)):
+        rows = slice(int(case.cu_lens[b]), int(case.cu_lens[b + 1]))
+        ramp = np.linspace(0.3, 1.0, int(case.lens[b])) if sign > 0 else np.linspace(1.0, 0.3, int(case.lens[b]))
+        case.K[rows] = (sign * size * ramp[:, None, None] * pattern).astype(np.float16)
+        case.K[rows.stop - 2] = case.K[rows.stop - 1] / 2     # (the ends of the ramp are apart in binary16 too)
+    case.V[:] = (case.V * np.exp2(rng.uniform(-8, 8, (len(case.V), 1, 1)))).astype(np.float16)
+    cfg = sa.make_config(d, 8, 1, k, nibble=nibble)
+    cache = sa.PagedCache(cfg, case.lens, dev)
+    cache.fill(up(case.K), up(case.V), case.cu_lens)
+    O = torch.zeros((len(lens), 8, d), dtype=torch.float32, device=dev)
+    (sa.decode_attention_fp16 if k == 16 else sa.decode_attention)(cfg, cache.handle, up(case.Q), O, cache.workspace)
+    torch.cuda.synchronize()
+    O = O.cpu().numpy()
+    assert np.isfinite(O).all()
+    for b in range(len(lens)):
+        rows = slice(int(case.cu_lens[b]), int(case.cu_lens[b + 1]))
+        score = case.K[rows, 0].astype(np.float64) @ pattern
+        z = np.sort(score)[::-1] * size * 0.5 / np.sqrt(d) * 1.4427
+        assert z[0] - z[1] >= 1024
+        best = case.V[rows, 0][np.argmax(score)]
+        vhat, g = ora.quantise_value(best[None])
+        want = best.astype(np.float64) if k == 16 else vhat[0] * 2.0 ** -float(g[0])
+        err = np.linalg.norm(O[b] - want, axis=1) / np.linalg.norm(want)
+        assert err.max() <= 1e-5, (b, err)
