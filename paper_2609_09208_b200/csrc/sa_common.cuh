@@ -224,10 +224,21 @@ SA_D float ex2_approx(float x) {
     return y;
 }
 
-// Packed FP32 pair multiply-add of sm_100: d = a * b + c on two lanes held in one 64-bit register.
-SA_D unsigned long long ffma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long d;
+// Packed FP32 pairs of sm_100, two lanes held in one 64-bit register: a * b + c, a * b, a + b.
+using f32x2 = unsigned long long;
+SA_D f32x2 ffma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+SA_D f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+SA_D f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 SA_D unsigned long long pack_f32x2(float lo, float hi) {

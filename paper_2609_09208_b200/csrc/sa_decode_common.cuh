@@ -30,7 +30,7 @@ struct DecodeArgs {
     float zscale;
     int gt, k;                // query heads per block; mantissa bits (the matrix kernels take both at run time)
     float score_unit;         // integer score = raw product sum of the matrix kernels * score_unit (test hook)
-    uint32_t one;             // the value 1, opaque to the compiler (adds issued as multiply-add)
+    uint32_t one;             // the value 1, opaque to the compiler (adds and shifts issued as multiply-adds)
     // Shift-based A.V option (eq. (6), (7)); all null / 0 on the default path.
     int32_t* zr;              // [batch][Hq][dbg_stride] rounded logits, written by the score pass
     int32_t* stat_m;          // [n_splits][batch][Hq] ceil of the largest logit of the split

@@ -155,9 +155,9 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         const int bq = b < 0 ? 0 : b;                              // (a block without work so far prepares sequence 0)
         const int len_g = (ranked ? bp.len : __ldcg(a.seq_lens + bq)) + (a.Knew ? 1 : 0);
         // ---- queries: reads only Q, which no kernel of a decode step writes, so it runs before the wait ----
-        const float qs = q.load(r < GT ? a.Q + ((size_t)bq * a.Hq + h0 + r) * D : nullptr, lane, a.hadamard != 0) * a.zscale;
-        qs0 = __shfl_sync(0xffffffffu, qs, 8 * c);
-        qs1 = __shfl_sync(0xffffffffu, qs, 8 * c + 4);
+        const float qd = q.load(r < GT ? a.Q + ((size_t)bq * a.Hq + h0 + r) * D : nullptr, lane, a.hadamard != 0) * a.zscale;
+        qs0 = __shfl_sync(0xffffffffu, qd, 8 * c);
+        qs1 = __shfl_sync(0xffffffffu, qd, 8 * c + 4);
         // A guess at this warp's first tile, only to ask L2 for it while the preceding kernel drains (loads that bypass
         // L1, so nothing stale can be read back later).
         n_tiles_g = (min(max(len_g, 0), a.max_pages * kPageTokens) + 31) >> 5;
@@ -258,7 +258,8 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
 
     float R0 = 0.0f, R1 = 0.0f;                    // references of queries 2 c, 2 c + 1 (integers)
     bool seen = false;                             // no key yet: R is not set
-    float l0 = 0.0f, l1 = 0.0f;                    // this lane's share of the normalisers
+    f32x2 l = pack_f32x2(0.0f, 0.0f);              // this lane's share of the normalisers
+    const f32x2 qs = pack_f32x2(qs0, qs1);
     float acc[MT][4];                              // O^T tiles: dims 16 mt + 2 r (c0, c1), + 1 (c2, c3) of queries 2 c, 2 c + 1
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt)
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
 
             // ---- scores ----
             float z[4][2], zh[SC::NACC == 2 ? 4 : 1][2];
-            q.tile(st, st + Stage::kPlaneOff, lane, z, zh);
+            q.tile(st, st + Stage::kPlaneOff, lane, a.one, z, zh);
             if (a.dbg_scores) {                               // parity tests only
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
@@ -300,22 +301,25 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
                         }
             }
             // ---- logits and weights ----
-            float zq[4][2], vs[4];                            // logit per score unit; 2^(14 - g_j)
+            // The lane's two queries as packed FP32: the same arithmetic in half the instructions, and in few enough registers
+            // (120 at d = 64) that a block of the merge kernel fits beside two of these: it is then there before the last of
+            // them ends.  A step of one sequence of 32 768 tokens took 10.85 us, 9.64 since.
+            f32x2 zq[4];                                      // logit per score unit
+            float vs[4];                                      // +- 2^(14 - g_j)
             uint32_t meta[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 if constexpr (kFp16) {                        // no scales
                     meta[j] = 0u;
                     vs[j] = (float)(1 << kWeightShift);
-                    zq[j][0] = qs0;
-                    zq[j][1] = qs1;
+                    zq[j] = qs;
                 } else {
                     meta[j] = lds_u32(st + Stage::kMetaOff + (8 * j + r) * 4);
                     const float sj = half_bits_to_float(meta[j] & 0xffffu);
-                    // byte 2 is g_j, in [-10, 30] for written tokens; byte 3 is zero: (g_j << 24) >> 1 = g_j << 23
-                    vs[j] = __int_as_float(((127 + kWeightShift) << 23) - ((int)__byte_perm(meta[j], 0u, 0x2444u) >> 1));
-                    zq[j][0] = qs0 * sj;
-                    zq[j][1] = qs1 * sj;
+                    // byte 2 is g_j, in [-10, 30] for written tokens: its place in the exponent field is 7 bits further up, by
+                    // a multiplication, for the pipe of the additions.  A negative g_j, 256 too large, toggles the sign bit.
+                    vs[j] = __uint_as_float(((127u + kWeightShift) << 23) - (meta[j] & 0x00ff0000u) * 128u);
+                    zq[j] = mul2(qs, pack_f32x2(sj, sj));
                 }
                 if constexpr (SC::NACC == 2) {                // rounded once, like the conversion of one integer sum
                     z[j][0] += zh[j][0];
@@ -332,8 +336,10 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
                     for (int j = 0; j < 4; ++j)
                         if (8 * j + r < n_valid) {
                             const float g = (float)((int)(meta[j] << 8) >> 24);
-                            y0 = fmaxf(y0, __fmaf_ru(z[j][0], zq[j][0], -g));
-                            y1 = fmaxf(y1, __fmaf_ru(z[j][1], zq[j][1], -g));
+                            float zq0, zq1;
+                            unpack_f32x2(zq[j], &zq0, &zq1);
+                            y0 = fmaxf(y0, __fmaf_ru(z[j][0], zq0, -g));
+                            y1 = fmaxf(y1, __fmaf_ru(z[j][1], zq1, -g));
                         }
 #pragma unroll
                     for (int o = 4; o < 32; o <<= 1) {
@@ -346,8 +352,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
                         y0 = fmaxf(R0, y0);
                         y1 = fmaxf(R1, y1);
                         const float f0 = pow2i_neg(__float2int_rn(R0 - y0)), f1 = pow2i_neg(__float2int_rn(R1 - y1));
-                        l0 *= f0;
-                        l1 *= f1;
+                        l = mul2(l, pack_f32x2(f0, f1));
 #pragma unroll
                         for (int mt = 0; mt < MT; ++mt) {
                             acc[mt][0] *= f0;
@@ -360,13 +365,16 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
                     R1 = y1;
                     seen = true;
                 }
+                const f32x2 nR = pack_f32x2(-R0, -R1);
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        p[j][e] = ex2_approx(fmaf(z[j][e], zq[j][e], e ? -R1 : -R0));
-                        w[j][e] = p[j][e] * vs[j];
-                    }
+                for (int j = 0; j < 4; ++j) {
+                    float x0, x1;
+                    unpack_f32x2(ffma2(pack_f32x2(z[j][0], z[j][1]), zq[j], nR), &x0, &x1);
+                    p[j][0] = ex2_approx(x0);
+                    p[j][1] = ex2_approx(x1);
+                    w[j][0] = p[j][0] * fabsf(vs[j]);
+                    w[j][1] = p[j][1] * fabsf(vs[j]);
+                }
                 if (n_valid < 32) {                           // the sequence's last tile: slots past its end may hold anything
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
@@ -386,12 +394,12 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
                 bh[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&h[j]));
                 if constexpr (kFp16) {
                     // one term; the normaliser sums the same rounded weights, so the result is an exact weighted mean
-                    l0 += hf.x;
-                    l1 += hf.y;
+                    l = add2(l, pack_f32x2(hf.x, hf.y));
                 } else {
-                    l0 += p[j][0];
-                    l1 += p[j][1];
-                    const __half2 lo = __floats2half2_rn(w[j][0] - hf.x, w[j][1] - hf.y);
+                    l = add2(l, pack_f32x2(p[j][0], p[j][1]));
+                    float x0, x1;                             // what the first term leaves
+                    unpack_f32x2(ffma2(pack_f32x2(hf.x, hf.y), pack_f32x2(-1.0f, -1.0f), pack_f32x2(w[j][0], w[j][1])), &x0, &x1);
+                    const __half2 lo = __floats2half2_rn(x0, x1);
                     bl[j] = movmatrix_trans(*reinterpret_cast<const uint32_t*>(&lo));
                 }
             }
@@ -442,6 +450,8 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     // block's largest, and writes it out; the rows are added in a fixed order.
     float* ref_s = reinterpret_cast<float*>(smem + SM::kRefOff);                   // [NW][8]
     float (*red_s)[8][D + 2] = reinterpret_cast<float (*)[8][D + 2]>(smem);        // {unused, l, O[D]}
+    float l0, l1;
+    unpack_f32x2(l, &l0, &l1);
 #pragma unroll
     for (int o = 4; o < 32; o <<= 1) {
         l0 += __shfl_xor_sync(0xffffffffu, l0, o);

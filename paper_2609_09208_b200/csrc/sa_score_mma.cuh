@@ -2,27 +2,34 @@
 //
 // A tile's key codes are the A operand (rows = keys) and the block's up to 8 quantised queries the B operand of
 // warp-level products; each code is decoded once, for all queries, into the small number it stands for:
-//   byte / planar containers  (1 + j/2^k) * 2^(g - c) with its sign, as a binary16 value (g = 7 - e; 0 for the zero
-//                             code).  Up to three mantissa bits (c = 7): sign, exponent field and mantissa field change
+//   byte / planar containers  (1 + j/2^k) * 2^(g - c) with its sign (g = 7 - e; 0 for the zero code).  Up to three
+//                             mantissa bits (c = 7): as a binary16 value.  Sign, exponent field and mantissa field change
 //                             places within the byte, four codes at a time, which makes it an FP8 (e4m3) value, and one
-//                             conversion instruction turns two of those into binary16.  PoT-M4 (c = 15): the fields are
-//                             moved to their places in binary16 directly.  Query integers are binary16 values too, so
-//                             every product is exact in FP32, and so is the sum: it is a whole number of units
-//                             2^-(c - 1 + k) below 2^24 (64 * 127 * 31 * 2^6 = 16 128 000 < 2^24 for PoT-M4).
+//                             conversion instruction turns two of those into binary16.  PoT-M4 (c = 127): as a bfloat16
+//                             value, where the mantissa field has its place already.  Query integers (PoT-M4: times
+//                             2^112) are values of the same type, so every product is exact in FP32, and so is the sum: it
+//                             is a whole number of units 2^-(c - 1 + k) (PoT-M4: 2^-18) below 2^24
+//                             (64 * 127 * 31 * 2^6 = 16 128 000 < 2^24 for PoT-M4).
 //                             At head_dim 128 PoT-M4 could reach 2^25: its two halves are accumulated apart.
 //   nibble container          2^(g - 1) <= 64 as an INT8 value: one byte permute looks four of them up, the sign bit of
 //                             the nibble (the permute's replicate-sign mode over non-negative bytes) turning the
 //                             others into 0; a second lookup with the signs flipped is multiplied by -q.  INT32 sums.
 //   INT8 keys                 as stored.  INT32 sums.
 //   binary16 keys             as stored, with the binary16 query; the sums are rounded like any FP32 sum.
-// So the INT32 scores are those of the shift-and-add datapath (sa_datapath.cuh) bit for bit.  (The decode is what a tile
-// costs most: for four codes 11 instructions in the direct form, 7 by way of FP8.  With FP8 operands of the product itself,
-// which are exact too, 32 x 32 768 tokens took 147 us against 116.)
+// So the INT32 scores are those of the shift-and-add datapath (sa_datapath.cuh) bit for bit.  The decode is what a tile
+// costs most: 7 instructions for four codes by way of FP8, 8 for PoT-M4 (11 as binary16).  The pipe of logic, shifts and
+// permutes, which issues every other clock, was 63 % busy in a call of 32 x 32 768 PoT-M4 tokens, the pipe of multiply-adds
+// 22 %, so shifts to the left are multiplications by a constant that the compiler cannot see (`one`, the value 1, is a kernel
+// argument).  With packed FP32 in the softmax (sa_decode_mma.cuh) that call went from 128 to 123.3 us, 32 x 4096 tokens of
+// head_dim 128 from 59.7 to 56.6.  Shifts to the right as the upper half of a product were slower (126.6), FP8 operands of
+// the product itself, which are exact too, far slower (116 -> 147).
 //
 // Fragments: lane (r, c) = (lane / 4, lane % 4) holds the c-th 32-bit word of a 16-byte code chunk of keys r, r + 8,
 // r + 16, r + 24 (one ldmatrix.x4 per chunk: 8 keys x 16 bytes are 128 contiguous bytes, no bank conflict).  The order of
 // the elements along the contraction is free as long as the queries are packed in the same order.
 #pragma once
+#include <cuda_bf16.h>
+
 #include "sa_common.cuh"
 #include "sa_datapath.cuh"
 #include "sa_mma.cuh"
@@ -33,16 +40,16 @@ namespace sa {
 // FMT_FP16: the unquantised cache; FMT_BYTE3: the byte container of the codes with at most three mantissa bits (all but PoT-M4)
 enum ScoreFormat { FMT_BYTE = 0, FMT_NIBBLE = 1, FMT_PLANAR1 = 2, FMT_PLANAR2 = 3, FMT_INT8 = 4, FMT_BYTE3 = 5, FMT_FP16 = 6 };
 
-// Bytes 0 and 2 (ODD: 1 and 3) of a word of the byte container (sign << 7 | mantissa << 3 | g) as a pair of binary16 values:
-// sign 7 -> 15, mantissa 6..3 -> 9..6, g 2..0 -> 12..10 of each half.
-template <bool ODD>
-SA_HD uint32_t byte_codes_to_half2(uint32_t w) {
-    return ODD ? ((w & 0x80008000u) | ((w >> 5) & 0x03c003c0u) | ((w << 2) & 0x1c001c00u))
-               : (((w << 8) & 0x80008000u) | ((w << 3) & 0x03c003c0u) | ((w << 10) & 0x1c001c00u));
+// Codes I, I + 1 of a word of the byte container (sign << 7 | mantissa << 3 | g) as a pair of bfloat16 values.  With the byte in
+// both halves of its value, the mantissa field and the sign are where bfloat16 has them; g moves to bits 9..7.
+template <int I>
+SA_D uint32_t byte_codes_to_bf16(uint32_t w, uint32_t one) {
+    const uint32_t h = __byte_perm(w, 0u, I ? 0x3322u : 0x1100u);
+    return (h & 0x80788078u) | ((h * (one * 128u)) & 0x03800380u);
 }
 // Four codes of the byte container with at most three mantissa bits as FP8 values (sign << 7 | g << 3 | mantissa >> 1).
-SA_HD uint32_t byte_codes_to_fp8(uint32_t w) {
-    return (w & 0x80808080u) | ((w << 3) & 0x38383838u) | ((w >> 4) & 0x07070707u);
+SA_HD uint32_t byte_codes_to_fp8(uint32_t w, uint32_t one) {
+    return (w & 0x80808080u) | ((w * (one * 8u)) & 0x38383838u) | ((w >> 4) & 0x07070707u);
 }
 // FP8 values 0 and 1 (HIGH: 2 and 3) of a word as a pair of binary16 values.
 template <bool HIGH>
@@ -54,8 +61,8 @@ SA_D uint32_t fp8_to_half2(uint32_t f) {
 }
 // Even (ODD: odd) elements of a word of nibbles (sign << 3 | g) as FP8 powers of two with their signs.
 template <bool ODD>
-SA_HD uint32_t nibble_codes_to_fp8(uint32_t w) {
-    return ODD ? ((w & 0x80808080u) | ((w >> 1) & 0x38383838u)) : (((w << 4) & 0x80808080u) | ((w << 3) & 0x38383838u));
+SA_HD uint32_t nibble_codes_to_fp8(uint32_t w, uint32_t one) {
+    return ODD ? ((w & 0x80808080u) | ((w >> 1) & 0x38383838u)) : (((w * (one * 16u)) & 0x80808080u) | ((w * (one * 8u)) & 0x38383838u));
 }
 // The mantissa bits of the even elements in a byte of a bit plane (odd ones: of the byte >> 1), bit 2 i to bit AT of byte
 // i: the product places copies of the byte at offsets 6 apart, the mask keeps the wanted bit of each.
@@ -177,13 +184,18 @@ struct ScoreMma {
         const __half2 h = __floats2half2_rn((float)lo, (float)hi);
         return *reinterpret_cast<const uint32_t*>(&h);
     }
+    // |integers| <= 127 times 2^112: exact.  The keys' exponent field starts at 2^-127; the factor makes the unit 2^-18.
+    SA_D static uint32_t bf2(int lo, int hi) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn((float)lo * 0x1p112f, (float)hi * 0x1p112f);
+        return *reinterpret_cast<const uint32_t*>(&h);
+    }
     // The order of the elements along the contraction: that of tile() below.
     SA_D void pack(const int (&v)[CH][E]) {
 #pragma unroll
         for (int k = 0; k < CH; ++k) {
             if constexpr (FMT == FMT_BYTE) {
-                q[2 * k] = h2(v[k][0], v[k][2]);
-                q[2 * k + 1] = h2(v[k][1], v[k][3]);
+                q[2 * k] = bf2(v[k][0], v[k][1]);
+                q[2 * k + 1] = bf2(v[k][2], v[k][3]);
             } else if constexpr (FMT == FMT_BYTE3) {
                 q[2 * k] = h2(v[k][0], v[k][1]);
                 q[2 * k + 1] = h2(v[k][2], v[k][3]);
@@ -207,8 +219,8 @@ struct ScoreMma {
 
     // Scores of the 32 keys of a staged tile: sc[j][e], j = 2 t + h: key 16 t + 8 h + r, query 2 c + e, in units of
     // 2^-(6 + k) (PoT-M4: 2^-18; integer formats: 1).  st: shared address of the tile's codes; planes: its mantissa bit planes.
-    // hi[][]: the part of dimensions 64 .. 127 of NACC == 2 (not yet added).
-    SA_D void tile(uint32_t st, uint32_t planes, int lane, float (&sc)[4][2], float (&hi)[NACC == 2 ? 4 : 1][2]) const {
+    // hi[][]: the part of dimensions 64 .. 127 of NACC == 2 (not yet added).  one: DecodeArgs::one.
+    SA_D void tile(uint32_t st, uint32_t planes, int lane, uint32_t one, float (&sc)[4][2], float (&hi)[NACC == 2 ? 4 : 1][2]) const {
         const uint32_t row = st + lane * 16;
         if constexpr (kInt) {
             int d[2][4] = {};
@@ -258,10 +270,10 @@ struct ScoreMma {
                     for (int t = 0; t < 2; ++t) {
                         float(&acc)[4] = d[(NACC == 2 && k >= CH / 2 ? 2 : 0) + t];
                         if constexpr (FMT == FMT_BYTE) {
-                            mma_f16_16816(acc, byte_codes_to_half2<false>(w[2 * t]), byte_codes_to_half2<false>(w[2 * t + 1]),
-                                          byte_codes_to_half2<true>(w[2 * t]), byte_codes_to_half2<true>(w[2 * t + 1]), q[2 * k], q[2 * k + 1]);
+                            mma_bf16_16816(acc, byte_codes_to_bf16<0>(w[2 * t], one), byte_codes_to_bf16<0>(w[2 * t + 1], one),
+                                           byte_codes_to_bf16<2>(w[2 * t], one), byte_codes_to_bf16<2>(w[2 * t + 1], one), q[2 * k], q[2 * k + 1]);
                         } else {
-                            const uint32_t f0 = byte_codes_to_fp8(w[2 * t]), f1 = byte_codes_to_fp8(w[2 * t + 1]);
+                            const uint32_t f0 = byte_codes_to_fp8(w[2 * t], one), f1 = byte_codes_to_fp8(w[2 * t + 1], one);
                             mma_f16_16816(acc, fp8_to_half2<false>(f0), fp8_to_half2<false>(f1), fp8_to_half2<true>(f0), fp8_to_half2<true>(f1),
                                           q[2 * k], q[2 * k + 1]);
                         }
@@ -278,8 +290,8 @@ struct ScoreMma {
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const int j = 2 * t + h;
-                            f[h][0] = nibble_codes_to_fp8<false>(w[j]);
-                            f[h][1] = nibble_codes_to_fp8<true>(w[j]);
+                            f[h][0] = nibble_codes_to_fp8<false>(w[j], one);
+                            f[h][1] = nibble_codes_to_fp8<true>(w[j], one);
                             const uint32_t pa = planes + (8 * j + (lane >> 2)) * (D / 8) + 4 * k + (lane & 3);
                             uint32_t p = lds_u8(pa);
                             f[h][0] |= plane_bits<FMT == FMT_PLANAR1 ? 2 : 1>(p);
