@@ -39,6 +39,11 @@ constexpr KernelShape mma_shape(int d, int kb) {
 }
 // ... over the binary16 cache (tiles of 8 and 16 KB).
 constexpr KernelShape fp16_shape(int d) { return d == 128 ? KernelShape{6, 2, 1} : KernelShape{5, 2, 2}; }
+// The kernel of one block per SM (sa_decode_stream.cuh).
+constexpr KernelShape stream_shape(int d, bool fp16) {
+    return fp16 ? KernelShape{12, 1, d == 128 ? 1 : 2} : d == 128 ? KernelShape{12, 1, 2} : KernelShape{16, 1, 2};
+}
+constexpr int stream_unit_cost(int d) { return d == 128 ? 14 : 32; }     // what a block pays for going on to another unit, in tiles
 constexpr int kClusterMost = 8;           // blocks of a thread-block cluster
 // Shift-and-add kernels (sa_decode_kernel.cuh): one stage buffer per warp where a second one would cost resident warps
 // (d = 128, where a tile is 8 KB, and PoT-M4 with its 32 KB table of query multiples).
@@ -87,8 +92,9 @@ sa_status make_plan(const sa_config* cfg, Plan* out);
 // a B200, where no device answers, so that the size queries also work on a machine without a GPU).
 int sm_count();
 // Number of splits of the key axis for a cache of this shape, and queries handled per block.  cluster (matrix kernel): the
-// splits form one thread-block cluster.
-void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster = nullptr);
+// splits form one thread-block cluster.  stream: the blocks of the kernel of one block per SM where that one serves the call
+// (n_splits then only says how much of the workspace it needs), else 0; null: not asked for.
+void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster = nullptr, int* stream = nullptr);
 
 // ---------------------------------------------------------------------------------------------
 // Exact helpers (usable on host for unit tests of the arithmetic, and on device).

@@ -11,6 +11,11 @@ void launch_mma_lost_copy(const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_mma_dense(int d, int k, const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_mma_int8(int d, const DecodeArgs& a, dim3 grid, cudaStream_t s);
 void launch_mma_fp16(int d, const DecodeArgs& a, dim3 grid, cudaStream_t s);
+void launch_stream_byte(int d, int k, const DecodeArgs& a, cudaStream_t s);                   // sa_decode_stream_*.cu
+void launch_stream_lost_copy(const DecodeArgs& a, cudaStream_t s);
+void launch_stream_dense(int d, int k, const DecodeArgs& a, cudaStream_t s);
+void launch_stream_int8(int d, const DecodeArgs& a, cudaStream_t s);
+void launch_stream_fp16(int d, const DecodeArgs& a, cudaStream_t s);
 void launch_shift_pot4(bool nib, int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);   // sa_decode_pot*.cu
 void launch_shift_potm1(bool nib, int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
 void launch_shift_potm2(bool nib, int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3 grid, cudaStream_t s);
@@ -20,7 +25,12 @@ void launch_shift_potm4(int d, ShiftMode mode, const DecodeArgs& a, int GT, dim3
 void launch_decode_main(const Plan& p, const DecodeArgs& a, int GT, cudaStream_t s) {
     const dim3 grid((unsigned)a.n_splits, (unsigned)(p.Hkv * (p.G / GT)), (unsigned)a.batch);
     const ShiftMode mode = a.zr ? SHIFT_SCORE_PASS : p.mulshift ? SHIFT_MUL : p.addalu ? SHIFT_ALU : SHIFT_FMA;
-    if (p.matrix) {
+    if (a.stream) {
+        if (p.fp16) launch_stream_fp16(p.d, a, s);
+        else if (p.int8) launch_stream_int8(p.d, a, s);
+        else if (p.nibble) launch_stream_dense(p.d, p.k, a, s);
+        else launch_stream_byte(p.d, p.k, a, s);
+    } else if (p.matrix) {
         if (p.fp16) launch_mma_fp16(p.d, a, grid, s);
         else if (p.int8) launch_mma_int8(p.d, a, grid, s);
         else if (p.nibble) launch_mma_dense(p.d, p.k, a, grid, s);
@@ -98,7 +108,8 @@ extern "C" sa_status sa_debug_decode_lost_copy(const sa_config* cfg, const sa_ca
     a.lost_tile = tile;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     settle_whole(workspace, p, &a);                              // the form that sa_decode_attention takes
-    launch_mma_lost_copy(a, dim3((unsigned)a.n_splits, (unsigned)p.Hkv, (unsigned)a.batch), s);
+    if (a.stream) launch_stream_lost_copy(a, s);
+    else launch_mma_lost_copy(a, dim3((unsigned)a.n_splits, (unsigned)p.Hkv, (unsigned)a.batch), s);
     if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
     return a.whole ? SA_OK : launch_merge(p, a, s);
 }
@@ -202,8 +213,8 @@ extern "C" sa_status sa_decode_attention_static(const sa_config* cfg, const sa_c
     if (st != SA_OK) return st;
     if (p.fp16) return SA_ERR_UNSUPPORTED;
     if (!cache || cache->batch <= 0 || cache->max_pages_per_seq <= 0) return SA_ERR_INVALID_ARG;
-    int S, GT;
-    split_plan(p, cache->batch, cache->max_pages_per_seq, &S, &GT);
+    int S, GT, plan_stream;
+    split_plan(p, cache->batch, cache->max_pages_per_seq, &S, &GT, nullptr, &plan_stream);
     const size_t need = decode_workspace_bytes(p, cache->batch, S);
     if (need > (size_t)SA_STATIC_SCRATCH_BYTES) return SA_ERR_CAPACITY;   // problem too large for the fixed scratch
     void* scratch = nullptr;

@@ -54,6 +54,11 @@ struct DecodeArgs {
     // read the lengths (last_to_arrive).
     int cluster, whole;
     unsigned long long* arrivals;
+    // The kernel of one block per SM (sa_decode_stream.cuh): its number of blocks (0: the other kernel); the tiles that going on to
+    // another unit costs a block.  Partials lie in slots of gt heads; `counters` has a word for every (query group, sequence) unit, at which
+    // the blocks that work on it meet (last_to_arrive); `plan`, where a merge kernel follows, {first slot, slots} of every unit.
+    int stream, unit_cost;
+    unsigned long long* counters;
 };
 
 // Batches of 2 .. kRankedBatchMax sequences: which (sequence, split) a block of the grid works on is decided on the
@@ -308,6 +313,7 @@ struct BumpArgs {
     int max_pages, n_pages, Hq;
     int early_release;        // release the dependents of the merge kernel before its own wait (see merge_kernel)
     const int32_t* plan;      // {first slot, splits} per sequence (plan_block), or null: slots split * batch + sequence
+    int unit_heads, batch;    // query heads of a slot where the plan is one per (query group, sequence) unit, 0 elsewhere
 };
 
 template <int D, int kMergeThreads>
@@ -343,7 +349,12 @@ __global__ void __launch_bounds__(kMergeThreads, 2048 / kMergeThreads) merge_ker
     size_t stride = (size_t)n_rows * (D + 2);
     const int ln = threadIdx.x % kMergeLanes, grp = threadIdx.x / kMergeLanes;
     const float* base = partials + (size_t)row * (D + 2);
-    if (bump.plan) {                                          // the sequence's splits sit in consecutive slots
+    if (bump.unit_heads) {                                    // the kernel of one block per SM
+        const int b = row / bump.Hq, h = row % bump.Hq, u = h / bump.unit_heads * bump.batch + b;
+        n_splits = bump.plan[2 * u + 1];
+        stride = (size_t)bump.unit_heads * (D + 2);
+        base = partials + ((size_t)bump.plan[2 * u] * bump.unit_heads + h % bump.unit_heads) * (D + 2);
+    } else if (bump.plan) {                                   // the sequence's splits sit in consecutive slots
         const int b = row / bump.Hq;
         const int first = bump.plan[2 * b];
         n_splits = bump.plan[2 * b + 1];
@@ -461,9 +472,34 @@ SA_D bool last_to_arrive(unsigned long long* word, unsigned blocks) {
     *word = kArrivalMark;
     return true;
 }
+// The lengths grow by one when the kernel appends the step's tokens and no merge kernel follows: by the hand of the last
+// block to get here, every block having read what it needs of them.  One warp per block.
+SA_D void bump_lengths(const DecodeArgs& a, int lane) {
+    bool last = false;
+    if (lane == 0) last = last_to_arrive(a.arrivals, gridDim.x * gridDim.y * gridDim.z);
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    for (int b = lane; b < a.batch; b += 32) {
+        const int len = __ldcg(a.seq_lens + b), lp = len / kPageTokens;
+        const int page = (len >= 0 && lp < a.max_pages) ? a.page_table[(size_t)b * a.max_pages + lp] : -1;
+        if (page >= 0 && page < a.n_pages) const_cast<int32_t*>(a.seq_lens)[b] = len + 1;
+    }
+}
+
+// Workspace of the kernel of one block per SM: slots of partials (one per block and unit boundary), the units' counting words
+// and one for the call, the plan.
+inline size_t stream_slot_bytes(const Plan& p, int gt, int blocks, long long units) {
+    return ((size_t)blocks + (size_t)units) * gt * (p.d + 2) * sizeof(float);
+}
+inline size_t stream_workspace_bytes(const Plan& p, int gt, int blocks, long long units) {
+    return stream_slot_bytes(p, gt, blocks, units) + (size_t)(units + 1) * 8 + (size_t)units * 2 * sizeof(int32_t);
+}
 // Settles the form of the call: one launch, unless it appends tokens with more blocks than the word can count.
 inline void settle_whole(void* workspace, const Plan& p, DecodeArgs* a) {
     const long long blocks = (long long)a->n_splits * p.Hkv * (p.G / a->gt) * a->batch;
+    if (a->stream) {
+        if (a->whole && a->Knew) a->arrivals = a->counters + (size_t)p.Hkv * (p.G / a->gt) * a->batch;
+        return;
+    }
     if (a->whole && a->Knew && blocks >= (1LL << kArrivalBits)) a->whole = 0;
     if (a->whole && a->Knew) a->arrivals = static_cast<unsigned long long*>(workspace);
     if (!a->whole) a->cluster = 1;
@@ -488,9 +524,9 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     auto mis = [](const void* ptr, size_t al) { return (reinterpret_cast<uintptr_t>(ptr) & (al - 1)) != 0; };
     if (mis(c->pages, p.lay.align) || mis(c->page_table, 4) || mis(c->seq_lens, 4) || mis(Q, 16) || mis(O, 16))
         return SA_ERR_ALIGNMENT;
-    int S, GT;
+    int S, GT, stream = 0;
     bool cluster;
-    split_plan(p, c->batch, c->max_pages_per_seq, &S, &GT, &cluster);
+    split_plan(p, c->batch, c->max_pages_per_seq, &S, &GT, &cluster, with_plan ? &stream : nullptr);
     // the kernels place the splits with 32-bit arithmetic: tiles * (splits + 1) must stay below 2^31
     if ((long long)c->max_pages_per_seq * (kPageTokens / kTileTokens) * (S + 1) >= (1LL << 31)) return SA_ERR_CAPACITY;
     const size_t need = decode_workspace_bytes(p, c->batch, S, with_plan);
@@ -537,7 +573,16 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     a->cluster = cluster ? S : 1;
     a->whole = p.matrix && S == a->cluster ? 1 : 0;
     a->arrivals = nullptr;
-    if (with_plan && batch_is_ranked(c->batch)) {
+    a->stream = stream;
+    a->unit_cost = 0;
+    a->counters = nullptr;
+    if (stream) {
+        const long long units = (long long)c->batch * p.Hkv * (p.G / GT);
+        a->counters = reinterpret_cast<unsigned long long*>(static_cast<char*>(workspace) + stream_slot_bytes(p, GT, stream, units));
+        a->plan = reinterpret_cast<int32_t*>(a->counters + units + 1);
+        a->whole = 1;
+        a->unit_cost = stream_unit_cost(p.d);
+    } else if (with_plan && batch_is_ranked(c->batch)) {
         a->plan = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)S * c->batch * p.Hq * (p.d + 2) * sizeof(float));
         // blocks per grid row that a batch of unequal lengths is cut into: the grid, rounded down to whole waves of
         // resident blocks (equal blocks gain nothing from a last, partly filled wave)
@@ -567,9 +612,10 @@ inline void set_scales(const Plan& p, DecodeArgs* a) {
 inline sa_status launch_merge(const Plan& p, const DecodeArgs& a, cudaStream_t s) {
     const int rows = a.batch * a.Hq;
     const int early = (!p.fp16 && p.shape.warps >= 8) ? 1 : 0;
-    BumpArgs bump{a.Knew ? const_cast<int32_t*>(a.seq_lens) : nullptr, a.page_table, a.max_pages, a.n_pages, a.Hq, early, a.plan};
+    BumpArgs bump{a.Knew ? const_cast<int32_t*>(a.seq_lens) : nullptr, a.page_table, a.max_pages, a.n_pages, a.Hq, early, a.plan,
+                  a.stream ? a.gt : 0, a.batch};
     cudaError_t err;
-    const bool small = a.n_splits <= kMergeSmallSplits;
+    const bool small = a.stream || a.n_splits <= kMergeSmallSplits;
     const dim3 grid(rows * (p.d / kMergeDims));
     const float* part = a.partials;
     if (p.d == 64) err = small ? launch_pdl(merge_kernel<64, 128>, grid, dim3(128), 0, s, part, a.O, a.n_splits, rows, bump)

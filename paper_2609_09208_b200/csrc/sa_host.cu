@@ -113,7 +113,30 @@ int sm_count() {
     return cached[dev];
 }
 
-void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster) {
+// Whether a call of this many units (query group, sequence), of at most `tiles` tiles each, goes to the kernel of one block
+// per SM (sa_decode_stream.cuh).  cost, S: the other kernel's by its cost model, and its splits.  Measured with both, in all
+// containers, on 119 shapes of 2 to 128 sequences; where the rule takes this kernel, calls of up to 1.35 times less time, and
+// one of 1.4 % more (INT8 keys, 24 x 8192 tokens).  us a call, the other kernel -> this one:
+//   PoT-M4, d = 64, 32 / 4 heads: 32 x 32 768 tokens 112.5 -> 98.4, 32 x 8192 38.7 -> 35.5, 16 x 16 384 35.8 -> 33.6, below the
+//     line 8 x 16 384 20.7 -> 21.4, 4 x 16 384 14.8 -> 15.8;
+//   PoT-M4, d = 128, 32 / 8 heads: 20 x 4096 tokens 48.6 -> 36.7, 13 x 8192 53.0 -> 43.1, 10 x 4000 25.0 -> 23.1, below the line
+//     3 x 8192 16.5 -> 16.7.
+// Not taken: less than 9 rounds of tiles (4.5 at d = 128, where a round takes longer), over which a block's prologue and end
+// (10 us, of which the other kernel hides a part behind the second block of an SM) have to be earned; less than 16 units, whose
+// partials one block after the other has to wait for and merge (one sequence of 131 072 tokens: 18.4 -> 27.7); and many short
+// units, of which every one after a block's first costs it 5 us, where the other kernel's grid happens to fill the machine
+// (32 x 4096 tokens, d = 128: 256 blocks on 296 slots, 52.6 -> 56.3).
+static bool stream_pays(const Plan& p, int batch, long long units, long long tiles, double cost, int S, int sms) {
+    if (!p.matrix || batch < 2 || batch > kRankedBatchMax || units < 16) return false;
+    if (units * (tiles + stream_unit_cost(p.d)) >= (1LL << 30)) return false;       // (the kernel counts all tiles in 32 bits)
+    const double rounds = (double)units * (double)tiles / ((double)sms * stream_shape(p.d, p.fp16).warps), u = (double)units / sms;
+    if (rounds < (p.d == 128 && !p.fp16 ? 4.5 : 9.0)) return false;
+    // both in rounds of the other kernel, fitted to the same measurements
+    if (p.d == 64) return 0.97 * rounds + 3.0 * u + 5.6 <= cost + (S > 1 ? 2.2 : 0.0) + 1.5;
+    return 0.88 * rounds + 2.2 * u + 2.9 <= cost + (S > 1 ? 3.3 : 0.0) - 2.4;
+}
+
+void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster, int* stream) {
     int GT = 1;
     for (int c = 8; c >= 1; c >>= 1)
         if (p.G % c == 0) { GT = c; break; }
@@ -135,6 +158,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     const int n_sms = sm_count();
     const long long slots = (long long)n_sms * bps;
     const long long tiles = (long long)max_pages * (kPageTokens / 32);
+    if (stream) *stream = 0;
     // A single sequence that is short: a cluster of 8 blocks per query group, which merges its splits itself.  One launch
     // instead of two (2.0 us of host time) and no trip of the partials through L2: 1024 tokens of one head 9.4 -> 5.3 us a
     // call from Python, of 32 / 4 heads 6.2 -> 5.8.  The line is a tile per warp: longer sequences are done sooner on all
@@ -151,16 +175,26 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     // over: every thread keeps its last answers.
     struct Kept {
         long long units, tiles;
-        double c_fix;
+        double c_fix, cost;
         int nw, bps, sms, S;
     };
     const double c_fix = !p.matrix ? 0.5 : p.int8 ? 3.5 : 2.5;        // (INT8 keys need no decoding: a shorter round)
     static thread_local Kept kept[8] = {};
     static thread_local unsigned turn = 0;
+    auto settle = [&](int S, double cost) {
+        *n_splits = S;
+        *gt = GT;
+        if (!stream || !stream_pays(p, batch, units, tiles, cost, S, n_sms)) return;
+        // its workspace, in whole splits of the other kernel's; not where the fixed scratch would hold only the other's
+        const size_t split = (size_t)batch * p.Hq * (p.d + 2) * sizeof(float);
+        const int own = (int)((stream_workspace_bytes(p, GT, n_sms, units) + split - 1) / split);
+        if (decode_workspace_bytes(p, batch, own) > (size_t)SA_STATIC_SCRATCH_BYTES && own > S) return;
+        *stream = n_sms;
+        *n_splits = own;
+    };
     for (const Kept& k : kept)
         if (k.units == units && k.tiles == tiles && k.c_fix == c_fix && k.nw == nw && k.bps == bps && k.sms == n_sms) {
-            *n_splits = k.S;
-            *gt = GT;
+            settle(k.S, k.cost);
             return;
         }
     long long cap = tiles / 2;                      // at least two tiles per block (short caches: spread them over the SMs)
@@ -185,9 +219,8 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
         }
         if (blocks > 16 * slots) break;             // more waves than this never pay
     }
-    kept[turn++ % 8] = Kept{units, tiles, c_fix, nw, bps, n_sms, (int)best_S};
-    *n_splits = (int)best_S;
-    *gt = GT;
+    kept[turn++ % 8] = Kept{units, tiles, c_fix, best, nw, bps, n_sms, (int)best_S};
+    settle((int)best_S, best);
 }
 
 // Inputs of one decode step from device-addressable pinned host memory into the staging buffer.
@@ -252,8 +285,8 @@ sa_status sa_workspace_bytes(const sa_config* cfg, int batch, int max_pages_per_
     Plan p;
     const sa_status st = make_plan(cfg, &p);
     if (st != SA_OK) return st;
-    int S, GT;
-    split_plan(p, batch, max_pages_per_seq, &S, &GT);
+    int S, GT, stream;
+    split_plan(p, batch, max_pages_per_seq, &S, &GT, nullptr, &stream);
     *out = decode_workspace_bytes(p, batch, S);
     return SA_OK;
 }
