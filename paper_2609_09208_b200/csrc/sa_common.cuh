@@ -45,6 +45,8 @@ constexpr KernelShape stream_shape(int d, bool fp16) {
 }
 constexpr int stream_unit_cost(int d) { return d == 128 ? 14 : 32; }     // what a block pays for going on to another unit, in tiles
 constexpr int kClusterMost = 8;           // blocks of a thread-block cluster
+// ... of the matrix kernels where the splits of a sequence form a cluster.  (fp16: fp16_shape.)
+constexpr KernelShape cluster_shape(int d) { return d == 128 ? KernelShape{6, 2, 2} : KernelShape{8, 2, 2}; }
 // Shift-and-add kernels (sa_decode_kernel.cuh): one stage buffer per warp where a second one would cost resident warps
 // (d = 128, where a tile is 8 KB, and PoT-M4 with its 32 KB table of query multiples).
 constexpr KernelShape shift_shape(int d, int kb) {

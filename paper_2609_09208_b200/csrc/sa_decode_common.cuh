@@ -525,7 +525,7 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     if (mis(c->pages, p.lay.align) || mis(c->page_table, 4) || mis(c->seq_lens, 4) || mis(Q, 16) || mis(O, 16))
         return SA_ERR_ALIGNMENT;
     int S, GT, stream = 0;
-    bool cluster;
+    bool cluster = false;
     split_plan(p, c->batch, c->max_pages_per_seq, &S, &GT, &cluster, with_plan ? &stream : nullptr);
     // the kernels place the splits with 32-bit arithmetic: tiles * (splits + 1) must stay below 2^31
     if ((long long)c->max_pages_per_seq * (kPageTokens / kTileTokens) * (S + 1) >= (1LL << 31)) return SA_ERR_CAPACITY;

@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     // plan_block deals it from the cached lengths.  The plan made here, from lengths the preceding kernel may be about
     // to change, is a guess that lets the query preparation run ahead of the dependency wait; the plan made after the
     // wait decides, and the preparation is repeated in the rare case that it names another sequence.
-    const bool ranked = batch_is_ranked(a.batch);
+    const bool ranked = batch_is_ranked(a.batch) && !(WHOLE && a.cluster > 1);     // (clusters: every sequence has its own)
     int* plan_scratch = reinterpret_cast<int*>(smem);
     BlockPlan bp{(int)blockIdx.z, (int)blockIdx.x, a.n_splits, 0};
     if (a.wait_first) pdl_wait();
@@ -281,7 +281,9 @@ static void launch_mma_as(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
 }
 template <int D, int FMT, int CODE, int NW, int BPS, int NS>
 static void launch_mma(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
-    if (a.whole) launch_mma_as<D, FMT, CODE, NW, BPS, NS, false, true>(a, grid, s);
+    constexpr KernelShape sh = FMT == FMT_FP16 ? KernelShape{NW, BPS, NS} : cluster_shape(D);
+    if (a.cluster > 1) launch_mma_as<D, FMT, CODE, sh.warps, sh.blocks_per_sm, sh.stages, false, true>(a, grid, s);
+    else if (a.whole) launch_mma_as<D, FMT, CODE, NW, BPS, NS, false, true>(a, grid, s);
     else launch_mma_as<D, FMT, CODE, NW, BPS, NS, false, false>(a, grid, s);
 }
 

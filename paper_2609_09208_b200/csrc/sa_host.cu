@@ -159,15 +159,23 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     const long long slots = (long long)n_sms * bps;
     const long long tiles = (long long)max_pages * (kPageTokens / 32);
     if (stream) *stream = 0;
-    // A single sequence that is short: a cluster of 8 blocks per query group, which merges its splits itself.  One launch
-    // instead of two (2.0 us of host time) and no trip of the partials through L2: 1024 tokens of one head 9.4 -> 5.3 us a
-    // call from Python, of 32 / 4 heads 6.2 -> 5.8.  The line is a tile per warp: longer sequences are done sooner on all
-    // SMs and with the merge kernel (PoT-4, 8192 tokens: 8.1 us in clusters, 5.8 without).  Batches have not been measured in
-    // this form: plan_block does not know clusters.
     if (cluster) *cluster = false;
-    if (p.matrix && batch == 1 && tiles <= kClusterMost * nw) {
-        if (cluster) *cluster = true;
-        *n_splits = (int)(tiles / 2 < 1 ? 1 : tiles / 2 > kClusterMost ? kClusterMost : tiles / 2);
+    // Short sequences: a cluster of up to 8 blocks per unit, which merges its splits itself.  One launch instead of two (2.0 us
+    // of host time) and no trip of the partials through L2.  us a call in a graph, with the merge kernel -> in clusters:
+    //   PoT-M4, 32 / 4 heads, d = 64: 2 x 2000 tokens 7.3 -> 5.5, 4 x 2000 7.0 -> 6.1, 4 x 4000 9.1 -> 8.1, 8 x 4000 10.9 -> 9.3;
+    //   d = 128, 32 / 8 heads: 2 x 2000 9.7 -> 7.6, 4 x 4000 13.9 -> 12.1; binary16 4 x 3000 9.0 -> 7.0.
+    // The line is a tile per warp for one sequence: longer ones are done sooner on all SMs (PoT-4, 4096 tokens: 6.1 against 6.5;
+    // PoT-M4 6.8 against 6.5, but 6.9 against 7.2 launched one by one); two tiles for batches, three where there are enough
+    // units for all SMs or rounds are long (4 x 6000 tokens, PoT-M1 planar: 9.7 -> 10.4, 8 x 6000 13.0 -> 11.4).  Fewer than 8
+    // units of a batch would leave most SMs idle.  256 blocks, two to an SM, are what the machine takes at a time in clusters of
+    // 8 (9 x 1000 tokens, 288 blocks: 7.3 -> 11.1).
+    const KernelShape whole = p.fp16 ? p.shape : cluster_shape(p.d);
+    long long blocks = tiles / 2 < 1 ? 1 : tiles / 2 > kClusterMost ? kClusterMost : tiles / 2;
+    if (units * blocks > n_sms && tiles <= kClusterMost / 2 * whole.warps && blocks > kClusterMost / 2) blocks = kClusterMost / 2;
+    const long long rounds = batch == 1 ? 1 : units > 16 || p.d == 128 || p.fp16 ? 3 : 2;
+    if (p.matrix && tiles <= rounds * kClusterMost * whole.warps && (batch == 1 || (units >= 8 && units * blocks <= 256))) {
+        if (cluster) *cluster = blocks > 1;
+        *n_splits = (int)blocks;
         *gt = GT;
         return;
     }
