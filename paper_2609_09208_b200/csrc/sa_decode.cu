@@ -121,10 +121,11 @@ extern "C" sa_status sa_decode_step(const sa_config* cfg, const sa_cache* cache,
 }
 
 // sa_decode_step; with q_after_wait the decode kernel reads Q only after its wait on the preceding kernel (the
-// host-buffer entry, whose staging kernel writes Q and releases its dependents early).
+// host-buffer entry, whose staging kernel writes Q and releases its dependents early).  host_in: Q, K_new and V_new are device
+// addresses of host memory, in a call whose blocks can fetch them (DecodeArgs::host_in).
 sa_status sa::decode_step_impl(const sa_config* cfg, const sa_cache* cache, const uint16_t* Q, const uint16_t* K_new,
                                const uint16_t* V_new, float* O, void* workspace, size_t workspace_bytes,
-                               sa_stream stream, bool q_after_wait) {
+                               sa_stream stream, bool q_after_wait, bool host_in) {
     Plan p;
     sa_status st = make_plan(cfg, &p);
     if (st != SA_OK) return st;
@@ -151,6 +152,7 @@ sa_status sa::decode_step_impl(const sa_config* cfg, const sa_cache* cache, cons
     a.Knew = K_new;
     a.Vnew = V_new;
     a.wait_first = q_after_wait ? 1 : 0;
+    a.host_in = host_in ? 1 : 0;
     set_scales(p, &a);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     settle_whole(workspace, p, &a);

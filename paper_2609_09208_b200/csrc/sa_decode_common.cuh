@@ -54,6 +54,9 @@ struct DecodeArgs {
     // read the lengths (last_to_arrive).
     int cluster, whole;
     unsigned long long* arrivals;
+    // Q, Knew and Vnew lie in host memory (whole; blocks that work on the sequence of their own grid coordinates): one block of
+    // every unit fetches them, for all of its cluster (fetch_inputs).
+    int host_in;
     // The kernel of one block per SM (sa_decode_stream.cuh): its number of blocks (0: the other kernel); the tiles that going on to
     // another unit costs a block.  Partials lie in slots of gt heads; `counters` has a word for every (query group, sequence) unit, at which
     // the blocks that work on it meet (last_to_arrive); `plan`, where a merge kernel follows, {first slot, slots} of every unit.
@@ -507,7 +510,7 @@ inline void settle_whole(void* workspace, const Plan& p, DecodeArgs* a) {
 
 sa_status decode_step_impl(const sa_config* cfg, const sa_cache* cache, const uint16_t* Q, const uint16_t* K_new,
                            const uint16_t* V_new, float* O, void* workspace, size_t workspace_bytes, sa_stream stream,
-                           bool q_after_wait);
+                           bool q_after_wait, bool host_in = false);
 
 // Bytes of the split-K workspace: the partials and, for the batches whose blocks are planned on the device, the plan.
 inline size_t decode_workspace_bytes(const Plan& p, int batch, int S, bool with_plan = true) {
@@ -573,6 +576,7 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     a->cluster = cluster ? S : 1;
     a->whole = p.matrix && S == a->cluster ? 1 : 0;
     a->arrivals = nullptr;
+    a->host_in = 0;
     a->stream = stream;
     a->unit_cost = 0;
     a->counters = nullptr;

@@ -26,6 +26,8 @@ struct MmaSmem {
     static constexpr int kRefOff = kMbarOff + ((NW * NS * 8 + 127) & ~127);
     static constexpr int kHeadOff = kRefOff + NW * 8 * 4;
     static constexpr int kBytes = kHeadOff + 8 * 8;
+    static constexpr int kInOff = kBytes;                     // WHOLE: the unit's queries, new key and new value (host_in)
+    static constexpr int kWholeBytes = kInOff + 10 * D * 2;
     static constexpr int kSumOff = NW * 8 * (D + 2) * 4;      // the block's O, behind the merge rows (within the stage buffers)
     static_assert(kSumOff + 8 * D * 4 <= NW * NS * Stage::kBytes, "merge rows and sums must fit in the stage buffers");
     static_assert(kHeadOff >= NW * NS * Stage::kBytes, "no copy may land on the marks");
@@ -69,12 +71,34 @@ SA_D void merge_cluster(const DecodeArgs& a, uint32_t sums, float* O) {
     }
 }
 
+// The unit's inputs from host memory into every block of the cluster: queries (gt rows), new key, new value at `in`.  The first
+// block fetches them (blocks that ask for the same lines of host memory at once are served one after another), while the others
+// start; nothing here waits for the preceding kernels, none of which writes host inputs.
+template <int D>
+SA_D void fetch_inputs(const DecodeArgs& a, uint32_t in, int b, int kvh) {
+    const int C = a.cluster, rank = blockIdx.x % C, nq = a.gt * (D / 8), nk = D / 8, i = threadIdx.x;
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    const bool mine = rank == 0 && i < nq + 2 * nk;
+    if (mine) {
+        const size_t unit = (size_t)b * a.Hkv + kvh;
+        const uint16_t* src = i < nq ? a.Q + unit * a.gt * D + i * 8 : (i < nq + nk ? a.Knew + (i - nq) * 8 : a.Vnew + (i - nq - nk) * 8) + unit * D;
+        x = __ldcv(reinterpret_cast<const uint4*>(src));      // host memory: never from a cache line of an earlier step
+    }
+    if (C > 1) cluster_sync();                                // every block of the cluster is there
+    if (mine)
+        for (int r = 0; r < C; ++r) sts_cluster_u4(C > 1 ? cluster_map(in + i * 16, r) : in + i * 16, x);
+    if (C > 1) cluster_sync();
+    else __syncthreads();
+}
+
 // CODE: the cache-write mode of the fused append (see write_token).  LOST: the test hook that never issues one chosen
 // tile's copy and makes its first plan for another block's coordinates (sa_debug_decode_lost_copy).
+// At most 112 registers at d = 64: what two blocks of 256 threads then leave of an SM are two blocks of the merge kernel, which
+// stand by while these end (8 x 19 323 tokens, 8 / 2 heads, PoT-4: 14.9 us a call with room for one, 13.9 for two).
 // WHOLE: the splits of a sequence form one cluster (or there is one split), which merges them (merge_cluster); an
 // instantiation of its own, as the code at the end costs the others 0.1 - 0.3 us.
 template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST, bool WHOLE>
-__global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_constant__ DecodeArgs a) {
+__global__ void __maxnreg__(D == 128 ? 168 : 112) decode_mma_kernel(const __grid_constant__ DecodeArgs a) {
     using SM = MmaSmem<D, FMT, NW, NS>;
     using Stage = typename SM::Stage;
     constexpr uint32_t kPolls = LOST ? (1u << 10) : kWaitLimit;
@@ -107,6 +131,12 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
     __syncwarp();
     pdl_launch_dependents();    // the split-K merge may be scheduled as soon as blocks of this grid retire
 
+    const uint16_t* host_rows = nullptr;
+    if constexpr (WHOLE)
+        if (a.host_in) {
+            fetch_inputs<D>(a, smem_addr(smem + SM::kInOff), blockIdx.z, kvh);
+            host_rows = reinterpret_cast<const uint16_t*>(smem + SM::kInOff);
+        }
     TileMma<D, FMT, false> t;
     int b = bp.b, n_tiles_g, first_g, tile1_g, pidx_g, lp_g, pnew_g;
     bool again;
@@ -116,7 +146,8 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         const int bq = b < 0 ? 0 : b;                              // (a block without work so far prepares sequence 0)
         const int len_g = (ranked ? bp.len : __ldcg(a.seq_lens + bq)) + (a.Knew ? 1 : 0);
         // ---- queries: reads only Q, which no kernel of a decode step writes, so it runs before the wait ----
-        t.load_queries((lane >> 2) < GT ? a.Q + ((size_t)bq * a.Hq + h0 + (lane >> 2)) * D : nullptr, lane, a.hadamard != 0, a.zscale);
+        const uint16_t* q_rows = WHOLE && host_rows ? host_rows : a.Q + ((size_t)bq * a.Hq + h0) * D;
+        t.load_queries((lane >> 2) < GT ? q_rows + (lane >> 2) * D : nullptr, lane, a.hadamard != 0, a.zscale);
         // A guess at this warp's first tile, only to ask L2 for it while the preceding kernel drains (loads that bypass
         // L1, so nothing stale can be read back later).
         n_tiles_g = (min(max(len_g, 0), a.max_pages * kPageTokens) + 31) >> 5;
@@ -136,7 +167,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         const int32_t* table_g = a.page_table + (size_t)bq * a.max_pages;
         pidx_g = first_g < tile1_g ? table_g[first_g >> 1] : -1;
         pnew_g = lp_g >= 0 ? table_g[lp_g] : -1;
-        if (lp_g >= 0 && n_tiles_g - 1 >= first_g && n_tiles_g == tile1_g && (n_tiles_g - 1 - first_g) % NW == 0) {
+        if (lp_g >= 0 && !a.host_in && n_tiles_g - 1 >= first_g && n_tiles_g == tile1_g && (n_tiles_g - 1 - first_g) % NW == 0) {
             const size_t row = ((size_t)bq * a.Hkv + kvh) * D;
             asm volatile("prefetch.global.L1 [%0];" ::"l"(a.Knew + row + lane * (D / 32)));
             asm volatile("prefetch.global.L1 [%0];" ::"l"(a.Vnew + row + lane * (D / 32)));
@@ -208,7 +239,9 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
         ca.k = a.k;
         uint8_t* block = const_cast<uint8_t*>(a.pages) + ((size_t)pidx_new * a.Hkv + kvh) * a.page_bytes;
         const size_t row = ((size_t)b * a.Hkv + kvh) * D;
-        write_token<D, CODE>(block, ca, (len - 1) % kPageTokens, lane, a.Knew + row, a.Vnew + row);
+        const bool fetched = WHOLE && host_rows;
+        write_token<D, CODE>(block, ca, (len - 1) % kPageTokens, lane, fetched ? host_rows + GT * D : a.Knew + row,
+                             fetched ? host_rows + (GT + 1) * D : a.Vnew + row);
         fence_proxy_async_global();
         __syncwarp();
 #pragma unroll
@@ -273,7 +306,7 @@ __global__ void __launch_bounds__(32 * NW, BPS) decode_mma_kernel(const __grid_c
 
 template <int D, int FMT, int CODE, int NW, int BPS, int NS, bool LOST, bool WHOLE>
 static void launch_mma_as(const DecodeArgs& a, dim3 grid, cudaStream_t s) {
-    constexpr int bytes = MmaSmem<D, FMT, NW, NS>::kBytes;
+    constexpr int bytes = WHOLE ? MmaSmem<D, FMT, NW, NS>::kWholeBytes : MmaSmem<D, FMT, NW, NS>::kBytes;
     static OncePerDevice once;
     if (!allow_shared(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST, WHOLE>, bytes, once)) return;      // (the caller asks for the last error)
     (void)launch_pdl_cluster(decode_mma_kernel<D, FMT, CODE, NW, BPS, NS, LOST, WHOLE>, grid, dim3(32 * NW), (size_t)bytes, s,

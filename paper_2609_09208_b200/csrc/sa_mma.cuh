@@ -73,6 +73,9 @@ SA_D float2 lds_cluster_f2(uint32_t addr) {
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
     return v;
 }
+SA_D void sts_cluster_u4(uint32_t addr, uint4 v) {
+    asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
 // Transpose of an 8 x 8 matrix of 16-bit elements held by the warp: in lane (g, t) M[g][2t], M[g][2t + 1];
 // out M[2t][g], M[2t + 1][g].
 SA_D uint32_t movmatrix_trans(uint32_t x) {

@@ -88,9 +88,9 @@ struct TileMma {
                     }
         }
         // ---- logits and weights ----
-        // The lane's two queries as packed FP32: the same arithmetic in half the instructions, and in few enough registers
-        // (120 at d = 64) that a block of the merge kernel fits beside a full set of decode blocks: it is then there before the
-        // last of them ends.  A step of one sequence of 32 768 tokens took 10.85 us, 9.64 since.
+        // The lane's two queries as packed FP32: the same arithmetic in half the instructions, and in few enough registers that
+        // blocks of the merge kernel fit beside a full set of decode blocks: they are then there before the last of these ends.
+        // A step of one sequence of 32 768 tokens took 10.85 us, 9.64 since.
         f32x2 zq[4];                                          // logit per score unit
         float vs[4];                                          // +- 2^(14 - g_j)
         uint32_t meta[4];
