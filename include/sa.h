@@ -146,8 +146,12 @@ sa_status sa_get_layout(const sa_config* cfg, sa_layout* out);
  * proportion to their cached lengths, so that a batch of unequal lengths keeps the machine as full as one
  * of equal lengths).  Host only; the one CUDA call it may make reads the number of
  * multiprocessors of the CURRENT device (once per device), because the split count is planned for it: ask on
- * the device the decode calls will run on (without a device the figure of a B200 is used).  The scratch needs
- * no initialisation and may be shared by calls that do not overlap on the GPU. */
+ * the device the decode calls will run on (without a device the figure of a B200 is used).  Large batches and
+ * steps of one launch also keep words there at which blocks of a call count themselves.  The scratch needs
+ * no initialisation, may be shared by calls that do not overlap on the GPU, whatever their shapes, and may be
+ * overwritten, in part too, between calls: a counting word that is not as a call left it is not taken for a count.
+ * (Calls of different shapes that do overlap on one scratch corrupt each other's output and may leave a false count
+ * behind: fill the scratch with any one byte value then.) */
 sa_status sa_workspace_bytes(const sa_config* cfg, int batch, int max_pages_per_seq, size_t* out);
 
 /* Key encode (eq. (2), eq. (5); nearest-in-log2 rounding, section II-D).
@@ -298,7 +302,8 @@ sa_status sa_decode_attention_fp16_stages(const sa_config* cfg, const sa_cache* 
  *     made with that device current, then cached).  Make that first call outside any stream
  *     capture; later calls on the same device do no such query.
  *   - All calls on a device share the one array, and it keeps whatever the previous call left.
- *     Nothing in it has to be cleared — each call overwrites every entry it later reads — but two
+ *     Nothing in it has to be cleared — each call writes every partial it later reads, and the words at
+ *     which its blocks count themselves are at rest after each — but two
  *     calls that overlap on the GPU (different streams, or graphs replayed concurrently) race on
  *     it and corrupt each other's output.  Serialise them, or give the overlapping ones their own
  *     workspace through sa_decode_attention.

@@ -222,8 +222,8 @@ extern "C" sa_status sa_decode_attention_static(const sa_config* cfg, const sa_c
     void* scratch = nullptr;
     st = static_scratch_address(&scratch);
     if (st != SA_OK) return st;
-    // Nothing in the scratch has to start at zero: the main kernel writes every partial that the
-    // merge kernel reads, so contents left by an earlier call are simply overwritten.
+    // Nothing in the scratch has to start at zero: the decode kernel writes every partial that is read later, and a
+    // counting word with other contents than a count is replaced (last_to_arrive).
     return sa_decode_attention_stages(cfg, cache, Q, O, scratch, (size_t)SA_STATIC_SCRATCH_BYTES, dbg_scores, 3,
                                       stream);
 }

@@ -451,35 +451,51 @@ __global__ void __launch_bounds__(kMergeThreads, 2048 / kMergeThreads) merge_ker
     }
 }
 
-// The blocks of a call that appends tokens and has no merge kernel meet at the first word of the workspace, which such a
-// call needs for nothing else (it writes no partials).  The workspace arrives with any contents: the word counts only while
-// its upper 40 bits are this mark.  A block adds one to the word whatever it holds; if it did not hold the mark, the block
-// arrives once more, as the one that replaces the word, stray additions included, by the mark and one arrival, or behind it.
-// Every call leaves the mark and no arrivals, so that the next one takes a single addition per block (with a look at the word
-// ahead of it a step of one sequence of 1000 tokens took 6.65 us instead of 6.29, of 400 x 500 tokens 63.0 instead of 61.1).
-// Nothing that this library writes into a workspace looks like the mark: its upper half is a NaN that no arithmetic produces
-// (where a partial has l or an output), and larger than any integer of a plan, a maximum or a rounded logit.  Other contents
-// would have to hit 40 chosen bits.
+// Blocks of a call that meet without a kernel boundary count themselves at a word of the workspace: those of a step without a
+// merge kernel, so that the last one moves the lengths (such a call of sa_decode_mma.cuh needs the workspace for nothing else),
+// and those that work on one unit of the kernel of one block per SM, so that the last one merges their partials.
+// The workspace arrives with any contents.  A word holds the count twice, each half of it above a number of its own
+// (arrivals_in), and counts only while the halves agree.  A block adds one to both whatever the word holds; if they did not
+// agree, the block arrives once more, as the one that replaces the word, stray additions included, by one arrival, or behind
+// it.  Every call leaves the word at rest, without arrivals, so that the next one takes a single addition per block (with a look
+// at the word ahead of it a step of one sequence of 1000 tokens took 6.65 us instead of 6.29, of 400 x 500 tokens 63.0 instead
+// of 61.1).
+// Other contents would have to agree in 32 bits and be within 2^24 of the numbers: a word at rest of which a part is
+// overwritten is not taken for a count, and nothing that this library writes into a workspace is (the upper half is a NaN that no
+// arithmetic produces, and larger than any integer of a plan, a maximum or a rounded logit).  What a call leaves of two that
+// overlapped by mistake, with the same number of blocks, is at rest again: arrivals are counted modulo the number of blocks, and
+// taken off by subtraction.
 constexpr int kArrivalBits = 24;
-constexpr unsigned long long kArrivalMark = 0x7fa5c3d296ull << kArrivalBits;
+constexpr unsigned long long kArrivalRest = 0x7fa5c3d296000000ull, kArrivalStep = (1ull << 32) + 1;
+// Arrivals counted in a word; -1: it is not a count.
+SA_HD int arrivals_in(unsigned long long word) {
+    const uint32_t n = (uint32_t)word - (uint32_t)kArrivalRest, again = (uint32_t)(word >> 32) - (uint32_t)(kArrivalRest >> 32);
+    return n == again && n < (1u << kArrivalBits) ? (int)n : -1;
+}
+struct GlobalWord {
+    unsigned long long* at;
+    SA_D unsigned long long add(unsigned long long x) const { return atomicAdd(at, x); }
+    SA_D unsigned long long swap(unsigned long long seen, unsigned long long x) const { return atomicCAS(at, seen, x); }
+};
 // Whether this is the last of `blocks` (< 2^24) blocks to call it with `word`.  One thread per block.
-SA_D bool last_to_arrive(unsigned long long* word, unsigned blocks) {
-    unsigned long long old = atomicAdd(word, 1ull);
-    while ((old >> kArrivalBits) != (kArrivalMark >> kArrivalBits)) {
+template <typename Word>
+SA_HD bool last_to_arrive(const Word& word, unsigned blocks) {
+    int n = arrivals_in(word.add(kArrivalStep));
+    while (n < 0) {
         // (an exchange fails only because another block has changed the word, which every block does at most three times)
-        const unsigned long long seen = atomicAdd(word, 0ull);
-        if ((seen >> kArrivalBits) == (kArrivalMark >> kArrivalBits)) old = atomicAdd(word, 1ull);
-        else if (atomicCAS(word, seen, kArrivalMark + 1) == seen) old = kArrivalMark;
+        const unsigned long long seen = word.add(0ull);
+        if (arrivals_in(seen) >= 0) n = arrivals_in(word.add(kArrivalStep));
+        else if (word.swap(seen, kArrivalRest + kArrivalStep) == seen) n = 0;
     }
-    if ((unsigned)(old - kArrivalMark) + 1 != blocks) return false;
-    *word = kArrivalMark;
+    if ((unsigned)n + 1 < blocks || ((unsigned)n + 1) % blocks != 0) return false;
+    word.add(0ull - blocks * kArrivalStep);
     return true;
 }
 // The lengths grow by one when the kernel appends the step's tokens and no merge kernel follows: by the hand of the last
 // block to get here, every block having read what it needs of them.  One warp per block.
 SA_D void bump_lengths(const DecodeArgs& a, int lane) {
     bool last = false;
-    if (lane == 0) last = last_to_arrive(a.arrivals, gridDim.x * gridDim.y * gridDim.z);
+    if (lane == 0) last = last_to_arrive(GlobalWord{a.arrivals}, gridDim.x * gridDim.y * gridDim.z);
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
     for (int b = lane; b < a.batch; b += 32) {
         const int len = __ldcg(a.seq_lens + b), lp = len / kPageTokens;

@@ -197,7 +197,7 @@ SA_D void finish_units(const FinishArgs& a, const UnitSums& j0, const float* row
     if ((threadIdx.x == 0 && meet0) || (threadIdx.x == 32 && meet1)) {
         const UnitSums& j = threadIdx.x ? j1 : j0;
         __threadfence();
-        last = last_to_arrive(a.counters + j.u, j.blocks) ? 1 : 0;
+        last = last_to_arrive(GlobalWord{a.counters + j.u}, j.blocks) ? 1 : 0;
         __threadfence();
     }
     const int merge0 = meet0 ? __syncthreads_or(threadIdx.x < 32 ? last : 0) : 0, merge1 = meet1 ? __syncthreads_or(threadIdx.x < 32 ? 0 : last) : 0;

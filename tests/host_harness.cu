@@ -143,6 +143,29 @@ int hh_settle_whole(int n_splits, int Hkv, int G, int gt, int batch, int appends
     settle_whole(workspace, p, &a);
     return a.whole | (a.arrivals ? 2 : 0) | (a.cluster == n_splits ? 4 : 0);
 }
+// last_to_arrive, `calls` times by one thread, on a word of any contents; late: what is taken off the count comes after the last
+// call, as where another call's blocks are in between.  Returns the word; last[i]: the answer to call i.
+struct HostWord {
+    mutable unsigned long long value;
+    mutable unsigned long long off;
+    bool late;
+    SA_HD unsigned long long add(unsigned long long x) const {
+        const unsigned long long old = value;
+        if (late && x >> 63) off += x;
+        else value += x;
+        return old;
+    }
+    SA_HD unsigned long long swap(unsigned long long seen, unsigned long long x) const {
+        const unsigned long long old = value;
+        if (old == seen) value = x;
+        return old;
+    }
+};
+uint64_t hh_arrive(uint64_t contents, int blocks, int calls, int late, uint8_t* last) {
+    const HostWord w{contents, 0, late != 0};
+    for (int i = 0; i < calls; ++i) last[i] = last_to_arrive(w, (unsigned)blocks) ? 1 : 0;
+    return w.value + w.off;
+}
 int hh_value_exponent(unsigned amax_bits) { return value_exponent(amax_bits); }
 void hh_score8(int k, const uint8_t* canon, const int8_t* q8, int d, int nibble_path, int32_t* out) {
     score8_any<0>(k, canon, q8, d, k == 0 ? nibble_path : 0, out);

@@ -175,3 +175,30 @@ def test_lengths_rewritten_by_the_kernel_in_front_and_a_copy_that_never_comes():
     assert bool(torch.isnan(O[3, 8:16]).all()) and bool(torch.isfinite(O[:, :8]).all())
     attend(cfg, c, Q, O)                                       # and the next call is an ordinary one
     assert torch.equal(O, outs[0])
+
+
+@pytest.mark.parametrize("byte", range(8))
+def test_words_at_rest_of_which_one_byte_was_overwritten(byte):
+    """The counting words that a call leaves are memory like any other: a byte written into each changes no later call."""
+    import torch
+    sa_build.build()
+    d, Hq, Hkv, code, dense, rot, lens, room = SHAPES[0]
+    case = synth.make_case("stream", lens, Hq, Hkv, d, code, seed=8500)
+    cfg = sa.make_config(d, Hq, Hkv, code)
+    c = wide_cache(cfg, lens, room, extra=1)
+    c.fill(up(case.K), up(case.V), case.cu_lens)
+    Q, K, V = up(case.Q), up(case.K[:len(lens)]), up(case.V[:len(lens)])
+    lens0, outs = c.seq_lens.clone(), []
+    for call in range(4):
+        if call:
+            words = c.workspace[:len(c.workspace) // 8 * 8].view(torch.int64)
+            rest = (words >> 24) == MARK
+            assert int(rest.sum()) > 1
+            words[rest] ^= 5 << (8 * byte)
+        c.seq_lens.copy_(lens0)
+        O = torch.full((len(lens), Hq, d), float("nan"), device="cuda")
+        sa.decode_step(cfg, c.handle, Q, K, V, O, c.workspace)
+        torch.cuda.synchronize()
+        outs.append(O)
+        assert torch.equal(c.seq_lens, lens0 + 1)
+        assert torch.equal(O, outs[0])

@@ -140,3 +140,29 @@ def test_kernel_attributes_are_set_once_per_device(hh, devs, fails, calls):
 def test_steps_of_one_launch_have_at_most_as_many_blocks_as_the_word_counts(hh, shape, appends, want):
     """settle_whole(splits, KV heads, group, queries per block, batch): one launch (1), counting word (2), cluster kept (4)."""
     assert hh.hh_settle_whole(*[C.c_int(x) for x in shape], C.c_int(appends)) == want
+
+
+REST = 0x7fa5c3d296 << 24                            # a counting word without arrivals
+
+
+def arrive(hh, contents, blocks, calls, late=False):
+    hh.hh_arrive.restype = C.c_uint64
+    last = np.zeros(calls, dtype=np.uint8)
+    word = hh.hh_arrive(C.c_uint64(contents), C.c_int(blocks), C.c_int(calls), C.c_int(late), last.ctypes.data_as(C.c_void_p))
+    return word, np.flatnonzero(last).tolist()
+
+
+@pytest.mark.parametrize("blocks", [1, 2, 5, 148])
+def test_counting_word_of_any_contents_names_the_last_block_and_ends_at_rest(hh, blocks):
+    """Every single byte of a word at rest changed, its halves overwritten, and words near it."""
+    words = [REST, 0, 2**64 - 1, 0xFFFFFFFF, REST - 1, REST - 2**32, REST - 1 - 2**32, REST + 1, REST + 2**32, (REST >> 32) << 32, REST & 0xFFFFFFFF]
+    words += [REST ^ (x << (8 * byte)) for byte in range(8) for x in (1, 2, 5, 0x80, 0xFF)]
+    words += [int(x) for x in np.random.default_rng(1).integers(0, 2**64, 200, dtype=np.uint64)]
+    for w in words:
+        assert arrive(hh, w, blocks, blocks) == (REST, [blocks - 1]), hex(w)
+        assert arrive(hh, w, blocks, 3 * blocks) == (REST, [blocks - 1, 2 * blocks - 1, 3 * blocks - 1]), hex(w)
+
+
+@pytest.mark.parametrize("blocks", [2, 5, 148])
+def test_counting_word_is_at_rest_again_after_calls_that_overlapped(hh, blocks):
+    assert arrive(hh, REST, blocks, 3 * blocks, late=True) == (REST, [blocks - 1, 2 * blocks - 1, 3 * blocks - 1])
