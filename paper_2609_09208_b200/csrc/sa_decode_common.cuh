@@ -487,16 +487,21 @@ SA_HD bool last_to_arrive(const Word& word, unsigned blocks) {
         if (arrivals_in(seen) >= 0) n = arrivals_in(word.add(kArrivalStep));
         else if (word.swap(seen, kArrivalRest + kArrivalStep) == seen) n = 0;
     }
-    if ((unsigned)n + 1 < blocks || ((unsigned)n + 1) % blocks != 0) return false;
+    return (unsigned)n + 1 == blocks || ((unsigned)n + 1 > blocks && ((unsigned)n + 1) % blocks == 0);
+}
+// For the last of them to call, then or later in its kernel.
+template <typename Word>
+SA_HD void leave_at_rest(const Word& word, unsigned blocks) {
     word.add(0ull - blocks * kArrivalStep);
-    return true;
 }
 // The lengths grow by one when the kernel appends the step's tokens and no merge kernel follows: by the hand of the last
 // block to get here, every block having read what it needs of them.  One warp per block.
 SA_D void bump_lengths(const DecodeArgs& a, int lane) {
     bool last = false;
-    if (lane == 0) last = last_to_arrive(GlobalWord{a.arrivals}, gridDim.x * gridDim.y * gridDim.z);
+    const unsigned blocks = gridDim.x * gridDim.y * gridDim.z;
+    if (lane == 0) last = last_to_arrive(GlobalWord{a.arrivals}, blocks);
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    if (lane == 0) leave_at_rest(GlobalWord{a.arrivals}, blocks);
     for (int b = lane; b < a.batch; b += 32) {
         const int len = __ldcg(a.seq_lens + b), lp = len / kPageTokens;
         const int page = (len >= 0 && lp < a.max_pages) ? a.page_table[(size_t)b * a.max_pages + lp] : -1;

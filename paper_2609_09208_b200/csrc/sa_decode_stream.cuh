@@ -199,6 +199,7 @@ SA_D void finish_units(const FinishArgs& a, const UnitSums& j0, const float* row
         __threadfence();
         last = last_to_arrive(GlobalWord{a.counters + j.u}, j.blocks) ? 1 : 0;
         __threadfence();
+        if (last) leave_at_rest(GlobalWord{a.counters + j.u}, j.blocks);      // (behind the fence, which would wait for it)
     }
     const int merge0 = meet0 ? __syncthreads_or(threadIdx.x < 32 ? last : 0) : 0, merge1 = meet1 ? __syncthreads_or(threadIdx.x < 32 ? 0 : last) : 0;
 #pragma unroll 1

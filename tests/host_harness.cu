@@ -163,7 +163,10 @@ struct HostWord {
 };
 uint64_t hh_arrive(uint64_t contents, int blocks, int calls, int late, uint8_t* last) {
     const HostWord w{contents, 0, late != 0};
-    for (int i = 0; i < calls; ++i) last[i] = last_to_arrive(w, (unsigned)blocks) ? 1 : 0;
+    for (int i = 0; i < calls; ++i) {
+        last[i] = last_to_arrive(w, (unsigned)blocks) ? 1 : 0;
+        if (last[i]) leave_at_rest(w, (unsigned)blocks);
+    }
     return w.value + w.off;
 }
 int hh_value_exponent(unsigned amax_bits) { return value_exponent(amax_bits); }
