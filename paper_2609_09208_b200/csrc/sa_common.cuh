@@ -95,8 +95,9 @@ sa_status make_plan(const sa_config* cfg, Plan* out);
 int sm_count();
 // Number of splits of the key axis for a cache of this shape, and queries handled per block.  cluster (matrix kernel): the
 // splits form one thread-block cluster.  stream: the blocks of the kernel of one block per SM where that one serves the call
-// (n_splits then only says how much of the workspace it needs), else 0; null: not asked for.
-void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster = nullptr, int* stream = nullptr);
+// (n_splits then only says how much of the workspace it needs), else 0; null: not asked for.  fine: that kernel's form (DecodeArgs).
+void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster = nullptr, int* stream = nullptr,
+                bool* fine = nullptr);
 
 // ---------------------------------------------------------------------------------------------
 // Exact helpers (usable on host for unit tests of the arithmetic, and on device).

@@ -60,7 +60,8 @@ struct DecodeArgs {
     // The kernel of one block per SM (sa_decode_stream.cuh): its number of blocks (0: the other kernel); the tiles that going on to
     // another unit costs a block.  Partials lie in slots of gt heads; `counters` has a word for every (query group, sequence) unit, at which
     // the blocks that work on it meet (last_to_arrive); `plan`, where a merge kernel follows, {first slot, slots} of every unit.
-    int stream, unit_cost;
+    // fine: the instantiation whose sums do not grow less exact with the length of a warp's stretch.
+    int stream, unit_cost, fine;
     unsigned long long* counters;
 };
 
@@ -549,8 +550,8 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     if (mis(c->pages, p.lay.align) || mis(c->page_table, 4) || mis(c->seq_lens, 4) || mis(Q, 16) || mis(O, 16))
         return SA_ERR_ALIGNMENT;
     int S, GT, stream = 0;
-    bool cluster = false;
-    split_plan(p, c->batch, c->max_pages_per_seq, &S, &GT, &cluster, with_plan ? &stream : nullptr);
+    bool cluster = false, fine = false;
+    split_plan(p, c->batch, c->max_pages_per_seq, &S, &GT, &cluster, with_plan ? &stream : nullptr, &fine);
     // the kernels place the splits with 32-bit arithmetic: tiles * (splits + 1) must stay below 2^31
     if ((long long)c->max_pages_per_seq * (kPageTokens / kTileTokens) * (S + 1) >= (1LL << 31)) return SA_ERR_CAPACITY;
     const size_t need = decode_workspace_bytes(p, c->batch, S, with_plan);
@@ -600,6 +601,7 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     a->host_in = 0;
     a->stream = stream;
     a->unit_cost = 0;
+    a->fine = fine ? 1 : 0;
     a->counters = nullptr;
     if (stream) {
         const long long units = (long long)c->batch * p.Hkv * (p.G / GT);

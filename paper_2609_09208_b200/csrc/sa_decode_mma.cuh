@@ -137,7 +137,7 @@ __global__ void __maxnreg__(D == 128 ? 168 : 112) decode_mma_kernel(const __grid
             fetch_inputs<D>(a, smem_addr(smem + SM::kInOff), blockIdx.z, kvh);
             host_rows = reinterpret_cast<const uint16_t*>(smem + SM::kInOff);
         }
-    TileMma<D, FMT, false> t;
+    TileMma<D, FMT, false, false> t;
     int b = bp.b, n_tiles_g, first_g, tile1_g, pidx_g, lp_g, pnew_g;
     bool again;
 #pragma unroll 1

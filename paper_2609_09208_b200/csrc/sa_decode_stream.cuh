@@ -36,7 +36,7 @@ struct StreamSmem {
     static constexpr int kFactorOff = kLenOff + kRankedBatchMax * 4;
     static constexpr int kHeadOff = kFactorOff + 2 * NW * 8 * 4;
     static constexpr int kRowOff = kHeadOff + 2 * NW * 8 * 8;
-    __host__ __device__ static constexpr int row_bytes(int heads) { return NW * heads * TileMma<D, FMT, true>::kRowStep * 4; }
+    __host__ __device__ static constexpr int row_bytes(int heads) { return NW * heads * TileMma<D, FMT, true, false>::kRowStep * 4; }
     __host__ __device__ static constexpr bool apart(int heads) { return kRowOff + row_bytes(heads) <= 227 * 1024; }
     static constexpr int bytes(int heads) { return kRowOff + (apart(heads) ? row_bytes(heads) : 0); }
     static_assert(row_bytes(8) <= NW * NS * Stage::kBytes, "the rows must fit in the stage buffers");
@@ -130,7 +130,7 @@ struct FinishArgs {
 // order of the blocks.
 template <int D, int FMT, int NW>
 SA_D void finish_units(const FinishArgs& a, const UnitSums& j0, const float* rows0, const UnitSums& j1, const float* rows1) {
-    constexpr int NT = 32 * NW, kStep = TileMma<D, FMT, true>::kRowStep;
+    constexpr int NT = 32 * NW, kStep = TileMma<D, FMT, true, false>::kRowStep;
     constexpr float kValueScale = 1.0f / (1 << kWeightShift), kSumScale = FMT == FMT_FP16 ? kValueScale : 1.0f;
     const int GT = a.GT;
     if (threadIdx.x < 2 * NW * 8) {                           // every warp's 2^(R - R of the block's largest), and l times that
@@ -246,8 +246,8 @@ SA_D void finish_units(const FinishArgs& a, const UnitSums& j0, const float* row
     }
 }
 
-// CODE, LOST: as in decode_mma_kernel.
-template <int D, int FMT, int CODE, int NW, int NS, bool LOST>
+// CODE, LOST: as in decode_mma_kernel.  FINE: as in TileMma.
+template <int D, int FMT, int CODE, int NW, int NS, bool FINE, bool LOST>
 __global__ void __maxnreg__(NW > 12 ? 128 : 168) decode_stream_kernel(const __grid_constant__ DecodeArgs a) {
     using SM = StreamSmem<D, FMT, NW, NS>;
     using Stage = typename SM::Stage;
@@ -281,7 +281,7 @@ __global__ void __maxnreg__(NW > 12 ? 128 : 168) decode_stream_kernel(const __gr
     __syncwarp();
     pdl_launch_dependents();
 
-    TileMma<D, FMT, true> t;
+    TileMma<D, FMT, true, FINE> t;
     auto load_queries = [&](int y, int b) {
         const int h0 = (y / chunks) * a.G + (y % chunks) * GT, r = lane >> 2;
         t.load_queries(r < GT ? a.Q + ((size_t)b * a.Hq + h0 + r) * D : nullptr, lane, a.hadamard != 0, a.zscale);
@@ -475,15 +475,20 @@ __global__ void __maxnreg__(NW > 12 ? 128 : 168) decode_stream_kernel(const __gr
     }
 }
 
-template <int D, int FMT, int CODE, bool LOST = false>
-static void launch_stream(const DecodeArgs& a, cudaStream_t s) {
+template <int D, int FMT, int CODE, bool FINE, bool LOST>
+static void launch_stream_as(const DecodeArgs& a, cudaStream_t s) {
     constexpr KernelShape sh = stream_shape(D, FMT == FMT_FP16);
     using SM = StreamSmem<D, FMT, sh.warps, sh.stages>;
     constexpr int most = SM::apart(8) ? SM::bytes(8) : SM::apart(4) ? SM::bytes(4) : SM::bytes(1);
     static OncePerDevice once;
-    auto kernel = decode_stream_kernel<D, FMT, CODE, sh.warps, sh.stages, LOST>;
+    auto kernel = decode_stream_kernel<D, FMT, CODE, sh.warps, sh.stages, FINE, LOST>;
     if (!allow_shared(kernel, most, once)) return;            // (the caller asks for the last error)
     (void)launch_pdl(kernel, dim3((unsigned)a.stream), dim3(32 * sh.warps), (size_t)SM::bytes(a.gt), s, a);
+}
+template <int D, int FMT, int CODE, bool LOST = false>
+static void launch_stream(const DecodeArgs& a, cudaStream_t s) {
+    if (FMT != FMT_FP16 && !LOST && a.fine) launch_stream_as<D, FMT, CODE, FMT != FMT_FP16 && !LOST, LOST>(a, s);
+    else launch_stream_as<D, FMT, CODE, false, LOST>(a, s);
 }
 
 }  // namespace sa

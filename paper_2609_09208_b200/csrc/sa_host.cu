@@ -136,7 +136,19 @@ static bool stream_pays(const Plan& p, int batch, long long units, long long til
     return 0.88 * rounds + 2.2 * u + 2.9 <= cost + (S > 1 ? 3.3 : 0.0) - 2.4;
 }
 
-void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster, int* stream) {
+// Whether the kernel of one block per SM adds every tile's sums on their own (FINE, sa_tile_mma.cuh): where a full cache has more
+// tiles for a warp in one unit than the other kernel, with S splits, would have, or more than 16.  So its outputs are no further off
+// than the other kernel's, and the error of the sums stays below that of 64 products.  Root mean square error against 64 bits
+// with values of mean 0 / 1, other kernel -> this one without -> with FINE (without where nothing else is said):
+//   PoT-M4, d = 64, 32 x 32 768 tokens 9.6e-7 / 1.2e-6 -> 2.5e-6 / 3.6e-6 -> 2.2e-7 / 1.1e-7; d = 128, 8 x 32 768
+//   9.1e-7 / 2.4e-6 -> 1.6e-6 / 4.2e-6 -> 3.2e-7 / 1.6e-7; PoT-4, 8 x 32 768 (14 tiles) 8.9e-7 / 1.8e-6 -> 7.3e-7 / 1.7e-6.
+static bool stream_is_fine(const Plan& p, long long units, long long tiles, int S, int sms) {
+    if (p.fp16) return false;
+    const double nw = stream_shape(p.d, false).warps, chain = (double)tiles / nw * (units < sms ? (double)units / sms : 1.0);
+    return chain > 16.0 || chain > 1.05 * (double)tiles / ((double)p.shape.warps * S);
+}
+
+void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster, int* stream, bool* fine) {
     int GT = 1;
     for (int c = 8; c >= 1; c >>= 1)
         if (p.G % c == 0) { GT = c; break; }
@@ -159,6 +171,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     const long long slots = (long long)n_sms * bps;
     const long long tiles = (long long)max_pages * (kPageTokens / 32);
     if (stream) *stream = 0;
+    if (fine) *fine = false;
     if (cluster) *cluster = false;
     // Short sequences: a cluster of up to 8 blocks per unit, which merges its splits itself.  One launch instead of two (2.0 us
     // of host time) and no trip of the partials through L2.  us a call in a graph, with the merge kernel -> in clusters:
@@ -199,6 +212,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
         if (decode_workspace_bytes(p, batch, own) > (size_t)SA_STATIC_SCRATCH_BYTES && own > S) return;
         *stream = n_sms;
         *n_splits = own;
+        if (fine) *fine = stream_is_fine(p, units, tiles, S, n_sms);
     };
     for (const Kept& k : kept)
         if (k.units == units && k.tiles == tiles && k.c_fix == c_fix && k.nw == nw && k.bps == bps && k.sms == n_sms) {

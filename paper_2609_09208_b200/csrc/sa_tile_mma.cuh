@@ -35,12 +35,18 @@ using MmaStage = TileStage<ScoreMma<D, FMT>::CH, FMT != FMT_FP16, FMT == FMT_FP1
 // LONG: for warps with many tiles.  Everything rare (a first tile, a reference that moves, slots past the sequence's end) is
 // then out of the way of the other tiles, behind one vote, which is worth 2.5 % of a call with 55 tiles a warp; of calls with two,
 // where every first tile takes the detour, it cost 2 to 5 %.
-template <int D, int FMT, bool LONG>
+// FINE: the products of a tile are summed from zero and then added to the sums of the tiles before, rounded to nearest.  The
+// matrix unit cuts its sums off, an error that grows with the number of products in one accumulator: 32 x 32 768 PoT-M4
+// tokens, 55 tiles a warp, outputs 2.0e-6 too small (3.4e-6 with values of mean 1), with FINE 7e-8.  The
+// additions cost 2 % at head_dim 64 (that call 98.5 -> 100.3 us, in a graph) and 1.5 - 4 % at 128 (8 x 32 768 tokens, PoT-M4 88.8 -> 89.9, PoT-M1
+// planar 86.7 -> 89.5), so warps with few tiles do without (see stream_is_fine).
+template <int D, int FMT, bool LONG, bool FINE>
 struct TileMma {
     using SC = ScoreMma<D, FMT>;
     using Stage = MmaStage<D, FMT>;
     static constexpr int MT = D / 16;              // 16-dim row tiles of O^T
     static constexpr bool kFp16 = FMT == FMT_FP16;
+    static_assert(!(FINE && kFp16), "binary16 values: the weights' rounding is an error 100 times as large");
     static constexpr int kNever = 0x7fffffff;
 
     SC q;
@@ -213,6 +219,8 @@ struct TileMma {
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
             uint32_t x[4];
+            float own[4];                                     // FINE: the sums of this tile
+            float(&sum)[4] = FINE ? own : acc[mt];
             if constexpr (kFp16) {                            // binary16 values: chunk 2 mt is rows r (dims 16 mt + r), chunk 2 mt + 1 rows r + 8
                 uint32_t y[4];
                 ldmatrix_x4_trans(x, st + Stage::kVOff + 2 * mt * 512 + lane * 16);
@@ -236,8 +244,13 @@ struct TileMma {
             for (int k = 0; k < 2; ++k) {
                 const uint32_t a0 = int8_to_half2<false>(x[2 * k]), a1 = int8_to_half2<true>(x[2 * k]);
                 const uint32_t a2 = int8_to_half2<false>(x[2 * k + 1]), a3 = int8_to_half2<true>(x[2 * k + 1]);
-                mma_f16_16816(acc[mt], a0, a1, a2, a3, bh[2 * k], bh[2 * k + 1]);
-                mma_f16_16816(acc[mt], a0, a1, a2, a3, bl[2 * k], bl[2 * k + 1]);
+                if (FINE && k == 0) mma_f16_16816_first(sum, a0, a1, a2, a3, bh[0], bh[1]);
+                else mma_f16_16816(sum, a0, a1, a2, a3, bh[2 * k], bh[2 * k + 1]);
+                mma_f16_16816(sum, a0, a1, a2, a3, bl[2 * k], bl[2 * k + 1]);
+            }
+            if constexpr (FINE) {
+                unpack_f32x2(add2(pack_f32x2(acc[mt][0], acc[mt][1]), pack_f32x2(own[0], own[1])), &acc[mt][0], &acc[mt][1]);
+                unpack_f32x2(add2(pack_f32x2(acc[mt][2], acc[mt][3]), pack_f32x2(own[2], own[3])), &acc[mt][2], &acc[mt][3]);
             }
         }
     }

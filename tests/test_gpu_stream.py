@@ -202,3 +202,40 @@ def test_words_at_rest_of_which_one_byte_was_overwritten(byte):
         outs.append(O)
         assert torch.equal(c.seq_lens, lens0 + 1)
         assert torch.equal(O, outs[0])
+
+
+@pytest.mark.parametrize("d,Hq,Hkv,code,batch", [(64, 32, 4, sa.SA_POTM4, 32), (64, 32, 4, sa.SA_INT8, 16), (128, 32, 8, sa.SA_POTM4, 8)])
+def test_sums_over_long_stretches_against_64_bits(d, Hq, Hkv, code, batch):
+    """Values of mean 1, whose sums grow with every tile: up to 55 tiles a warp.  The matrix unit cuts its sums off, by up to 2^-23;
+    four of them make a tile: 4.8e-7.  Weights of 21 bits (2.4e-7) and the tiles' sums, rounded to nearest
+    (sqrt(55) 2^-24, 4.4e-7), are added: 1.2e-6 of the largest output at most, 1e-6 in the mean square."""
+    import torch
+    sa_build.build()
+    n = 32768
+    gen = torch.Generator(device="cuda").manual_seed(8600 + d + code)
+    cfg = sa.make_config(d, Hq, Hkv, code)
+    c = sa.PagedCache(cfg, [n] * batch, "cuda", permutation=synth.page_permutation(batch * n // 64, 3))
+    K = torch.randn((batch * n, Hkv, d), generator=gen, device="cuda").half()
+    V = (torch.randn((batch * n, Hkv, d), generator=gen, device="cuda") + 1).half()
+    c.fill(K, V, np.arange(batch + 1) * n)
+    del K, V
+    Q = torch.randn((batch, Hq, d), generator=gen, device="cuda").half()
+    O = torch.full((batch, Hq, d), float("nan"), device="cuda")
+    c.workspace.fill_(255)
+    attend(cfg, c, Q, O)
+    assert marks(c.workspace) > 0
+    q_hat, delta = torch.zeros((batch, Hq, d), dtype=torch.int8, device="cuda"), torch.zeros((batch, Hq), device="cuda")
+    sa.quantise_query(cfg, Q, q_hat, delta)
+    q = (q_hat.double() * delta.double()[..., None])[0]
+    codes, v_hat = [torch.zeros((n, Hkv, d), dtype=t, device="cuda") for t in (torch.uint8, torch.int8)]
+    scales, g = [torch.zeros((n, Hkv), dtype=t, device="cuda") for t in (torch.float16, torch.int8)]
+    sa.debug_unpack(cfg, c.handle, 0, n, codes, scales, v_hat, g)
+    if code == sa.SA_INT8:
+        keys = codes.view(torch.int8).double() / 127
+    else:
+        keys = torch.where(codes >= 128, -1.0, 1.0).double() * (1 + (codes & 15).double() / 16) * torch.exp2(-((codes >> 4) & 7).double())
+        keys[((codes >> 4) & 7) == 7] = 0
+    keys, values, G = keys * scales.double()[..., None], v_hat.double() * torch.exp2(-g.double())[..., None], Hq // Hkv
+    want = torch.cat([torch.softmax(q[h * G:(h + 1) * G] @ keys[:, h].T / d ** 0.5, -1) @ values[:, h] for h in range(Hkv)])
+    off = O[0].double() - want
+    assert float(off.abs().max() / want.abs().max()) <= 1.2e-6 and float(off.norm() / want.norm()) <= 1e-6
