@@ -402,7 +402,7 @@ __global__ void __maxnreg__(NW > 12 ? 128 : 168) decode_stream_kernel(const __gr
                 __syncwarp();
 #pragma unroll
                 for (int i = 0; i < NS; ++i)
-                    if (i == i_new) n_keys[i] = issue(tile_new, pidx_new, stage0 + (done + i) % NS * Stage::kBytes, mbar0 + (done + i) % NS * 8);
+                    if (i == i_new && i < n_my) n_keys[i] = issue(tile_new, pidx_new, stage0 + (done + i) % NS * Stage::kBytes, mbar0 + (done + i) % NS * 8);
             }
             if (next) load_queries(s.y, b);
             t.start();
