@@ -380,6 +380,7 @@ __global__ void __maxnreg__(NW > 12 ? 128 : 168) decode_stream_kernel(const __gr
                 return mapped ? len - tile * 32 : 0;
             };
             int n_keys[NS];
+            if (next && lane == 0) fence_proxy_async();       // (the stages were read, as before every copy in the loop)
 #pragma unroll
             for (int i = 0; i < NS; ++i)
                 if (i < n_my && i != i_new) {
@@ -463,7 +464,7 @@ __global__ void __maxnreg__(NW > 12 ? 128 : 168) decode_stream_kernel(const __gr
                                      second_job, rows_alias);
             if (!more) break;
             held.any = false;
-            fence_proxy_async();                              // (the next copies land where the rows were)
+            fence_proxy_async();                              // (the next copies land where the rows of all warps were)
             __syncthreads();
         }
         s.start += s.free + s.tiles;
@@ -480,6 +481,7 @@ static void launch_stream_as(const DecodeArgs& a, cudaStream_t s) {
     constexpr KernelShape sh = stream_shape(D, FMT == FMT_FP16);
     using SM = StreamSmem<D, FMT, sh.warps, sh.stages>;
     constexpr int most = SM::apart(8) ? SM::bytes(8) : SM::apart(4) ? SM::bytes(4) : SM::bytes(1);
+    static_assert(most >= SM::bytes(1) && most >= SM::bytes(2) && most >= SM::bytes(4) && most >= SM::bytes(8), "for any number of heads");
     static OncePerDevice once;
     auto kernel = decode_stream_kernel<D, FMT, CODE, sh.warps, sh.stages, FINE, LOST>;
     if (!allow_shared(kernel, most, once)) return;            // (the caller asks for the last error)
