@@ -468,10 +468,10 @@ __global__ void __launch_bounds__(kMergeThreads, 2048 / kMergeThreads) merge_ker
 // taken off by subtraction.
 constexpr int kArrivalBits = 24;
 constexpr unsigned long long kArrivalRest = 0x7fa5c3d296000000ull, kArrivalStep = (1ull << 32) + 1;
-// Arrivals counted in a word; -1: it is not a count.
-SA_HD int arrivals_in(unsigned long long word) {
+// Arrivals counted in a word; 2^24 or more: it is not a count.
+SA_HD uint32_t arrivals_in(unsigned long long word) {
     const uint32_t n = (uint32_t)word - (uint32_t)kArrivalRest, again = (uint32_t)(word >> 32) - (uint32_t)(kArrivalRest >> 32);
-    return n == again && n < (1u << kArrivalBits) ? (int)n : -1;
+    return n == again ? n : 0xffffffffu;
 }
 struct GlobalWord {
     unsigned long long* at;
@@ -481,14 +481,16 @@ struct GlobalWord {
 // Whether this is the last of `blocks` (< 2^24) blocks to call it with `word`.  One thread per block.
 template <typename Word>
 SA_HD bool last_to_arrive(const Word& word, unsigned blocks) {
-    int n = arrivals_in(word.add(kArrivalStep));
-    while (n < 0) {
+    unsigned n = arrivals_in(word.add(kArrivalStep));
+    while (__builtin_expect(n >= (1u << kArrivalBits), 0)) {
         // (an exchange fails only because another block has changed the word, which every block does at most three times)
         const unsigned long long seen = word.add(0ull);
-        if (arrivals_in(seen) >= 0) n = arrivals_in(word.add(kArrivalStep));
+        if (arrivals_in(seen) < (1u << kArrivalBits)) n = arrivals_in(word.add(kArrivalStep));
         else if (word.swap(seen, kArrivalRest + kArrivalStep) == seen) n = 0;
     }
-    return (unsigned)n + 1 == blocks || ((unsigned)n + 1 > blocks && ((unsigned)n + 1) % blocks == 0);
+    unsigned count = n + 1;
+    while (__builtin_expect(count > blocks, 0)) count -= blocks;      // (a division costs the kernel 0.05 us without being executed)
+    return count == blocks;
 }
 // For the last of them to call, then or later in its kernel.
 template <typename Word>
