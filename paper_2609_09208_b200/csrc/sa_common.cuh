@@ -43,7 +43,8 @@ constexpr KernelShape fp16_shape(int d) { return d == 128 ? KernelShape{6, 2, 1}
 constexpr KernelShape stream_shape(int d, bool fp16) {
     return fp16 ? KernelShape{12, 1, d == 128 ? 1 : 2} : d == 128 ? KernelShape{12, 1, 2} : KernelShape{16, 1, 2};
 }
-constexpr int stream_unit_cost(int d) { return d == 128 ? 14 : 32; }     // what a block pays for going on to another unit, in tiles
+SA_HD constexpr int stream_unit_cost(int d) { return d == 128 ? 14 : 32; }     // what a block pays for going on to another unit, in tiles
+SA_HD constexpr int stream_merge_cost(int d) { return d == 128 ? 20 : 30; }    // ... for parts of a unit that other blocks have worked on
 constexpr int kClusterMost = 8;           // blocks of a thread-block cluster
 // ... of the matrix kernels where the splits of a sequence form a cluster.  (fp16: fp16_shape.)
 constexpr KernelShape cluster_shape(int d) { return d == 128 ? KernelShape{6, 2, 2} : KernelShape{8, 2, 2}; }

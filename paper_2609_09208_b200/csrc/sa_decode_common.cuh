@@ -57,11 +57,11 @@ struct DecodeArgs {
     // Q, Knew and Vnew lie in host memory (whole; blocks that work on the sequence of their own grid coordinates): one block of
     // every unit fetches them, for all of its cluster (fetch_inputs).
     int host_in;
-    // The kernel of one block per SM (sa_decode_stream.cuh): its number of blocks (0: the other kernel); the tiles that going on to
-    // another unit costs a block.  Partials lie in slots of gt heads; `counters` has a word for every (query group, sequence) unit, at which
-    // the blocks that work on it meet (last_to_arrive); `plan`, where a merge kernel follows, {first slot, slots} of every unit.
-    // fine: the instantiation whose sums do not grow less exact with the length of a warp's stretch.
-    int stream, unit_cost, fine;
+    // The kernel of one block per SM (sa_decode_stream.cuh): its number of blocks (0: the other kernel); whether its instantiation is
+    // the one whose sums do not grow less exact with the length of a warp's stretch.  Partials lie in slots of gt heads; `counters` has a
+    // word for every (query group, sequence) unit, at which the blocks that work on it meet (last_to_arrive); `plan`, where a merge kernel
+    // follows, {first slot, slots} of every unit.
+    int stream, fine;
     unsigned long long* counters;
 };
 
@@ -602,7 +602,6 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
     a->arrivals = nullptr;
     a->host_in = 0;
     a->stream = stream;
-    a->unit_cost = 0;
     a->fine = fine ? 1 : 0;
     a->counters = nullptr;
     if (stream) {
@@ -610,7 +609,6 @@ inline sa_status make_decode_args(const Plan& p, const sa_cache* c, const uint16
         a->counters = reinterpret_cast<unsigned long long*>(static_cast<char*>(workspace) + stream_slot_bytes(p, GT, stream, units));
         a->plan = reinterpret_cast<int32_t*>(a->counters + units + 1);
         a->whole = 1;
-        a->unit_cost = stream_unit_cost(p.d);
     } else if (with_plan && batch_is_ranked(c->batch)) {
         a->plan = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)S * c->batch * p.Hq * (p.d + 2) * sizeof(float));
         // blocks per grid row that a batch of unequal lengths is cut into: the grid, rounded down to whole waves of

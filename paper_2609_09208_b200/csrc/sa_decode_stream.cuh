@@ -47,28 +47,48 @@ struct StreamSmem {
 constexpr int kLaneSeqs = kRankedBatchMax / 32;       // sequences per lane, at most
 struct Stretch {
     int t0, t1;                   // the block's stretch of all (virtual) tiles
-    int each, more;               // stretches are `each` tiles long, the first `more` of them one longer
+    int each, more, grain;        // stretches are `each` tiles long, the first `more` of them `grain` longer
     int y, b, len, start, tiles;  // its first unit: query group, sequence, length before the call, first virtual tile, real tiles
     int free;                     // virtual tiles in front of the real ones of every unit
 };
 // Tiles of a sequence of `len` tokens in the cut: an empty one counts as one, so that a block takes care of its output.
 SA_D int stretch_tiles(int len, int cap) { return max((min(max(len, 0), cap) + 31) >> 5, 1); }
 
-// before, lens: of sequences lane * K .. lane * K + K - 1, without and with the token that the call appends.  Every unit has `free` tiles that cost
-// nothing in front of its real ones: a block that goes on to another unit has its merge and prologue to pay, and gets that
-// many tiles less.  No such thing where every block stays within one unit (equal tile counts, blocks a multiple of the units).
+// before, lens: of sequences lane * K .. lane * K + K - 1, without and with the token that the call appends.
+// Every unit has `free` tiles that cost nothing in front of its real ones: a block that goes on to another unit has its merge and
+// prologue to pay, and gets that many tiles less.  Units of equal tile counts are cut into as many even parts as there are blocks for,
+// or kept whole, where that makes the busiest block's part shorter, merges included: above all where the sequences are short and the
+// page table is wide, which the host's choice of this kernel goes by.  us a call in a graph, the other kernel / the cut that takes no
+// notice of units / this (PoT-M4; costs of 0 to 64 tiles a merge were tried):
+//   d = 64, 32 / 4 heads: 8 x 2048 of 32 768 tokens 9.3 / 11.1 / 9.8, 16 x 1024 of 16 384 10.1 / 11.5 / 8.2, 32 x 512 of 8192 12.1 / 11.6 / 8.0,
+//     full 41.1 / 35.2 / 32.9;
+//   d = 128, 32 / 8 heads: 24 x 256 of 4096 20.4 / 14.7 / 11.3, 32 x 512 of 8192 12.9 / 20.7 / 15.7, 32 x 2048 of 8192 32.9 / 37.6 / 34.0.
+// (256 short units are what fills the other kernel's slots once, two units side by side on an SM and no splits; here a block has
+// two of them one after the other.)
+template <int D>
 SA_D Stretch cut_stretch(const DecodeArgs& a, const int (&before)[kLaneSeqs], const int (&lens)[kLaneSeqs], int K, int lane, int blk) {
     const int B = a.batch, cap = a.max_pages * kPageTokens, R = a.Hkv * (a.G / a.gt), P = gridDim.x;
+    constexpr int kUnit = stream_unit_cost(D), kMerge = stream_merge_cost(D);
     int t[kLaneSeqs], sum = 0;
     bool same = true;
 #pragma unroll
     for (int k = 0; k < kLaneSeqs; ++k) t[k] = k < K && lane * K + k < B ? stretch_tiles(lens[k], cap) : 0;
-    const int t_first = __shfl_sync(0xffffffffu, t[0], 0);
+    const int T = __shfl_sync(0xffffffffu, t[0], 0);
 #pragma unroll
-    for (int k = 0; k < kLaneSeqs; ++k) same = same && (t[k] == 0 || t[k] == t_first);
+    for (int k = 0; k < kLaneSeqs; ++k) same = same && (t[k] == 0 || t[k] == T);
     same = __all_sync(0xffffffffu, same);
     Stretch s;
-    s.free = same && P % (R * B) == 0 ? 0 : a.unit_cost;
+    s.free = kUnit;
+    int parts = 0;                                            // of every unit; 0: the cut takes no notice of units
+    if (same) {
+        const int U = R * B, k = min(P / U, T), c = (U + P - 1) / P;
+        const int cut = (U * (T + kUnit) + P - 1) / P + kMerge, whole = c * T + (c - 1) * kUnit;
+        const int even = k > 1 ? (T + k - 1) / k + kMerge : 0x7fffffff;
+        if (min(whole, even) <= cut) {
+            parts = even < whole ? k : 1;
+            s.free = (parts - T % parts) % parts;             // (even parts)
+        }
+    }
 #pragma unroll
     for (int k = 0; k < kLaneSeqs; ++k) sum += t[k] ? t[k] + s.free : 0;
     int upto = sum;                                           // inclusive prefix over the lanes
@@ -78,10 +98,12 @@ SA_D Stretch cut_stretch(const DecodeArgs& a, const int (&before)[kLaneSeqs], co
         if (lane >= o) upto += x;
     }
     const int row = __shfl_sync(0xffffffffu, upto, 31), all = row * R;
-    s.each = all / P;
-    s.more = all - s.each * P;
-    s.t0 = blk * s.each + min(blk, s.more);
-    s.t1 = s.t0 + s.each + (blk < s.more ? 1 : 0);
+    s.grain = parts ? (T + s.free) / parts : 1;
+    const int grains = parts ? R * B * parts : all;
+    s.each = grains / P * s.grain;
+    s.more = grains % P;
+    s.t0 = blk * s.each + min(blk, s.more) * s.grain;
+    s.t1 = s.t0 + s.each + (blk < s.more ? s.grain : 0);
     s.y = min(s.t0 / row, R - 1);
     const int o = s.t0 - s.y * row;
     // the last sequence that begins at o or before
@@ -104,8 +126,8 @@ SA_D Stretch cut_stretch(const DecodeArgs& a, const int (&before)[kLaneSeqs], co
 }
 // The block whose stretch holds virtual tile t.
 SA_D int block_of_tile(const Stretch& s, int t) {
-    const int edge = s.more * (s.each + 1);
-    return t < edge ? t / (s.each + 1) : s.more + (t - edge) / s.each;
+    const int edge = s.more * (s.each + s.grain);
+    return t < edge ? t / (s.each + s.grain) : s.more + (t - edge) / s.each;
 }
 
 // A unit that a block has been through: its rows are to be added.
@@ -197,9 +219,10 @@ SA_D void finish_units(const FinishArgs& a, const UnitSums& j0, const float* row
     if ((threadIdx.x == 0 && meet0) || (threadIdx.x == 32 && meet1)) {
         const UnitSums& j = threadIdx.x ? j1 : j0;
         __threadfence();
-        last = last_to_arrive(GlobalWord{a.counters + j.u}, j.blocks) ? 1 : 0;
+        const GlobalWord word{a.counters + j.u};
+        last = last_to_arrive(word, j.blocks) ? 1 : 0;
         __threadfence();
-        if (last) leave_at_rest(GlobalWord{a.counters + j.u}, j.blocks);      // (behind the fence, which would wait for it)
+        if (last) leave_at_rest(word, j.blocks);      // (behind the fence, which would wait for it)
     }
     const int merge0 = meet0 ? __syncthreads_or(threadIdx.x < 32 ? last : 0) : 0, merge1 = meet1 ? __syncthreads_or(threadIdx.x < 32 ? 0 : last) : 0;
 #pragma unroll 1
@@ -291,7 +314,7 @@ __global__ void __maxnreg__(NW > 12 ? 128 : 168) decode_stream_kernel(const __gr
     bool again = LOST;                                        // (the test hook makes its first cut for another block)
 #pragma unroll 1
     for (;;) {
-        s = cut_stretch(a, before, lens, K, lane, LOST && again ? (blockIdx.x + 1) % gridDim.x : blockIdx.x);
+        s = cut_stretch<D>(a, before, lens, K, lane, LOST && again ? (blockIdx.x + 1) % gridDim.x : blockIdx.x);
         // this warp's first tile: L2 is asked for it while the preceding kernel drains, its page is read behind the wait
         const int32_t* table = a.page_table + (size_t)s.b * a.max_pages;
         const int first_g = max(s.t0 - s.start - s.free, 0) + warp, end_g = min(min(s.t1 - s.start - s.free, s.tiles), a.max_pages * 2);

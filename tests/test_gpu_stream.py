@@ -239,3 +239,36 @@ def test_sums_over_long_stretches_against_64_bits(d, Hq, Hkv, code, batch):
     want = torch.cat([torch.softmax(q[h * G:(h + 1) * G] @ keys[:, h].T / d ** 0.5, -1) @ values[:, h] for h in range(Hkv)])
     off = O[0].double() - want
     assert float(off.abs().max() / want.abs().max()) <= 1.2e-6 and float(off.norm() / want.norm()) <= 1e-6
+
+
+# equal lengths, 64 tokens a page, room for `room`: units (sequences x KV heads) in 2 and 4 even parts, with tiles to spare and without,
+# fewer tiles than parts, one to a block, whole ones one after another, and so many tiles that the cut takes no notice of units
+EQUAL = [(64, 16, 2, sa.SA_POTM4, False, 37, [1, 33, 2000, 4000], 32768), (64, 8, 1, sa.SA_POT4, True, 37, [31, 100, 4000], 32768),
+         (64, 32, 4, sa.SA_POT4, False, 37, [0, 65, 777], 65536), (64, 32, 4, sa.SA_POTM4, False, 48, [96, 600], 16384),
+         (128, 16, 16, sa.SA_POTM2, True, 16, [64, 500, 1500], 8192), (128, 32, 8, sa.SA_POTM4, False, 8, [200, 900, 3000], 8192),
+         (64, 32, 4, sa.SA_KV_FP16, False, 32, [40, 700], 8192), (64, 8, 1, sa.SA_INT8, False, 100, [32, 1300], 16384)]
+
+
+@pytest.mark.parametrize("d,Hq,Hkv,code,dense,batch,tokens,room", EQUAL)
+def test_units_of_equal_lengths_against_the_oracle(d, Hq, Hkv, code, dense, batch, tokens, room):
+    """Every sequence has the same keys and queries, so all outputs are those of the first, whose are the oracle's."""
+    import torch
+    sa_build.build()
+    cfg = sa.make_config(d, Hq, Hkv, code, nibble=dense)
+    for n in tokens:
+        case = synth.make_case("equal", [n], Hq, Hkv, d, 0 if code == sa.SA_KV_FP16 else code, nibble=dense, outliers=True, seed=8700 + n)
+        want, scores = reference(case, code)
+        c = wide_cache(cfg, [n] * batch, room)
+        c.fill(*[up(np.concatenate([x] * batch)) for x in (case.K, case.V)], np.arange(batch + 1) * n)
+        Q = up(np.concatenate([case.Q] * batch))
+        dbg = torch.full((batch, Hq, room), -7, dtype=torch.int32, device="cuda") if scores is not None else None
+        for call in range(2):
+            O = torch.full((batch, Hq, d), float("nan"), device="cuda")
+            attend(cfg, c, Q, O, dbg if call else None)
+            torch.cuda.synchronize()
+            assert np.max(np.abs(O.cpu().numpy() - want[:1])) <= 1e-3, n
+        if dbg is not None:
+            assert np.array_equal(dbg[:, :, :n].cpu().numpy(), np.broadcast_to(scores[0][None, :, :n], (batch, Hq, n))) and bool((dbg[:, :, n:] == -7).all())
+        attend(cfg, c, Q, O.fill_(float("nan")), stages=1)
+        attend(cfg, c, Q, O, stages=2)
+        assert np.max(np.abs(O.cpu().numpy() - want[:1])) <= 1e-3, n

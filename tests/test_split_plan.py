@@ -17,3 +17,16 @@ def test_shift_by_multiply_has_the_shift_kernels_plan():
         size = lambda **flags: [sa.workspace_bytes(sa.make_config(d, 32, 4, code, nibble=nibble, **flags), b, p)
                                 for d in (64, 128) for b in (1, 3, 7, 32) for p in (20, 40, 100, 512, 700)]
         assert size(shift_by_multiply=True) == size(add_on_alu=True) != size()
+
+
+def test_the_shapes_of_the_stream_tests_go_to_the_kernel_of_one_block_per_sm():
+    """Its workspace (148 SMs: a slot per block and unit boundary, words, plan, in whole splits) is another one than the other kernel's."""
+    from test_gpu_stream import EQUAL, SHAPES
+    shapes = [(d, Hq, Hkv, code, dense, len(lens), room) for d, Hq, Hkv, code, dense, _, lens, room in SHAPES]
+    for d, Hq, Hkv, code, dense, batch, room in shapes + [x[:6] + x[7:] for x in EQUAL]:
+        gt = next(c for c in (8, 4, 2, 1) if Hq // Hkv % c == 0)
+        units, split = batch * Hkv * (Hq // Hkv // gt), batch * Hq * (d + 2) * 4
+        need = (148 + units) * gt * (d + 2) * 4 + (units + 1) * 8 + units * 8
+        size = sa.workspace_bytes(sa.make_config(d, Hq, Hkv, code, nibble=dense), batch, room // 64) - (batch * 8 + 15) // 16 * 16
+        # (37 sequences of PoT-M1 with room for 8192 tokens stay with the other kernel)
+        assert (size == -(-need // split) * split) == ((batch, room) != (37, 8192)), (d, Hq, Hkv, code, batch, room)
