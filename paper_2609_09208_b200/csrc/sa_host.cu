@@ -131,6 +131,10 @@ static bool stream_pays(const Plan& p, int batch, long long units, long long til
     if (units * (tiles + stream_unit_cost(p.d)) >= (1LL << 30)) return false;       // (the kernel counts all tiles in 32 bits)
     const double rounds = (double)units * (double)tiles / ((double)sms * stream_shape(p.d, p.fp16).warps), u = (double)units / sms;
     if (rounds < (p.d == 128 && !p.fp16 ? 4.5 : 9.0)) return false;
+    // binary16 tiles come at the copy rate in either kernel: nothing to gain on units that fill the other one's slots, once and unsplit
+    // (d = 64, 64 x 4096 tokens 43.5 -> 45.3 us, 64 x 8192 83.5 -> 86.5; 64 x 1024 of 8192 11.5 -> 14.0)
+    const long long slots = (long long)sms * p.shape.blocks_per_sm;
+    if (p.fp16 && S == 1 && units <= slots && 5 * units >= 4 * slots) return false;
     // both in rounds of the other kernel, fitted to the same measurements
     if (p.d == 64) return 0.97 * rounds + 3.0 * u + 5.6 <= cost + (S > 1 ? 2.2 : 0.0) + 1.5;
     return 0.88 * rounds + 2.2 * u + 2.9 <= cost + (S > 1 ? 3.3 : 0.0) - 2.4;

@@ -30,3 +30,10 @@ def test_the_shapes_of_the_stream_tests_go_to_the_kernel_of_one_block_per_sm():
         size = sa.workspace_bytes(sa.make_config(d, Hq, Hkv, code, nibble=dense), batch, room // 64) - (batch * 8 + 15) // 16 * 16
         # (37 sequences of PoT-M1 with room for 8192 tokens stay with the other kernel)
         assert (size == -(-need // split) * split) == ((batch, room) != (37, 8192)), (d, Hq, Hkv, code, batch, room)
+
+
+def test_binary16_units_that_fill_the_machine_once_stay_unsplit():
+    """64 sequences of 4 KV heads, 256 units on 296 slots: one split and no workspace of the kernel of one block per SM."""
+    cfg = sa.make_config(64, 32, 4, sa.SA_KV_FP16)
+    for tokens in (4096, 8192):
+        assert sa.workspace_bytes(cfg, 64, tokens // 64) == 64 * 32 * 66 * 4 + 64 * 8
