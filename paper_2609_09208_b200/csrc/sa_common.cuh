@@ -45,6 +45,13 @@ constexpr KernelShape stream_shape(int d, bool fp16) {
 }
 SA_HD constexpr int stream_unit_cost(int d) { return d == 128 ? 14 : 32; }     // what a block pays for going on to another unit, in tiles
 SA_HD constexpr int stream_merge_cost(int d) { return d == 128 ? 20 : 30; }    // ... for parts of a unit that other blocks have worked on
+// U units of T tiles each on P blocks: parts that every unit is cut into (1: units stay whole), where the busiest block, merges
+// included, is then done sooner than with a cut that takes no notice of units (0).
+SA_HD int stream_parts(int T, int U, int P, int d) {
+    const int unit = stream_unit_cost(d), merge = stream_merge_cost(d), k = P / U < T ? P / U : T, c = (U + P - 1) / P;
+    const int cut = (U * (T + unit) + P - 1) / P + merge, whole = c * T + (c - 1) * unit, even = k > 1 ? (T + k - 1) / k + merge : 0x7fffffff;
+    return (whole < even ? whole : even) > cut ? 0 : even < whole ? k : 1;
+}
 constexpr int kClusterMost = 8;           // blocks of a thread-block cluster
 // ... of the matrix kernels where the splits of a sequence form a cluster.  (fp16: fp16_shape.)
 constexpr KernelShape cluster_shape(int d) { return d == 128 ? KernelShape{6, 2, 2} : KernelShape{8, 2, 2}; }

@@ -68,7 +68,6 @@ SA_D int stretch_tiles(int len, int cap) { return max((min(max(len, 0), cap) + 3
 template <int D>
 SA_D Stretch cut_stretch(const DecodeArgs& a, const int (&before)[kLaneSeqs], const int (&lens)[kLaneSeqs], int K, int lane, int blk) {
     const int B = a.batch, cap = a.max_pages * kPageTokens, R = a.Hkv * (a.G / a.gt), P = gridDim.x;
-    constexpr int kUnit = stream_unit_cost(D), kMerge = stream_merge_cost(D);
     int t[kLaneSeqs], sum = 0;
     bool same = true;
 #pragma unroll
@@ -78,17 +77,8 @@ SA_D Stretch cut_stretch(const DecodeArgs& a, const int (&before)[kLaneSeqs], co
     for (int k = 0; k < kLaneSeqs; ++k) same = same && (t[k] == 0 || t[k] == T);
     same = __all_sync(0xffffffffu, same);
     Stretch s;
-    s.free = kUnit;
-    int parts = 0;                                            // of every unit; 0: the cut takes no notice of units
-    if (same) {
-        const int U = R * B, k = min(P / U, T), c = (U + P - 1) / P;
-        const int cut = (U * (T + kUnit) + P - 1) / P + kMerge, whole = c * T + (c - 1) * kUnit;
-        const int even = k > 1 ? (T + k - 1) / k + kMerge : 0x7fffffff;
-        if (min(whole, even) <= cut) {
-            parts = even < whole ? k : 1;
-            s.free = (parts - T % parts) % parts;             // (even parts)
-        }
-    }
+    const int parts = same ? stream_parts(T, R * B, P, D) : 0;
+    s.free = parts ? (parts - T % parts) % parts : stream_unit_cost(D);            // (even parts)
 #pragma unroll
     for (int k = 0; k < kLaneSeqs; ++k) sum += t[k] ? t[k] + s.free : 0;
     int upto = sum;                                           // inclusive prefix over the lanes

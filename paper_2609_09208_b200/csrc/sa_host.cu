@@ -141,15 +141,18 @@ static bool stream_pays(const Plan& p, int batch, long long units, long long til
 }
 
 // Whether the kernel of one block per SM adds every tile's sums on their own (FINE, sa_tile_mma.cuh): where a full cache has more
-// tiles for a warp in one unit than the other kernel, with S splits, would have, or more than 16.  So its outputs are no further off
-// than the other kernel's, and the error of the sums stays below that of 64 products.  Root mean square error against 64 bits
-// with values of mean 0 / 1, other kernel -> this one without -> with FINE (without where nothing else is said):
-//   PoT-M4, d = 64, 32 x 32 768 tokens 9.6e-7 / 1.2e-6 -> 2.5e-6 / 3.6e-6 -> 2.2e-7 / 1.1e-7; d = 128, 8 x 32 768
-//   9.1e-7 / 2.4e-6 -> 1.6e-6 / 4.2e-6 -> 3.2e-7 / 1.6e-7; PoT-4, 8 x 32 768 (14 tiles) 8.9e-7 / 1.8e-6 -> 7.3e-7 / 1.7e-6.
-static bool stream_is_fine(const Plan& p, long long units, long long tiles, int S, int sms) {
+// than 15 tiles for a warp in one unit.  Root mean square error against 64 bits with values of mean 0 / 1, the other kernel / this one
+// without FINE / with it where the rule takes it:
+//   up to 15 tiles: 20 x 4096 tokens, d = 128, 5.4e-7 / 5.6e-7 (8.7e-7 / 9.3e-7 with mean 1), 24 x 4096 PoT-M1 planar 5.5e-7 / 6.4e-7 (9.4e-7 /
+//     1.1e-6), 13 x 8192 9.1e-7 / 8.9e-7 (1.3e-6 / 1.4e-6), PoT-4, 8 x 32 768 8.9e-7 / 7.3e-7 (1.8e-6 / 1.7e-6);
+//   above: 40 x 8192, d = 64, 8.7e-7 / 9.4e-7 / 3.3e-7 (1.3e-6 / 1.6e-6 / 1.8e-7), 32 x 32 768 9.6e-7 / 2.5e-6 / 2.2e-7 (1.2e-6 / 3.6e-6 / 1.1e-7), 8 x 32 768, d = 128,
+//     9.1e-7 / 1.6e-6 / 3.2e-7 (2.4e-6 / 4.2e-6 / 1.6e-7).
+// (With the line at the other kernel's own number of tiles 20 x 4096 and 13 x 8192 tokens took 39.2 and 45.5 us instead of 36.6 and 43.2.)
+static bool stream_is_fine(const Plan& p, long long units, long long tiles, int sms) {
     if (p.fp16) return false;
-    const double nw = stream_shape(p.d, false).warps, chain = (double)tiles / nw * (units < sms ? (double)units / sms : 1.0);
-    return chain > 16.0 || chain > 1.05 * (double)tiles / ((double)p.shape.warps * S);
+    const int parts = stream_parts((int)tiles, (int)units, sms, p.d);
+    const double most = parts ? (double)tiles / parts : units < sms ? (double)tiles * (double)units / sms : (double)tiles;
+    return most > 15.0 * stream_shape(p.d, false).warps;
 }
 
 void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt, bool* cluster, int* stream, bool* fine) {
@@ -216,7 +219,7 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
         if (decode_workspace_bytes(p, batch, own) > (size_t)SA_STATIC_SCRATCH_BYTES && own > S) return;
         *stream = n_sms;
         *n_splits = own;
-        if (fine) *fine = stream_is_fine(p, units, tiles, S, n_sms);
+        if (fine) *fine = stream_is_fine(p, units, tiles, n_sms);
     };
     for (const Kept& k : kept)
         if (k.units == units && k.tiles == tiles && k.c_fix == c_fix && k.nw == nw && k.bps == bps && k.sms == n_sms) {
