@@ -141,7 +141,8 @@ sa_status sa_get_layout(const sa_config* cfg, sa_layout* out);
 
 /* Bytes of scratch that sa_decode_attention / sa_decode_attention_fp16 need for a cache with
  * `batch` sequences of at most `max_pages_per_seq` pages (split-K partial results, section II-F:
- * the kernel grid has a split dimension; for batches of 2 to 128 sequences also two words per sequence,
+ * the kernel grid has a split dimension, or, in large batches, blocks that leave a partial at every boundary of
+ * a sequence; for batches of 2 to 128 sequences also two words per sequence,
  * in which the decode kernel tells the merge kernel how it dealt the grid's blocks to the sequences: in
  * proportion to their cached lengths, so that a batch of unequal lengths keeps the machine as full as one
  * of equal lengths).  Host only; the one CUDA call it may make reads the number of
@@ -232,9 +233,9 @@ sa_status sa_decode_attention_fp16(const sa_config* cfg, const sa_cache* cache, 
  * The warp of the decode kernel that owns the new token's 32-key tile encodes and writes the token
  * before it stages that tile, so the separate append kernel and its launch disappear from the
  * step; seq_lens[b] is incremented after every block has read it: by the split-K merge kernel, or, where the
- * plan needs no merge kernel (a short single sequence, whose splits form a thread-block cluster, or one split per
- * sequence), by the last block of the decode kernel itself (the blocks are counted in the workspace, which such a
- * step needs for nothing else and which needs no initialisation for it).
+ * plan needs no merge kernel (short sequences, whose splits form a thread-block cluster; one split per sequence; large
+ * batches, in which the last block to work on a sequence merges its partials), by the last block of the decode kernel
+ * itself (the blocks are counted in the workspace, which needs no initialisation for it).
  * As with sa_append_kv the token's page must already be mapped; if it is not, the token is not
  * written, the length stays, and the step attends over the old cache.
  * With more than 8 query heads per KV head the call runs the two kernels separately.  A binary16
@@ -357,8 +358,9 @@ sa_status sa_debug_unpack(const sa_config* cfg, const sa_cache* cache, int b, in
  * (quantised or SA_KV_FP16) and copies O [batch, n_q_heads, head_dim] float to O_host.
  * Everything is asynchronous on `stream`; synchronise it before reading O_host.
  * If all four host buffers are pinned and device-addressable (cudaHostAlloc / cudaHostRegister
- * memory under unified addressing), no copy engine is used: a small kernel fetches the inputs
- * and the merge kernel stores O directly into host memory.  That kernel reads the three input buffers
+ * memory under unified addressing), no copy engine is used: a small kernel, or, in steps of one launch whose blocks
+ * know their sequence, the decode kernel itself, fetches the inputs (`staging` is not written then), and the kernel that
+ * ends the call stores O directly into host memory.  The three input buffers are read
  * without waiting for kernels enqueued earlier on `stream` (they are host inputs): their contents must
  * be in place when the call is enqueued (or the graph holding it is launched), written by the host or by
  * work that has completed, not produced by a kernel still pending on the same stream.  Otherwise the buffers are copied

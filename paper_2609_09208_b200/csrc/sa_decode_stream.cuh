@@ -1,8 +1,8 @@
 // The decode kernel for calls with work for every SM: one block per SM, which takes a contiguous stretch of the call's tiles.
 //
 // The tiles of all (query group, sequence) units follow one another, group by group, and are cut into gridDim.x stretches of
-// the same length, whatever the lengths of the sequences are; a block works through the units of its stretch one after
-// another.  A unit that lies within one block is finished there; of the others every block leaves a partial, and the last one
+// the same length, whatever the lengths of the sequences are (equal short units into even parts, or not at all: cut_stretch); a
+// block works through the units of its stretch one after another.  A unit that lies within one block is finished there; of the others every block leaves a partial, and the last one
 // to do so merges them: one launch.  Next to the kernel of sa_decode_mma.cuh, whose blocks each work on one unit, several of them to an SM:
 //   * no last wave and no idle SM, whatever the shape;
 //   * one prologue and one block merge per SM and unit boundary instead of one per block (about 925 warp instructions for

@@ -114,18 +114,19 @@ int sm_count() {
 }
 
 // Whether a call of this many units (query group, sequence), of at most `tiles` tiles each, goes to the kernel of one block
-// per SM (sa_decode_stream.cuh).  cost, S: the other kernel's by its cost model, and its splits.  Measured with both, in all
-// containers, on 119 shapes of 2 to 128 sequences; where the rule takes this kernel, calls of up to 1.35 times less time, and
-// one of 1.4 % more (INT8 keys, 24 x 8192 tokens).  us a call, the other kernel -> this one:
-//   PoT-M4, d = 64, 32 / 4 heads: 32 x 32 768 tokens 112.5 -> 98.4, 32 x 8192 38.7 -> 35.5, 16 x 16 384 35.8 -> 33.6, below the
-//     line 8 x 16 384 20.7 -> 21.4, 4 x 16 384 14.8 -> 15.8;
-//   PoT-M4, d = 128, 32 / 8 heads: 20 x 4096 tokens 48.6 -> 36.7, 13 x 8192 53.0 -> 43.1, 10 x 4000 25.0 -> 23.1, below the line
+// per SM (sa_decode_stream.cuh).  cost, S: the other kernel's by its cost model, and its splits.  The constants are a fit to times of both
+// kernels, in all containers, on 119 shapes of 2 to 128 sequences with full caches.  us a call of eight in a graph (SM clock 1965 MHz; in long
+// runs under the power cap 32 x 32 768 tokens take 129 and 116), the other kernel -> this one:
+//   PoT-M4, d = 64, 32 / 4 heads: 32 x 32 768 tokens 118.5 -> 100.3, 32 x 8192 41.0 -> 33.0, 16 x 16 384 38.2 -> 33.5; INT8 keys 32 x 32 768
+//     94.1 -> 88.4, 16 x 16 384 30.5 -> 30.4; below the line 8 x 16 384 20.7 -> 21.4, 4 x 16 384 14.8 -> 15.8;
+//   PoT-M4, d = 128, 32 / 8 heads: 20 x 4096 tokens 51.7 -> 36.5, 13 x 8192 55.9 -> 43.1, 10 x 4032 27.3 -> 22.7, below the line
 //     3 x 8192 16.5 -> 16.7.
+// (Below the line: with the cut that took no notice of units.)  Sequences that fill a part of the page table: see cut_stretch.
 // Not taken: less than 9 rounds of tiles (4.5 at d = 128, where a round takes longer), over which a block's prologue and end
 // (10 us, of which the other kernel hides a part behind the second block of an SM) have to be earned; less than 16 units, whose
 // partials one block after the other has to wait for and merge (one sequence of 131 072 tokens: 18.4 -> 27.7); and many short
 // units, of which every one after a block's first costs it 5 us, where the other kernel's grid happens to fill the machine
-// (32 x 4096 tokens, d = 128: 256 blocks on 296 slots, 52.6 -> 56.3).
+// (32 x 4096 tokens, d = 128: 256 blocks on 296 slots, 51.2 us, 56.3 in this kernel when that took 52.6).
 static bool stream_pays(const Plan& p, int batch, long long units, long long tiles, double cost, int S, int sms) {
     if (!p.matrix || batch < 2 || batch > kRankedBatchMax || units < 16) return false;
     if (units * (tiles + stream_unit_cost(p.d)) >= (1LL << 30)) return false;       // (the kernel counts all tiles in 32 bits)
@@ -169,8 +170,9 @@ void split_plan(const Plan& p, int batch, int max_pages, int* n_splits, int* gt,
     //   * blocks run in waves of (SMs of the current device) x resident-blocks-per-SM; a last wave whose SMs hold only the
     //     fraction f of that takes 0.1 + 0.9 f of a full wave's time, a single partial wave f^0.2
     //     (an SM's throughput falls almost in proportion to its resident warps).  f is taken from the SM with the most blocks,
-    //     so 256 blocks on 296 slots count as a full wave, which they are not: PoT-M4, 32 sequences, gets 2 splits at 513 to
-    //     520 pages (122.6 us) and 8 at 512 and at 530 (116.0 us; 8 splits at 513 to 520 pages take 116.0 us as well).
+    //     so 256 blocks on 296 slots count as a full wave, which they are not: PoT-M4, 32 sequences, got 2 splits at 513 to
+    //     520 pages (122.6 us) and 8 at 512 and at 530 (116.0 us; 8 splits at 513 to 520 pages took 116.0 us as well), before such
+    //     calls went to the kernel of one block per SM.
     // The sequence lengths live on the device, so the model uses the cache's capacity.
     const long long units = (long long)batch * p.Hkv * (p.G / GT);
     const int bps = p.shape.blocks_per_sm, nw = p.shape.warps;

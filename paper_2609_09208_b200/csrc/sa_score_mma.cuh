@@ -18,10 +18,10 @@
 //   binary16 keys             as stored, with the binary16 query; the sums are rounded like any FP32 sum.
 // So the INT32 scores are those of the shift-and-add datapath (sa_datapath.cuh) bit for bit.  The decode is what a tile
 // costs most: 7 instructions for four codes by way of FP8, 8 for PoT-M4 (11 as binary16).  The pipe of logic, shifts and
-// permutes, which issues every other clock, was 63 % busy in a call of 32 x 32 768 PoT-M4 tokens, the pipe of multiply-adds
-// 22 %, so shifts to the left are multiplications by a constant that the compiler cannot see (`one`, the value 1, is a kernel
-// argument).  With packed FP32 in the softmax (sa_decode_mma.cuh) that call went from 128 to 123.3 us, 32 x 4096 tokens of
-// head_dim 128 from 59.7 to 56.6.  Shifts to the right as the upper half of a product were slower (126.6), FP8 operands of
+// permutes, which issues every other clock, is the fullest, the pipe of multiply-adds has room (62 and 20 % in a call of 32 x 32 768
+// PoT-M4 tokens before; 63 and 19 now, with a fifth less time), so shifts to the left are multiplications by a constant that the
+// compiler cannot see (`one`, the value 1, is a kernel argument).  With packed FP32 in the softmax (sa_tile_mma.cuh) that call of
+// decode_mma_kernel, in a long run under the power cap, went from 128 to 123.3 us, 32 x 4096 tokens of head_dim 128 from 59.7 to 56.6.  Shifts to the right as the upper half of a product were slower (126.6), FP8 operands of
 // the product itself, which are exact too, far slower (116 -> 147).
 //
 // Fragments: lane (r, c) = (lane / 4, lane % 4) holds the c-th 32-bit word of a 16-byte code chunk of keys r, r + 8,

@@ -38,8 +38,9 @@ using MmaStage = TileStage<ScoreMma<D, FMT>::CH, FMT != FMT_FP16, FMT == FMT_FP1
 // FINE: the products of a tile are summed from zero and then added to the sums of the tiles before, rounded to nearest.  The
 // matrix unit cuts its sums off, an error that grows with the number of products in one accumulator: 32 x 32 768 PoT-M4
 // tokens, 55 tiles a warp, outputs 2.0e-6 too small (3.4e-6 with values of mean 1), with FINE 7e-8.  The
-// additions cost 2 % at head_dim 64 (that call 98.5 -> 100.3 us, in a graph) and 1.5 - 4 % at 128 (8 x 32 768 tokens, PoT-M4 88.8 -> 89.9, PoT-M1
-// planar 86.7 -> 89.5), so warps with few tiles do without (see stream_is_fine).
+// additions cost 2 % at head_dim 64 (that call 98.3 -> 100.3 us, in a graph) and 1.5 - 7 % at 128, most where stretches are short
+// (8 x 32 768 tokens, PoT-M4 88.8 -> 89.9, PoT-M1 planar 86.7 -> 89.5; 20 x 4096 36.6 -> 39.2), so warps with few tiles do without (see
+// stream_is_fine).  (Sums put aside in tensor memory every 4 or 8 tiles instead: 1.2e-6 and 6 % at 4 tiles, a larger error at 8.)
 template <int D, int FMT, bool LONG, bool FINE>
 struct TileMma {
     using SC = ScoreMma<D, FMT>;
