@@ -202,7 +202,7 @@ sa_status sa_fill_kv(const sa_config* cfg, const sa_cache* cache, const uint16_t
  *   The A.V products run on the tensor cores with FP32 accumulation: the INT8 values are exact in binary16,
  *   and every weight enters as the sum of two binary16 terms (22 significant bits down to 2^-17 of the
  *   largest weight, an absolute 2^-38 of it below that).  Against 64 bits, root mean square relative to the outputs:
- *   3e-7 to 1.4e-6 over 1 to 32 sequences of 4096 to 131 072 tokens with values of mean 0, 1e-7 to 2.8e-6 with values of
+ *   2e-7 to 1.4e-6 over 1 to 32 sequences of 4096 to 131 072 tokens with values of mean 0, 1e-7 to 2.8e-6 with values of
  *   mean 1, which the matrix unit, cutting its sums off, makes too small.
  * Q [batch, n_q_heads, head_dim] binary16; O [batch, n_q_heads, head_dim] float.
  * A sequence with seq_lens[b] == 0 yields zeros.
